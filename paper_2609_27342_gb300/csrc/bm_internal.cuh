@@ -24,6 +24,21 @@
 #define BM_HIST 16           // pair-contact history entries per particle
 #define BM_NBR 64            // pair-contact candidates kept per particle (Verlet list)
 #define BM_WRENCH_W 6
+#define BM_BRICK_CODES 64    // distinct codes kept per brick (more raise the slot-overflow flag)
+#define BM_LAT_POS 512       // particle places of a lattice brick: 8 planes per axis
+
+// Place of lattice particle (x, y, z) of a brick (plane indices 0..7, two per
+// base cell) in the shared-memory arrays of the lattice kernels, and the XOR
+// of its 16-byte chunks.  The low bit and the XOR mix cell bits with plane
+// bits, so that both the 8 particles of one cell (stored together) and one
+// particle of 8 neighbouring cells (read together) fall on all 8 groups of
+// banks.
+__host__ __device__ inline int bm_lat_place(int x, int y, int z) {
+  return z * 64 + y * 8 + (x & 4) + ((x & 1) << 1) + ((x ^ (x >> 1)) & 1);
+}
+__host__ __device__ inline int bm_lat_xor(int place) {
+  return (((place >> 2) ^ (place >> 3)) & 1) | ((((place >> 4) ^ (place >> 6)) & 1) << 1);
+}
 
 struct DevSeg {
   int n_steps, cut_id;
@@ -97,7 +112,7 @@ struct DevScene {
   int label_pending;
   int need_rebuild;
   int n_slots;
-  int pad_[1];
+  int lattice;              // the lattice kernels (bm_lattice.cu) carry this scene's transfers
 };
 
 struct PPool {
@@ -112,6 +127,8 @@ struct PPool {
   float *J[3];              // pair-contact impulse of this substep (k_pair -> k_p2g_brick)
   uint8_t *pend;            // side digit assigned this substep (0: none), committed by k_fupd
   int *perm;                // pool index -> caller's particle index
+  uint16_t *lpos;           // lattice scenes: the particle's place in its brick (bm_lat_place)
+  uint8_t *cid;             // lattice scenes: index of the particle's code in its brick's list
   // pair contact
   int *hkey;                // bucket of each particle's current-configuration cell
   int *horder;              // particles ordered by bucket, by pool index inside a bucket
@@ -151,6 +168,11 @@ struct BPool {              // brick-tile partial sums
   int *ptot;                // slots in each brick's tile
   int *tdesc;               // [brick * BM_TILE_NODES]: first tile slot | slot count << 16
   int *tgoff;               // [brick * BM_TILE_NODES]: first pool slot of each tile node
+  // lattice scenes
+  float *lf;                // [brick * 24]: fractional offset of the 8 particle planes per axis
+  uint2 *bcode;             // [brick * BM_BRICK_CODES]: distinct codes of the brick's particles
+  int *binfo;               // number of those codes | 1 << 8 when no tile node holds several slots
+  uint8_t *bdirty;          // a particle of the brick gained a label since its codes were listed
 };
 
 struct HashPool {           // pair-contact spatial hash (world-wide table)
@@ -186,6 +208,7 @@ struct LaunchSet {
   int n_scenes;
   int any_pair;             // some scene has pair contact
   int any_inelastic;        // some scene has plasticity or viscosity
+  int any_lattice, any_general;  // some scene takes the lattice kernels; some the general ones
   int pair_n_particles;     // particles of pair-contact scenes (hash sizing)
 };
 
@@ -225,6 +248,12 @@ cudaError_t bm_launch_surface_embed(const World &w, const SurfParams &sp, int n_
 #define BM_NUM_VARIANTS 27  // 3 occupancy choices for each of the 3 brick kernels
 extern const char *const bm_kernel_names[BM_NUM_KERNELS];
 cudaError_t bm_kernels_init();  // per device: shared-memory limits of the brick kernels
+
+// lattice brick kernels (bm_lattice.cu)
+cudaError_t bm_lattice_init();
+void bm_launch_p2g_lat(const World &w, const LaunchSet &ls, cudaStream_t st);
+void bm_launch_g2p_lat(const World &w, const LaunchSet &ls, cudaStream_t st);
+void bm_launch_fupd_lat(const World &w, const LaunchSet &ls, cudaStream_t st);
 
 // adjoint of the substep (bm_adjoint.cu); the work record is opaque here
 size_t bm_adj_work_struct_size();

@@ -121,6 +121,9 @@ struct bm_scene_s {
   std::vector<float> h_fx[3];
   std::vector<uint32_t> h_base;
   std::vector<int> h_perm;
+  bool lattice = false;               // particles on planes of at most two per base cell and axis
+  std::vector<float> h_lf;            // lattice: 24 plane offsets per brick (BPool::lf)
+  std::vector<uint16_t> h_lpos;       // lattice: place of every particle in its brick, pool order
   bool fresh = true;
   cudaStream_t home_stream = nullptr;  // stream and allocator given at creation
   bm_alloc home_alloc{};
@@ -220,6 +223,9 @@ int world_alloc(WorldH *W) {
   U(pp.s1, P);
   U(pp.s2, P);
   I(pp.perm, P);
+  pp.lpos = W->get<uint16_t>(P);
+  pp.cid = W->get<uint8_t>(P);
+  ok &= pp.lpos && pp.cid;
   pp.pend = W->get<uint8_t>(P);
   ok &= pp.pend != nullptr;
   if (W->pair) {
@@ -271,7 +277,11 @@ int world_alloc(WorldH *W) {
   bp.ptot = W->get<int>(W->cap_brick);
   bp.tdesc = W->get<int>(W->cap_brick * BM_TILE_NODES);
   bp.tgoff = W->get<int>(W->cap_brick * BM_TILE_NODES);
-  ok &= bp.pm && bp.pd && bp.poff && bp.ptot && bp.tdesc && bp.tgoff;
+  bp.lf = W->get<float>(W->cap_brick * 24);
+  bp.bcode = W->get<uint2>(W->cap_brick * BM_BRICK_CODES);
+  bp.binfo = W->get<int>(W->cap_brick);
+  bp.bdirty = W->get<uint8_t>(W->cap_brick);
+  ok &= bp.pm && bp.pd && bp.poff && bp.ptot && bp.tdesc && bp.tgoff && bp.lf && bp.bcode && bp.binfo && bp.bdirty;
   W->w.scenes = W->get<DevScene>(W->cap_scenes);
   W->w.wpart = W->get<double>(W->cap_brick * 6);
   W->w.whist = W->get<double>(std::max<int64_t>(W->cap_hist, 1) * 6);
@@ -359,6 +369,8 @@ LaunchSet scene_set(const WorldH *W, const bm_scene_s *s) {
   ls.n_scenes = 1;
   ls.any_pair = s->desc.pair_contact;
   ls.any_inelastic = s->desc.yield_stress > 0 || s->desc.viscosity > 0;
+  ls.any_lattice = s->lattice;
+  ls.any_general = !s->lattice;
   return ls;
 }
 
@@ -375,7 +387,9 @@ LaunchSet world_set(const WorldH *W) {
   for (auto *s : W->members) {
     ls.any_pair |= s->desc.pair_contact;
     ls.any_inelastic |= s->desc.yield_stress > 0 || s->desc.viscosity > 0;
-    ls.ppc16 |= s->ppc_max > 8;
+    ls.ppc16 |= !s->lattice && s->ppc_max > 8;
+    ls.any_lattice |= s->lattice;
+    ls.any_general |= !s->lattice;
   }
   return ls;
 }
@@ -389,6 +403,7 @@ void fill_template(bm_scene_s *s) {
   t.nn[0] = s->nn[0]; t.nn[1] = s->nn[1]; t.nn[2] = s->nn[2];
   t.nbr[0] = s->nbr[0]; t.nbr[1] = s->nbr[1]; t.nbr[2] = s->nbr[2];
   t.n_brick = (int)s->n_brick;
+  t.lattice = s->lattice;
   t.n_p = (int)s->n;
   t.n_node = (int)s->n_node;
   t.n_cell = (int)s->n_cell;
@@ -584,6 +599,11 @@ int place_fresh(WorldH *W, bm_scene_s *s) {
   CK(cudaMemsetAsync(P.s2 + pb, 0, sizeof(uint32_t) * n, st));
   CK(cudaMemcpyAsync(P.base + pb, s->h_base.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(P.perm + pb, s->h_perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
+  if (s->lattice) {
+    CK(cudaMemcpyAsync(P.lpos + pb, s->h_lpos.data(), sizeof(uint16_t) * n, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(W->w.B.lf + s->brick_begin * 24, s->h_lf.data(), sizeof(float) * s->h_lf.size(),
+                       cudaMemcpyHostToDevice, st));
+  }
   if (W->pair) {
     for (int b = 0; b < 2; ++b)
       CK(cudaMemsetAsync(P.hist_partner[b] + pb * BM_HIST, 0xff, sizeof(int) * n * BM_HIST, st));
@@ -600,6 +620,8 @@ int place_fresh(WorldH *W, bm_scene_s *s) {
   s->fresh = false;
   s->h_fx[0].clear(); s->h_fx[1].clear(); s->h_fx[2].clear();
   s->h_base.clear();
+  s->h_lpos.clear();
+  s->h_lf.clear();
   return BM_OK;
 }
 
@@ -662,6 +684,10 @@ int move_scene(bm_scene_s *s, WorldH *W) {
   CK(cp(B.s1 + pd, A.s1 + ps, sizeof(uint32_t) * n));
   CK(cp(B.s2 + pd, A.s2 + ps, sizeof(uint32_t) * n));
   CK(cp(B.perm + pd, A.perm + ps, sizeof(int) * n));
+  if (s->lattice) {
+    CK(cp(B.lpos + pd, A.lpos + ps, sizeof(uint16_t) * n));
+    CK(cp(W->w.B.lf + s->brick_begin * 24, S->w.B.lf + old.brick_begin * 24, sizeof(float) * 24 * s->n_brick));
+  }
   CK(cudaMemsetAsync(B.pend + pd, 0, n, st));
   for (int a = 0; a < 3; ++a) CK(cudaMemsetAsync(B.J[a] + pd, 0, sizeof(float) * n, st));
   if (W->pair) {
@@ -760,6 +786,62 @@ int validate_desc(const bm_scene_desc *d) {
   return BM_OK;
 }
 
+// Whether the lattice kernels can carry the scene: along each axis the
+// particles of a base-cell layer lie on at most two planes (one float32
+// fractional offset each), and the caller lists a cell's particles in
+// ascending (x, y, z) plane order, no two at one place (the order in which
+// both kernel forms sum them).  Then the places and the planes' offsets are
+// laid out per brick.  A lattice cell of more than 2 x 2 x 2 particles,
+// another order, or positions off the planes (a jittered or scanned body)
+// take the general kernels.
+void find_lattice(bm_scene_s *s, const std::vector<double> &f3, const std::vector<int> &b3, const int lo[3]) {
+  s->lattice = false;
+  if (s->ppc_max > 8) return;
+  const int64_t n = s->n;
+  std::vector<float> pl[3];  // per axis and base-cell layer: the planes' offsets, ascending (-1: none)
+  for (int a = 0; a < 3; ++a) {
+    pl[a].assign((size_t)s->nb[a] * 2, -1.0f);
+    for (int64_t i = 0; i < n; ++i) {
+      float *q = &pl[a][2 * (size_t)(b3[3 * i + a] - lo[a])];
+      const float f = (float)f3[3 * i + a];
+      if (f == q[0] || f == q[1]) continue;
+      if (q[1] >= 0.0f) return;  // a third plane
+      if (q[0] < 0.0f) q[0] = f;
+      else q[1] = f;
+    }
+    for (int c = 0; c < s->nb[a]; ++c)
+      if (pl[a][2 * c + 1] >= 0.0f && pl[a][2 * c + 1] < pl[a][2 * c]) std::swap(pl[a][2 * c], pl[a][2 * c + 1]);
+  }
+  s->h_lpos.resize((size_t)n);
+  int64_t last_cell = -1;
+  int last_key = -1;
+  for (int64_t j = 0; j < n; ++j) {
+    const int64_t i = s->h_perm[j];
+    int x[3], b[3];
+    for (int a = 0; a < 3; ++a) {
+      b[a] = b3[3 * i + a] - lo[a];
+      x[a] = 2 * (b[a] & 3) + ((float)f3[3 * i + a] != pl[a][2 * (size_t)b[a]]);
+    }
+    const int64_t cell = ((int64_t)b[2] * s->nb[1] + b[1]) * s->nb[0] + b[0];
+    const int key = ((x[0] & 1) * 2 + (x[1] & 1)) * 2 + (x[2] & 1);
+    if (cell == last_cell && key <= last_key) return;  // another order, or two particles at one place
+    last_cell = cell;
+    last_key = key;
+    s->h_lpos[(size_t)j] = (uint16_t)bm_lat_place(x[0], x[1], x[2]);
+  }
+  s->h_lf.assign((size_t)s->n_brick * 24, 1.0f);
+  for (int64_t br = 0; br < s->n_brick; ++br) {
+    const int64_t c[3] = {br % s->nbr[0], (br / s->nbr[0]) % s->nbr[1], br / ((int64_t)s->nbr[0] * s->nbr[1])};
+    for (int a = 0; a < 3; ++a)
+      for (int k = 0; k < 8; ++k) {
+        const int64_t cell = 4 * c[a] + (k >> 1);
+        if (cell < s->nb[a] && pl[a][2 * cell + (k & 1)] >= 0.0f)
+          s->h_lf[(size_t)br * 24 + a * 8 + k] = pl[a][2 * cell + (k & 1)];
+      }
+  }
+  s->lattice = true;
+}
+
 // stencil table: base cell, fractional offset, sort by base cell (Eq. 1)
 int build_layout(bm_scene_s *s) {
   const int64_t n = s->n;
@@ -816,6 +898,7 @@ int build_layout(bm_scene_s *s) {
              bz = (uint32_t)(b3[3 * i + 2] - lo[2]);
     s->h_base[j] = bx | (by << 10) | (bz << 20);
   }
+  find_lattice(s, f3, b3, lo);
   s->slot_cap = std::max<int64_t>(4 * s->n_node, 64);
   // brick-tile partial sums: a node appears in <= 8 tiles, ~3.4 on average;
   // 6 entries per node covers ~1.8 logical grids per node on average
@@ -1245,6 +1328,7 @@ int bm_checkpoint_restore(bm_scene_t s, const void *src, int src_on_device) {
   sv.slot_cap = cur.slot_cap;
   sv.label_pending = 0;
   sv.need_rebuild = 0;
+  sv.lattice = cur.lattice;  // decided by the scene's positions, not by the saved record
   sv.stop_at = cur.stop_at;  // the stop substep is a control of the caller's, not state
   sv.frozen = (sv.stop_at >= 0 && sv.step >= sv.stop_at) ? 1 : 0;
   CK(cudaMemcpy(W->w.scenes + s->slot, &sv, sizeof sv, cudaMemcpyHostToDevice));
@@ -1501,13 +1585,13 @@ int bm_scene_footprint(const bm_scene_desc *desc, const float *X_ref, int64_t n,
   if (nodes) *nodes = s.n_node;
   if (bricks) *bricks = s.n_brick;
   // fx, x, v, u_t, J (3 each); F, Fp^-1, dF/dt (9 each); D; base, masks, perm; pending label;
-  // the D / u_t flag;
+  // the D / u_t flag; lattice place and code index;
   // with pair contact: hash key, order, entries with their base cells and cell keys, the double-buffered history,
   // the candidate list and the positions at its build
-  const int64_t per_p = 4 * (3 * 5 + 9 * 3 + 1) + 4 * 4 + 1 + 1 +
+  const int64_t per_p = 4 * (3 * 5 + 9 * 3 + 1) + 4 * 4 + 1 + 1 + 2 + 1 +
                         (desc->pair_contact ? (4 + 4 + 16 + 4 + 16 + 2 * BM_HIST * 16 + 4 * BM_NBR + 1 + 12) : 0);
   const int64_t per_node = 4 + 1 + 8 * BM_MAXS + 4 * (3 * 16 + 8) + 6 * 32;
-  const int64_t per_brick = 3 * BM_TILE_NODES + 48 + 16 + 8;
+  const int64_t per_brick = 3 * BM_TILE_NODES + 48 + 16 + 8 + 4 * 24 + 8 * BM_BRICK_CODES + 4 + 1;
   if (bytes) *bytes = n * per_p + s.n_node * per_node + (s.n_cell + 1) * 4 + s.n_brick * per_brick + s.hist_cap * 48;
   return BM_OK;
 }
