@@ -429,20 +429,6 @@ __device__ __forceinline__ int side_label(const DevScene &sc, const float x[3], 
   return s < 0.0f ? 1 : 2;
 }
 
-// deterministic block sum of a double (fixed shuffle tree, warps in order)
-__device__ __forceinline__ double block_sum(double v, double *sm) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-  __syncthreads();
-  if (lane == 0) sm[wid] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < nw; ++i) t += sm[i];
-  return t;  // valid in thread 0
-}
-
 // exclusive block scan of one int per thread (fixed order); total in all threads
 __device__ __forceinline__ int block_excl_scan(int v, int *sm, int &total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -518,30 +504,6 @@ __device__ __forceinline__ void particle_base(uint32_t b, int &bx, int &by, int 
   bx = (int)(b & 1023u);
   by = (int)((b >> 10) & 1023u);
   bz = (int)((b >> 20) & 1023u);
-}
-
-// Eq. 8 on ns logical grids with masses m and states S[a][nc]
-template <int NC>
-__device__ __forceinline__ void couple(int ns, const uint2 *codes, const float *m, float (*S)[NC]) {
-  float M = 0.f;
-  for (int a = 0; a < ns; ++a) M += m[a];
-  if (!(M > 0.f)) return;
-  const float iM = 1.0f / M;
-  float out[BM_MAXS][NC];
-  for (int a = 0; a < ns; ++a) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      float acc = 0.f;
-      for (int b = 0; b < ns; ++b) {
-        if (b == a || conflict(codes[a].x, codes[a].y, codes[b].x, codes[b].y)) continue;
-        acc += m[a] * S[b][c] - m[b] * S[a][c];
-      }
-      out[a][c] = S[a][c] + acc * iM;
-    }
-  }
-  for (int a = 0; a < ns; ++a)
-#pragma unroll
-    for (int c = 0; c < NC; ++c) S[a][c] = out[a][c];
 }
 
 // The node tile of one brick: for each of its 6x6x6 nodes the first tile
