@@ -271,4 +271,7 @@ cudaError_t bm_launch_prepare(const World &w, const LaunchSet &ls, cudaStream_t 
 cudaError_t bm_launch_rebuild(const World &w, const LaunchSet &ls, cudaStream_t st, int force);
 cudaError_t bm_launch_io(const World &w, int scene_slot, int p_begin, int n, int field, void *buf,
                          int to_device_pool, cudaStream_t st);
+// the fields of `mask` (BM_FIELD_* but X and CODE) into device buffers buf[field], one launch
+cudaError_t bm_launch_read(const World &w, int scene_slot, int p_begin, int n, uint32_t mask, void *const *buf,
+                           cudaStream_t st);
 cudaError_t bm_launch_code(const World &w, int p_begin, int n, int64_t *out, cudaStream_t st);

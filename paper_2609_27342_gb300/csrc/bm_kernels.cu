@@ -2027,11 +2027,8 @@ __global__ void k_slot_fill(World w, LaunchSet ls, int force) {
 // --------------------------------------------------------------------------
 // state I/O between pool order and the caller's order
 // --------------------------------------------------------------------------
-__global__ void k_io(World w, int scene_slot, int p_begin, int n, int field, void *buf, int to_pool) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int p = p_begin + i;
-  const int o = w.P.perm[p];
+__device__ __forceinline__ void io_field(const World &w, int scene_slot, int p, int o, int field, void *buf,
+                                         int to_pool) {
   const PPool &P = w.P;
   float *fb = (float *)buf;
   uint32_t *ub = (uint32_t *)buf;
@@ -2097,6 +2094,26 @@ __global__ void k_io(World w, int scene_slot, int p_begin, int n, int field, voi
       break;
     }
   }
+}
+
+__global__ void k_io(World w, int scene_slot, int p_begin, int n, int field, void *buf, int to_pool) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int p = p_begin + i;
+  io_field(w, scene_slot, p, w.P.perm[p], field, buf, to_pool);
+}
+
+struct ReadSet {
+  void *buf[BM_NUM_FIELDS];
+  int field[BM_NUM_FIELDS];
+};
+
+// blockIdx.y: which of the requested fields
+__global__ void k_read(World w, int scene_slot, int p_begin, int n, ReadSet r) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int p = p_begin + i;
+  io_field(w, scene_slot, p, w.P.perm[p], r.field[blockIdx.y], r.buf[blockIdx.y], 0);
 }
 
 __global__ void k_code(World w, int p_begin, int n, int64_t *out) {
@@ -2355,6 +2372,20 @@ cudaError_t bm_launch_io(const World &w, int scene_slot, int p_begin, int n, int
                          int to_pool, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   k_io<<<(n + 255) / 256, 256, 0, st>>>(w, scene_slot, p_begin, n, field, buf, to_pool);
+  return cudaGetLastError();
+}
+
+cudaError_t bm_launch_read(const World &w, int scene_slot, int p_begin, int n, uint32_t mask, void *const *buf,
+                           cudaStream_t st) {
+  ReadSet r{};
+  int k = 0;
+  for (int f = 0; f < BM_NUM_FIELDS; ++f)
+    if (mask & (1u << f)) {
+      r.buf[k] = buf[f];
+      r.field[k++] = f;
+    }
+  if (n == 0 || k == 0) return cudaSuccess;
+  k_read<<<dim3((unsigned)(n + 255) / 256, (unsigned)k), 256, 0, st>>>(w, scene_slot, p_begin, n, r);
   return cudaGetLastError();
 }
 
