@@ -221,8 +221,6 @@ struct SurfParams {
   double Xmin[3], h[3];      // lattice point j sits at Xmin + j h
   double origin[3], dx;      // the scene's reference grid
   int lo[3];                 // absolute index of the scene's local base cell 0
-  int bmin[3], bmax[3];      // stencil base cells of the first and last lattice point per axis
-  const int *jstart[3];      // [B - bmin]: first lattice index whose base cell is >= B
   int *lat;                  // lattice point (x fastest) -> scene-relative pool index, -1 empty
   float *Xr[3];              // scene-relative reference positions
   int p_begin, slot;         // the scene's first pool particle and its record in the world
@@ -230,6 +228,11 @@ struct SurfParams {
   uint32_t *cell_reg;        // per cell: 4 bits per corner, vertex ordinal of its region (15: none)
   int *pt_cnt, *pt_off;      // per link lower end: triangles, first triangle (n_cells + 1)
   int *scan_tmp;             // block sums of the scans
+  int *totals;               // vertices, triangles
+  uint8_t *nmark;            // per scene-local grid node: some vertex's embedding reads it
+  float4 *nval;              // per scene-relative slot of a marked node: sum N, sum N (x - X)
+  int *vcell;                // per vertex: its lattice cell
+  uint8_t *vord;             // per vertex: its region's ordinal in the cell
   float *ref[3], *cur[3];    // vertex reference and current positions
   int *anchor;               // vertex anchor particle (scene-relative)
   uint32_t *vmask[2];        // vertex code
@@ -237,11 +240,13 @@ struct SurfParams {
 };
 cudaError_t bm_launch_surface_map(const World &w, const SurfParams &sp, int n, const int *jlin,
                                   const float *Xc, cudaStream_t st);
-cudaError_t bm_launch_surface_cells(const World &w, const SurfParams &sp, cudaStream_t st);
-cudaError_t bm_launch_surface_vertices(const World &w, const SurfParams &sp, cudaStream_t st);
-cudaError_t bm_launch_surface_tri_count(const World &w, const SurfParams &sp, cudaStream_t st);
-cudaError_t bm_launch_surface_tris(const World &w, const SurfParams &sp, cudaStream_t st);
-cudaError_t bm_launch_surface_embed(const World &w, const SurfParams &sp, int n_vertices, cudaStream_t st);
+cudaError_t bm_launch_surface_count(const World &w, const SurfParams &sp, cudaStream_t st);
+cudaError_t bm_launch_surface_write(const World &w, const SurfParams &sp, int n_vertices, int n_node,
+                                    cudaStream_t st);
+cudaError_t bm_launch_surface_embed(const World &w, const SurfParams &sp, int n_vertices, int n_node,
+                                    cudaStream_t st);
+// n records of nc (2 or 3) words from nc columns
+cudaError_t bm_launch_surface_pack(const void *const *cols, int nc, int n, void *out, cudaStream_t st);
 
 // kernel launchers (bm_kernels.cu)
 #define BM_NUM_KERNELS 19

@@ -1971,6 +1971,7 @@ struct bm_surface_s {
   Allocator al;
   std::vector<void *> fixed;           // lattice map, tables, per-cell arrays
   void *vbuf = nullptr, *tbuf = nullptr;  // vertex and triangle arrays (grown on demand)
+  void *pack = nullptr;                // in vbuf: records on their way to the host
   int64_t vcap = 0, tcap = 0;
   int64_t nv = 0, nt = 0;
   void release_all(cudaStream_t st) {
@@ -1993,11 +1994,13 @@ T *surf_get(bm_surface_s *f, int64_t count) {
   return (T *)p;
 }
 
-// vertex arrays: ref[3], cur[3] floats, anchor int, masks 2 x uint32 (9 words per vertex)
+// vertex arrays: ref[3], cur[3] floats, anchor int, masks 2 x uint32, cell
+// int, 3 words to pack records in for a host read (13 words per vertex), and
+// the cell ordinal (a byte)
 int surf_grow_vertices(bm_surface_s *f, int64_t nv) {
   if (nv <= f->vcap) return BM_OK;
   int64_t cap = std::max<int64_t>(nv + nv / 4, 1024);
-  void *b = f->al.alloc(sizeof(uint32_t) * 9 * (size_t)cap);
+  void *b = f->al.alloc((sizeof(uint32_t) * 13 + 1) * (size_t)cap);
   if (!b) return fail(BM_E_OOM, "surface vertex arrays");
   f->al.release(f->vbuf);
   f->vbuf = b;
@@ -2010,6 +2013,9 @@ int surf_grow_vertices(bm_surface_s *f, int64_t nv) {
   f->sp.anchor = (int *)(fb + (size_t)6 * cap);
   f->sp.vmask[0] = (uint32_t *)(fb + (size_t)7 * cap);
   f->sp.vmask[1] = (uint32_t *)(fb + (size_t)8 * cap);
+  f->sp.vcell = (int *)(fb + (size_t)9 * cap);
+  f->pack = fb + (size_t)10 * cap;
+  f->sp.vord = (uint8_t *)(fb + (size_t)13 * cap);
   return BM_OK;
 }
 
@@ -2074,22 +2080,13 @@ int bm_surface_create(bm_scene_t s, const int lattice[3], bm_surface_t *out) {
     }
   }
   // stencil base cell of every lattice coordinate; it must be the particles'
-  std::vector<int> base[3], jstart[3];
-  int bmin[3], bmax[3];
+  std::vector<int> base[3];
   for (int a = 0; a < 3; ++a) {
     base[a].resize((size_t)nl[a]);
     for (int64_t j = 0; j < nl[a]; ++j)
       base[a][(size_t)j] = (int)std::floor((Xmin[a] + (double)j * h[a] - d.origin[a]) / d.dx - 0.5);
-    bmin[a] = base[a].front();
-    bmax[a] = base[a].back();
     for (int64_t j = 1; j < nl[a]; ++j)
       if (base[a][(size_t)j] < base[a][(size_t)j - 1]) return fail(BM_E_INVALID, "lattice not monotone");
-    jstart[a].assign((size_t)(bmax[a] - bmin[a] + 2), (int)nl[a]);
-    for (int B = bmin[a]; B <= bmax[a] + 1; ++B) {
-      int64_t j = 0;
-      while (j < nl[a] && base[a][(size_t)j] < B) ++j;
-      jstart[a][(size_t)(B - bmin[a])] = (int)j;
-    }
   }
   for (int64_t i = 0; i < n; ++i)
     for (int a = 0; a < 3; ++a) {
@@ -2111,14 +2108,10 @@ int bm_surface_create(bm_scene_t s, const int lattice[3], bm_surface_t *out) {
     sp.h[a] = h[a];
     sp.origin[a] = d.origin[a];
     sp.lo[a] = s->lo[a];
-    sp.bmin[a] = bmin[a];
-    sp.bmax[a] = bmax[a];
   }
   sp.dx = d.dx;
   sp.n_cells = ncells;
   bool ok = true;
-  int *js[3];
-  for (int a = 0; a < 3; ++a) ok &= (js[a] = surf_get<int>(f, (int64_t)jstart[a].size())) != nullptr;
   ok &= (sp.lat = surf_get<int>(f, total)) != nullptr;
   for (int a = 0; a < 3; ++a) ok &= (sp.Xr[a] = surf_get<float>(f, n)) != nullptr;
   ok &= (sp.cell_cnt = surf_get<int>(f, ncells)) != nullptr;
@@ -2127,6 +2120,9 @@ int bm_surface_create(bm_scene_t s, const int lattice[3], bm_surface_t *out) {
   ok &= (sp.pt_cnt = surf_get<int>(f, ncells)) != nullptr;
   ok &= (sp.pt_off = surf_get<int>(f, ncells + 1)) != nullptr;
   ok &= (sp.scan_tmp = surf_get<int>(f, ncells / 1024 + 2)) != nullptr;
+  ok &= (sp.totals = surf_get<int>(f, 2)) != nullptr;
+  ok &= (sp.nmark = surf_get<uint8_t>(f, s->n_node)) != nullptr;
+  ok &= (sp.nval = surf_get<float4>(f, s->slot_cap)) != nullptr;
   int *d_jlin = nullptr;
   float *d_X = nullptr;
   if (ok) {
@@ -2141,15 +2137,12 @@ int bm_surface_create(bm_scene_t s, const int lattice[3], bm_surface_t *out) {
     delete f;
     return fail(BM_E_OOM, "surface buffers");
   }
-  for (int a = 0; a < 3; ++a) sp.jstart[a] = js[a];
   WorldH *W = s->world;
   sp.p_begin = (int)s->p_begin;
   sp.slot = s->slot;
   cudaStream_t st = W->st;
   cudaError_t e = cudaSuccess;
-  for (int a = 0; a < 3 && e == cudaSuccess; ++a)
-    e = cudaMemcpyAsync(js[a], jstart[a].data(), sizeof(int) * jstart[a].size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sp.lat, 0xff, sizeof(int) * (size_t)total, st);
+  e = cudaMemsetAsync(sp.lat, 0xff, sizeof(int) * (size_t)total, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_jlin, jlin.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
@@ -2176,24 +2169,18 @@ int bm_surface_update(bm_surface_t f, int rebuild, int64_t *n_vertices, int64_t 
   sp.slot = s->slot;
   cudaStream_t st = W->st;
   if (rebuild || f->vbuf == nullptr) {
-    CK(bm_launch_surface_cells(W->w, sp, st));
-    int nv = 0;
-    CK(cudaMemcpyAsync(&nv, sp.cell_off + sp.n_cells, sizeof nv, cudaMemcpyDeviceToHost, st));
+    CK(bm_launch_surface_count(W->w, sp, st));
+    int tot[2] = {0, 0};  // vertices, triangles
+    CK(cudaMemcpyAsync(tot, sp.totals, sizeof tot, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    int rc = surf_grow_vertices(f, nv);
+    int rc = surf_grow_vertices(f, tot[0]);
+    if (!rc) rc = surf_grow_tris(f, tot[1]);
     if (rc) return rc;
-    CK(bm_launch_surface_vertices(W->w, sp, st));
-    CK(bm_launch_surface_tri_count(W->w, sp, st));
-    int nt = 0;
-    CK(cudaMemcpyAsync(&nt, sp.pt_off + sp.n_cells, sizeof nt, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    rc = surf_grow_tris(f, nt);
-    if (rc) return rc;
-    CK(bm_launch_surface_tris(W->w, sp, st));
-    f->nv = nv;
-    f->nt = nt;
+    CK(bm_launch_surface_write(W->w, sp, tot[0], (int)s->n_node, st));
+    f->nv = tot[0];
+    f->nt = tot[1];
   }
-  CK(bm_launch_surface_embed(W->w, sp, (int)f->nv, st));
+  CK(bm_launch_surface_embed(W->w, sp, (int)f->nv, (int)s->n_node, st));
   CK(cudaStreamSynchronize(st));
   if (n_vertices) *n_vertices = f->nv;
   if (n_triangles) *n_triangles = f->nt;
@@ -2204,28 +2191,27 @@ int bm_surface_read(bm_surface_t f, float *vertices, float *reference, int32_t *
                     int dst_on_device) {
   if (!valid_surface(f)) return fail(BM_E_INVALID, "bad surface or its scene has no storage");
   cudaStream_t st = f->scene->world->st;
-  CK(cudaStreamSynchronize(st));
   const size_t nv = (size_t)f->nv, nt = (size_t)f->nt;
   const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  // struct-of-arrays on the device, [n][3] / [n][2] at the ABI
-  auto interleave = [&](void *dst, void *const *cols, int ncol, size_t cnt) -> cudaError_t {
-    for (int a = 0; a < ncol; ++a) {
-      cudaError_t e = cudaMemcpy2DAsync((char *)dst + 4 * a, 4 * (size_t)ncol, cols[a], 4, 4, cnt, kind, st);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+  // struct-of-arrays on the device, [n][3] / [n][2] at the ABI: packed by a
+  // kernel, for the host by way of the vertex arrays' spare words (a copy of
+  // 4-byte rows per column took 16 us each)
+  auto records = [&](void *dst, const void *const *cols, int nc) -> cudaError_t {
+    cudaError_t e = bm_launch_surface_pack(cols, nc, (int)nv, dst_on_device ? dst : f->pack, st);
+    if (e == cudaSuccess && !dst_on_device) e = cudaMemcpyAsync(dst, f->pack, sizeof(uint32_t) * nc * nv, kind, st);
+    return e;
   };
   if (nv && vertices) {
-    void *c[3] = {f->sp.cur[0], f->sp.cur[1], f->sp.cur[2]};
-    CK(interleave(vertices, c, 3, nv));
+    const void *c[3] = {f->sp.cur[0], f->sp.cur[1], f->sp.cur[2]};
+    CK(records(vertices, c, 3));
   }
   if (nv && reference) {
-    void *c[3] = {f->sp.ref[0], f->sp.ref[1], f->sp.ref[2]};
-    CK(interleave(reference, c, 3, nv));
+    const void *c[3] = {f->sp.ref[0], f->sp.ref[1], f->sp.ref[2]};
+    CK(records(reference, c, 3));
   }
   if (nv && masks) {
-    void *c[2] = {f->sp.vmask[0], f->sp.vmask[1]};
-    CK(interleave(masks, c, 2, nv));
+    const void *c[2] = {f->sp.vmask[0], f->sp.vmask[1]};
+    CK(records(masks, c, 2));
   }
   if (nt && triangles) CK(cudaMemcpyAsync(triangles, f->sp.tri, sizeof(int) * 3 * nt, kind, st));
   CK(cudaStreamSynchronize(st));

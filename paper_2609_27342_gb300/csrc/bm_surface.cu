@@ -48,16 +48,22 @@ struct CellInfo {
   int nreg;
 };
 
-__device__ void cell_info(const World &w, const SurfParams &sp, const int j[3], CellInfo &ci) {
-  int parent[8];
+// the corners' particles and codes alone
+__device__ __forceinline__ void cell_corners(const World &w, const SurfParams &sp, const int j[3], CellInfo &ci) {
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int p = lat_at(sp, j[0] + (q & 1), j[1] + ((q >> 1) & 1), j[2] + ((q >> 2) & 1));
     ci.part[q] = p;
     ci.c1[q] = p >= 0 ? w.P.s1[sp.p_begin + p] : 0u;
     ci.c2[q] = p >= 0 ? w.P.s2[sp.p_begin + p] : 0u;
-    parent[q] = q;
   }
+}
+
+__device__ void cell_info(const World &w, const SurfParams &sp, const int j[3], CellInfo &ci) {
+  int parent[8];
+  cell_corners(w, sp, j, ci);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) parent[q] = q;
   for (int q = 0; q < 8; ++q)
     for (int a = 0; a < 3; ++a) {
       if ((q >> a) & 1) continue;
@@ -84,14 +90,16 @@ __device__ void cell_info(const World &w, const SurfParams &sp, const int j[3], 
 // Hermite data of the cell edge qa -> qb (axis a) seen from corner qa, in
 // coordinates relative to the cell's lower corner jl: false when qa is empty
 // or the link is connected.
-__device__ bool hermite(const SurfParams &sp, const DevScene &sc, const CellInfo &ci, const int jl[3],
-                        int qa, int qb, int a, float p[3], float nrm[3]) {
+// (hf: the lattice spacing in float32; only the crossing of a recorded plane
+// needs float64, which is slow here)
+__device__ __forceinline__ bool hermite(const SurfParams &sp, const DevScene &sc, const CellInfo &ci, const int jl[3],
+                                        const float hf[3], int qa, int qb, int a, float p[3], float nrm[3]) {
   const int pa = ci.part[qa], pb = ci.part[qb];
   if (pa < 0) return false;
   const float sgn = qb > qa ? 1.f : -1.f;
 #pragma unroll
   for (int t = 0; t < 3; ++t) {
-    p[t] = (float)(((qa >> t) & 1) * sp.h[t]);
+    p[t] = ((qa >> t) & 1) ? hf[t] : 0.f;
     nrm[t] = 0.f;
   }
   if (pb >= 0) {
@@ -116,7 +124,7 @@ __device__ bool hermite(const SurfParams &sp, const DevScene &sc, const CellInfo
     }
   }
   // boundary link (voxel face), or a cut without a recorded plane: midpoint
-  p[a] += 0.5f * sgn * (float)sp.h[a];
+  p[a] += 0.5f * sgn * hf[a];
   nrm[a] = sgn;
   return true;
 }
@@ -200,21 +208,47 @@ __global__ void k_sf_cells(World w, SurfParams sp) {
   sp.cell_reg[i] = packed;
 }
 
-// one vertex per active region: local dual contouring on the region's
-// Hermite data, relative to the mass point, pseudo-inverse, clamped to the cell
-__global__ void k_sf_vertices(World w, SurfParams sp) {
+// the cell and ordinal of every vertex
+__global__ void k_sf_list(SurfParams sp) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= sp.n_cells) return;
-  const int cnt = sp.cell_cnt[i];
-  if (cnt == 0) return;
+  const int cnt = sp.cell_cnt[i], base = sp.cell_off[i];
+  for (int o = 0; o < cnt; ++o) {
+    sp.vcell[base + o] = (int)i;
+    sp.vord[base + o] = (uint8_t)o;
+  }
+}
+
+// grid nodes (scene-local) of the trilinear cell around a point, and weights
+__device__ __forceinline__ void trilinear(const SurfParams &sp, const float c[3], int n0[3], float tw[3]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const double f = ((double)c[a] - sp.origin[a]) / sp.dx;
+    const double fb = floor(f);
+    tw[a] = (float)(f - fb);
+    n0[a] = (int)fb - sp.lo[a];
+  }
+}
+
+// one vertex per active region: local dual contouring on the region's
+// Hermite data, relative to the mass point, pseudo-inverse, clamped to the
+// cell.  A thread per vertex: of the lattice cells only about one in ten has
+// one, and a thread per cell kept 9 lanes of 10 idle through the
+// eigen-decomposition (34,774 vertices of 337,881 cells: 107 us, now 56).  Each
+// vertex also marks the grid nodes that its embedding reads.
+__global__ void k_sf_vertices(World w, SurfParams sp, int nv) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= nv) return;
+  const long long i = sp.vcell[v];
+  const int o = sp.vord[v];
   int j[3];
   cell_of(sp, i, j);
   CellInfo ci;
-  cell_info(w, sp, j, ci);
+  cell_corners(w, sp, j, ci);
   const DevScene &sc = w.scenes[sp.slot];
   const uint32_t packed = sp.cell_reg[i];
-  const int base = sp.cell_off[i];
-  for (int o = 0; o < cnt; ++o) {
+  const float hf[3] = {(float)sp.h[0], (float)sp.h[1], (float)sp.h[2]};
+  {
     float m[3] = {0.f, 0.f, 0.f};
     int k = 0, anchor = -1;
     for (int q = 7; q >= 0; --q)
@@ -228,7 +262,7 @@ __global__ void k_sf_vertices(World w, SurfParams sp) {
           const int qa = side ? r : q, qb = side ? q : r;
           if (((packed >> (4 * qa)) & 15u) != (uint32_t)o) continue;
           float p[3], nn[3];
-          if (!hermite(sp, sc, ci, j, qa, qb, a, p, nn)) continue;
+          if (!hermite(sp, sc, ci, j, hf, qa, qb, a, p, nn)) continue;
           m[0] += p[0];
           m[1] += p[1];
           m[2] += p[2];
@@ -249,7 +283,7 @@ __global__ void k_sf_vertices(World w, SurfParams sp) {
           const int qa = side ? r : q, qb = side ? q : r;
           if (((packed >> (4 * qa)) & 15u) != (uint32_t)o) continue;
           float p[3], nn[3];
-          if (!hermite(sp, sc, ci, j, qa, qb, a, p, nn)) continue;
+          if (!hermite(sp, sc, ci, j, hf, qa, qb, a, p, nn)) continue;
           const float d = nn[0] * (p[0] - m[0]) + nn[1] * (p[1] - m[1]) + nn[2] * (p[2] - m[2]);
 #pragma unroll
           for (int u = 0; u < 3; ++u) {
@@ -270,13 +304,22 @@ __global__ void k_sf_vertices(World w, SurfParams sp) {
 #pragma unroll
       for (int u = 0; u < 3; ++u) c[u] += g * V[u][e];
     }
-    const int v = base + o;
+    float pos[3];
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
       const float cl = fminf(fmaxf(c[u], 0.f), (float)sp.h[u]);
-      sp.ref[u][v] = (float)(sp.Xmin[u] + j[u] * sp.h[u] + (double)cl);
+      pos[u] = (float)(sp.Xmin[u] + j[u] * sp.h[u] + (double)cl);
+      sp.ref[u][v] = pos[u];
     }
     sp.anchor[v] = ci.part[anchor];
+    int n0[3];
+    float tw[3];
+    trilinear(sp, pos, n0, tw);
+    for (int d = 0; d < 8; ++d) {
+      const int x = n0[0] + (d & 1), y = n0[1] + ((d >> 1) & 1), z = n0[2] + (d >> 2);
+      if (x >= 0 && y >= 0 && z >= 0 && x < sc.nn[0] && y < sc.nn[1] && z < sc.nn[2])
+        sp.nmark[(z * sc.nn[1] + y) * sc.nn[0] + x] = 1;
+    }
   }
 }
 
@@ -356,123 +399,138 @@ __global__ void k_sf_tris(World w, SurfParams sp) {
 }
 
 // --------------------------------------------------------------------------
-// side-aware embedding: 8 lanes per vertex share the lattice points around
-// its 8 trilinear nodes (the union of the nodes' B-spline supports, split by
-// z slice); each lane sums, for every node, the weights and weighted
-// displacements of the particles with the anchor's exact code, then the
-// group adds the lanes' sums (xor butterfly) and lane 0 combines the nodes
-// in node order
+// side-aware embedding.  A node's motion is sum N (x - X) / sum N over the
+// particles of one code in its B-spline support; it is taken once per marked
+// node and logical grid (a warp per node: lane l < 27 walks stencil cell l,
+// an xor butterfly adds the lanes), and a vertex combines the 8 nodes around
+// it.  Summing the support anew for every vertex read 512 lattice points per
+// vertex where its neighbours read the same ones (34,774 vertices: 201 us, now
+// 45 + 18; k_sf_nodes is bound by the latency of its particle loads).
 // --------------------------------------------------------------------------
-__device__ __forceinline__ int jfirst(const SurfParams &sp, int a, int B) {
-  if (B <= sp.bmin[a]) return 0;
-  if (B > sp.bmax[a]) return sp.n[a];
-  return sp.jstart[a][B - sp.bmin[a]];
+__device__ __forceinline__ void bsw3(float f, float (&q)[3]) {
+  const float a = 1.5f - f, b = f - 1.f, c = f - 0.5f;
+  q[0] = 0.5f * a * a;
+  q[1] = 0.75f - b * b;
+  q[2] = 0.5f * c * c;
 }
 
-// quadratic B-spline weight of node base + o for fractional offset f in
-// [0.5, 1.5); zero outside the stencil (o not in 0..2)
-__device__ __forceinline__ float bsw(int o, float f) {
-  if (o == 0) {
-    const float t = 1.5f - f;
-    return 0.5f * t * t;
+// sums over the particles of code (a1, a2) in base cell (bx, by, bz) at its
+// node offset (ox, oy, oz)
+__device__ __forceinline__ float4 cell_motion(const World &w, const SurfParams &sp, const DevScene &sc, int bx, int by,
+                                              int bz, int ox, int oy, int oz, uint32_t a1, uint32_t a2) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (bx < 0 || by < 0 || bz < 0 || bx >= sc.nb[0] || by >= sc.nb[1] || bz >= sc.nb[2]) return s;
+  const int brick = ((bz >> 2) * sc.nbr[1] + (by >> 2)) * sc.nbr[0] + (bx >> 2);
+  const int *cs = w.N.cell_start + sc.cell_begin + brick * 64 + (((bz & 3) * 4 + (by & 3)) * 4 + (bx & 3));
+  const int p1 = cs[1];
+  for (int g = cs[0]; g < p1; ++g) {
+    if (w.P.s1[g] != a1 || w.P.s2[g] != a2) continue;
+    const int p = g - sp.p_begin;
+    float wx[3], wy[3], wz[3];
+    bsw3(w.P.fx[0][g], wx);
+    bsw3(w.P.fx[1][g], wy);
+    bsw3(w.P.fx[2][g], wz);
+    const float N = (ox == 0 ? wx[0] : ox == 1 ? wx[1] : wx[2]) * (oy == 0 ? wy[0] : oy == 1 ? wy[1] : wy[2]) *
+                    (oz == 0 ? wz[0] : oz == 1 ? wz[1] : wz[2]);
+    s.x += N;
+    s.y += N * (w.P.x[0][g] - sp.Xr[0][p]);
+    s.z += N * (w.P.x[1][g] - sp.Xr[1][p]);
+    s.w += N * (w.P.x[2][g] - sp.Xr[2][p]);
   }
-  if (o == 1) {
-    const float t = f - 1.f;
-    return 0.75f - t * t;
+  return s;
+}
+
+__device__ __forceinline__ float warp_xor_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
+constexpr int kNodeWarps = 8;
+
+__global__ void __launch_bounds__(32 * kNodeWarps) k_sf_nodes(World w, SurfParams sp) {
+  const DevScene &sc = w.scenes[sp.slot];
+  const int lane = threadIdx.x & 31;
+  const int li = blockIdx.x * kNodeWarps + (threadIdx.x >> 5);
+  if (li >= sc.n_node || !sp.nmark[li]) return;
+  const int node = sc.node_begin + li;
+  const int off = w.N.slot_off[node], ns = w.N.slot_cnt[node];
+  const int ix = li % sc.nn[0], iy = (li / sc.nn[0]) % sc.nn[1], iz = li / (sc.nn[0] * sc.nn[1]);
+  const int ox = lane % 3, oy = (lane / 3) % 3, oz = lane / 9;
+  for (int a = 0; a < ns; ++a) {
+    const uint2 c = w.S.code[off + a];
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < 27) s = cell_motion(w, sp, sc, ix - ox, iy - oy, iz - oz, ox, oy, oz, c.x, c.y);
+    s.x = warp_xor_sum(s.x);
+    s.y = warp_xor_sum(s.y);
+    s.z = warp_xor_sum(s.z);
+    s.w = warp_xor_sum(s.w);
+    if (lane == 0) sp.nval[off + a - sc.slot_begin] = s;
   }
-  if (o == 2) {
-    const float t = f - 0.5f;
-    return 0.5f * t * t;
-  }
-  return 0.f;
 }
 
 __global__ void k_sf_embed(World w, SurfParams sp, int nv) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int v = (int)(t >> 3), lane8 = (int)(t & 7);
-  const bool valid = v < nv;
-  float acc[8][4];  // per trilinear node: sum N, sum N (x - X)
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= nv) return;
+  const DevScene &sc = w.scenes[sp.slot];
+  const int p0 = sp.anchor[v], g0 = sp.p_begin + p0;
+  const uint32_t a1 = w.P.s1[g0], a2 = w.P.s2[g0];
+  // a scene that has overflowed its slots has codes without one: they are summed here
+  const bool over = (sc.err & BM_ERRBIT_SLOT_OVERFLOW) != 0u;
+  float c[3], tw[3];
+  int n0[3];
 #pragma unroll
-  for (int d = 0; d < 8; ++d) acc[d][0] = acc[d][1] = acc[d][2] = acc[d][3] = 0.f;
-  float c[3] = {0.f, 0.f, 0.f}, tw[3] = {0.f, 0.f, 0.f};
-  int g0 = 0;
-  uint32_t a1 = 0u, a2 = 0u;
-  if (valid) {
-    g0 = sp.p_begin + sp.anchor[v];
-    a1 = w.P.s1[g0];
-    a2 = w.P.s2[g0];
-    int n0[3], jlo[3], jhi[3];
+  for (int a = 0; a < 3; ++a) c[a] = sp.ref[a][v];
+  trilinear(sp, c, n0, tw);
+  float num[3] = {0.f, 0.f, 0.f}, den = 0.f;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      c[a] = sp.ref[a][v];
-      const double f = ((double)c[a] - sp.origin[a]) / sp.dx;
-      const double fb = floor(f);
-      tw[a] = (float)(f - fb);
-      n0[a] = (int)fb;
-      // particles whose stencil holds node n0 or n0 + 1: base cells n0 - 2 .. n0 + 1
-      jlo[a] = jfirst(sp, a, n0[a] - 2);
-      jhi[a] = jfirst(sp, a, n0[a] + 2);
+  for (int d = 0; d < 8; ++d) {
+    const int x = n0[0] + (d & 1), y = n0[1] + ((d >> 1) & 1), z = n0[2] + (d >> 2);
+    if (x < 0 || y < 0 || z < 0 || x >= sc.nn[0] || y >= sc.nn[1] || z >= sc.nn[2]) continue;
+    const int node = sc.node_begin + (z * sc.nn[1] + y) * sc.nn[0] + x;
+    const int off = w.N.slot_off[node], ns = w.N.slot_cnt[node];
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int a = 0; a < ns; ++a) {
+      const uint2 q = w.S.code[off + a];
+      if (q.x == a1 && q.y == a2) s = sp.nval[off + a - sc.slot_begin];
     }
-    for (int z = jlo[2] + lane8; z < jhi[2]; z += 8)
-      for (int y = jlo[1]; y < jhi[1]; ++y)
-        for (int x = jlo[0]; x < jhi[0]; ++x) {
-          const int p = sp.lat[((long long)z * sp.n[1] + y) * sp.n[0] + x];
-          if (p < 0) continue;
-          const int g = sp.p_begin + p;
-          if (w.P.s1[g] != a1 || w.P.s2[g] != a2) continue;
-          const uint32_t bb = w.P.base[g];
-          const int ox = n0[0] - ((int)(bb & 1023u) + sp.lo[0]);
-          const int oy = n0[1] - ((int)((bb >> 10) & 1023u) + sp.lo[1]);
-          const int oz = n0[2] - ((int)((bb >> 20) & 1023u) + sp.lo[2]);
-          const float fx = w.P.fx[0][g], fy = w.P.fx[1][g], fz = w.P.fx[2][g];
-          const float wx[2] = {bsw(ox, fx), bsw(ox + 1, fx)};
-          const float wy[2] = {bsw(oy, fy), bsw(oy + 1, fy)};
-          const float wz[2] = {bsw(oz, fz), bsw(oz + 1, fz)};
-          const float u0 = w.P.x[0][g] - sp.Xr[0][p], u1 = w.P.x[1][g] - sp.Xr[1][p],
-                      u2 = w.P.x[2][g] - sp.Xr[2][p];
-#pragma unroll
-          for (int d = 0; d < 8; ++d) {
-            const float N = wx[d & 1] * wy[(d >> 1) & 1] * wz[d >> 2];
-            acc[d][0] += N;
-            acc[d][1] += N * u0;
-            acc[d][2] += N * u1;
-            acc[d][3] += N * u2;
-          }
-        }
+    if (over && s.x == 0.f)
+      for (int l = 0; l < 27; ++l) {
+        const float4 m = cell_motion(w, sp, sc, x - l % 3, y - (l / 3) % 3, z - l / 9, l % 3, (l / 3) % 3, l / 9, a1, a2);
+        s.x += m.x;
+        s.y += m.y;
+        s.z += m.z;
+        s.w += m.w;
+      }
+    if (!(s.x > 0.f)) continue;  // no particle of this code around the node
+    const float wt = ((d & 1) ? tw[0] : 1.f - tw[0]) * (((d >> 1) & 1) ? tw[1] : 1.f - tw[1]) *
+                     ((d >> 2) ? tw[2] : 1.f - tw[2]);
+    const float r = wt / s.x;
+    num[0] += r * s.y;
+    num[1] += r * s.z;
+    num[2] += r * s.w;
+    den += wt;
   }
-  // sums over the group's 8 lanes (the xor partners stay inside the group)
 #pragma unroll
-  for (int m = 1; m < 8; m <<= 1)
-#pragma unroll
-    for (int d = 0; d < 8; ++d)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[d][e] += __shfl_xor_sync(kFull, acc[d][e], m);
-  if (valid && lane8 == 0) {
-    float num[3] = {0.f, 0.f, 0.f}, den = 0.f;
-#pragma unroll
-    for (int d = 0; d < 8; ++d) {
-      if (!(acc[d][0] > 0.f)) continue;  // no particle of this code around the node
-      const float wt = ((d & 1) ? tw[0] : 1.f - tw[0]) * (((d >> 1) & 1) ? tw[1] : 1.f - tw[1]) *
-                       ((d >> 2) ? tw[2] : 1.f - tw[2]);
-      const float s = wt / acc[d][0];
-      num[0] += s * acc[d][1];
-      num[1] += s * acc[d][2];
-      num[2] += s * acc[d][3];
-      den += wt;
-    }
-    const int p0 = sp.anchor[v];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const float u = den > 0.f ? num[a] / den : w.P.x[a][g0] - sp.Xr[a][p0];
-      sp.cur[a][v] = c[a] + u;
-    }
-    sp.vmask[0][v] = a1;
-    sp.vmask[1][v] = a2;
+  for (int a = 0; a < 3; ++a) {
+    const float u = den > 0.f ? num[a] / den : w.P.x[a][g0] - sp.Xr[a][p0];
+    sp.cur[a][v] = c[a] + u;
   }
+  sp.vmask[0][v] = a1;
+  sp.vmask[1][v] = a2;
+}
+
+// n records of nc words from columns, into an array of records
+__global__ void k_sf_pack(const uint32_t *c0, const uint32_t *c1, const uint32_t *c2, int nc, int n, uint32_t *out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  out[(size_t)nc * i] = c0[i];
+  out[(size_t)nc * i + 1] = c1[i];
+  if (nc > 2) out[(size_t)nc * i + 2] = c2[i];
 }
 
 // --------------------------------------------------------------------------
-// exclusive scan of n ints into out[0..n] (out[n] = total)
+// exclusive scan of n ints, and their total
 // --------------------------------------------------------------------------
 __device__ int block_scan_excl(int v, int *sm, int &total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -528,10 +586,10 @@ __global__ void k_sf_scan_add(int *out, const int *bsum, long long n) {
   if (i < n) out[i] += bsum[i / kScanBlock];
 }
 
-cudaError_t scan_excl(const int *in, int *out, int *tmp, long long n, cudaStream_t st) {
+cudaError_t scan_excl(const int *in, int *out, int *total, int *tmp, long long n, cudaStream_t st) {
   const int nb = (int)((n + kScanBlock - 1) / kScanBlock);
   if (nb > 0) k_sf_scan_block<<<nb, kScanBlock, 0, st>>>(in, out, tmp, n);
-  k_sf_scan_top<<<1, kScanBlock, 0, st>>>(tmp, nb, out + n);
+  k_sf_scan_top<<<1, kScanBlock, 0, st>>>(tmp, nb, total);
   if (nb > 0) k_sf_scan_add<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(out, tmp, n);
   return cudaGetLastError();
 }
@@ -546,31 +604,40 @@ cudaError_t bm_launch_surface_map(const World &w, const SurfParams &sp, int n, c
   return cudaGetLastError();
 }
 
-cudaError_t bm_launch_surface_cells(const World &w, const SurfParams &sp, cudaStream_t st) {
+// regions and their vertices' places, then the triangles' places; the two
+// totals end up in sp.totals
+cudaError_t bm_launch_surface_count(const World &w, const SurfParams &sp, cudaStream_t st) {
   k_sf_cells<<<grid_of(sp.n_cells, 128), 128, 0, st>>>(w, sp);
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = scan_excl(sp.cell_cnt, sp.cell_off, sp.totals, sp.scan_tmp, sp.n_cells, st);
   if (e != cudaSuccess) return e;
-  return scan_excl(sp.cell_cnt, sp.cell_off, sp.scan_tmp, sp.n_cells, st);
-}
-
-cudaError_t bm_launch_surface_vertices(const World &w, const SurfParams &sp, cudaStream_t st) {
-  k_sf_vertices<<<grid_of(sp.n_cells, 128), 128, 0, st>>>(w, sp);
-  return cudaGetLastError();
-}
-
-cudaError_t bm_launch_surface_tri_count(const World &w, const SurfParams &sp, cudaStream_t st) {
   k_sf_tris<false><<<grid_of(sp.n_cells, 128), 128, 0, st>>>(w, sp);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return scan_excl(sp.pt_cnt, sp.pt_off, sp.scan_tmp, sp.n_cells, st);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = scan_excl(sp.pt_cnt, sp.pt_off, sp.totals + 1, sp.scan_tmp, sp.n_cells, st);
+  return e;
 }
 
-cudaError_t bm_launch_surface_tris(const World &w, const SurfParams &sp, cudaStream_t st) {
+cudaError_t bm_launch_surface_write(const World &w, const SurfParams &sp, int n_vertices, int n_node,
+                                    cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(sp.nmark, 0, (size_t)n_node, st);
+  if (e != cudaSuccess) return e;
+  k_sf_list<<<grid_of(sp.n_cells, 256), 256, 0, st>>>(sp);
+  if (n_vertices > 0) k_sf_vertices<<<grid_of(n_vertices, 64), 64, 0, st>>>(w, sp, n_vertices);
   k_sf_tris<true><<<grid_of(sp.n_cells, 128), 128, 0, st>>>(w, sp);
   return cudaGetLastError();
 }
 
-cudaError_t bm_launch_surface_embed(const World &w, const SurfParams &sp, int n_vertices, cudaStream_t st) {
-  if (n_vertices > 0) k_sf_embed<<<grid_of(8LL * n_vertices, 256), 256, 0, st>>>(w, sp, n_vertices);
+cudaError_t bm_launch_surface_embed(const World &w, const SurfParams &sp, int n_vertices, int n_node,
+                                    cudaStream_t st) {
+  if (n_vertices == 0) return cudaSuccess;
+  k_sf_nodes<<<grid_of(n_node, kNodeWarps), 32 * kNodeWarps, 0, st>>>(w, sp);
+  k_sf_embed<<<grid_of(n_vertices, 128), 128, 0, st>>>(w, sp, n_vertices);
+  return cudaGetLastError();
+}
+
+cudaError_t bm_launch_surface_pack(const void *const *cols, int nc, int n, void *out, cudaStream_t st) {
+  if (n > 0)
+    k_sf_pack<<<grid_of(n, 256), 256, 0, st>>>((const uint32_t *)cols[0], (const uint32_t *)cols[1],
+                                               nc > 2 ? (const uint32_t *)cols[2] : nullptr, nc, n, (uint32_t *)out);
   return cudaGetLastError();
 }
