@@ -21,7 +21,7 @@
 //                 change (Eq. 17 and x update), through Eq. 8 transposed
 //   k_adj_part    per particle: P2G (Eq. 2) transposed, stress, blade and
 //                 floor contact; block partials of the parameter adjoints
-//   k_adj_reduce  one block: partials summed in block order (float64), tool
+//   k_adj_reduce  one block: the blocks' partials summed (float64), tool
 //                 position and segment velocity adjoints updated
 // Scope: kinematic blade translating without rotation, rigid interval 1, no
 // material-material contact (checked on the host).
@@ -67,15 +67,33 @@ __device__ __forceinline__ int node_at(const DevScene &sc, int ix, int iy, int i
   return (iz * sc.nn[1] + iy) * sc.nn[0] + ix;
 }
 
-// slot (pool index) holding code c at scene-local node li, or -1
-__device__ __forceinline__ int find_slot(const World &w, const DevScene &sc, int li, uint2 c) {
-  const int node = sc.node_begin + li;
-  const int off = w.N.slot_off[node], cnt = w.N.slot_cnt[node];
-  for (int a = 0; a < cnt; ++a) {
-    const uint2 k = w.S.code[off + a];
-    if (k.x == c.x && k.y == c.y) return off + a;
+// Pool slots of code c at the 9 nodes of stencil layer oz of a particle with
+// base cell (bx, by, bz) (-1: none), index 3 oy + ox.  The layer's slot table
+// entries are read together: looked up one node after the other, the 27
+// dependent reads were most of k_adj_v1 and k_adj_part.  A node with one slot
+// needs no look at its code: it holds the particle's.
+__device__ __forceinline__ void layer_slots(const World &w, const DevScene &sc, int bx, int by, int bz, uint2 c,
+                                            int (&slot)[9]) {
+  int cnt[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int node = sc.node_begin + node_at(sc, bx + k % 3, by + k / 3, bz);
+    slot[k] = w.N.slot_off[node];
+    cnt[k] = w.N.slot_cnt[node];
   }
-  return -1;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    if (cnt[k] == 1) continue;
+    int found = -1;
+    for (int a = 0; a < cnt[k]; ++a) {
+      const uint2 q = w.S.code[slot[k] + a];
+      if (q.x == c.x && q.y == c.y) {
+        found = slot[k] + a;
+        break;
+      }
+    }
+    slot[k] = found;
+  }
 }
 
 struct AdjWork {
@@ -114,25 +132,50 @@ __device__ __forceinline__ void couple_T(int ns, const uint2 *codes, const float
     for (int c = 0; c < NC; ++c) S[b][c] = out[b][c];
 }
 
-// Visit the (particle, weight, gradient) pairs of scene-local node li whose
-// particle lies in stencil cell l (< 27: ox = l % 3, oy = l / 3 % 3,
-// oz = l / 9, the base cell li - (ox, oy, oz)), in pool order.
-template <class Fn>
-__device__ __forceinline__ void for_cell_particles(const World &w, const DevScene &sc, int li, int l, Fn fn) {
+// Particle range [p0, p1) of stencil cell l of scene-local node li (l < 27:
+// ox = l % 3, oy = l / 3 % 3, oz = l / 9, the base cell li - (ox, oy, oz)).
+__device__ __forceinline__ void stencil_cell(const World &w, const DevScene &sc, int li, int l, int &p0, int &p1) {
+  p0 = p1 = 0;
+  if (l >= 27) return;
   const int ix = li % sc.nn[0], iy = (li / sc.nn[0]) % sc.nn[1], iz = li / (sc.nn[0] * sc.nn[1]);
-  const int ox = l % 3, oy = (l / 3) % 3, oz = l / 9;
-  const int bx = ix - ox, by = iy - oy, bz = iz - oz;
+  const int bx = ix - l % 3, by = iy - (l / 3) % 3, bz = iz - l / 9;
   if (bx < 0 || by < 0 || bz < 0 || bx >= sc.nb[0] || by >= sc.nb[1] || bz >= sc.nb[2]) return;
-  const int *cs = w.N.cell_start + sc.cell_begin;
-  const int c = cell_at(sc, bx, by, bz);
-  for (int p = cs[c]; p < cs[c + 1]; ++p) {
-    float wx, wy, wz, dx, dy, dz;
-    wgt(ox, w.P.fx[0][p], wx, dx);
-    wgt(oy, w.P.fx[1][p], wy, dy);
-    wgt(oz, w.P.fx[2][p], wz, dz);
-    const float N = wx * wy * wz;
-    const float gN[3] = {dx * wy * wz * sc.inv_dx, wx * dy * wz * sc.inv_dx, wx * wy * dz * sc.inv_dx};
-    fn(p, N, gN);
+  const int *cs = w.N.cell_start + sc.cell_begin + cell_at(sc, bx, by, bz);
+  p0 = cs[0];
+  p1 = cs[1];
+}
+
+// Walk a cell's particles of code c in pool order, U at a time: the NV values
+// val[.][particle - pb] and the weights of U particles are read before any is
+// used (one after the other, the reads' latency set the kernel's time), then
+// fn(values, N, grad N) takes them in order.
+template <int U, int NV, class Fn>
+__device__ __forceinline__ void walk_cell(const World &w, const DevScene &sc, int l, int p0, int p1, uint2 c,
+                                          float *const (&val)[NV], Fn fn) {
+  const int ox = l % 3, oy = (l / 3) % 3, oz = l / 9, pb = sc.p_begin;
+  for (int q = p0; q < p1; q += U) {
+    bool on[U];
+    float f[U][3], v[U][NV];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int p = min(q + u, p1 - 1);
+      on[u] = q + u < p1 && w.P.s1[p] == c.x && w.P.s2[p] == c.y;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) f[u][a] = w.P.fx[a][p];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[u][k] = val[k][p - pb];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (!on[u]) continue;
+      float wx, wy, wz, dx, dy, dz;
+      wgt(ox, f[u][0], wx, dx);
+      wgt(oy, f[u][1], wy, dy);
+      wgt(oz, f[u][2], wz, dz);
+      const float N = wx * wy * wz;
+      const float gN[3] = {dx * wy * wz * sc.inv_dx, wx * dy * wz * sc.inv_dx, wx * wy * dz * sc.inv_dx};
+      fn(v[u], N, gN);
+    }
   }
 }
 
@@ -160,20 +203,18 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_musl(World w, AdjWork aw) {
   const int node = sc.node_begin + li;
   const int off = w.N.slot_off[node], ns = w.N.slot_cnt[node];
   if (ns == 0) return;
-  const int pb = sc.p_begin;
   const float dt = sc.dt, mp = sc.mp;
+  int p0, p1;
+  stencil_cell(w, sc, li, lane, p0, p1);
   for (int a = 0; a < ns; ++a) {
     const uint2 ca = w.S.code[off + a];
     float m = 0.f, S0 = 0.f, S1 = 0.f, S2 = 0.f;
-    if (lane < 27)
-      for_cell_particles(w, sc, li, lane, [&](int p, float N, const float *gN) {
-        if (w.P.s1[p] != ca.x || w.P.s2[p] != ca.y) return;
-        m += N * mp;
-        const int i = p - pb;
-        S0 += dt * (aw.Fb[0][i] * gN[0] + aw.Fb[1][i] * gN[1] + aw.Fb[2][i] * gN[2]);
-        S1 += dt * (aw.Fb[3][i] * gN[0] + aw.Fb[4][i] * gN[1] + aw.Fb[5][i] * gN[2]);
-        S2 += dt * (aw.Fb[6][i] * gN[0] + aw.Fb[7][i] * gN[1] + aw.Fb[8][i] * gN[2]);
-      });
+    walk_cell<4>(w, sc, lane, p0, p1, ca, aw.Fb, [&](const float *F, float N, const float *gN) {
+      m += N * mp;
+      S0 += dt * (F[0] * gN[0] + F[1] * gN[1] + F[2] * gN[2]);
+      S1 += dt * (F[3] * gN[0] + F[4] * gN[1] + F[5] * gN[2]);
+      S2 += dt * (F[6] * gN[0] + F[7] * gN[1] + F[8] * gN[2]);
+    });
     m = warp_sum(m);
     S0 = warp_sum(S0);
     S1 = warp_sum(S1);
@@ -215,20 +256,27 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_v1(World w, AdjWork aw) {
   const uint2 c = make_uint2(w.P.s1[p], w.P.s2[p]);
   float acc[3] = {aw.vb[0][i], aw.vb[1][i], aw.vb[2][i]};
   const float mp = sc.mp;
-  for (int oz = 0; oz < 3; ++oz)
-    for (int oy = 0; oy < 3; ++oy)
-      for (int ox = 0; ox < 3; ++ox) {
-        float wx, wy, wz, d0, d1, d2;
-        wgt(ox, w.P.fx[0][p], wx, d0);
-        wgt(oy, w.P.fx[1][p], wy, d1);
-        wgt(oz, w.P.fx[2][p], wz, d2);
-        const int s = find_slot(w, sc, node_at(sc, bx + ox, by + oy, bz + oz), c);
-        if (s < 0) continue;
-        const float N = wx * wy * wz;
-        const int rel = s - sc.slot_begin;
+  const float f[3] = {w.P.fx[0][p], w.P.fx[1][p], w.P.fx[2][p]};
+  for (int oz = 0; oz < 3; ++oz) {
+    int slot[9];
+    layer_slots(w, sc, bx, by, bz + oz, c, slot);
+    float s3[9][3];
 #pragma unroll
-        for (int r = 0; r < 3; ++r) acc[r] += N * mp * aw.s3[r][rel];
-      }
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) s3[k][r] = slot[k] >= 0 ? aw.s3[r][slot[k] - sc.slot_begin] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      if (slot[k] < 0) continue;
+      float wx, wy, wz, d0, d1, d2;
+      wgt(k % 3, f[0], wx, d0);
+      wgt(k / 3, f[1], wy, d1);
+      wgt(oz, f[2], wz, d2);
+      const float N = wx * wy * wz;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) acc[r] += N * mp * s3[k][r];
+    }
+  }
 #pragma unroll
   for (int r = 0; r < 3; ++r) aw.v1b[r][i] = acc[r];
 }
@@ -246,20 +294,20 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_g2p(World w, AdjWork aw) {
   const int off = w.N.slot_off[node], ns = w.N.slot_cnt[node];
   if (ns == 0) return;
   const int rel = off - sc.slot_begin;
-  const int pb = sc.p_begin;
   const float dt = sc.dt, beta = sc.beta;
+  float *const val[6] = {aw.v1b[0], aw.v1b[1], aw.v1b[2], aw.xb[0], aw.xb[1], aw.xb[2]};
+  int p0, p1;
+  stencil_cell(w, sc, li, lane, p0, p1);
   for (int a = 0; a < ns; ++a) {
     const uint2 ca = w.S.code[off + a];
     const float ma = aw.sm[rel + a];
     float S[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (lane < 27 && ma > 0.f)
-      for_cell_particles(w, sc, li, lane, [&](int p, float N, const float *) {
-        if (w.P.s1[p] != ca.x || w.P.s2[p] != ca.y) return;
+    if (ma > 0.f)
+      walk_cell<4>(w, sc, lane, p0, p1, ca, val, [&](const float *v, float N, const float *) {
         const float q = N / ma;
-        const int i = p - pb;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
-          const float v1 = aw.v1b[r][i], xx = dt * aw.xb[r][i];
+          const float v1 = v[r], xx = dt * v[3 + r];
           S[r] += q * ((1.0f - beta) * v1 + xx);
           S[3 + r] += q * (v1 + xx);
         }
@@ -351,21 +399,30 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_part(World w, AdjWork aw) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) Pb[k] = 0.f;
     const float cA = -dt * sc.V0;
-    for (int oz = 0; oz < 3; ++oz)
-      for (int oy = 0; oy < 3; ++oy)
+    const float f[3] = {w.P.fx[0][p], w.P.fx[1][p], w.P.fx[2][p]};
+    for (int oz = 0; oz < 3; ++oz) {
+      int slot[9];
+      layer_slots(w, sc, bx, by, bz + oz, code, slot);
+#pragma unroll
+      for (int oy = 0; oy < 3; ++oy) {
+        float s6[3][6];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+          for (int r = 0; r < 6; ++r)
+            s6[k][r] = slot[3 * oy + k] >= 0 ? aw.s6[r][slot[3 * oy + k] - sc.slot_begin] : 0.f;
+#pragma unroll
         for (int ox = 0; ox < 3; ++ox) {
+          if (slot[3 * oy + ox] < 0) continue;
           float wx, wy, wz, d0, d1, d2;
-          wgt(ox, w.P.fx[0][p], wx, d0);
-          wgt(oy, w.P.fx[1][p], wy, d1);
-          wgt(oz, w.P.fx[2][p], wz, d2);
-          const int s = find_slot(w, sc, node_at(sc, bx + ox, by + oy, bz + oz), code);
-          if (s < 0) continue;
-          const int rel = s - sc.slot_begin;
+          wgt(ox, f[0], wx, d0);
+          wgt(oy, f[1], wy, d1);
+          wgt(oz, f[2], wz, d2);
           const float N = wx * wy * wz;
           const float gN[3] = {d0 * wy * wz * sc.inv_dx, wx * d1 * wz * sc.inv_dx, wx * wy * d2 * sc.inv_dx};
 #pragma unroll
           for (int r = 0; r < 3; ++r) {
-            const float pbar = aw.s6[r][rel], dpbar = aw.s6[3 + r][rel];
+            const float pbar = s6[ox][r], dpbar = s6[ox][3 + r];
             vb[r] += N * mp * pbar;
             Jb[r] += N * dpbar;
             Pb[3 * r] += cA * dpbar * gN[0];
@@ -373,6 +430,8 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_part(World w, AdjWork aw) {
             Pb[3 * r + 2] += cA * dpbar * gN[2];
           }
         }
+      }
+    }
     // stress
     float F[9], Fb[9];
 #pragma unroll
@@ -593,15 +652,20 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_part(World w, AdjWork aw) {
   }
 }
 
-// one block: partials summed in block order; x_B^{n+1} = x_B^n + dt v_B^n
+// one block: the blocks' partials summed; x_B^{n+1} = x_B^n + dt v_B^n
 // with v_B^n the velocity of the segment active at this substep
-__global__ void k_adj_reduce(World w, AdjWork aw, int nblocks) {
+// (warp k sums partial k: its lanes stride the blocks, a fixed shuffle tree
+// adds them; one thread adding the blocks in turn took 16 us for 250 of them)
+__global__ void __launch_bounds__(32 * kParts) k_adj_reduce(World w, AdjWork aw, int nblocks) {
   __shared__ double tot[kParts];
   const DevScene &sc = w.scenes[aw.slot];
-  if (threadIdx.x < kParts) {
+  {
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += aw.part[(size_t)b * kParts + threadIdx.x];
-    tot[threadIdx.x] = s;
+    for (int b = lane; b < nblocks; b += 32) s += aw.part[(size_t)b * kParts + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) tot[k] = s;
   }
   __syncthreads();
   if (threadIdx.x != 0) return;
@@ -697,7 +761,7 @@ cudaError_t bm_launch_adjoint_substep(const World &w, const void *work, const do
   k_adj_v1<<<gp, kAdjBlock, 0, st>>>(w, aw);
   k_adj_g2p<<<gn, kAdjBlock, 0, st>>>(w, aw);
   k_adj_part<<<gp, kAdjBlock, 0, st>>>(w, aw);
-  k_adj_reduce<<<1, 32, 0, st>>>(w, aw, gp);
+  k_adj_reduce<<<1, 32 * kParts, 0, st>>>(w, aw, gp);
   return cudaGetLastError();
 }
 

@@ -1750,99 +1750,114 @@ __global__ void k_tool(World w, LaunchSet ls) {
 // --------------------------------------------------------------------------
 
 
-// Distinct codes at every node of a node tile.  Nodes next to a newly
-// labelled particle (dirty) are recounted, the others keep their distinct
-// codes from the last rebuild.  A recount takes one warp per node: lane l <
-// 27 holds base cell (i - l % 3, j - l / 3 % 3, k - l / 9) of the node's
-// stencil, and the node's codes are found in ascending order of the key
-// (mask2 << 32 | mask1) as repeated warp-wide minima over the lanes' particles
-// of the keys above the last one found.
+// Recount of the distinct codes at one node, by one warp: lane l < 27 holds
+// base cell (i - l % 3, j - l / 3 % 3, k - l / 9) of the node's stencil, and
+// the node's codes are found in ascending order of the key (mask2 << 32 |
+// mask1) as repeated warp-wide minima over the lanes' particles of the keys
+// above the last one found.  Returns the count.
 // KR: particles per cell whose label keys a lane keeps in registers across
 // the passes (8 or 16, the launch set's largest cell)
 template <int KR>
+__device__ __forceinline__ int recount_node(const World &w, DevScene &sc, int nd, int lane) {
+  const int *cs = w.N.cell_start + sc.cell_begin;
+  int ix, iy, iz;
+  node_coords(sc, nd - sc.node_begin, ix, iy, iz);
+  int p0 = 0, p1 = 0;
+  if (lane < 27) {
+    const int bx = ix - lane % 3, by = iy - (lane / 3) % 3, bz = iz - lane / 9;
+    if (bx >= 0 && by >= 0 && bz >= 0 && bx < sc.nb[0] && by < sc.nb[1] && bz < sc.nb[2]) {
+      const int c = cell_index(sc, bx, by, bz);
+      p0 = cs[c];
+      p1 = cs[c + 1];
+    }
+  }
+  int cnt = 0;
+  bool over = false;
+  unsigned long long last = 0;
+  bool first = true;
+  // a cell of up to KR particles keeps its keys in registers across the
+  // passes (the all-ones key is never a code: a cut has one side per particle)
+  const bool inreg = p1 - p0 <= KR;
+  unsigned long long kr[KR];
+#pragma unroll
+  for (int j = 0; j < KR; ++j)
+    kr[j] = (inreg && p0 + j < p1) ? ((unsigned long long)w.P.s2[p0 + j] << 32) | w.P.s1[p0 + j] : ~0ull;
+  for (;;) {
+    unsigned long long m = ~0ull;
+    if (inreg) {
+#pragma unroll
+      for (int j = 0; j < KR; ++j)
+        if ((first || kr[j] > last) && kr[j] < m) m = kr[j];
+    } else {
+      for (int p = p0; p < p1; ++p) {
+        const unsigned long long k = ((unsigned long long)w.P.s2[p] << 32) | w.P.s1[p];
+        if ((first || k > last) && k < m) m = k;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(FULL, m, o);
+      m = y < m ? y : m;
+    }
+    if (m == ~0ull) break;
+    if (cnt < BM_MAXS) {
+      if (lane == 0) w.N.tmp_codes[(size_t)nd * BM_MAXS + cnt] = make_uint2((uint32_t)m, (uint32_t)(m >> 32));
+      ++cnt;
+    } else {
+      over = true;
+      break;
+    }
+    last = m;
+    first = false;
+  }
+  if (lane == 0) {
+    if (over) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
+    w.N.ncodes[nd] = (uint8_t)cnt;
+    w.N.dirty[nd] = 0;
+  }
+  return cnt;
+}
+
+// Recount of a tile's dirty nodes (all of them when forced) by the warps of
+// gridDim.y CTAs, ahead of k_slot_count<.., true>.
+template <int KR>
+__global__ void k_recount(World w, LaunchSet ls, int force) {
+  const int4 t = ls.ntiles[blockIdx.x];
+  DevScene &sc = w.scenes[t.x];
+  if (!force && !sc.need_rebuild) return;
+  const int lane = threadIdx.x & 31;
+  const int warp = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = gridDim.y * (blockDim.x >> 5);
+  for (int li = warp; li < t.z; li += nw)
+    if (force || w.N.dirty[t.y + li]) recount_node<KR>(w, sc, t.y + li, lane);
+}
+
+// Slot counts of a node tile's nodes and their sum.  Nodes next to a newly
+// labelled particle (dirty) are recounted, a warp each (COUNTED: k_recount
+// has done so), the others keep their distinct codes from the last rebuild.
+template <int KR, bool COUNTED>
 __global__ void k_slot_count(World w, LaunchSet ls, int force) {
   const int4 t = ls.ntiles[blockIdx.x];
   DevScene &sc = w.scenes[t.x];
   if (!force && !sc.need_rebuild) return;
   __shared__ int sm[33];
-  __shared__ int dlist[512];   // node tile <= 512 nodes
-  __shared__ int dcnt[512];
-  __shared__ int ndirty;
   const int i = threadIdx.x;
   const int node = t.y + i;
-  bool recount = false;
-  if (i < t.z) recount = force != 0 || w.N.dirty[node] != 0;
-  if (i == 0) ndirty = 0;
-  __syncthreads();
-  if (recount) dlist[atomicAdd(&ndirty, 1)] = i;
-  __syncthreads();
-  const int lane = i & 31, wid = i >> 5, nw = blockDim.x >> 5;
-  const int *cs = w.N.cell_start + sc.cell_begin;
-  for (int j = wid; j < ndirty; j += nw) {
-    const int li = dlist[j];
-    const int nd = t.y + li;
-    int ix, iy, iz;
-    node_coords(sc, nd - sc.node_begin, ix, iy, iz);
-    int p0 = 0, p1 = 0;
-    if (lane < 27) {
-      const int bx = ix - lane % 3, by = iy - (lane / 3) % 3, bz = iz - lane / 9;
-      if (bx >= 0 && by >= 0 && bz >= 0 && bx < sc.nb[0] && by < sc.nb[1] && bz < sc.nb[2]) {
-        const int c = cell_index(sc, bx, by, bz);
-        p0 = cs[c];
-        p1 = cs[c + 1];
-      }
-    }
-    int cnt = 0;
-    bool over = false;
-    unsigned long long last = 0;
-    bool first = true;
-    // a cell of up to KR particles keeps its keys in registers across the
-    // passes (the all-ones key is never a code: a cut has one side per particle)
-    const bool inreg = p1 - p0 <= KR;
-    unsigned long long kr[KR];
-#pragma unroll
-    for (int j = 0; j < KR; ++j)
-      kr[j] = (inreg && p0 + j < p1) ? ((unsigned long long)w.P.s2[p0 + j] << 32) | w.P.s1[p0 + j] : ~0ull;
-    for (;;) {
-      unsigned long long m = ~0ull;
-      if (inreg) {
-#pragma unroll
-        for (int j = 0; j < KR; ++j)
-          if ((first || kr[j] > last) && kr[j] < m) m = kr[j];
-      } else {
-        for (int p = p0; p < p1; ++p) {
-          const unsigned long long k = ((unsigned long long)w.P.s2[p] << 32) | w.P.s1[p];
-          if ((first || k > last) && k < m) m = k;
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(FULL, m, o);
-        m = y < m ? y : m;
-      }
-      if (m == ~0ull) break;
-      if (cnt < BM_MAXS) {
-        if (lane == 0)
-          w.N.tmp_codes[(size_t)nd * BM_MAXS + cnt] = make_uint2((uint32_t)m, (uint32_t)(m >> 32));
-        ++cnt;
-      } else {
-        over = true;
-        break;
-      }
-      last = m;
-      first = false;
-    }
-    if (lane == 0) {
-      if (over) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
-      w.N.ncodes[nd] = (uint8_t)cnt;
-      w.N.dirty[nd] = 0;
-      dcnt[li] = cnt;
-    }
-  }
-  __syncthreads();
   int cnt = 0;
-  if (i < t.z) cnt = recount ? dcnt[i] : w.N.ncodes[node];
-  if (i < t.z) w.N.slot_cnt[node] = (uint8_t)cnt;
+  if (!COUNTED) {
+    __shared__ int dlist[512];   // node tile <= 512 nodes
+    __shared__ int ndirty;
+    if (i == 0) ndirty = 0;
+    __syncthreads();
+    if (i < t.z && (force != 0 || w.N.dirty[node] != 0)) dlist[atomicAdd(&ndirty, 1)] = i;
+    __syncthreads();
+    const int lane = i & 31, wid = i >> 5, nw = blockDim.x >> 5;
+    for (int j = wid; j < ndirty; j += nw) recount_node<KR>(w, sc, t.y + dlist[j], lane);
+    __syncthreads();
+  }
+  if (i < t.z) {
+    cnt = w.N.ncodes[node];
+    w.N.slot_cnt[node] = (uint8_t)cnt;
+  }
   int total;
   block_excl_scan(cnt, sm, total);
   if (threadIdx.x == 0) w.N.tile_sum[t.w] = total;
@@ -2152,22 +2167,30 @@ static inline void rec(cudaEvent_t *ev, int k, int after, cudaStream_t st) {
   if (ev) cudaEventRecord(ev[2 * k + after], st);
 }
 
-// Threads per CTA of the recount, whose warps share out a node tile's dirty
-// nodes.  New labels fall on a few tiles, so while the whole grid fits the
-// chip at 512 threads (4 CTAs on each of 152 SMs) the extra warps shorten the
-// chain (16,000-particle scene 15.7 -> 8.6 us, 477k particles 12.2 -> 10.2);
-// beyond that most CTAs have no dirty node and the smaller CTA is cheaper
-// (256-scene batch 47 us at 128 threads, 91 at 512).
-static int recount_threads(const LaunchSet &ls) { return ls.n_ntiles <= 4 * 152 ? 512 : ls.ntile_size; }
+// New labels fall on a few node tiles.  While the tiles are too few to fill
+// the chip, their dirty nodes are shared out over several CTAs per tile in a
+// launch of their own; beyond that (four CTAs on each of 152 SMs) a tile's own
+// CTA recounts them.  16,000-particle scene 15.7 us in one launch -> 5 in two; 3,887 nodes
+// all recounted after a restore 24 -> 7 us; the 256-scene batch takes 47 us
+// in one launch.
+#define RECOUNT_CTAS (4 * 152)
+template <int KR>
+static void launch_count(const World &w, const LaunchSet &ls, cudaStream_t st, int force) {
+  if (ls.n_ntiles > RECOUNT_CTAS) {
+    k_slot_count<KR, false><<<ls.n_ntiles, ls.ntile_size, 0, st>>>(w, ls, force);
+    return;
+  }
+  const int parts = min(max(RECOUNT_CTAS / ls.n_ntiles, 1), 16);
+  k_recount<KR><<<dim3((unsigned)ls.n_ntiles, (unsigned)parts), 256, 0, st>>>(w, ls, force);
+  k_slot_count<KR, true><<<ls.n_ntiles, ls.ntile_size, 0, st>>>(w, ls, force);
+}
 
 static cudaError_t launch_rebuild(const World &w, const LaunchSet &ls, cudaStream_t st, int force,
                                   cudaEvent_t *ev) {
   if (ls.n_ntiles == 0) return cudaSuccess;
   rec(ev, 6, 0, st);
-  if (ls.ppc16)
-    k_slot_count<16><<<ls.n_ntiles, recount_threads(ls), 0, st>>>(w, ls, force);
-  else
-    k_slot_count<8><<<ls.n_ntiles, recount_threads(ls), 0, st>>>(w, ls, force);
+  if (ls.ppc16) launch_count<16>(w, ls, st, force);
+  else launch_count<8>(w, ls, st, force);
   rec(ev, 6, 1, st);
   rec(ev, 9, 0, st);
   k_brick_tiles<<<(ls.n_btiles + BTILE_WARPS - 1) / BTILE_WARPS, 32 * BTILE_WARPS, 0, st>>>(w, ls, force);
