@@ -132,51 +132,49 @@ __device__ __forceinline__ void couple_T(int ns, const uint2 *codes, const float
     for (int c = 0; c < NC; ++c) S[b][c] = out[b][c];
 }
 
-// Particle range [p0, p1) of stencil cell l of scene-local node li (l < 27:
-// ox = l % 3, oy = l / 3 % 3, oz = l / 9, the base cell li - (ox, oy, oz)).
-__device__ __forceinline__ void stencil_cell(const World &w, const DevScene &sc, int li, int l, int &p0, int &p1) {
-  p0 = p1 = 0;
-  if (l >= 27) return;
-  const int ix = li % sc.nn[0], iy = (li / sc.nn[0]) % sc.nn[1], iz = li / (sc.nn[0] * sc.nn[1]);
-  const int bx = ix - l % 3, by = iy - (l / 3) % 3, bz = iz - l / 9;
-  if (bx < 0 || by < 0 || bz < 0 || bx >= sc.nb[0] || by >= sc.nb[1] || bz >= sc.nb[2]) return;
-  const int *cs = w.N.cell_start + sc.cell_begin + cell_at(sc, bx, by, bz);
-  p0 = cs[0];
-  p1 = cs[1];
-}
-
-// Walk a cell's particles of code c in pool order, U at a time: the NV values
-// val[.][particle - pb] and the weights of U particles are read before any is
-// used (one after the other, the reads' latency set the kernel's time), then
-// fn(values, N, grad N) takes them in order.
-template <int U, int NV, class Fn>
-__device__ __forceinline__ void walk_cell(const World &w, const DevScene &sc, int l, int p0, int p1, uint2 c,
+// Walk the particles of code c in the stencil of scene-local node li with the
+// warp's lanes: for each of the 9 (y, z) rows of base cells the particles of
+// its three cells lie together in the pool (in two pieces where the row
+// crosses a brick), and consecutive lanes take consecutive particles, so the
+// reads of the NV values val[.][particle - p_begin] coalesce.  (A lane per
+// cell touched 27 sectors with every read, and the kernels were bound by
+// that.)  fn(values, N, grad N) for each.
+template <int NV, class Fn>
+__device__ __forceinline__ void walk_rows(const World &w, const DevScene &sc, int li, int lane, uint2 c,
                                           float *const (&val)[NV], Fn fn) {
-  const int ox = l % 3, oy = (l / 3) % 3, oz = l / 9, pb = sc.p_begin;
-  for (int q = p0; q < p1; q += U) {
-    bool on[U];
-    float f[U][3], v[U][NV];
+  const int ix = li % sc.nn[0], iy = (li / sc.nn[0]) % sc.nn[1], iz = li / (sc.nn[0] * sc.nn[1]);
+  const int *cs = w.N.cell_start + sc.cell_begin;
+  const int x0 = max(ix - 2, 0), x1 = min(ix, sc.nb[0] - 1);
+  const int xs = min(x0 | 3, x1);  // last cell of the first piece
+  const int pb = sc.p_begin;
+  for (int oz = 0; oz < 3; ++oz)
+    for (int oy = 0; oy < 3; ++oy) {
+      const int by = iy - oy, bz = iz - oz;
+      if (by < 0 || bz < 0 || by >= sc.nb[1] || bz >= sc.nb[2] || x0 > x1) continue;
+      const int a0 = cs[cell_at(sc, x0, by, bz)], a1 = cs[cell_at(sc, xs, by, bz) + 1];
+      int b0 = 0, b1 = 0;
+      if (xs < x1) {
+        b0 = cs[cell_at(sc, xs + 1, by, bz)];
+        b1 = cs[cell_at(sc, x1, by, bz) + 1];
+      }
+      const int na = a1 - a0, n = na + b1 - b0;
+      for (int i = lane; i < n; i += 32) {
+        const int p = i < na ? a0 + i : b0 + (i - na);
+        float v[NV];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int p = min(q + u, p1 - 1);
-      on[u] = q + u < p1 && w.P.s1[p] == c.x && w.P.s2[p] == c.y;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) f[u][a] = w.P.fx[a][p];
-#pragma unroll
-      for (int k = 0; k < NV; ++k) v[u][k] = val[k][p - pb];
+        for (int k = 0; k < NV; ++k) v[k] = val[k][p - pb];
+        const float f0 = w.P.fx[0][p], f1 = w.P.fx[1][p], f2 = w.P.fx[2][p];
+        const int ox = ix - (int)(w.P.base[p] & 1023u);
+        if (w.P.s1[p] != c.x || w.P.s2[p] != c.y) continue;
+        float wx, wy, wz, dx, dy, dz;
+        wgt(ox, f0, wx, dx);
+        wgt(oy, f1, wy, dy);
+        wgt(oz, f2, wz, dz);
+        const float N = wx * wy * wz;
+        const float gN[3] = {dx * wy * wz * sc.inv_dx, wx * dy * wz * sc.inv_dx, wx * wy * dz * sc.inv_dx};
+        fn(v, N, gN);
+      }
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!on[u]) continue;
-      float wx, wy, wz, dx, dy, dz;
-      wgt(ox, f[u][0], wx, dx);
-      wgt(oy, f[u][1], wy, dy);
-      wgt(oz, f[u][2], wz, dz);
-      const float N = wx * wy * wz;
-      const float gN[3] = {dx * wy * wz * sc.inv_dx, wx * dy * wz * sc.inv_dx, wx * wy * dz * sc.inv_dx};
-      fn(v[u], N, gN);
-    }
-  }
 }
 
 // sum over the warp's lanes in a fixed butterfly order (every lane gets it)
@@ -186,8 +184,8 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// The per-node adjoint kernels run one warp per node: lane l < 27 walks the
-// node's particles in stencil cell l, the lanes' sums are combined by
+// The per-node adjoint kernels run one warp per node: the lanes walk the
+// node's particles (walk_rows), their sums are combined by
 // warp_sum, one pass per logical grid of the node (codes fixed), and lane 0
 // applies the transposed coupling to the node's slot sums.
 constexpr int kAdjNodesPerBlock = kAdjBlock / 32;
@@ -204,12 +202,10 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_musl(World w, AdjWork aw) {
   const int off = w.N.slot_off[node], ns = w.N.slot_cnt[node];
   if (ns == 0) return;
   const float dt = sc.dt, mp = sc.mp;
-  int p0, p1;
-  stencil_cell(w, sc, li, lane, p0, p1);
   for (int a = 0; a < ns; ++a) {
     const uint2 ca = w.S.code[off + a];
     float m = 0.f, S0 = 0.f, S1 = 0.f, S2 = 0.f;
-    walk_cell<4>(w, sc, lane, p0, p1, ca, aw.Fb, [&](const float *F, float N, const float *gN) {
+    walk_rows(w, sc, li, lane, ca, aw.Fb, [&](const float *F, float N, const float *gN) {
       m += N * mp;
       S0 += dt * (F[0] * gN[0] + F[1] * gN[1] + F[2] * gN[2]);
       S1 += dt * (F[3] * gN[0] + F[4] * gN[1] + F[5] * gN[2]);
@@ -296,14 +292,12 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_g2p(World w, AdjWork aw) {
   const int rel = off - sc.slot_begin;
   const float dt = sc.dt, beta = sc.beta;
   float *const val[6] = {aw.v1b[0], aw.v1b[1], aw.v1b[2], aw.xb[0], aw.xb[1], aw.xb[2]};
-  int p0, p1;
-  stencil_cell(w, sc, li, lane, p0, p1);
   for (int a = 0; a < ns; ++a) {
     const uint2 ca = w.S.code[off + a];
     const float ma = aw.sm[rel + a];
     float S[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (ma > 0.f)
-      walk_cell<4>(w, sc, lane, p0, p1, ca, val, [&](const float *v, float N, const float *) {
+      walk_rows(w, sc, li, lane, ca, val, [&](const float *v, float N, const float *) {
         const float q = N / ma;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
