@@ -154,11 +154,16 @@ struct WorldH {
   int n_btiles = 0, n_ntiles = 0;
   std::map<int, cudaGraphExec_t> graphs;
 
+  // The pools are pieces of one allocation (some 80 of their own took 1 ms of
+  // a scene's creation and release): world_alloc walks them twice, first with
+  // no slab to add up their sizes.
+  char *slab = nullptr;
+  size_t slab_used = 0;
   template <class T>
   T *get(int64_t count) {
-    void *p = al.alloc(sizeof(T) * (size_t)std::max<int64_t>(count, 1));
-    if (p) allocs.push_back(p);
-    return (T *)p;
+    const size_t at = slab_used;
+    slab_used += (sizeof(T) * (size_t)std::max<int64_t>(count, 1) + 255) & ~size_t(255);
+    return (T *)(slab + at);
   }
   void drop_graphs() {
     for (auto &kv : graphs) cudaGraphExecDestroy(kv.second);
@@ -187,24 +192,18 @@ int rebase_candidate(int e, int from, int to) {
   return (int)((u & 0x80000000u) | q);
 }
 
-int world_alloc(WorldH *W) {
+void carve_pools(WorldH *W) {
   const int64_t P = W->cap_p;
   PPool &pp = W->w.P;
-  bool ok = true;
   auto F = [&](float *&ptr, int64_t c) {
     ptr = W->get<float>(c);
-    ok &= ptr != nullptr;
   };
   auto U = [&](uint32_t *&ptr, int64_t c) {
     ptr = W->get<uint32_t>(c);
-    ok &= ptr != nullptr;
   };
   auto I = [&](int *&ptr, int64_t c) {
     ptr = W->get<int>(c);
-    ok &= ptr != nullptr;
   };
-  cudaError_t ie = bm_kernels_init();
-  if (ie != cudaSuccess) return fail(BM_E_CUDA, std::string("kernel set-up: ") + cudaGetErrorString(ie));
   for (int a = 0; a < 3; ++a) {
     F(pp.fx[a], P);
     F(pp.x[a], P);
@@ -219,32 +218,26 @@ int world_alloc(WorldH *W) {
   }
   F(pp.D, P);
   pp.tflag = W->get<uint8_t>(P);
-  ok &= pp.tflag != nullptr;
   U(pp.base, P);
   U(pp.s1, P);
   U(pp.s2, P);
   I(pp.perm, P);
   pp.lpos = W->get<uint16_t>(P);
   pp.cid = W->get<uint8_t>(P);
-  ok &= pp.lpos && pp.cid;
   pp.pend = W->get<uint8_t>(P);
-  ok &= pp.pend != nullptr;
   if (W->pair) {
     I(pp.hkey, P);
     I(pp.horder, P);
     pp.hent = W->get<float4>(P);
-    ok &= pp.hent != nullptr;
     U(pp.hbase, P);
     pp.hcell = W->get<unsigned long long>(P);
     pp.hentk = W->get<unsigned long long>(P);
-    ok &= pp.hcell && pp.hentk;
     for (int b = 0; b < 2; ++b) {
       I(pp.hist_partner[b], P * BM_HIST);
       F(pp.hist_u[b], P * BM_HIST * 3);
     }
     I(pp.nbr, P * BM_NBR);
     pp.nbr_n = W->get<uint8_t>(P);
-    ok &= pp.nbr_n != nullptr;
     for (int a = 0; a < 3; ++a) F(pp.xb[a], P);
     int nb = 1024;
     while (nb < 2 * P && nb < (1 << 28)) nb <<= 1;
@@ -261,16 +254,13 @@ int world_alloc(WorldH *W) {
   np.slot_cnt = W->get<uint8_t>(W->cap_node);
   np.ncodes = W->get<uint8_t>(W->cap_node);
   np.dirty = W->get<uint8_t>(W->cap_node);
-  ok &= np.slot_cnt && np.ncodes && np.dirty;
   np.tmp_codes = W->get<uint2>(W->cap_node * BM_MAXS);
-  ok &= np.tmp_codes != nullptr;
   I(np.tile_sum, W->cap_ntile);
   SPool &sp = W->w.S;
   sp.vold = W->get<float4>(W->cap_slot);
   sp.vnew = W->get<float4>(W->cap_slot);
   sp.vstar = W->get<float4>(W->cap_slot);
   sp.code = W->get<uint2>(W->cap_slot);
-  ok &= sp.vold && sp.vnew && sp.vstar && sp.code;
   BPool &bp = W->w.B;
   bp.pm = W->get<float4>(W->cap_ppool);
   bp.pd = W->get<float4>(W->cap_ppool);
@@ -282,7 +272,6 @@ int world_alloc(WorldH *W) {
   bp.bcode = W->get<uint2>(W->cap_brick * BM_BRICK_CODES);
   bp.binfo = W->get<int>(W->cap_brick);
   bp.bdirty = W->get<uint8_t>(W->cap_brick);
-  ok &= bp.pm && bp.pd && bp.poff && bp.ptot && bp.tdesc && bp.tgoff && bp.lf && bp.bcode && bp.binfo && bp.bdirty;
   W->w.scenes = W->get<DevScene>(W->cap_scenes);
   W->w.wpart = W->get<double>(W->cap_brick * 6);
   W->w.whist = W->get<double>(std::max<int64_t>(W->cap_hist, 1) * 6);
@@ -291,9 +280,17 @@ int world_alloc(WorldH *W) {
   W->d_scene_ids = W->get<int>(W->cap_scenes);
   W->d_slot_ids = W->get<int>(W->cap_scenes);
   W->d_stage = W->get<double>((int64_t)W->cap_scenes * 18);
-  ok &= W->w.scenes && W->w.wpart && W->w.whist && W->d_btiles && W->d_ntiles && W->d_scene_ids &&
-        W->d_slot_ids && W->d_stage;
-  if (!ok) return fail(BM_E_OOM, "device allocation failed");
+}
+
+int world_alloc(WorldH *W) {
+  cudaError_t ie = bm_kernels_init();
+  if (ie != cudaSuccess) return fail(BM_E_CUDA, std::string("kernel set-up: ") + cudaGetErrorString(ie));
+  carve_pools(W);
+  W->slab = (char *)W->al.alloc(W->slab_used);
+  if (!W->slab) return fail(BM_E_OOM, "device allocation failed");
+  W->allocs.push_back(W->slab);
+  W->slab_used = 0;
+  carve_pools(W);
   W->rp.init(W->cap_p);
   W->rcell.init(W->cap_cell);
   W->rnode.init(W->cap_node);
