@@ -506,68 +506,109 @@ __device__ __forceinline__ void particle_base(uint32_t b, int &bx, int &by, int 
   bz = (int)((b >> 20) & 1023u);
 }
 
-// The node tile of one brick: for each of its 6x6x6 nodes the first tile
-// slot (the node's logical grids laid out node by node in each node's own
-// slot order), the slot count and the node's first pool slot.  A tile holds
-// at most 216 x BM_MAXS slots; shared-memory working sets cover windows of
-// TSCAP slots at a time.
-struct Tile {
-  uint16_t lo[TN];
-  uint8_t cnt[TN];
-  int goff[TN];
-  int total;
-};
-
 __device__ __forceinline__ void brick_coords(const DevScene &sc, int lb, int &c0x, int &c0y, int &c0z) {
   c0x = (lb % sc.nbr[0]) * BR;
   c0y = ((lb / sc.nbr[0]) % sc.nbr[1]) * BR;
   c0z = (lb / (sc.nbr[0] * sc.nbr[1])) * BR;
 }
 
-// Cooperative load of a brick's tile (all threads; ends with a barrier).  The
-// per-node slot counts and first tile slots come from the descriptor the
-// slot rebuild wrote for this brick; the nodes' first pool slots from the
-// slot table.  Returns (in every thread) whether every tile node holds at
-// most one logical grid; the kernels then keep the tile's values by node
-// (entry t for tile node t) instead of by tile slot.
-__device__ bool tile_load(const World &w, const DevScene &sc, int brick, int c0x, int c0y, int c0z,
-                          Tile &T) {
-  bool single = true;
-  for (int t = threadIdx.x; t < TN; t += blockDim.x) {
-    const int d = w.B.tdesc[(size_t)brick * TN + t];
-    const int cnt = d >> 16;
-    const int off = w.B.tgoff[(size_t)brick * TN + t];  // valid where cnt > 0
-    T.lo[t] = (uint16_t)(d & 0xffff);
-    T.cnt[t] = (uint8_t)cnt;
-    T.goff[t] = off;
-    single &= cnt <= 1;
+// --------------------------------------------------------------------------
+// The node tile of one brick: for each of its 6x6x6 nodes the first pool
+// slot, the first tile slot (the node's logical grids laid out node by node
+// in each node's own slot order) and the slot count; and, for the codes of
+// the brick's particles (BPool::bcode; PPool::cid is a particle's index in
+// the list), the slot (index at its node) of each code at each node.  Looked
+// up in this table, a particle of a brick at a cut finds its 27 slots with
+// one byte each; comparing its code with the slots' codes took two to four
+// 8-byte reads a node.
+// --------------------------------------------------------------------------
+#define BRICK_SLOT_CODES 8  // codes with a slot table in shared memory (further codes compare)
+#define NOSLOT 0xff
+
+struct BrickTile {
+  uint2 bcode[BM_BRICK_CODES];
+  int goff[TN];
+  uint16_t lo[TN];
+  uint8_t cnt[TN];
+  uint8_t slot[BRICK_SLOT_CODES][TN];
+};
+
+// slot of the brick's code b at tile node t (an index at the node), or NOSLOT
+__device__ __forceinline__ int brick_slot(const World &w, const BrickTile &T, int nbc, int b, int t) {
+  if (nbc <= BRICK_SLOT_CODES) return T.slot[b][t];
+  const uint2 k = T.bcode[b];
+  for (int a = 0; a < T.cnt[t]; ++a) {
+    const uint2 c = w.S.code[T.goff[t] + a];
+    if (c.x == k.x && c.y == k.y) return a;
   }
-  if (threadIdx.x == 0) T.total = w.B.ptot[brick];
-  return __syncthreads_and(single) != 0;
+  return NOSLOT;
 }
 
-// tile slot holding code (s1, s2) at tile node t, or -1.  Nodes with several
-// logical grids compare against the tile's codes in shared memory when the
-// tile fits the window (codes != nullptr), else against the pool's codes.
-__device__ __forceinline__ int tile_slot(const World &w, const Tile &T, const uint2 *codes, int t,
-                                         uint32_t s1, uint32_t s2) {
-  const int n = T.cnt[t];
-  const int lo = T.lo[t];
-  if (n == 1) return lo;
-  if (codes) {
-    for (int a = 0; a < n; ++a) {
-      const uint2 c = codes[lo + a];
-      if (c.x == s1 && c.y == s2) return lo + a;
-    }
-    return -1;
+// Tile and codes of brick `brick` (nt threads); ends without a barrier.
+__device__ __forceinline__ void brick_tile(const World &w, int brick, int nbc, BrickTile &T, int nt) {
+  const int tid = threadIdx.x;
+  for (int t = tid; t < TN; t += nt) {
+    const int d = w.B.tdesc[(size_t)brick * TN + t];
+    T.lo[t] = (uint16_t)(d & 0xffff);
+    T.cnt[t] = (uint8_t)(d >> 16);
+    T.goff[t] = w.B.tgoff[(size_t)brick * TN + t];  // valid where the count is not zero
   }
-  const int off = T.goff[t];
-  for (int a = 0; a < n; ++a) {
-    const uint2 c = w.S.code[off + a];
-    if (c.x == s1 && c.y == s2) return lo + a;
-  }
-  return -1;
+  if (tid < nbc) T.bcode[tid] = w.B.bcode[(size_t)brick * BM_BRICK_CODES + tid];
 }
+
+// Slot table of a brick with several codes or slots (after a barrier on
+// brick_tile).  Slots whose code no particle of the brick carries get zero
+// partial sums, mass and momentum and with FORCE the force too (pbase < 0:
+// none are written).
+template <bool FORCE>
+__device__ __forceinline__ void brick_slots(const World &w, BrickTile &T, int nbc, int pbase, int nt) {
+  for (int t = threadIdx.x; t < TN; t += nt) {
+    const int n = T.cnt[t], g = T.goff[t];
+    if (nbc <= BRICK_SLOT_CODES)
+      for (int b = 0; b < nbc; ++b) T.slot[b][t] = NOSLOT;
+    for (int a = 0; a < n; ++a) {
+      const uint2 c = w.S.code[g + a];
+      int id = -1;
+      for (int b = 0; b < nbc; ++b)
+        if (T.bcode[b].x == c.x && T.bcode[b].y == c.y) id = b;
+      if (id >= 0) {
+        if (nbc <= BRICK_SLOT_CODES) T.slot[id][t] = (uint8_t)a;
+      } else if (pbase >= 0) {
+        const size_t e = (size_t)pbase + T.lo[t] + a;
+        w.B.pm[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (FORCE) w.B.pd[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  }
+}
+
+// What a brick kernel needs to know of its brick (of at most `places` particles).
+struct BrickInfo {
+  int nbc;        // distinct codes of the brick's particles
+  bool single;    // no tile node holds several logical grids
+  bool uniform;   // and at most one code: one pass, no code tests
+  bool mask;      // empty places or several codes
+  int pbase;      // partial-sum range (negative: pool overflow)
+  int npass;      // a brick without particles still runs one pass: it writes zeros to its tile
+  __device__ __forceinline__ BrickInfo(const World &w, const int4 &bt, int places) {
+    const int info = w.B.binfo[bt.y];
+    nbc = info & 0xff;
+    single = (info >> 8) != 0;
+    uniform = single && nbc <= 1;
+    mask = bt.w < places || nbc > 1;
+    pbase = w.B.poff[bt.y];
+    npass = max(nbc, 1);
+  }
+  // slot of pass b's code at tile node t (an index at the node), or NOSLOT
+  __device__ __forceinline__ int slot(const World &w, const BrickTile &T, int b, int t) const {
+    return T.cnt[t] == 0 ? NOSLOT : uniform ? 0 : nbc == 0 ? NOSLOT : brick_slot(w, T, nbc, b, t);
+  }
+  // partial-sum entry of that slot, or -1
+  __device__ __forceinline__ long long entry(const World &w, const BrickTile &T, int b, int t) const {
+    const int sl = slot(w, T, b, t);
+    return sl == NOSLOT || pbase < 0 ? -1 : (long long)pbase + T.lo[t] + sl;
+  }
+};
 
 // --------------------------------------------------------------------------
 // Per-particle work ahead of P2G (one thread per particle, inside the P2G

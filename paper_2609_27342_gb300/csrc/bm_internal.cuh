@@ -128,7 +128,7 @@ struct PPool {
   uint8_t *pend;            // side digit assigned this substep (0: none), committed by k_fupd
   int *perm;                // pool index -> caller's particle index
   uint16_t *lpos;           // lattice scenes: the particle's place in its brick (bm_lat_place)
-  uint8_t *cid;             // lattice scenes: index of the particle's code in its brick's list
+  uint8_t *cid;             // index of the particle's code in its brick's list (BPool::bcode)
   // pair contact
   int *hkey;                // bucket of each particle's current-configuration cell
   int *horder;              // particles ordered by bucket, by pool index inside a bucket
@@ -168,8 +168,7 @@ struct BPool {              // brick-tile partial sums
   int *ptot;                // slots in each brick's tile
   int *tdesc;               // [brick * BM_TILE_NODES]: first tile slot | slot count << 16
   int *tgoff;               // [brick * BM_TILE_NODES]: first pool slot of each tile node
-  // lattice scenes
-  float *lf;                // [brick * 24]: fractional offset of the 8 particle planes per axis
+  float *lf;                // lattice scenes, [brick * 24]: fractional offset of the 8 particle planes per axis
   uint2 *bcode;             // [brick * BM_BRICK_CODES]: distinct codes of the brick's particles
   int *binfo;               // number of those codes | 1 << 8 when no tile node holds several slots
   uint8_t *bdirty;          // a particle of the brick gained a label since its codes were listed

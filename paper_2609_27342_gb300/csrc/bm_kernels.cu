@@ -38,68 +38,30 @@ namespace {
 // k_p2g_brick: the brick's share of P2G (Eq. 2) into its node tile, per
 // logical grid, from the particles' A, J, v staged in shared memory.
 // --------------------------------------------------------------------------
-// Distinct codes of the brick's particles (one warp, lane L holding cells 2L
-// and 2L + 1): the next code not yet listed is taken from the lowest lane
-// that has one, so the list is in first-occurrence order over the cells.
-template <int PPC>
-__device__ void brick_codes(const uint32_t *ps1, const uint32_t *ps2, const uint8_t (*ccode)[PPC],
-                            const uint8_t *ncode, uint2 *bcode, int *nbcode, unsigned int *err) {
-  const int lane = threadIdx.x & 31;
-  const int c0 = 2 * lane;
-  const int tot = ncode[c0] + ncode[c0 + 1];
-  int cur = 0, n = 0;
-  auto code_of = [&](int q, uint32_t &a, uint32_t &b) {
-    const int c = q < ncode[c0] ? c0 : c0 + 1;
-    const int j = ccode[c][q < ncode[c0] ? q : q - ncode[c0]];
-    const int k = pic(j, c);
-    a = ps1[k];
-    b = ps2[k];
-  };
-  for (;;) {
-    // advance past candidates already listed
-    uint32_t a = 0, b = 0;
-    while (cur < tot) {
-      code_of(cur, a, b);
-      bool seen = false;
-      for (int q = 0; q < n; ++q)
-        if (bcode[q].x == a && bcode[q].y == b) {
-          seen = true;
-          break;
-        }
-      if (!seen) break;
-      ++cur;
-    }
-    const unsigned pend = __ballot_sync(FULL, cur < tot);
-    if (!pend) break;
-    const int src = __ffs(pend) - 1;
-    const uint32_t ka = __shfl_sync(FULL, a, src), kb = __shfl_sync(FULL, b, src);
-    if (n < BM_BRICK_CODES) {
-      if (lane == 0) bcode[n] = make_uint2(ka, kb);
-      __syncwarp();
-    } else if (lane == 0) {
-      atomicOr(err, BM_ERRBIT_SLOT_OVERFLOW);
-    }
-    ++n;
-    if (n > BM_BRICK_CODES) break;
-  }
-  if (lane == 0) *nbcode = min(n, BM_BRICK_CODES);
-}
-
 template <int PPC>
 struct K2S {
-  Tile T;
+  BrickTile T;
   float part[18][PPC * BR3];   // the brick's particles (fx, v, A, J), [particle-in-cell][cell]
   float sz[7][3][TZ];          // one pass's (node, z-offset) sums
-  uint32_t ps1[PPC * BR3], ps2[PPC * BR3];
-  uint2 bcode[BM_BRICK_CODES]; // distinct codes of the brick's particles
+  unsigned long long cmask[BR3];  // several codes: which of the brick's codes each cell's particles carry
   float red[6][BT / 32];       // wrench partials of the warps
-  uint8_t ccode[BR3][PPC];  // distinct codes of each cell: particle-in-cell index of the
-                            // first particle with each code (first-occurrence order)
-  uint8_t ncode[BR3];
   int cs[BR3 + 1];
-  int maxcodes;
-  int nbcode;
+  uint8_t pid[PPC * BR3];      // several codes: code index of each particle
 };
+
+// Which of the brick's codes each cell's particles carry (threads of z-offset
+// 0), from the [particle-in-cell][cell] staging of the code indices.
+__device__ __forceinline__ void cell_codes(const uint8_t *pid, const int *cs, unsigned long long *cmask) {
+  const int c = threadIdx.x;
+  if (c >= BR3) return;
+  const int n = cs[c + 1] - cs[c];
+  unsigned long long m = 0;
+  for (int j = 0; j < n; ++j) {
+    const int b = pid[pic(j, c)];
+    if (b < BM_BRICK_CODES) m |= 1ull << b;
+  }
+  cmask[c] = m;
+}
 
 // The brick's particles into shared memory, transposed to
 // [particle-in-cell][cell] so that the (cell, z-offset) threads read
@@ -107,8 +69,8 @@ struct K2S {
 // that pre_particle computes from x, v, F, D, u_t and the codes.  The caller
 // provides the barrier that publishes it.
 template <int PPC, bool INELASTIC>
-__device__ void stage_particles(const World &w, const DevScene &sc, const int4 &bt, int c0x, int c0y, int c0z,
-                                K2S<PPC> &S, float wr[6], bool &clamped, bool &anyc) {
+__device__ void stage_particles(const World &w, const DevScene &sc, const int4 &bt, bool coded, K2S<PPC> &S,
+                                float wr[6], bool &clamped, bool &anyc) {
   const PPool &P = w.P;
   // each thread fetches its next particle's flag one iteration ahead, so the
   // loads of D and u_t it gates do not wait on it
@@ -119,10 +81,11 @@ __device__ void stage_particles(const World &w, const DevScene &sc, const int4 &
     if (i + (int)blockDim.x < bt.w) tf_next = P.tflag[p + blockDim.x];
     const float x[3] = {P.x[0][p], P.x[1][p], P.x[2][p]};
     const float v[3] = {P.v[0][p], P.v[1][p], P.v[2][p]};
-    const uint32_t s1 = P.s1[p], s2 = P.s2[p];
+    const int id = P.cid[p];
+    const uint2 code = id < BM_BRICK_CODES ? S.T.bcode[id] : make_uint2(0u, 0u);
     const float f0 = P.fx[0][p], f1 = P.fx[1][p], f2 = P.fx[2][p];
     float A[9], J[3];
-    pre_particle<INELASTIC>(sc, P, p, tf, x, v, s1, s2, A, J, wr, clamped, anyc);
+    pre_particle<INELASTIC>(sc, P, p, tf, x, v, code.x, code.y, A, J, wr, clamped, anyc);
     const int c = cell_of(S.cs, i);
     const int si = pic(i - S.cs[c], c);
     S.part[0][si] = f0;
@@ -136,77 +99,8 @@ __device__ void stage_particles(const World &w, const DevScene &sc, const int4 &
     S.part[15][si] = J[0];
     S.part[16][si] = J[1];
     S.part[17][si] = J[2];
-    S.ps1[si] = s1;
-    S.ps2[si] = s2;
+    if (coded) S.pid[si] = (uint8_t)id;
   }
-}
-
-// distinct codes of each cell, once per cell (threads of z-offset 0), from
-// the [particle-in-cell][cell] staging of the codes: each code is kept as the
-// particle-in-cell index of its first particle.
-template <int PPC>
-__device__ __forceinline__ void cell_codes(const uint32_t *s1, const uint32_t *s2, const int *cs,
-                                           uint8_t (*ccode)[PPC], uint8_t *ncode, int *maxcodes) {
-  const int c = threadIdx.x;
-  if (c >= BR3) return;
-  const int n = cs[c + 1] - cs[c];
-  int cnt = 0;
-  for (int j = 0; j < n; ++j) {
-    const int k = pic(j, c);
-    const uint32_t a = s1[k], b = s2[k];
-    bool seen = false;
-    for (int q = 0; q < cnt; ++q) {
-      const int kq = pic(ccode[c][q], c);
-      if (s1[kq] == a && s2[kq] == b) {
-        seen = true;
-        break;
-      }
-    }
-    if (!seen) ccode[c][cnt++] = (uint8_t)j;
-  }
-  ncode[c] = (uint8_t)cnt;
-  atomicMax(maxcodes, cnt);
-}
-
-// Whether cell c holds particles with code (k1, k2), and whether they are
-// all of the cell's particles.
-template <int PPC>
-__device__ __forceinline__ bool cell_has_code(const uint32_t *ps1, const uint32_t *ps2,
-                                              const uint8_t (*ccode)[PPC], const uint8_t *ncode, int c,
-                                              uint32_t k1, uint32_t k2) {
-  for (int q = 0; q < ncode[c]; ++q) {
-    const int k = pic(ccode[c][q], c);
-    if (ps1[k] == k1 && ps2[k] == k2) return true;
-  }
-  return false;
-}
-
-// Tile slot of node t holding code (k1, k2) as an index into the node's
-// slots, or -1; `uniform`: one code in the brick and one slot per node.
-// tcodes: the tile's slot codes in shared memory (by tile slot), or null to
-// read them from the slot pool.
-__device__ __forceinline__ uint2 tile_code(const World &w, const Tile &T, const uint2 *tcodes, int t, int a) {
-  return tcodes ? tcodes[T.lo[t] + a] : w.S.code[T.goff[t] + a];
-}
-
-__device__ __forceinline__ int node_slot_of(const World &w, const Tile &T, const uint2 *tcodes, int t,
-                                            bool uniform, uint32_t k1, uint32_t k2) {
-  const int n = T.cnt[t];
-  if (uniform) return n > 0 ? 0 : -1;
-  for (int a = 0; a < n; ++a) {
-    const uint2 c = tile_code(w, T, tcodes, t, a);
-    if (c.x == k1 && c.y == k2) return a;
-  }
-  return -1;
-}
-
-// In the first pass over a multi-code brick, the tile slots whose code no
-// particle of the brick carries get zero partial sums (every other slot is
-// written by the pass of its code).
-__device__ __forceinline__ bool code_listed(const uint2 *bcode, int n, uint2 c) {
-  for (int q = 0; q < n; ++q)
-    if (bcode[q].x == c.x && bcode[q].y == c.y) return true;
-  return false;
 }
 
 template <int PPC, int MB, bool INELASTIC>
@@ -219,32 +113,23 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
   if (sc.frozen || sc.lattice) return;
   const int tid = threadIdx.x;
   const int lb = bt.y - sc.brick_begin;
-  int c0x, c0y, c0z;
-  brick_coords(sc, lb, c0x, c0y, c0z);
+  const BrickInfo B(w, bt, PPC * BR3);
+  const bool several = B.nbc > 1;
   const int *csg = w.N.cell_start + sc.cell_begin + lb * BR3;
   for (int i = tid; i <= BR3; i += BT) S.cs[i] = csg[i] - bt.z;
-  if (tid == 0) S.maxcodes = 0;
+  brick_tile(w, bt.y, B.nbc, S.T, BT);
   __syncthreads();
-  // the particles (with contact, labels and stress) and the tile descriptors
-  // load together
   float wr[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   bool clamped = false, anyc = false;
-  stage_particles<PPC, INELASTIC>(w, sc, bt, c0x, c0y, c0z, S, wr, clamped, anyc);
+  stage_particles<PPC, INELASTIC>(w, sc, bt, several, S, wr, clamped, anyc);
   if (clamped) atomicOr(&scm.err, BM_ERRBIT_INVERTED);
-  const bool single = tile_load(w, sc, bt.y, c0x, c0y, c0z, S.T);
-  if (sc.has_blade) brick_wrench(w, bt.y, wr, anyc, S.red);  // (its barriers publish the copy too)
-  cell_codes<PPC>(S.ps1, S.ps2, S.cs, S.ccode, S.ncode, &S.maxcodes);
+  if (!B.uniform) brick_slots<true>(w, S.T, B.nbc, B.pbase, BT);
+  if (sc.has_blade) brick_wrench(w, bt.y, wr, anyc, S.red);
   __syncthreads();
-  // every tile node holds one logical grid (so all the brick's particles
-  // share one code): one pass, no code tests
-  const bool uniform = single && S.maxcodes <= 1;
-  if (!uniform) {
-    if (tid < 32) brick_codes<PPC>(S.ps1, S.ps2, S.ccode, S.ncode, S.bcode, &S.nbcode, &scm.err);
+  if (several) {
+    cell_codes(S.pid, S.cs, S.cmask);
     __syncthreads();
   }
-  // a brick without particles still runs one pass: it writes zeros to its tile
-  const int nbc = uniform ? 1 : S.nbcode;
-  const int npass = max(nbc, 1);
 
   // ---- one pass per code of the brick ----
   // Each thread sums, for its cell and one z-offset, m N, m v N and
@@ -256,13 +141,10 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
   const int c = tid % BR3, oz = tid / BR3;
   const int cx = c & 3, cy = (c >> 2) & 3, cz = c >> 4;
   const int n_c = S.cs[c + 1] - S.cs[c];
-  const int pbase = w.B.poff[bt.y];  // this brick's partial-sum range (negative: pool overflow)
-  for (int b = 0; b < npass; ++b) {
-    const bool coded = b < nbc;  // false only in the single pass of a brick without particles
-    const uint32_t k1 = (uniform || !coded) ? 0u : S.bcode[b].x, k2 = (uniform || !coded) ? 0u : S.bcode[b].y;
-    const bool has = coded && n_c > 0 &&
-                     (uniform || cell_has_code<PPC>(S.ps1, S.ps2, S.ccode, S.ncode, c, k1, k2));
-    const bool filt = !uniform && S.ncode[c] > 1;
+  const unsigned long long codes = several ? S.cmask[c] : 0ull;
+  const bool filt = (codes & (codes - 1)) != 0;  // the cell's particles carry several codes
+  for (int b = 0; b < B.npass; ++b) {
+    const bool has = n_c > 0 && (!several || ((codes >> b) & 1u));
     // two walks over the cell's particles, each reducing its own values, so
     // that fewer sums are live at once: (m N, m v N), then A grad N + N J
     {
@@ -276,7 +158,7 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
       if (has) {
         for (int j = 0; j < n_c; ++j) {
           const int si = pic(j, c);
-          if (filt && (S.ps1[si] != k1 || S.ps2[si] != k2)) continue;
+          if (filt && S.pid[si] != b) continue;
           float wx[3], wy[3], wz, d;
           const float f0 = S.part[0][si], f1 = S.part[1][si], f2 = S.part[2][si];
           bs<0>(f0, wx[0], d); bs<1>(f0, wx[1], d); bs<2>(f0, wx[2], d);
@@ -313,7 +195,7 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
       if (has) {
         for (int j = 0; j < n_c; ++j) {
           const int si = pic(j, c);
-          if (filt && (S.ps1[si] != k1 || S.ps2[si] != k2)) continue;
+          if (filt && S.pid[si] != b) continue;
           float wx[3], dwx[3], wy[3], dwy[3], wz, dwz;
           const float f0 = S.part[0][si], f1 = S.part[1][si], f2 = S.part[2][si];
           bs<0>(f0, wx[0], dwx[0]); bs<1>(f0, wx[1], dwx[1]); bs<2>(f0, wx[2], dwx[2]);
@@ -347,26 +229,15 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
       stage_layer<3, TZ>(S.sz + 4, a, cx, cy, cz, oz);
     }
     __syncthreads();
-    if (pbase >= 0) {
-      for (int t = tid; t < TN; t += BT) {
-        const int n = S.T.cnt[t];
-        if (n == 0) continue;
-        const size_t e0 = (size_t)pbase + S.T.lo[t];
-        if (b == 0 && !uniform)
-          for (int q = 0; q < n; ++q)
-            if (!code_listed(S.bcode, S.nbcode, tile_code(w, S.T, nullptr, t, q))) {
-              w.B.pm[e0 + q] = make_float4(0.f, 0.f, 0.f, 0.f);
-              w.B.pd[e0 + q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        const int sl = coded ? node_slot_of(w, S.T, nullptr, t, uniform, k1, k2) : -1;
-        if (sl < 0) continue;
-        float acc[7];
-        gather_z<7, TZ>(S.sz, t, acc);
-        w.B.pm[e0 + sl] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        w.B.pd[e0 + sl] = make_float4(acc[4], acc[5], acc[6], 0.f);
-      }
+    for (int t = tid; t < TN; t += BT) {
+      const long long e = B.entry(w, S.T, b, t);
+      if (e < 0) continue;
+      float acc[7];
+      gather_z<7, TZ>(S.sz, t, acc);
+      w.B.pm[e] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      w.B.pd[e] = make_float4(acc[4], acc[5], acc[6], 0.f);
     }
-    if (b + 1 < npass) __syncthreads();  // the next pass overwrites the z stage
+    if (b + 1 < B.npass) __syncthreads();  // the next pass overwrites the z stage
   }
 }
 
@@ -577,10 +448,18 @@ __global__ void k_p2g_node(World w, LaunchSet ls) {
 // grid velocities, then the brick's share of the MUSL re-scatter sum m v^{n+1}
 // N per logical grid, committed in the same fixed phase order as P2G.
 // --------------------------------------------------------------------------
+// tile slot of code index id at tile node t, or -1 (a node with one slot holds
+// the code of every particle it touches)
+__device__ __forceinline__ int tile_slot(const World &w, const BrickTile &T, int nbc, int t, int id) {
+  if (T.cnt[t] == 1) return T.lo[t];
+  if (id >= nbc) return -1;
+  const int a = brick_slot(w, T, nbc, id, t);
+  return a == NOSLOT ? -1 : T.lo[t] + a;
+}
+
 template <int PPC>
 struct K4S {
-  Tile T;
-  uint2 codes[TSCAP];
+  BrickTile T;
   union {
     struct {
       float4 tvo[TSCAP];      // v_old xyz, m of the tile slots (G2P)
@@ -590,13 +469,9 @@ struct K4S {
   };
   float pf[3][PPC * BR3];
   float pv[3][PPC * BR3];
-  uint32_t ps1[PPC * BR3], ps2[PPC * BR3];
-  uint2 bcode[BM_BRICK_CODES];  // as in K2S
-  uint8_t ccode[BR3][PPC];
-  uint8_t ncode[BR3];
+  unsigned long long cmask[BR3];  // as in K2S
   int cs[BR3 + 1];
-  int maxcodes;
-  int nbcode;
+  uint8_t pid[PPC * BR3];
 };
 
 template <int PPC, int MB>
@@ -610,15 +485,15 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
   const PPool &P = w.P;
   const int tid = threadIdx.x;
   const int lb = bt.y - sc.brick_begin;
-  int c0x, c0y, c0z;
-  brick_coords(sc, lb, c0x, c0y, c0z);
+  const BrickInfo B(w, bt, PPC * BR3);
+  const bool several = B.nbc > 1, single = B.single;
+  const int total = w.B.ptot[bt.y];
+  const bool in_smem = total <= TSCAP;  // otherwise G2P reads the pool slots directly
   const int *csg = w.N.cell_start + sc.cell_begin + lb * BR3;
   for (int i = tid; i <= BR3; i += BT) S.cs[i] = csg[i] - bt.z;
-  if (tid == 0) S.maxcodes = 0;
-  const bool single = tile_load(w, sc, bt.y, c0x, c0y, c0z, S.T);
-  const int total = S.T.total;
-  const bool in_smem = total <= TSCAP;  // otherwise G2P reads the pool slots directly
-  const uint2 *tcodes = in_smem ? S.codes : nullptr;
+  brick_tile(w, bt.y, B.nbc, S.T, BT);
+  __syncthreads();
+  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, B.pbase, BT);
   if (single) {  // by node: a particle's node t holds its (only) logical grid
     for (int t = tid; t < TN; t += BT) {
       const bool has = S.T.cnt[t] != 0;
@@ -630,7 +505,6 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
     for (int t = tid; t < TN; t += BT) {
       const int n = S.T.cnt[t], lo = S.T.lo[t], g = S.T.goff[t];
       for (int a = 0; a < n; ++a) {
-        S.codes[lo + a] = w.S.code[g + a];  // every slot: the MUSL passes look codes up by slot
         S.tvo[lo + a] = w.S.vold[g + a];
         S.tvn[lo + a] = w.S.vnew[g + a];
       }
@@ -645,7 +519,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
     const int c = cell_of(S.cs, i);
     const int lx = c & 3, ly = (c >> 2) & 3, lz = c >> 4;
     const int si = pic(i - S.cs[c], c);
-    const uint32_t s1 = P.s1[p], s2 = P.s2[p];
+    const int id = several ? P.cid[p] : 0;
     const float f0 = P.fx[0][p], f1 = P.fx[1][p], f2 = P.fx[2][p];
     float wx[3], wy[3], wz[3], d;
     bs<0>(f0, wx[0], d); bs<1>(f0, wx[1], d); bs<2>(f0, wx[2], d);
@@ -685,7 +559,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
           const float wyz = wy[oy] * wz[oz];
 #pragma unroll
           for (int ox = 0; ox < 3; ++ox) {
-            const int s = tile_slot(w, S.T, tcodes, t0 + (oz * TE + oy) * TE + ox, s1, s2);
+            const int s = tile_slot(w, S.T, B.nbc, t0 + (oz * TE + oy) * TE + ox, id);
             const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
             const float4 vo = s >= 0 ? S.tvo[s] : zero, vn = s >= 0 ? S.tvn[s] : zero;
             const float N = vo.w > 0.f ? wx[ox] * wyz : 0.f;
@@ -705,7 +579,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
 #pragma unroll
         for (int ox = 0; ox < 3; ++ox) {
           const int t = ((lz + oz) * TE + (ly + oy)) * TE + (lx + ox);
-          const int s = tile_slot(w, S.T, tcodes, t, s1, s2);
+          const int s = tile_slot(w, S.T, B.nbc, t, id);
           if (s < 0) continue;
           float4 vo, vn;
           {
@@ -734,8 +608,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
     S.pf[0][si] = f0;
     S.pf[1][si] = f1;
     S.pf[2][si] = f2;
-    S.ps1[si] = s1;
-    S.ps2[si] = s2;
+    if (several) S.pid[si] = (uint8_t)id;
   }
   if (bad) atomicOr(&scm.err, BM_ERRBIT_NONFINITE);
   // ---- phase 1: MUSL sums m v^{n+1} N, one pass per code of the brick,
@@ -744,22 +617,14 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
   const int cx = c & 3, cy = (c >> 2) & 3, cz = c >> 4;
   const int n_c = S.cs[c + 1] - S.cs[c];
   __syncthreads();  // G2P reads of the tile velocities are done: the z stage may reuse them
-  cell_codes<PPC>(S.ps1, S.ps2, S.cs, S.ccode, S.ncode, &S.maxcodes);
-  __syncthreads();
-  const bool uniform = single && S.maxcodes <= 1;
-  if (!uniform) {
-    if (tid < 32) brick_codes<PPC>(S.ps1, S.ps2, S.ccode, S.ncode, S.bcode, &S.nbcode, &scm.err);
+  if (several) {
+    cell_codes(S.pid, S.cs, S.cmask);
     __syncthreads();
   }
-  const int nbc = uniform ? 1 : S.nbcode;
-  const int npass = max(nbc, 1);  // a brick without particles writes zeros in one pass
-  const int pbase = w.B.poff[bt.y];
-  for (int b = 0; b < npass; ++b) {
-    const bool coded = b < nbc;
-    const uint32_t k1 = (uniform || !coded) ? 0u : S.bcode[b].x, k2 = (uniform || !coded) ? 0u : S.bcode[b].y;
-    const bool has = coded && n_c > 0 &&
-                     (uniform || cell_has_code<PPC>(S.ps1, S.ps2, S.ccode, S.ncode, c, k1, k2));
-    const bool filt = !uniform && S.ncode[c] > 1;
+  const unsigned long long codes = several ? S.cmask[c] : 0ull;
+  const bool filt = (codes & (codes - 1)) != 0;
+  for (int b = 0; b < B.npass; ++b) {
+    const bool has = n_c > 0 && (!several || ((codes >> b) & 1u));
     float a[3][3][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -768,7 +633,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
     if (has) {
       for (int j = 0; j < n_c; ++j) {
         const int si = pic(j, c);
-        if (filt && (S.ps1[si] != k1 || S.ps2[si] != k2)) continue;
+        if (filt && S.pid[si] != b) continue;
         float wx[3], wy[3], wz, d;
         const float f0 = S.pf[0][si], f1 = S.pf[1][si], f2 = S.pf[2][si];
         bs<0>(f0, wx[0], d); bs<1>(f0, wx[1], d); bs<2>(f0, wx[2], d);
@@ -791,23 +656,14 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
     xy_reduce<3>(a, cx, cy);
     stage_layer<3, TN>(S.sz, a, cx, cy, cz, oz);
     __syncthreads();
-    if (pbase >= 0) {
-      for (int t = tid; t < TN; t += BT) {
-        const int n = S.T.cnt[t];
-        if (n == 0) continue;
-        const size_t e0 = (size_t)pbase + S.T.lo[t];
-        if (b == 0 && !uniform)
-          for (int q = 0; q < n; ++q)
-            if (!code_listed(S.bcode, S.nbcode, tile_code(w, S.T, tcodes, t, q)))
-              w.B.pm[e0 + q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int sl = coded ? node_slot_of(w, S.T, tcodes, t, uniform, k1, k2) : -1;
-        if (sl < 0) continue;
-        float acc[3];
-        gather_z<3, TN>(S.sz, t, acc);
-        w.B.pm[e0 + sl] = make_float4(acc[0], acc[1], acc[2], 0.f);
-      }
+    for (int t = tid; t < TN; t += BT) {
+      const long long e = B.entry(w, S.T, b, t);
+      if (e < 0) continue;
+      float acc[3];
+      gather_z<3, TN>(S.sz, t, acc);
+      w.B.pm[e] = make_float4(acc[0], acc[1], acc[2], 0.f);
     }
-    if (b + 1 < npass) __syncthreads();  // the next pass overwrites the z stage
+    if (b + 1 < B.npass) __syncthreads();  // the next pass overwrites the z stage
   }
 }
 
@@ -875,8 +731,7 @@ __global__ void k_musl_node(World w, LaunchSet ls) {
 // commit the side labels assigned this substep (they act from the next one)
 // --------------------------------------------------------------------------
 struct K1S {
-  Tile T;
-  uint2 codes[TSCAP];
+  BrickTile T;
   float4 tvs[TSCAP];
   int any;
 };
@@ -894,19 +749,19 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
   int c0x, c0y, c0z;
   brick_coords(sc, lb, c0x, c0y, c0z);
   if (tid == 0) S.any = 0;
-  const bool single = tile_load(w, sc, bt.y, c0x, c0y, c0z, S.T);
-  const bool in_smem = S.T.total <= TSCAP;
-  const uint2 *tcodes = in_smem ? S.codes : nullptr;
+  const BrickInfo B(w, bt, 0);
+  const bool several = B.nbc > 1, single = B.single;
+  const bool in_smem = w.B.ptot[bt.y] <= TSCAP;
+  brick_tile(w, bt.y, B.nbc, S.T, BT);
+  __syncthreads();
+  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, -1, BT);
   if (single) {  // by node
     for (int t = tid; t < TN; t += BT)
       S.tvs[t] = S.T.cnt[t] ? w.S.vstar[S.T.goff[t]] : make_float4(0.f, 0.f, 0.f, 0.f);
   } else if (in_smem) {
     for (int t = tid; t < TN; t += BT) {
       const int n = S.T.cnt[t], lo = S.T.lo[t], g = S.T.goff[t];
-      for (int a = 0; a < n; ++a) {
-        if (n > 1) S.codes[lo + a] = w.S.code[g + a];
-        S.tvs[lo + a] = w.S.vstar[g + a];
-      }
+      for (int a = 0; a < n; ++a) S.tvs[lo + a] = w.S.vstar[g + a];
     }
   }
   __syncthreads();
@@ -918,7 +773,7 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
     int bx, by, bz;
     particle_base(P.base[p], bx, by, bz);
     const int lx = bx - c0x, ly = by - c0y, lz = bz - c0z;
-    const uint32_t s1 = P.s1[p], s2 = P.s2[p];
+    const int id = several ? P.cid[p] : 0;
     const float f0 = P.fx[0][p], f1 = P.fx[1][p], f2 = P.fx[2][p];
     float wx[3], wy[3], wz[3], gx[3], gy[3], gz[3];
     bs<0>(f0, wx[0], gx[0]); bs<1>(f0, wx[1], gx[1]); bs<2>(f0, wx[2], gx[2]);
@@ -945,7 +800,7 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
 #pragma unroll
           for (int ox = 0; ox < 3; ++ox) {
             const int t = t0 + (oz * TE + oy) * TE + ox;
-            const int s = tile_slot(w, S.T, tcodes, t, s1, s2);
+            const int s = tile_slot(w, S.T, B.nbc, t, id);
             if (s < 0) continue;
             const float4 v = in_smem ? S.tvs[s] : w.S.vstar[S.T.goff[t] + s - S.T.lo[t]];
             sx[0] += v.x * gx[ox]; sx[1] += v.y * gx[ox]; sx[2] += v.z * gx[ox];
@@ -966,8 +821,8 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
       for (int k = 0; k < 9; ++k) P.Fdot[k][p] = sc.inv_dx * G[k];
     const uint8_t pend = P.pend[p];
     if (pend && cut >= 0) {
-      if (pend == 1) P.s1[p] = s1 | (1u << cut);
-      else P.s2[p] = s2 | (1u << cut);
+      if (pend == 1) P.s1[p] |= 1u << cut;
+      else P.s2[p] |= 1u << cut;
       any = true;
       // the nodes of this particle's stencil need their codes recounted
       for (int oz = 0; oz < 3; ++oz)
@@ -978,7 +833,10 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
   }
   if (any) S.any = 1;
   __syncthreads();
-  if (tid == 0 && S.any) atomicOr(&scm.label_pending, 1);
+  if (tid == 0 && S.any) {
+    w.B.bdirty[bt.y] = 1;  // its particles' codes are listed anew by the slot rebuild
+    atomicOr(&scm.label_pending, 1);
+  }
 }
 
 // --------------------------------------------------------------------------
@@ -1869,12 +1727,13 @@ __global__ void k_slot_count(World w, LaunchSet ls, int force) {
 // nodes 7l .. 7l + 6, an exclusive warp scan orders them)
 #define BTILE_WARPS 8
 
-// Distinct codes of a lattice brick's particles and each particle's index in
+// Distinct codes of a brick's particles and each particle's index in
 // the list (one warp; a lane keeps the codes of its particles lane + 32 j in
 // registers).  The next code is that of the lowest particle not yet listed,
 // so the list is in first-occurrence order.
+// (PER: 32 PER particles at most)
+template <int PER>
 __device__ __forceinline__ int list_brick_codes(const World &w, DevScene &sc, const int4 &bt, int lane) {
-  constexpr int PER = BM_LAT_POS / 32;
   uint32_t a[PER], b[PER];
   unsigned todo = 0;
 #pragma unroll
@@ -1912,6 +1771,7 @@ __device__ __forceinline__ int list_brick_codes(const World &w, DevScene &sc, co
   return n;
 }
 
+template <int PPC>
 __global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, LaunchSet ls, int force) {
   const int lane = threadIdx.x & 31;
   const int bi = blockIdx.x * BTILE_WARPS + (threadIdx.x >> 5);
@@ -1919,14 +1779,12 @@ __global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, Launc
   const int4 bt = ls.btiles[bi];
   DevScene &sc = w.scenes[bt.x];
   if (!force && !sc.need_rebuild) return;
-  int ncode = 0;
-  if (sc.lattice) {
-    if (force || w.B.bdirty[bt.y]) {
-      ncode = list_brick_codes(w, sc, bt, lane);
-      if (lane == 0) w.B.bdirty[bt.y] = 0;
-    } else {
-      ncode = w.B.binfo[bt.y] & 0xff;
-    }
+  int ncode;
+  if (force || w.B.bdirty[bt.y]) {
+    ncode = list_brick_codes<PPC * BR3 / 32>(w, sc, bt, lane);
+    if (lane == 0) w.B.bdirty[bt.y] = 0;
+  } else {
+    ncode = w.B.binfo[bt.y] & 0xff;
   }
   int c0x, c0y, c0z;
   brick_coords(sc, bt.y - sc.brick_begin, c0x, c0y, c0z);
@@ -1948,7 +1806,7 @@ __global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, Launc
 #pragma unroll
   for (int j = 0; j < PER; ++j) several |= cnt[j] > 1;
   const bool single = !__any_sync(FULL, several);
-  if (lane == 0 && sc.lattice) w.B.binfo[bt.y] = ncode | (single ? 256 : 0);
+  if (lane == 0) w.B.binfo[bt.y] = ncode | (single ? 256 : 0);
   int incl = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -2193,7 +2051,9 @@ static cudaError_t launch_rebuild(const World &w, const LaunchSet &ls, cudaStrea
   else launch_count<8>(w, ls, st, force);
   rec(ev, 6, 1, st);
   rec(ev, 9, 0, st);
-  k_brick_tiles<<<(ls.n_btiles + BTILE_WARPS - 1) / BTILE_WARPS, 32 * BTILE_WARPS, 0, st>>>(w, ls, force);
+  const int tgrid = (ls.n_btiles + BTILE_WARPS - 1) / BTILE_WARPS;
+  if (ls.ppc16) k_brick_tiles<16><<<tgrid, 32 * BTILE_WARPS, 0, st>>>(w, ls, force);
+  else k_brick_tiles<8><<<tgrid, 32 * BTILE_WARPS, 0, st>>>(w, ls, force);
   rec(ev, 9, 1, st);
   rec(ev, 7, 0, st);
   k_slot_scan<<<ls.n_scenes, 256, 0, st>>>(w, ls, force);

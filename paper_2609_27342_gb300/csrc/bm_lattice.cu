@@ -40,8 +40,6 @@
 namespace {
 
 constexpr int LP = BM_LAT_POS;     // particle places of a brick
-constexpr int LCODES = 8;          // codes per brick with a slot table in shared memory
-constexpr int NOSLOT = 0xff;
 
 // B-spline weights of one particle plane: w0 w1 w2 d0 | d1 d2
 struct __align__(16) PlaneW {
@@ -100,38 +98,15 @@ __device__ __forceinline__ f2 force_u2(f2 A1, f2 dyz, f2 A2, f2 wyd, f2 J, f2 wy
 }
 __device__ __forceinline__ f2 force_acc2(f2 q, f2 w, f2 U, f2 d, f2 V) { return add2(q, fma2(w, U, mul2(d, V))); }
 
-// The brick's node tile: first pool slot, first tile slot and slot count of
-// each node; with several codes also the slot (index at its node) of every
-// code of the brick.
-struct LatTile {
+// the brick's node tile and the weights of its planes
+struct LatTile : BrickTile {
   PlaneW wt[3][8];
-  uint2 bcode[BM_BRICK_CODES];
-  int goff[TN];
-  uint16_t lo[TN];
-  uint8_t cnt[TN];
-  uint8_t slot[LCODES][TN];
 };
-
-__device__ __forceinline__ int lat_slot(const World &w, const LatTile &T, int nbc, int b, int t) {
-  if (nbc <= LCODES) return T.slot[b][t];
-  const uint2 k = T.bcode[b];
-  for (int a = 0; a < T.cnt[t]; ++a) {
-    const uint2 c = w.S.code[T.goff[t] + a];
-    if (c.x == k.x && c.y == k.y) return a;
-  }
-  return NOSLOT;
-}
 
 // Tile and weights of brick `brick` (nt threads); ends without a barrier.
 __device__ __forceinline__ void lat_tile(const World &w, int brick, int nbc, LatTile &T, int nt) {
+  brick_tile(w, brick, nbc, T, nt);
   const int tid = threadIdx.x;
-  for (int t = tid; t < TN; t += nt) {
-    const int d = w.B.tdesc[(size_t)brick * TN + t];
-    T.lo[t] = (uint16_t)(d & 0xffff);
-    T.cnt[t] = (uint8_t)(d >> 16);
-    T.goff[t] = w.B.tgoff[(size_t)brick * TN + t];
-  }
-  if (tid < nbc) T.bcode[tid] = w.B.bcode[(size_t)brick * BM_BRICK_CODES + tid];
   if (tid >= nt - 24) {
     const int k = tid - (nt - 24);
     const float f = w.B.lf[(size_t)brick * 24 + k];
@@ -143,57 +118,6 @@ __device__ __forceinline__ void lat_tile(const World &w, int brick, int nbc, Lat
     T.wt[k >> 3][k & 7].b = make_float4(d[1], d[2], 0.f, 0.f);
   }
 }
-
-// Slot table of a brick with several codes or slots (after a barrier on
-// lat_tile).  Slots whose code no particle of the brick carries get zero
-// partial sums (pbase < 0: none are written).
-template <bool FORCE>
-__device__ __forceinline__ void lat_slots(const World &w, LatTile &T, int nbc, int pbase, int nt) {
-  for (int t = threadIdx.x; t < TN; t += nt) {
-    const int n = T.cnt[t], g = T.goff[t];
-    if (nbc <= LCODES)
-      for (int b = 0; b < nbc; ++b) T.slot[b][t] = NOSLOT;
-    for (int a = 0; a < n; ++a) {
-      const uint2 c = w.S.code[g + a];
-      int id = -1;
-      for (int b = 0; b < nbc; ++b)
-        if (T.bcode[b].x == c.x && T.bcode[b].y == c.y) id = b;
-      if (id >= 0) {
-        if (nbc <= LCODES) T.slot[id][t] = (uint8_t)a;
-      } else if (pbase >= 0) {
-        const size_t e = (size_t)pbase + T.lo[t] + a;
-        w.B.pm[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (FORCE) w.B.pd[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-  }
-}
-
-// What a brick kernel needs to know of its brick.
-struct LatBrick {
-  int nbc;        // distinct codes of the brick's particles
-  bool uniform;   // at most one code, and one logical grid at every tile node
-  bool mask;      // empty places or several codes
-  int pbase;      // partial-sum range (negative: pool overflow)
-  int npass;      // a brick without particles still runs one pass: it writes zeros to its tile
-  __device__ __forceinline__ LatBrick(const World &w, const int4 &bt) {
-    const int info = w.B.binfo[bt.y];
-    nbc = info & 0xff;
-    uniform = (info >> 8) != 0 && nbc <= 1;
-    mask = bt.w < LP || nbc > 1;
-    pbase = w.B.poff[bt.y];
-    npass = max(nbc, 1);
-  }
-  // slot of pass b's code at tile node t (an index at the node), or NOSLOT
-  __device__ __forceinline__ int slot(const World &w, const LatTile &T, int b, int t) const {
-    return T.cnt[t] == 0 ? NOSLOT : uniform ? 0 : nbc == 0 ? NOSLOT : lat_slot(w, T, nbc, b, t);
-  }
-  // partial-sum entry of that slot, or -1
-  __device__ __forceinline__ long long entry(const World &w, const LatTile &T, int b, int t) const {
-    const int sl = slot(w, T, b, t);
-    return sl == NOSLOT || pbase < 0 ? -1 : (long long)pbase + T.lo[t] + sl;
-  }
-};
 
 // plane indices of a place (inverse of bm_lat_place), its base cell in the
 // brick (x fastest) and its particle's number in the cell's (x, y, z) order
@@ -358,7 +282,7 @@ __global__ void __launch_bounds__(PT, MB) k_p2g_lat(World w, LaunchSet ls) {
   if (sc.frozen || !sc.lattice) return;
   const PPool &P = w.P;
   const int tid = threadIdx.x;
-  const LatBrick B(w, bt);
+  const BrickInfo B(w, bt, LP);
   lat_tile(w, bt.y, B.nbc, S.T, PT);
   if (B.mask && tid < LP / 4) reinterpret_cast<unsigned *>(S.cid)[tid] = 0xffffffffu;
   __syncthreads();
@@ -383,7 +307,7 @@ __global__ void __launch_bounds__(PT, MB) k_p2g_lat(World w, LaunchSet ls) {
     if (B.mask) S.cid[place_cell8(q)] = (uint8_t)c;
   }
   if (clamped) atomicOr(&scm.err, BM_ERRBIT_INVERTED);
-  if (!B.uniform) lat_slots<true>(w, S.T, B.nbc, B.pbase, PT);
+  if (!B.uniform) brick_slots<true>(w, S.T, B.nbc, B.pbase, PT);
   if (sc.has_blade) brick_wrench(w, bt.y, wr, anyc, S.red);
   __syncthreads();
   const CellOz q(tid);
@@ -482,7 +406,7 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
   if (sc.frozen || !sc.lattice) return;
   const PPool &P = w.P;
   const int tid = threadIdx.x;
-  const LatBrick B(w, bt);
+  const BrickInfo B(w, bt, LP);
   // the general kernel multiplies the weights of a tile beyond its slot
   // window in another order: (wx wy) wz, not wx (wy wz)
   const bool wide = w.B.ptot[bt.y] > TSCAP;
@@ -495,7 +419,7 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
     S.inv[q] = (uint16_t)i;
     if (B.mask) S.cid[place_cell8(q)] = P.cid[bt.z + i];
   }
-  if (!B.uniform) lat_slots<false>(w, S.T, B.nbc, B.pbase, GT);
+  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, B.pbase, GT);
   __syncthreads();
   const int cell = tid >> 2, jx = (tid >> 1) & 1, jy = tid & 1;
   const int cx = cell & 3, cy = (cell >> 2) & 3, cz = cell >> 4;
@@ -632,7 +556,7 @@ __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
   if (sc.frozen || !sc.lattice) return;
   const PPool &P = w.P;
   const int tid = threadIdx.x;
-  const LatBrick B(w, bt);
+  const BrickInfo B(w, bt, LP);
   if (tid == 0) S.any = 0;
   float F[NPT][9];  // read up front: the latency passes under the tile
   int pq[NPT], pc[NPT];
@@ -650,7 +574,7 @@ __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
   lat_tile(w, bt.y, B.nbc, S.T, FT);
   __syncthreads();
   if (!B.uniform) {
-    lat_slots<false>(w, S.T, B.nbc, -1, FT);
+    brick_slots<false>(w, S.T, B.nbc, -1, FT);
     __syncthreads();
   }
   const float c = sc.dt * sc.inv_dx;
