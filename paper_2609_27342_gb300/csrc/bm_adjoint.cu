@@ -193,6 +193,7 @@ constexpr int kAdjNodesPerBlock = kAdjBlock / 32;
 // per node: slot masses, adjoint of v* from F' = F + dt sum v* (x) grad N,
 // then through v* = C p* / m
 __global__ void __launch_bounds__(kAdjBlock) k_adj_musl(World w, AdjWork aw) {
+  chain_wait();
   __shared__ float red[kAdjNodesPerBlock][BM_MAXS][4];
   const DevScene &sc = w.scenes[aw.slot];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -243,6 +244,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_musl(World w, AdjWork aw) {
 
 // per particle: adjoint of v^{n+1} = incoming adjoint + MUSL re-scatter term
 __global__ void __launch_bounds__(kAdjBlock) k_adj_v1(World w, AdjWork aw) {
+  chain_wait();
   const DevScene &sc = w.scenes[aw.slot];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= sc.n_p) return;
@@ -281,6 +283,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_v1(World w, AdjWork aw) {
 // from v^{n+1} = beta v + sum N/m ((1-beta) p + dp) and x^{n+1} = x + dt sum
 // N (p + dp)/m, then through Eq. 8 transposed
 __global__ void __launch_bounds__(kAdjBlock) k_adj_g2p(World w, AdjWork aw) {
+  chain_wait();
   __shared__ float red[kAdjNodesPerBlock][BM_MAXS][6];
   const DevScene &sc = w.scenes[aw.slot];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -377,6 +380,7 @@ __device__ void piola_vjp(const float F[9], float mu, float lam, const float Pb[
 // per particle: P2G transposed, stress, blade contact (with friction and the
 // D release) and floor contact; block partials of the parameter adjoints
 __global__ void __launch_bounds__(kAdjBlock) k_adj_part(World w, AdjWork aw) {
+  chain_wait();
   __shared__ double red[kParts][kAdjBlock / 32];
   const DevScene &sc = w.scenes[aw.slot];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -651,6 +655,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_part(World w, AdjWork aw) {
 // (warp k sums partial k: its lanes stride the blocks, a fixed shuffle tree
 // adds them; one thread adding the blocks in turn took 16 us for 250 of them)
 __global__ void __launch_bounds__(32 * kParts) k_adj_reduce(World w, AdjWork aw, int nblocks) {
+  chain_wait();
   __shared__ double tot[kParts];
   const DevScene &sc = w.scenes[aw.slot];
   {
@@ -684,6 +689,7 @@ __global__ void __launch_bounds__(32 * kParts) k_adj_reduce(World w, AdjWork aw,
 
 // state adjoints <-> caller order (perm maps pool index -> caller index)
 __global__ void k_adj_io(World w, AdjWork aw, int field, float *buf, int to_work) {
+  chain_wait();
   const DevScene &sc = w.scenes[aw.slot];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= sc.n_p) return;
@@ -751,11 +757,11 @@ cudaError_t bm_launch_adjoint_substep(const World &w, const void *work, const do
   if (n_p == 0) return cudaSuccess;
   // per-node kernels: a warp per node; per-particle kernels: a thread per particle
   const int gn = (n_node + kAdjNodesPerBlock - 1) / kAdjNodesPerBlock, gp = (n_p + kAdjBlock - 1) / kAdjBlock;
-  k_adj_musl<<<gn, kAdjBlock, 0, st>>>(w, aw);
-  k_adj_v1<<<gp, kAdjBlock, 0, st>>>(w, aw);
-  k_adj_g2p<<<gn, kAdjBlock, 0, st>>>(w, aw);
-  k_adj_part<<<gp, kAdjBlock, 0, st>>>(w, aw);
-  k_adj_reduce<<<1, 32 * kParts, 0, st>>>(w, aw, gp);
+  chain_launch(k_adj_musl, dim3((unsigned)gn), kAdjBlock, 0, st, w, aw);
+  chain_launch(k_adj_v1, dim3((unsigned)gp), kAdjBlock, 0, st, w, aw);
+  chain_launch(k_adj_g2p, dim3((unsigned)gn), kAdjBlock, 0, st, w, aw);
+  chain_launch(k_adj_part, dim3((unsigned)gp), kAdjBlock, 0, st, w, aw);
+  chain_launch(k_adj_reduce, dim3(1), 32 * kParts, 0, st, w, aw, gp);
   return cudaGetLastError();
 }
 
@@ -763,6 +769,6 @@ cudaError_t bm_launch_adjoint_io(const World &w, const void *work, int field, fl
                                  int n_p, cudaStream_t st) {
   if (n_p == 0) return cudaSuccess;
   const AdjWork aw = *reinterpret_cast<const AdjWork *>(work);
-  k_adj_io<<<(n_p + 255) / 256, 256, 0, st>>>(w, aw, field, buf, to_work);
+  chain_launch(k_adj_io, dim3((unsigned)((n_p + 255) / 256)), 256, 0, st, w, aw, field, buf, to_work);
   return cudaGetLastError();
 }

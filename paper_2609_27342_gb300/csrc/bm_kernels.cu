@@ -105,6 +105,7 @@ __device__ void stage_particles(const World &w, const DevScene &sc, const int4 &
 
 template <int PPC, int MB, bool INELASTIC>
 __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   K2S<PPC> &S = *reinterpret_cast<K2S<PPC> *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];  // scene, pool brick, first particle, count
@@ -368,6 +369,7 @@ __device__ __forceinline__ void coupled_slots(const World &w, NodeS<NC> &N, int 
 }
 
 __global__ void k_p2g_node(World w, LaunchSet ls) {
+  chain_wait();
   __shared__ NodeS<6> N;
   const int4 t = ls.ntiles[blockIdx.x];
   const int i = threadIdx.x;
@@ -476,6 +478,7 @@ struct K4S {
 
 template <int PPC, int MB>
 __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   K4S<PPC> &S = *reinterpret_cast<K4S<PPC> *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];
@@ -671,6 +674,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
 // k_musl_node: per slot, MUSL sums of the covering bricks, coupling, v*
 // --------------------------------------------------------------------------
 __global__ void k_musl_node(World w, LaunchSet ls) {
+  chain_wait();
   __shared__ NodeS<3> N;
   const int4 t = ls.ntiles[blockIdx.x];
   const int i = threadIdx.x;
@@ -738,6 +742,7 @@ struct K1S {
 
 template <int MB, bool INELASTIC>
 __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
+  chain_wait();
   __shared__ K1S S;
   const int4 bt = ls.btiles[blockIdx.x];
   DevScene &scm = w.scenes[bt.x];
@@ -871,6 +876,7 @@ __device__ __forceinline__ unsigned long long cell_key(int scene, int cx, int cy
 
 // per-substep reset of the scenes' reductions and of the world's build flag
 __global__ void k_pair_reset(World w, LaunchSet ls) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) *w.H.build = 0;
   if (i < ls.n_scenes) {
@@ -883,6 +889,7 @@ __global__ void k_pair_reset(World w, LaunchSet ls) {
 // per scene: largest particle speed, and largest displacement since the
 // candidate lists were built (non-negative floats order like their bits)
 __global__ void k_pair_vmax(World w, LaunchSet ls) {
+  chain_wait();
   const int4 bt = ls.btiles[blockIdx.x];
   DevScene &sc = w.scenes[bt.x];
   if (!sc.pair_on || sc.frozen) return;
@@ -912,6 +919,7 @@ __global__ void k_pair_vmax(World w, LaunchSet ls) {
 
 // per scene: whether the candidate lists are rebuilt this substep
 __global__ void k_pair_decide(World w, LaunchSet ls) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ls.n_scenes) return;
   DevScene &sc = w.scenes[ls.scene_ids[i]];
@@ -934,6 +942,7 @@ __global__ void k_pair_decide(World w, LaunchSet ls) {
 }
 
 __global__ void k_pair_hash(World w, LaunchSet ls) {
+  chain_wait();
   const int4 bt = ls.btiles[blockIdx.x];
   const DevScene &sc = w.scenes[bt.x];
   if (!sc.pair_on || !sc.pair_build) return;
@@ -952,6 +961,7 @@ __global__ void k_pair_hash(World w, LaunchSet ls) {
 }
 
 __global__ void k_scan_local(World w) {
+  chain_wait();
   if (!*w.H.build) return;
   __shared__ int sm[33];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -963,6 +973,7 @@ __global__ void k_scan_local(World w) {
 }
 
 __global__ void k_scan_top(World w, int nblocks) {
+  chain_wait();
   if (!*w.H.build) return;
   __shared__ int sm[33];
   int carry = 0;
@@ -979,12 +990,14 @@ __global__ void k_scan_top(World w, int nblocks) {
 }
 
 __global__ void k_scan_add(World w) {
+  chain_wait();
   if (!*w.H.build) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < w.H.n_buckets) w.H.bucket_start[i] += w.H.block_sum[blockIdx.x];
 }
 
 __global__ void k_pair_fill(World w, LaunchSet ls) {
+  chain_wait();
   const int4 bt = ls.btiles[blockIdx.x];
   const DevScene &sc = w.scenes[bt.x];
   if (!sc.pair_on || !sc.pair_build) return;
@@ -998,6 +1011,7 @@ __global__ void k_pair_fill(World w, LaunchSet ls) {
 // order each bucket by pool index (buckets are short), then lay out its
 // entries (position, pool index, base cell, cell key) for the list build
 __global__ void k_pair_sort(World w) {
+  chain_wait();
   if (!*w.H.build) return;
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < w.H.n_buckets; b += gridDim.x * blockDim.x) {
     const int s0 = w.H.bucket_start[b], s1 = w.H.bucket_start[b + 1];
@@ -1137,6 +1151,7 @@ __device__ __forceinline__ void bucket_lists(const World &w, int c0, int c1, int
 // particles of each non-empty one, 32 entries at a time.  The positions of
 // the build are kept.
 __global__ void __launch_bounds__(256) k_pair_list(World w) {
+  chain_wait();
   if (!*w.H.build) return;
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1159,6 +1174,7 @@ __global__ void __launch_bounds__(256) k_pair_list(World w) {
 // skipped unless the two are on opposite sides of a cut, before its state
 // is read.
 __global__ void k_pair(World w, LaunchSet ls) {
+  chain_wait();
   const int4 bt = ls.btiles[blockIdx.x];
   DevScene &scm = w.scenes[bt.x];
   const DevScene &sc = scm;
@@ -1348,6 +1364,7 @@ __device__ void rot_exp(const double th[3], double Rm[9]) {
 }
 
 __global__ void k_prepare(World w, LaunchSet ls) {
+  chain_wait();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= ls.n_scenes) return;
   prepare_substep(w.scenes[ls.scene_ids[idx]]);
@@ -1355,6 +1372,7 @@ __global__ void k_prepare(World w, LaunchSet ls) {
 
 // tool states {x_B, R, v_B, omega_B} of several scenes, then their frames
 __global__ void k_set_tools(World w, const int *ids, int n, const double *states) {
+  chain_wait();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n) return;
   DevScene &sc = w.scenes[ids[idx]];
@@ -1369,6 +1387,7 @@ __global__ void k_set_tools(World w, const int *ids, int n, const double *states
 }
 
 __global__ void k_get_wrenches(World w, const int *ids, int n, double *out) {
+  chain_wait();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n) return;
   const DevScene &sc = w.scenes[ids[idx]];
@@ -1556,6 +1575,7 @@ __device__ __forceinline__ void tool_step(const World &w, DevScene &sc, ToolTmp 
 }
 
 __global__ void k_tool(World w, LaunchSet ls) {
+  chain_wait();
   const int sid = ls.scene_ids[blockIdx.x];
   DevScene &g = w.scenes[sid];
   if (g.frozen) {  // a scene that has taken its substeps: nothing moves, nothing to rebuild
@@ -1680,6 +1700,7 @@ __device__ __forceinline__ int recount_node(const World &w, DevScene &sc, int nd
 // gridDim.y CTAs, ahead of k_slot_count<.., true>.
 template <int KR>
 __global__ void k_recount(World w, LaunchSet ls, int force) {
+  chain_wait();
   const int4 t = ls.ntiles[blockIdx.x];
   DevScene &sc = w.scenes[t.x];
   if (!force && !sc.need_rebuild) return;
@@ -1694,6 +1715,7 @@ __global__ void k_recount(World w, LaunchSet ls, int force) {
 // has done so), the others keep their distinct codes from the last rebuild.
 template <int KR, bool COUNTED>
 __global__ void k_slot_count(World w, LaunchSet ls, int force) {
+  chain_wait();
   const int4 t = ls.ntiles[blockIdx.x];
   DevScene &sc = w.scenes[t.x];
   if (!force && !sc.need_rebuild) return;
@@ -1773,6 +1795,7 @@ __device__ __forceinline__ int list_brick_codes(const World &w, DevScene &sc, co
 
 template <int PPC>
 __global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, LaunchSet ls, int force) {
+  chain_wait();
   const int lane = threadIdx.x & 31;
   const int bi = blockIdx.x * BTILE_WARPS + (threadIdx.x >> 5);
   if (bi >= ls.n_btiles) return;
@@ -1825,6 +1848,7 @@ __global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, Launc
 
 // per scene: slot offsets of the node tiles, and partial-sum ranges of the bricks
 __global__ void k_slot_scan(World w, LaunchSet ls, int force) {
+  chain_wait();
   DevScene &sc = w.scenes[ls.scene_ids[blockIdx.x]];
   if (!force && !sc.need_rebuild) return;
   __shared__ int sm[33];
@@ -1861,6 +1885,7 @@ __global__ void k_slot_scan(World w, LaunchSet ls, int force) {
 }
 
 __global__ void k_slot_fill(World w, LaunchSet ls, int force) {
+  chain_wait();
   const int4 t = ls.ntiles[blockIdx.x];
   DevScene &sc = w.scenes[t.x];
   if (!force && !sc.need_rebuild) return;
@@ -1970,6 +1995,7 @@ __device__ __forceinline__ void io_field(const World &w, int scene_slot, int p, 
 }
 
 __global__ void k_io(World w, int scene_slot, int p_begin, int n, int field, void *buf, int to_pool) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int p = p_begin + i;
@@ -1983,6 +2009,7 @@ struct ReadSet {
 
 // blockIdx.y: which of the requested fields
 __global__ void k_read(World w, int scene_slot, int p_begin, int n, ReadSet r) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int p = p_begin + i;
@@ -1990,6 +2017,7 @@ __global__ void k_read(World w, int scene_slot, int p_begin, int n, ReadSet r) {
 }
 
 __global__ void k_code(World w, int p_begin, int n, int64_t *out) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int p = p_begin + i;
@@ -2010,7 +2038,7 @@ __global__ void k_code(World w, int p_begin, int n, int64_t *out) {
 // ----------------------------------------------------------------------------
 cudaError_t bm_launch_prepare(const World &w, const LaunchSet &ls, cudaStream_t st) {
   if (ls.n_scenes == 0) return cudaSuccess;
-  k_prepare<<<(ls.n_scenes + 63) / 64, 64, 0, st>>>(w, ls);
+  chain_launch(k_prepare, dim3((unsigned)((ls.n_scenes + 63) / 64)), 64, 0, st, w, ls);
   return cudaGetLastError();
 }
 
@@ -2035,12 +2063,12 @@ static inline void rec(cudaEvent_t *ev, int k, int after, cudaStream_t st) {
 template <int KR>
 static void launch_count(const World &w, const LaunchSet &ls, cudaStream_t st, int force) {
   if (ls.n_ntiles > RECOUNT_CTAS) {
-    k_slot_count<KR, false><<<ls.n_ntiles, ls.ntile_size, 0, st>>>(w, ls, force);
+    chain_launch(k_slot_count<KR, false>, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
     return;
   }
   const int parts = min(max(RECOUNT_CTAS / ls.n_ntiles, 1), 16);
-  k_recount<KR><<<dim3((unsigned)ls.n_ntiles, (unsigned)parts), 256, 0, st>>>(w, ls, force);
-  k_slot_count<KR, true><<<ls.n_ntiles, ls.ntile_size, 0, st>>>(w, ls, force);
+  chain_launch(k_recount<KR>, dim3((unsigned)ls.n_ntiles, (unsigned)parts), 256, 0, st, w, ls, force);
+  chain_launch(k_slot_count<KR, true>, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
 }
 
 static cudaError_t launch_rebuild(const World &w, const LaunchSet &ls, cudaStream_t st, int force,
@@ -2052,14 +2080,14 @@ static cudaError_t launch_rebuild(const World &w, const LaunchSet &ls, cudaStrea
   rec(ev, 6, 1, st);
   rec(ev, 9, 0, st);
   const int tgrid = (ls.n_btiles + BTILE_WARPS - 1) / BTILE_WARPS;
-  if (ls.ppc16) k_brick_tiles<16><<<tgrid, 32 * BTILE_WARPS, 0, st>>>(w, ls, force);
-  else k_brick_tiles<8><<<tgrid, 32 * BTILE_WARPS, 0, st>>>(w, ls, force);
+  if (ls.ppc16) chain_launch(k_brick_tiles<16>, dim3(tgrid), 32 * BTILE_WARPS, 0, st, w, ls, force);
+  else chain_launch(k_brick_tiles<8>, dim3(tgrid), 32 * BTILE_WARPS, 0, st, w, ls, force);
   rec(ev, 9, 1, st);
   rec(ev, 7, 0, st);
-  k_slot_scan<<<ls.n_scenes, 256, 0, st>>>(w, ls, force);
+  chain_launch(k_slot_scan, dim3(ls.n_scenes), 256, 0, st, w, ls, force);
   rec(ev, 7, 1, st);
   rec(ev, 8, 0, st);
-  k_slot_fill<<<ls.n_ntiles, ls.ntile_size, 0, st>>>(w, ls, force);
+  chain_launch(k_slot_fill, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
   rec(ev, 8, 1, st);
   return cudaGetLastError();
 }
@@ -2130,20 +2158,20 @@ cudaError_t bm_kernels_init() {
 template <int PPC, int C>
 static void launch_p2g(const World &w, const LaunchSet &ls, cudaStream_t st) {
   if (ls.any_inelastic)
-    k_p2g_brick<PPC, OccP2G<C, true>::v, true><<<ls.n_btiles, BT, sizeof(K2S<PPC>), st>>>(w, ls);
+    chain_launch(k_p2g_brick<PPC, OccP2G<C, true>::v, true>, dim3(ls.n_btiles), BT, sizeof(K2S<PPC>), st, w, ls);
   else
-    k_p2g_brick<PPC, OccP2G<C, false>::v, false><<<ls.n_btiles, BT, sizeof(K2S<PPC>), st>>>(w, ls);
+    chain_launch(k_p2g_brick<PPC, OccP2G<C, false>::v, false>, dim3(ls.n_btiles), BT, sizeof(K2S<PPC>), st, w, ls);
 }
 
 template <int PPC, int C>
 static void launch_g2p(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  k_g2p_musl<PPC, OccG2P<C>::v><<<ls.n_btiles, BT, sizeof(K4S<PPC>), st>>>(w, ls);
+  chain_launch(k_g2p_musl<PPC, OccG2P<C>::v>, dim3(ls.n_btiles), BT, sizeof(K4S<PPC>), st, w, ls);
 }
 
 template <int C>
 static void launch_fupd(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  if (ls.any_inelastic) k_fupd<OccFupd<C>::v, true><<<ls.n_btiles, BT, 0, st>>>(w, ls);
-  else k_fupd<OccFupd<C>::v, false><<<ls.n_btiles, BT, 0, st>>>(w, ls);
+  if (ls.any_inelastic) chain_launch(k_fupd<OccFupd<C>::v, true>, dim3(ls.n_btiles), BT, 0, st, w, ls);
+  else chain_launch(k_fupd<OccFupd<C>::v, false>, dim3(ls.n_btiles), BT, 0, st, w, ls);
 }
 
 template <int PPC>
@@ -2180,7 +2208,7 @@ static void launch_bricks(const World &w, const LaunchSet &ls, cudaStream_t st, 
   }
   rec(ev, 0, 1, st);
   rec(ev, 1, 0, st);
-  k_p2g_node<<<ls.n_ntiles, ls.ntile_size, 0, st>>>(w, ls);
+  chain_launch(k_p2g_node, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls);
   rec(ev, 1, 1, st);
   rec(ev, 2, 0, st);
   if (ls.any_lattice) bm_launch_g2p_lat(w, ls, st);
@@ -2190,7 +2218,7 @@ static void launch_bricks(const World &w, const LaunchSet &ls, cudaStream_t st, 
   }
   rec(ev, 2, 1, st);
   rec(ev, 3, 0, st);
-  k_musl_node<<<ls.n_ntiles, ls.ntile_size, 0, st>>>(w, ls);
+  chain_launch(k_musl_node, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls);
   rec(ev, 3, 1, st);
   rec(ev, 4, 0, st);
   if (ls.any_lattice) bm_launch_fupd_lat(w, ls, st);
@@ -2202,36 +2230,36 @@ static void launch_pairs(const World &w, const LaunchSet &ls, cudaStream_t st, c
   const int nb = w.H.n_buckets;
   const int nblk = (nb + 1023) / 1024;
   rec(ev, 10, 0, st);
-  k_pair_reset<<<(ls.n_scenes + 255) / 256, 256, 0, st>>>(w, ls);
-  k_pair_vmax<<<ls.n_btiles, BT, 0, st>>>(w, ls);
-  k_pair_decide<<<(ls.n_scenes + 63) / 64, 64, 0, st>>>(w, ls);
+  chain_launch(k_pair_reset, dim3((ls.n_scenes + 255) / 256), 256, 0, st, w, ls);
+  chain_launch(k_pair_vmax, dim3(ls.n_btiles), BT, 0, st, w, ls);
+  chain_launch(k_pair_decide, dim3((ls.n_scenes + 63) / 64), 64, 0, st, w, ls);
   cudaMemsetAsync(w.H.bucket_start, 0, sizeof(int) * ((size_t)nb + 1), st);
   cudaMemsetAsync(w.H.bucket_fill, 0, sizeof(int) * (size_t)nb, st);
   rec(ev, 10, 1, st);
   rec(ev, 11, 0, st);
-  k_pair_hash<<<ls.n_btiles, BT, 0, st>>>(w, ls);
+  chain_launch(k_pair_hash, dim3(ls.n_btiles), BT, 0, st, w, ls);
   rec(ev, 11, 1, st);
   rec(ev, 12, 0, st);
-  k_scan_local<<<nblk, 1024, 0, st>>>(w);
+  chain_launch(k_scan_local, dim3(nblk), 1024, 0, st, w);
   rec(ev, 12, 1, st);
   rec(ev, 13, 0, st);
-  k_scan_top<<<1, 1024, 0, st>>>(w, nblk);
+  chain_launch(k_scan_top, dim3(1), 1024, 0, st, w, nblk);
   rec(ev, 13, 1, st);
   rec(ev, 14, 0, st);
-  k_scan_add<<<nblk, 1024, 0, st>>>(w);
+  chain_launch(k_scan_add, dim3(nblk), 1024, 0, st, w);
   rec(ev, 14, 1, st);
   rec(ev, 15, 0, st);
-  k_pair_fill<<<ls.n_btiles, BT, 0, st>>>(w, ls);
+  chain_launch(k_pair_fill, dim3(ls.n_btiles), BT, 0, st, w, ls);
   rec(ev, 15, 1, st);
   rec(ev, 16, 0, st);
-  k_pair_sort<<<(nb + 255) / 256, 256, 0, st>>>(w);
+  chain_launch(k_pair_sort, dim3((nb + 255) / 256), 256, 0, st, w);
   rec(ev, 16, 1, st);
   rec(ev, 18, 0, st);
   const int lgrid = (nb / 32 + 7) / 8;  // 8 warps per CTA, a warp per 32 buckets, at most 8 CTAs per SM
-  k_pair_list<<<lgrid < 152 * 8 ? lgrid : 152 * 8, 256, 0, st>>>(w);
+  chain_launch(k_pair_list, dim3(lgrid < 152 * 8 ? lgrid : 152 * 8), 256, 0, st, w);
   rec(ev, 18, 1, st);
   rec(ev, 17, 0, st);
-  k_pair<<<dim3(ls.n_btiles, 4), 128, 0, st>>>(w, ls);
+  chain_launch(k_pair, dim3(ls.n_btiles, 4), 128, 0, st, w, ls);
   rec(ev, 17, 1, st);
 }
 
@@ -2240,7 +2268,7 @@ cudaError_t bm_launch_substep_ev(const World &w, const LaunchSet &ls, cudaStream
   if (ls.any_pair && w.H.n_buckets > 0) launch_pairs(w, ls, st, ev);
   launch_bricks(w, ls, st, ev);
   rec(ev, 5, 0, st);
-  k_tool<<<ls.n_scenes, 256, 0, st>>>(w, ls);
+  chain_launch(k_tool, dim3(ls.n_scenes), 256, 0, st, w, ls);
   rec(ev, 5, 1, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -2254,7 +2282,7 @@ cudaError_t bm_launch_substep(const World &w, const LaunchSet &ls, cudaStream_t 
 cudaError_t bm_launch_io(const World &w, int scene_slot, int p_begin, int n, int field, void *buf,
                          int to_pool, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_io<<<(n + 255) / 256, 256, 0, st>>>(w, scene_slot, p_begin, n, field, buf, to_pool);
+  chain_launch(k_io, dim3((unsigned)((n + 255) / 256)), 256, 0, st, w, scene_slot, p_begin, n, field, buf, to_pool);
   return cudaGetLastError();
 }
 
@@ -2268,26 +2296,26 @@ cudaError_t bm_launch_read(const World &w, int scene_slot, int p_begin, int n, u
       r.field[k++] = f;
     }
   if (n == 0 || k == 0) return cudaSuccess;
-  k_read<<<dim3((unsigned)(n + 255) / 256, (unsigned)k), 256, 0, st>>>(w, scene_slot, p_begin, n, r);
+  chain_launch(k_read, dim3((unsigned)(n + 255) / 256, (unsigned)k), 256, 0, st, w, scene_slot, p_begin, n, r);
   return cudaGetLastError();
 }
 
 cudaError_t bm_launch_set_tools(const World &w, const int *scene_ids, int n, const double *states,
                                 cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_set_tools<<<(n + 63) / 64, 64, 0, st>>>(w, scene_ids, n, states);
+  chain_launch(k_set_tools, dim3((unsigned)((n + 63) / 64)), 64, 0, st, w, scene_ids, n, states);
   return cudaGetLastError();
 }
 
 cudaError_t bm_launch_get_wrenches(const World &w, const int *scene_ids, int n, double *out,
                                    cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_get_wrenches<<<(n + 63) / 64, 64, 0, st>>>(w, scene_ids, n, out);
+  chain_launch(k_get_wrenches, dim3((unsigned)((n + 63) / 64)), 64, 0, st, w, scene_ids, n, out);
   return cudaGetLastError();
 }
 
 cudaError_t bm_launch_code(const World &w, int p_begin, int n, int64_t *out, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_code<<<(n + 255) / 256, 256, 0, st>>>(w, p_begin, n, out);
+  chain_launch(k_code, dim3((unsigned)((n + 255) / 256)), 256, 0, st, w, p_begin, n, out);
   return cudaGetLastError();
 }

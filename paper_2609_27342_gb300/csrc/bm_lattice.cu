@@ -274,6 +274,7 @@ __device__ __forceinline__ void p2g_force(P2GS &S, const CellOz &q, unsigned m) 
 
 template <int MB, bool INELASTIC>
 __global__ void __launch_bounds__(PT, MB) k_p2g_lat(World w, LaunchSet ls) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   P2GS &S = *reinterpret_cast<P2GS *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];  // scene, pool brick, first particle, count
@@ -398,6 +399,7 @@ __device__ __forceinline__ void musl_cell(G2PS &S, const CellOz &q, unsigned m) 
 
 template <int MB>
 __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   G2PS &S = *reinterpret_cast<G2PS *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];
@@ -549,6 +551,7 @@ struct FupdS {
 
 template <int MB, bool INELASTIC>
 __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
+  chain_wait();
   __shared__ FupdS S;
   const int4 bt = ls.btiles[blockIdx.x];
   DevScene &scm = w.scenes[bt.x];
@@ -684,15 +687,15 @@ cudaError_t bm_lattice_init() {
 }
 
 void bm_launch_p2g_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  if (ls.any_inelastic) k_p2g_lat<OCC_P2G, true><<<ls.n_btiles, PT, sizeof(P2GS), st>>>(w, ls);
-  else k_p2g_lat<OCC_P2G, false><<<ls.n_btiles, PT, sizeof(P2GS), st>>>(w, ls);
+  if (ls.any_inelastic) chain_launch(k_p2g_lat<OCC_P2G, true>, dim3(ls.n_btiles), PT, sizeof(P2GS), st, w, ls);
+  else chain_launch(k_p2g_lat<OCC_P2G, false>, dim3(ls.n_btiles), PT, sizeof(P2GS), st, w, ls);
 }
 
 void bm_launch_g2p_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  k_g2p_lat<OCC_G2P><<<ls.n_btiles, GT, sizeof(G2PS), st>>>(w, ls);
+  chain_launch(k_g2p_lat<OCC_G2P>, dim3(ls.n_btiles), GT, sizeof(G2PS), st, w, ls);
 }
 
 void bm_launch_fupd_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  if (ls.any_inelastic) k_fupd_lat<OCC_FUPD, true><<<ls.n_btiles, FT, 0, st>>>(w, ls);
-  else k_fupd_lat<OCC_FUPD, false><<<ls.n_btiles, FT, 0, st>>>(w, ls);
+  if (ls.any_inelastic) chain_launch(k_fupd_lat<OCC_FUPD, true>, dim3(ls.n_btiles), FT, 0, st, w, ls);
+  else chain_launch(k_fupd_lat<OCC_FUPD, false>, dim3(ls.n_btiles), FT, 0, st, w, ls);
 }

@@ -1306,6 +1306,7 @@ __device__ __forceinline__ void copy_words(char *d, const char *s, long long n) 
 }
 
 __global__ void __launch_bounds__(kCopyBlock) k_copy_sections(CopySet c) {
+  chain_wait();
   char *d = c.dst[blockIdx.y];
   const char *s = c.src[blockIdx.y];
   const long long n = c.bytes[blockIdx.y];
@@ -1320,7 +1321,7 @@ cudaError_t launch_copies(const CopySet &c, cudaStream_t st) {
   for (int i = 0; i < c.n; ++i) most = std::max(most, c.bytes[i]);
   // 16 bytes per thread and step; at most two CTAs per SM for the longest section
   const unsigned gx = (unsigned)std::min<long long>(std::max<long long>(most / (16 * kCopyBlock) + 1, 1), 2 * 152);
-  k_copy_sections<<<dim3(gx, (unsigned)c.n), kCopyBlock, 0, st>>>(c);
+  chain_launch(k_copy_sections, dim3(gx, (unsigned)c.n), kCopyBlock, 0, st, c);
   return cudaGetLastError();
 }
 

@@ -170,6 +170,7 @@ __device__ void jacobi3(float A[3][3], float V[3][3]) {
 // lattice map: lattice point -> particle, and the reference positions
 // --------------------------------------------------------------------------
 __global__ void k_sf_map(World w, SurfParams sp, int n, const int *jlin, const float *Xc) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;  // scene-relative pool index
   if (i >= n) return;
   const int c = w.P.perm[sp.p_begin + i];                // caller index
@@ -183,6 +184,7 @@ __global__ void k_sf_map(World w, SurfParams sp, int n, const int *jlin, const f
 // one of their corners) and each corner's vertex ordinal
 // --------------------------------------------------------------------------
 __global__ void k_sf_cells(World w, SurfParams sp) {
+  chain_wait();
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= sp.n_cells) return;
   int j[3];
@@ -210,6 +212,7 @@ __global__ void k_sf_cells(World w, SurfParams sp) {
 
 // the cell and ordinal of every vertex
 __global__ void k_sf_list(SurfParams sp) {
+  chain_wait();
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= sp.n_cells) return;
   const int cnt = sp.cell_cnt[i], base = sp.cell_off[i];
@@ -237,6 +240,7 @@ __device__ __forceinline__ void trilinear(const SurfParams &sp, const float c[3]
 // eigen-decomposition (34,774 vertices of 337,881 cells: 107 us, now 56).  Each
 // vertex also marks the grid nodes that its embedding reads.
 __global__ void k_sf_vertices(World w, SurfParams sp, int nv) {
+  chain_wait();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= nv) return;
   const long long i = sp.vcell[v];
@@ -330,6 +334,7 @@ __global__ void k_sf_vertices(World w, SurfParams sp, int nv) {
 // --------------------------------------------------------------------------
 template <bool WRITE>
 __global__ void k_sf_tris(World w, SurfParams sp) {
+  chain_wait();
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= sp.n_cells) return;
   if (sp.cell_cnt[i] == 0) {  // the link's own cell (lower corner j) carries a vertex
@@ -449,6 +454,7 @@ __device__ __forceinline__ float warp_xor_sum(float v) {
 constexpr int kNodeWarps = 8;
 
 __global__ void __launch_bounds__(32 * kNodeWarps) k_sf_nodes(World w, SurfParams sp) {
+  chain_wait();
   const DevScene &sc = w.scenes[sp.slot];
   const int lane = threadIdx.x & 31;
   const int li = blockIdx.x * kNodeWarps + (threadIdx.x >> 5);
@@ -470,6 +476,7 @@ __global__ void __launch_bounds__(32 * kNodeWarps) k_sf_nodes(World w, SurfParam
 }
 
 __global__ void k_sf_embed(World w, SurfParams sp, int nv) {
+  chain_wait();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= nv) return;
   const DevScene &sc = w.scenes[sp.slot];
@@ -522,6 +529,7 @@ __global__ void k_sf_embed(World w, SurfParams sp, int nv) {
 
 // n records of nc words from columns, into an array of records
 __global__ void k_sf_pack(const uint32_t *c0, const uint32_t *c1, const uint32_t *c2, int nc, int n, uint32_t *out) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   out[(size_t)nc * i] = c0[i];
@@ -560,6 +568,7 @@ __device__ int block_scan_excl(int v, int *sm, int &total) {
 }
 
 __global__ void __launch_bounds__(kScanBlock) k_sf_scan_block(const int *in, int *out, int *bsum, long long n) {
+  chain_wait();
   __shared__ int sm[kScanBlock / 32 + 1];
   const long long i = blockIdx.x * (long long)kScanBlock + threadIdx.x;
   int total;
@@ -569,6 +578,7 @@ __global__ void __launch_bounds__(kScanBlock) k_sf_scan_block(const int *in, int
 }
 
 __global__ void __launch_bounds__(kScanBlock) k_sf_scan_top(int *bsum, int nb, int *total_out) {
+  chain_wait();
   __shared__ int sm[kScanBlock / 32 + 1];
   int carry = 0;
   for (int b0 = 0; b0 < nb; b0 += kScanBlock) {
@@ -582,15 +592,16 @@ __global__ void __launch_bounds__(kScanBlock) k_sf_scan_top(int *bsum, int nb, i
 }
 
 __global__ void k_sf_scan_add(int *out, const int *bsum, long long n) {
+  chain_wait();
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i < n) out[i] += bsum[i / kScanBlock];
 }
 
 cudaError_t scan_excl(const int *in, int *out, int *total, int *tmp, long long n, cudaStream_t st) {
   const int nb = (int)((n + kScanBlock - 1) / kScanBlock);
-  if (nb > 0) k_sf_scan_block<<<nb, kScanBlock, 0, st>>>(in, out, tmp, n);
-  k_sf_scan_top<<<1, kScanBlock, 0, st>>>(tmp, nb, total);
-  if (nb > 0) k_sf_scan_add<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(out, tmp, n);
+  if (nb > 0) chain_launch(k_sf_scan_block, dim3((unsigned)nb), kScanBlock, 0, st, in, out, tmp, n);
+  chain_launch(k_sf_scan_top, dim3(1), kScanBlock, 0, st, tmp, nb, total);
+  if (nb > 0) chain_launch(k_sf_scan_add, dim3((unsigned)((n + 255) / 256)), 256, 0, st, out, tmp, n);
   return cudaGetLastError();
 }
 
@@ -600,18 +611,18 @@ inline unsigned grid_of(long long n, int bs) { return (unsigned)((n + bs - 1) / 
 
 cudaError_t bm_launch_surface_map(const World &w, const SurfParams &sp, int n, const int *jlin,
                                   const float *Xc, cudaStream_t st) {
-  if (n > 0) k_sf_map<<<grid_of(n, 256), 256, 0, st>>>(w, sp, n, jlin, Xc);
+  if (n > 0) chain_launch(k_sf_map, dim3(grid_of(n, 256)), 256, 0, st, w, sp, n, jlin, Xc);
   return cudaGetLastError();
 }
 
 // regions and their vertices' places, then the triangles' places; the two
 // totals end up in sp.totals
 cudaError_t bm_launch_surface_count(const World &w, const SurfParams &sp, cudaStream_t st) {
-  k_sf_cells<<<grid_of(sp.n_cells, 128), 128, 0, st>>>(w, sp);
+  chain_launch(k_sf_cells, dim3(grid_of(sp.n_cells, 128)), 128, 0, st, w, sp);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = scan_excl(sp.cell_cnt, sp.cell_off, sp.totals, sp.scan_tmp, sp.n_cells, st);
   if (e != cudaSuccess) return e;
-  k_sf_tris<false><<<grid_of(sp.n_cells, 128), 128, 0, st>>>(w, sp);
+  chain_launch(k_sf_tris<false>, dim3(grid_of(sp.n_cells, 128)), 128, 0, st, w, sp);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = scan_excl(sp.pt_cnt, sp.pt_off, sp.totals + 1, sp.scan_tmp, sp.n_cells, st);
   return e;
@@ -621,23 +632,23 @@ cudaError_t bm_launch_surface_write(const World &w, const SurfParams &sp, int n_
                                     cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(sp.nmark, 0, (size_t)n_node, st);
   if (e != cudaSuccess) return e;
-  k_sf_list<<<grid_of(sp.n_cells, 256), 256, 0, st>>>(sp);
-  if (n_vertices > 0) k_sf_vertices<<<grid_of(n_vertices, 64), 64, 0, st>>>(w, sp, n_vertices);
-  k_sf_tris<true><<<grid_of(sp.n_cells, 128), 128, 0, st>>>(w, sp);
+  chain_launch(k_sf_list, dim3(grid_of(sp.n_cells, 256)), 256, 0, st, sp);
+  if (n_vertices > 0) chain_launch(k_sf_vertices, dim3(grid_of(n_vertices, 64)), 64, 0, st, w, sp, n_vertices);
+  chain_launch(k_sf_tris<true>, dim3(grid_of(sp.n_cells, 128)), 128, 0, st, w, sp);
   return cudaGetLastError();
 }
 
 cudaError_t bm_launch_surface_embed(const World &w, const SurfParams &sp, int n_vertices, int n_node,
                                     cudaStream_t st) {
   if (n_vertices == 0) return cudaSuccess;
-  k_sf_nodes<<<grid_of(n_node, kNodeWarps), 32 * kNodeWarps, 0, st>>>(w, sp);
-  k_sf_embed<<<grid_of(n_vertices, 128), 128, 0, st>>>(w, sp, n_vertices);
+  chain_launch(k_sf_nodes, dim3(grid_of(n_node, kNodeWarps)), 32 * kNodeWarps, 0, st, w, sp);
+  chain_launch(k_sf_embed, dim3(grid_of(n_vertices, 128)), 128, 0, st, w, sp, n_vertices);
   return cudaGetLastError();
 }
 
 cudaError_t bm_launch_surface_pack(const void *const *cols, int nc, int n, void *out, cudaStream_t st) {
   if (n > 0)
-    k_sf_pack<<<grid_of(n, 256), 256, 0, st>>>((const uint32_t *)cols[0], (const uint32_t *)cols[1],
+    chain_launch(k_sf_pack, dim3(grid_of(n, 256)), 256, 0, st, (const uint32_t *)cols[0], (const uint32_t *)cols[1],
                                                nc > 2 ? (const uint32_t *)cols[2] : nullptr, nc, n, (uint32_t *)out);
   return cudaGetLastError();
 }
