@@ -116,6 +116,7 @@ struct bm_scene_s {
   int64_t p_begin = 0, cell_begin = 0, node_begin = 0, slot_begin = 0, hist_begin = 0, brick_begin = 0,
           ppool_begin = 0;
   int ntile_begin = 0, n_ntile = 0;
+  int dev_ntile[2] = {-1, -1};        // the same as last uploaded to the scene's record (-1: not since it was placed)
   DevScene tmpl{};                    // static fields (host template)
   // staged fresh state, uploaded when the scene first enters a world
   std::vector<float> h_fx[3];
@@ -334,6 +335,9 @@ int rebuild_tiles(WorldH *W) {
   if (!ids.empty()) CK(cudaMemcpy(W->d_scene_ids, ids.data(), sizeof(int) * ids.size(), cudaMemcpyHostToDevice));
   for (bm_scene_s *s : W->members) {
     int r[2] = {s->ntile_begin, s->n_ntile};
+    if (r[0] == s->dev_ntile[0] && r[1] == s->dev_ntile[1]) continue;  // as in the record already
+    s->dev_ntile[0] = r[0];
+    s->dev_ntile[1] = r[1];
     CK(cudaMemcpy((char *)(W->w.scenes + s->slot) + offsetof(DevScene, ntile_begin), r, sizeof r,
                   cudaMemcpyHostToDevice));
   }
@@ -527,6 +531,7 @@ int reserve(WorldH *W, bm_scene_s *s) {
     if (hb >= 0) W->rhist.give(hb, s->hist_cap);
     return fail(BM_E_CAPACITY, "batch pools have no room for the scene");
   }
+  s->dev_ntile[0] = s->dev_ntile[1] = -1;
   s->slot = W->free_slots.back();
   W->free_slots.pop_back();
   s->p_begin = pb;
@@ -792,38 +797,38 @@ int validate_desc(const bm_scene_desc *d) {
 // laid out per brick.  A lattice cell of more than 2 x 2 x 2 particles,
 // another order, or positions off the planes (a jittered or scanned body)
 // take the general kernels.
-void find_lattice(bm_scene_s *s, const std::vector<double> &f3, const std::vector<int> &b3, const int lo[3]) {
+void find_lattice(bm_scene_s *s) {
   s->lattice = false;
   if (s->ppc_max > 8) return;
   const int64_t n = s->n;
+  const float *f[3] = {s->h_fx[0].data(), s->h_fx[1].data(), s->h_fx[2].data()};
+  const uint32_t *base = s->h_base.data();
   std::vector<float> pl[3];  // per axis and base-cell layer: the planes' offsets, ascending (-1: none)
-  for (int a = 0; a < 3; ++a) {
-    pl[a].assign((size_t)s->nb[a] * 2, -1.0f);
-    for (int64_t i = 0; i < n; ++i) {
-      float *q = &pl[a][2 * (size_t)(b3[3 * i + a] - lo[a])];
-      const float f = (float)f3[3 * i + a];
-      if (f == q[0] || f == q[1]) continue;
+  for (int a = 0; a < 3; ++a) pl[a].assign((size_t)s->nb[a] * 2, -1.0f);
+  for (int64_t j = 0; j < n; ++j)
+    for (int a = 0; a < 3; ++a) {
+      float *q = &pl[a][2 * (size_t)((base[j] >> (10 * a)) & 1023u)];
+      const float v = f[a][j];
+      if (v == q[0] || v == q[1]) continue;
       if (q[1] >= 0.0f) return;  // a third plane
-      if (q[0] < 0.0f) q[0] = f;
-      else q[1] = f;
+      if (q[0] < 0.0f) q[0] = v;
+      else q[1] = v;
     }
+  for (int a = 0; a < 3; ++a)
     for (int c = 0; c < s->nb[a]; ++c)
       if (pl[a][2 * c + 1] >= 0.0f && pl[a][2 * c + 1] < pl[a][2 * c]) std::swap(pl[a][2 * c], pl[a][2 * c + 1]);
-  }
   s->h_lpos.resize((size_t)n);
-  int64_t last_cell = -1;
+  uint32_t last_cell = 0xffffffffu;
   int last_key = -1;
   for (int64_t j = 0; j < n; ++j) {
-    const int64_t i = s->h_perm[j];
-    int x[3], b[3];
+    int x[3];
     for (int a = 0; a < 3; ++a) {
-      b[a] = b3[3 * i + a] - lo[a];
-      x[a] = 2 * (b[a] & 3) + ((float)f3[3 * i + a] != pl[a][2 * (size_t)b[a]]);
+      const int c = (int)((base[j] >> (10 * a)) & 1023u);
+      x[a] = 2 * (c & 3) + (f[a][j] != pl[a][2 * (size_t)c]);
     }
-    const int64_t cell = ((int64_t)b[2] * s->nb[1] + b[1]) * s->nb[0] + b[0];
     const int key = ((x[0] & 1) * 2 + (x[1] & 1)) * 2 + (x[2] & 1);
-    if (cell == last_cell && key <= last_key) return;  // another order, or two particles at one place
-    last_cell = cell;
+    if (base[j] == last_cell && key <= last_key) return;  // another order, or two particles at one place
+    last_cell = base[j];
     last_key = key;
     s->h_lpos[(size_t)j] = (uint16_t)bm_lat_place(x[0], x[1], x[2]);
   }
@@ -896,7 +901,7 @@ int build_layout(bm_scene_s *s) {
              bz = (uint32_t)(b3[3 * i + 2] - lo[2]);
     s->h_base[j] = bx | (by << 10) | (bz << 20);
   }
-  find_lattice(s, f3, b3, lo);
+  find_lattice(s);
   s->slot_cap = std::max<int64_t>(4 * s->n_node, 64);
   // brick-tile partial sums: a node appears in <= 8 tiles, ~3.4 on average;
   // 6 entries per node covers ~1.8 logical grids per node on average
