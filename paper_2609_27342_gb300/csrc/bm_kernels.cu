@@ -1008,28 +1008,25 @@ __global__ void k_pair_fill(World w, LaunchSet ls) {
   }
 }
 
-// order each bucket by pool index (buckets are short), then lay out its
-// entries (position, pool index, base cell, cell key) for the list build
+// the entries of each bucket in pool-index order (position, pool index, base
+// cell, cell key), for the list build.  A thread per entry counts the
+// bucket's smaller indices (buckets are short); sorting a bucket in place, a
+// thread per bucket, took 30 us on the 252,800-particle cylinder, most of
+// 524,288 buckets being empty and the others a chain of global reads and
+// writes.
 __global__ void k_pair_sort(World w) {
   chain_wait();
   if (!*w.H.build) return;
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < w.H.n_buckets; b += gridDim.x * blockDim.x) {
+  const int total = w.H.bucket_start[w.H.n_buckets];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+    const int q = w.P.horder[e];
+    const int b = w.P.hkey[q];
     const int s0 = w.H.bucket_start[b], s1 = w.H.bucket_start[b + 1];
-    for (int i = s0 + 1; i < s1; ++i) {
-      const int key = w.P.horder[i];
-      int j = i - 1;
-      while (j >= s0 && w.P.horder[j] > key) {
-        w.P.horder[j + 1] = w.P.horder[j];
-        --j;
-      }
-      w.P.horder[j + 1] = key;
-    }
-    for (int i = s0; i < s1; ++i) {
-      const int q = w.P.horder[i];
-      w.P.hent[i] = make_float4(w.P.x[0][q], w.P.x[1][q], w.P.x[2][q], __int_as_float(q));
-      w.P.hbase[i] = w.P.base[q];
-      w.P.hentk[i] = w.P.hcell[q];
-    }
+    int i = s0;
+    for (int k = s0; k < s1; ++k) i += w.P.horder[k] < q ? 1 : 0;
+    w.P.hent[i] = make_float4(w.P.x[0][q], w.P.x[1][q], w.P.x[2][q], __int_as_float(q));
+    w.P.hbase[i] = w.P.base[q];
+    w.P.hentk[i] = w.P.hcell[q];
   }
 }
 
@@ -1047,18 +1044,32 @@ __device__ __forceinline__ bool share_stencil(uint32_t bp, uint32_t bq) {
 // 32, lane i holding entry c0 + i), by one warp.  The particles are taken in
 // groups of one cell (and scene); a group shares its 27 neighbour cells
 // (dz, dy, dx in -1..1, x fastest), whose bucket entries are laid end to end
-// and tested 32 at a time, one per lane, against each member in turn: an
+// and tested 64 at a time, two per lane, against each member in turn (read
+// from the warp's shared memory: five shuffles a member for every 32 entries
+// were a third of the kernel's instructions): an
 // entry counts when it belongs to the neighbour cell (its key; a bucket's
 // hash may be shared), is another particle and lies within r_l = 2 R_p +
 // skin.  A ballot gives each accepted entry its place, so every list is in
 // (cell, pool index) order, as a walk of the cells in order would give;
-// bit 31 of an entry marks a pair whose reference stencils overlap.
-__device__ __forceinline__ void bucket_lists(const World &w, int c0, int c1, int lane) {
+// bit 31 of an entry marks a pair whose reference stencils overlap, and a
+// list of only such pairs is marked by NBR_SHARED in its count.
+#define NBR_SHARED 0x80
+#define LIST_WARPS 8
+
+struct ListMembers {
+  float4 me[32];
+  uint32_t base[32];
+};
+
+__device__ __forceinline__ void bucket_lists(const World &w, ListMembers &M, int c0, int c1, int lane) {
   const PPool &P = w.P;
   const bool mine = lane < c1 - c0;
   const float4 me = mine ? P.hent[c0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
   const unsigned long long mkey = mine ? P.hentk[c0 + lane] : ~0ull;
-  const uint32_t mbase = mine ? P.hbase[c0 + lane] : 0u;
+  __syncwarp();
+  M.me[lane] = me;
+  M.base[lane] = mine ? P.hbase[c0 + lane] : 0u;
+  __syncwarp();
   const int mscene = (int)(mkey >> 48);
   int mx = 0, my = 0, mz = 0;
   if (mine) {
@@ -1068,6 +1079,7 @@ __device__ __forceinline__ void bucket_lists(const World &w, int c0, int c1, int
     mz = (int)floorf(me.z * ih);
   }
   int cnt = 0;
+  bool apart = false;  // some pair of the lane's list shares no stencil
   unsigned todo = __ballot_sync(FULL, mine);
   while (todo) {
     const int lead = __ffs(todo) - 1;
@@ -1096,49 +1108,65 @@ __device__ __forceinline__ void bucket_lists(const World &w, int c0, int c1, int
     }
     const int T = __shfl_sync(FULL, incl, 31);
     const int excl = incl - sz;
-    for (int base = 0; base < T; base += 32) {
-      const int j = base + lane;
-      // neighbour cell of candidate j: the last cell whose entries start at or before j
-      int L = 0;
+    for (int base = 0; base < T; base += 64) {
+      float4 e[2];
+      uint32_t eb[2];
+      bool valid[2];
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const int t = L + step;
-        const int ex = __shfl_sync(FULL, excl, t < 27 ? t : 26);
-        if (t < 27 && ex <= j) L = t;
+      for (int h = 0; h < 2; ++h) {
+        const int j = base + 32 * h + lane;
+        // neighbour cell of candidate j: the last cell whose entries start at or before j
+        int L = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+          const int t = L + step;
+          const int ex = __shfl_sync(FULL, excl, t < 27 ? t : 26);
+          if (t < 27 && ex <= j) L = t;
+        }
+        const int aL = __shfl_sync(FULL, a0, L), exL = __shfl_sync(FULL, excl, L);
+        const unsigned long long kL = __shfl_sync(FULL, nk, L);
+        const bool inr = j < T;
+        const int k = aL + (j - exL);
+        e[h] = inr ? P.hent[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const unsigned long long ek = inr ? P.hentk[k] : 0ull;
+        eb[h] = inr ? P.hbase[k] : 0u;
+        valid[h] = inr && ek == kL;
       }
-      const int aL = __shfl_sync(FULL, a0, L), exL = __shfl_sync(FULL, excl, L);
-      const unsigned long long kL = __shfl_sync(FULL, nk, L);
-      const bool inr = j < T;
-      const int k = aL + (j - exL);
-      const float4 e = inr ? P.hent[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-      const unsigned long long ek = inr ? P.hentk[k] : 0ull;
-      const uint32_t eb = inr ? P.hbase[k] : 0u;
-      const bool valid = inr && ek == kL;
-      const int q = __float_as_int(e.w);
       unsigned g = grp;
       while (g) {
         const int m = __ffs(g) - 1;
         g &= g - 1;
-        const float px = __shfl_sync(FULL, me.x, m), py = __shfl_sync(FULL, me.y, m),
-                    pz = __shfl_sync(FULL, me.z, m);
-        const int p = __float_as_int(__shfl_sync(FULL, me.w, m));
-        const uint32_t bp = __shfl_sync(FULL, mbase, m);
-        const float d0 = px - e.x, d1 = py - e.y, d2 = pz - e.z;
-        const bool acc = valid && q != p && d0 * d0 + d1 * d1 + d2 * d2 <= rl2;
-        const unsigned am = __ballot_sync(FULL, acc);
-        const int c = __shfl_sync(FULL, cnt, m);
-        if (acc) {
-          const int pos = c + __popc(am & ((1u << lane) - 1u));
-          if (pos < BM_NBR)
-            P.nbr[(size_t)p * BM_NBR + pos] = share_stencil(bp, eb) ? (int)((uint32_t)q | 0x80000000u) : q;
+        const float4 mp = M.me[m];
+        const uint32_t bp = M.base[m];
+        const int p = __float_as_int(mp.w);
+        int c = __shfl_sync(FULL, cnt, m);
+        const int c_in = c;
+        bool far = false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int q = __float_as_int(e[h].w);
+          const float d0 = mp.x - e[h].x, d1 = mp.y - e[h].y, d2 = mp.z - e[h].z;
+          const bool acc = valid[h] && q != p && d0 * d0 + d1 * d1 + d2 * d2 <= rl2;
+          const unsigned am = __ballot_sync(FULL, acc);
+          if (acc) {
+            const int pos = c + __popc(am & ((1u << lane) - 1u));
+            const bool share = share_stencil(bp, eb[h]);
+            far |= !share;
+            if (pos < BM_NBR) P.nbr[(size_t)p * BM_NBR + pos] = share ? (int)((uint32_t)q | 0x80000000u) : q;
+          }
+          c += __popc(am);
         }
-        if (lane == m) cnt += __popc(am);
+        const bool any_far = __any_sync(FULL, far);
+        if (lane == m) {
+          cnt += c - c_in;
+          apart |= any_far;
+        }
       }
     }
   }
   if (mine) {
     const int p = __float_as_int(me.w);
-    P.nbr_n[p] = (uint8_t)min(cnt, BM_NBR);
+    P.nbr_n[p] = (uint8_t)(min(cnt, BM_NBR) | (apart ? 0 : NBR_SHARED));
     P.xb[0][p] = me.x;
     P.xb[1][p] = me.y;
     P.xb[2][p] = me.z;
@@ -1150,9 +1178,10 @@ __device__ __forceinline__ void bucket_lists(const World &w, int c0, int c1, int
 // warp takes groups of 32 buckets (grid-stride) and builds the lists of the
 // particles of each non-empty one, 32 entries at a time.  The positions of
 // the build are kept.
-__global__ void __launch_bounds__(256) k_pair_list(World w) {
+__global__ void __launch_bounds__(32 * LIST_WARPS) k_pair_list(World w) {
   chain_wait();
   if (!*w.H.build) return;
+  __shared__ ListMembers members[LIST_WARPS];
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
   const int nb = w.H.n_buckets;
@@ -1164,7 +1193,7 @@ __global__ void __launch_bounds__(256) k_pair_list(World w) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
       const int k0 = __shfl_sync(FULL, e0, src), k1 = __shfl_sync(FULL, e1, src);
-      for (int c = k0; c < k1; c += 32) bucket_lists(w, c, min(k1, c + 32), lane);
+      for (int c = k0; c < k1; c += 32) bucket_lists(w, members[threadIdx.x >> 5], c, min(k1, c + 32), lane);
     }
   }
 }
@@ -1172,7 +1201,8 @@ __global__ void __launch_bounds__(256) k_pair_list(World w) {
 // Pair impulses (Eq. 10-13), one thread per particle walking its list
 // (gridDim.y CTAs per brick).  A candidate sharing p's reference stencil is
 // skipped unless the two are on opposite sides of a cut, before its state
-// is read.
+// is read; a particle without labels is on no side, so such candidates of it
+// are skipped unread, and a list of nothing else (NBR_SHARED) is not walked.
 __global__ void k_pair(World w, LaunchSet ls) {
   chain_wait();
   const int4 bt = ls.btiles[blockIdx.x];
@@ -1191,12 +1221,14 @@ __global__ void k_pair(World w, LaunchSet ls) {
     const uint32_t a1 = P.s1[p], a2 = P.s2[p];
     float J[3] = {0.f, 0.f, 0.f};
     int cnt = 0;
-    const int n = P.nbr_n[p];
+    const int nn8 = P.nbr_n[p];
+    const bool uncut = (a1 | a2) == 0u;
+    const int n = uncut && (nn8 & NBR_SHARED) ? 0 : nn8 & (NBR_SHARED - 1);
     const int *lst = P.nbr + (size_t)p * BM_NBR;
     for (int k = 0; k < n; ++k) {
       const int ent = lst[k];
       const int q = ent & 0x7fffffff;
-      if (ent < 0 && !conflict(a1, a2, P.s1[q], P.s2[q])) continue;  // self-contact exclusion
+      if (ent < 0 && (uncut || !conflict(a1, a2, P.s1[q], P.s2[q]))) continue;  // self-contact exclusion
       const float xq[3] = {P.x[0][q], P.x[1][q], P.x[2][q]};
       const float vq[3] = {P.v[0][q], P.v[1][q], P.v[2][q]};
       const bool plo = p < q;
@@ -2252,11 +2284,11 @@ static void launch_pairs(const World &w, const LaunchSet &ls, cudaStream_t st, c
   chain_launch(k_pair_fill, dim3(ls.n_btiles), BT, 0, st, w, ls);
   rec(ev, 15, 1, st);
   rec(ev, 16, 0, st);
-  chain_launch(k_pair_sort, dim3((nb + 255) / 256), 256, 0, st, w);
+  chain_launch(k_pair_sort, dim3((nb / 2 + 255) / 256), 256, 0, st, w);  // at least a thread per particle
   rec(ev, 16, 1, st);
   rec(ev, 18, 0, st);
   const int lgrid = (nb / 32 + 7) / 8;  // 8 warps per CTA, a warp per 32 buckets, at most 8 CTAs per SM
-  chain_launch(k_pair_list, dim3(lgrid < 152 * 8 ? lgrid : 152 * 8), 256, 0, st, w);
+  chain_launch(k_pair_list, dim3(lgrid < 152 * 8 ? lgrid : 152 * 8), 32 * LIST_WARPS, 0, st, w);
   rec(ev, 18, 1, st);
   rec(ev, 17, 0, st);
   chain_launch(k_pair, dim3(ls.n_btiles, 4), 128, 0, st, w, ls);
