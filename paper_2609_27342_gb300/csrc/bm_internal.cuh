@@ -137,11 +137,11 @@ struct DevScene {
   // counters and flags
   long long step;
   long long stop_at;        // >= 0: the scene stops advancing once step reaches it
-  int frozen;               // set by the tool kernel when step reaches stop_at; every
+  int frozen;               // set by the tool step when step reaches stop_at; every
                             // substep kernel then leaves the scene untouched
   unsigned int err;
-  int label_pending;
-  int need_rebuild;
+  int label_pending;        // k_fupd committed labels: the slot table is rebuilt this substep
+  int reserved;             // (saved records keep their layout)
   int n_slots;
   int lattice;              // the lattice kernels (bm_lattice.cu) carry this scene's transfers
 };
@@ -220,6 +220,7 @@ struct World {
   SPool S;
   BPool B;
   HashPool H;
+  DevScene *scenes_next;    // each scene's tool block, step and frozen after this substep
   double *wpart;            // per brick wrench partials (6 doubles)
   double *whist;            // wrench history records (6 doubles)
 };

@@ -670,13 +670,275 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
   }
 }
 
+__device__ const DevSeg *seg_at(const DevScene &sc, long long step) {
+  long long acc = 0;
+  for (int i = 0; i < sc.nseg; ++i) {
+    acc += sc.seg[i].n_steps;
+    if (step < acc) return &sc.seg[i];
+  }
+  return nullptr;
+}
+
+// The tool step by one warp on the shared-memory copy of the scene record:
+// wrench history, interval-averaged rigid tool step, and the frame of the
+// next substep.  Float64 operations are slow here (about 2 lanes per clock
+// and SM), so each component of a vector or matrix is its own lane's, in the
+// expression of the one-thread code: a serial thread spent most of the
+// kernel's 16.5 us (a 16,000-particle scene) on some 400 of them; 9.2 us now.
+__device__ __forceinline__ double matmul_at(const double A[9], const double B[9], int k) {
+  const int i = k / 3, j = k % 3;
+  return A[3 * i] * B[j] + A[3 * i + 1] * B[3 + j] + A[3 * i + 2] * B[6 + j];
+}
+
+struct ToolTmp {
+  double Fa[3], Ta[3], th[3], A[9], Iw[9], K[9], K2[9], Rinc[9];
+};
+
+__device__ __forceinline__ void prepare_substep_warp(DevScene &sc, ToolTmp &T, int lane) {
+  if (!sc.has_blade) {
+    if (lane == 0) {
+      sc.cut = -1;
+      sc.reset_D = 0;
+    }
+    return;
+  }
+  const DevSeg *sg = seg_at(sc, sc.step);
+  const int cut = sg ? sg->cut_id : -1;
+  const bool dynamic = sc.mass > 0.0;
+  const int reset = (cut >= 0 && cut != sc.cur_cut) ? 1 : 0;
+  if (!dynamic && sg && lane < 3) {
+    sc.vB[lane] = sg->v[lane];
+    sc.wB[lane] = sg->w[lane];
+  }
+  if (lane == 0) {
+    sc.cut = cut;
+    sc.reset_D = reset;
+  }
+  // edge point and blade axes: lane 3 q + i holds component i of vector q
+  if (lane < 12) {
+    const int q = lane / 3, i = lane % 3;
+    const double *v = q == 0 ? sc.edgeT : q == 1 ? sc.nT : q == 2 ? sc.eT : sc.dT;
+    const double y = __dadd_rn(__dadd_rn(__dmul_rn(sc.R[3 * i], v[0]), __dmul_rn(sc.R[3 * i + 1], v[1])),
+                               __dmul_rn(sc.R[3 * i + 2], v[2]));
+    double *o = q == 0 ? sc.dxe : q == 1 ? sc.dn : q == 2 ? sc.de : sc.dd;
+    o[i] = q == 0 ? __dadd_rn(sc.xB[i], y) : y;
+  }
+  __syncwarp();
+  if (lane < 3) {
+    const int i = lane, j = (lane + 1) % 3, k = (lane + 2) % 3;
+    const double rj = __dsub_rn(sc.dxe[j], sc.xB[j]), rk = __dsub_rn(sc.dxe[k], sc.xB[k]);
+    const double wr = __dsub_rn(__dmul_rn(sc.wB[j], rk), __dmul_rn(sc.wB[k], rj));
+    sc.dve[i] = __dadd_rn(sc.vB[i], wr);
+  }
+  if (dynamic && lane < 9) T.A[lane] = matmul_at(sc.R, sc.Ib_inv, lane);
+  __syncwarp();
+  if (reset) {  // a new cut begins: keep its plane for the cut faces
+    if (lane < 3) sc.cutpl[cut][lane] = sc.dn[lane];
+    if (lane == 3) {
+      sc.cutpl[cut][3] = __dadd_rn(__dadd_rn(__dmul_rn(sc.dn[0], sc.dxe[0]), __dmul_rn(sc.dn[1], sc.dxe[1])),
+                                   __dmul_rn(sc.dn[2], sc.dxe[2]));
+      sc.cutpl_set |= 1u << cut;
+    }
+  }
+  if (lane < 3) {
+    const int i = lane;
+    sc.fxe[i] = (float)sc.dxe[i];
+    sc.fn[i] = (float)sc.dn[i];
+    sc.fe[i] = (float)sc.de[i];
+    sc.fd[i] = (float)sc.dd[i];
+    sc.fve[i] = (float)sc.dve[i];
+    sc.fc[i] = (float)(sc.dxe[i] - sc.half_height * sc.dd[i]);
+    sc.fxB[i] = (float)sc.xB[i];
+    sc.fvB[i] = (float)sc.vB[i];
+    sc.fwB[i] = (float)sc.wB[i];
+  }
+  if (lane == 3) {
+    sc.fhext[0] = (float)sc.half_thick;
+    sc.fhext[1] = (float)sc.half_len;
+    sc.fhext[2] = (float)sc.half_height;
+    sc.fL = (float)sc.L_d;
+    sc.fmu_s = (float)sc.mu_s;
+    sc.fmu_d = (float)sc.mu_d;
+    sc.finv_mass = dynamic ? (float)(1.0 / sc.mass) : 0.f;
+  }
+  if (lane < 9) {  // world inverse inertia R Ib^-1 R^T
+    const int i = lane / 3, j = lane % 3;
+    sc.fIinv[lane] =
+        dynamic ? (float)(T.A[3 * i] * sc.R[3 * j] + T.A[3 * i + 1] * sc.R[3 * j + 1] + T.A[3 * i + 2] * sc.R[3 * j + 2])
+                : 0.f;
+  }
+}
+
+__device__ __forceinline__ void tool_step(const World &w, DevScene &sc, ToolTmp &T, const double W[6], int lane) {
+  if (sc.has_blade) {
+    const long long st = sc.step;
+    if (st < sc.hist_cap && lane < 6) w.whist[(size_t)(sc.hist_begin + st) * 6 + lane] = W[lane];
+    const int cnt = sc.acc_cnt + 1;
+    if (lane < 3) {
+      sc.accF[lane] += W[lane];
+      sc.accT[lane] += W[3 + lane];
+    }
+    __syncwarp();
+    if (cnt >= sc.rigid_interval) {
+      const double H = sc.dt_d * cnt;
+      if (lane < 3) {
+        T.Fa[lane] = sc.accF[lane] / cnt;
+        T.Ta[lane] = sc.accT[lane] / cnt;
+      }
+      if (sc.mass > 0.0) {
+        const DevSeg *tg = seg_at(sc, st);
+        if (lane < 9) T.A[lane] = matmul_at(sc.R, sc.Ib_inv, lane);
+        __syncwarp();
+        if (lane < 9) {
+          const int i = lane / 3, j = lane % 3;
+          T.Iw[lane] = T.A[3 * i] * sc.R[3 * j] + T.A[3 * i + 1] * sc.R[3 * j + 1] + T.A[3 * i + 2] * sc.R[3 * j + 2];
+        }
+        __syncwarp();
+        if (lane < 3) {
+          const int k = lane;
+          const double dw = T.Iw[3 * k] * T.Ta[0] + T.Iw[3 * k + 1] * T.Ta[1] + T.Iw[3 * k + 2] * T.Ta[2];
+          const double vt = tg ? tg->v[k] : 0.0, wt = tg ? tg->w[k] : 0.0;
+          sc.vB[k] += H * (sc.kv * (vt - sc.vB[k]) + T.Fa[k] / sc.mass);
+          sc.wB[k] += H * (sc.kv * (wt - sc.wB[k]) + dw);
+        }
+      }
+      __syncwarp();
+      if (lane < 3) T.th[lane] = H * sc.wB[lane];
+      __syncwarp();
+      // rotation increment exp(th): I + sin a K + (1 - cos a) K^2
+      const double th0 = T.th[0], th1 = T.th[1], th2 = T.th[2];
+      const double a = sqrt(th0 * th0 + th1 * th1 + th2 * th2);
+      if (a > 0) {
+        const double k0 = th0 / a, k1 = th1 / a, k2 = th2 / a;
+        if (lane == 0) {
+          T.K[0] = T.K[4] = T.K[8] = 0;
+          T.K[1] = -k2;
+          T.K[2] = k1;
+          T.K[3] = k2;
+          T.K[5] = -k0;
+          T.K[6] = -k1;
+          T.K[7] = k0;
+        }
+        __syncwarp();
+        if (lane < 9) {
+          const double sa = sin(a), ca = 1.0 - cos(a);
+          double r = (lane % 4 == 0) ? 1.0 : 0.0;
+          r += sa * T.K[lane] + ca * matmul_at(T.K, T.K, lane);
+          T.Rinc[lane] = r;
+        }
+      } else if (lane < 9) {
+        T.Rinc[lane] = (lane % 4 == 0) ? 1.0 : 0.0;
+      }
+      __syncwarp();
+      const double Rn = lane < 9 ? matmul_at(T.Rinc, sc.R, lane) : 0.0;
+      __syncwarp();
+      if (lane < 9) sc.R[lane] = Rn;
+      if (lane < 3) {
+        sc.xB[lane] += H * sc.vB[lane];
+        sc.lastW[lane] = T.Fa[lane];
+        sc.lastW[3 + lane] = T.Ta[lane];
+        sc.accF[lane] = sc.accT[lane] = 0.0;
+      }
+    }
+    __syncwarp();
+    if (lane == 0) {
+      sc.acc_cnt = cnt >= sc.rigid_interval ? 0 : cnt;
+      if (sc.cut >= 0) sc.cur_cut = sc.cut;
+    }
+  }
+  if (lane == 0) {
+    sc.step++;
+    if (sc.stop_at >= 0 && sc.step >= sc.stop_at) sc.frozen = 1;
+  }
+  __syncwarp();
+  prepare_substep_warp(sc, T, lane);
+}
+
+// The tool step of a scene, as one CTA of k_musl_node: it needs the wrench
+// partials, which P2G has left, and nothing later in the substep; k_fupd still
+// reads this substep's frame, so the result goes to the scene's record in
+// scenes_next and commit_tool takes it over when the particles are done.  As a
+// kernel of its own after k_fupd it was 9.2 us of a 16,000-particle scene's 98 us
+// substep and 16 of the 256-scene batch's 1,460.
+struct ToolS {
+  DevScene sc;
+  ToolTmp T;
+  double part[6][8], W[6];
+};
+
+// the part of the record that the tool step writes, in words
+constexpr int kToolWord0 = (int)(offsetof(DevScene, xB) / sizeof(int));
+constexpr int kToolWords = (int)(offsetof(DevScene, err) / sizeof(int)) - kToolWord0;
+
+__device__ __forceinline__ void next_tool(const World &w, int sid, ToolS &S) {
+  DevScene &g = w.scenes[sid];
+  // the labels of the last substep are in the slot table; k_fupd sets this anew
+  if (threadIdx.x == 0) g.label_pending = 0;
+  if (g.frozen) return;  // a scene that has taken its substeps: nothing moves
+  // the scene record into shared memory (coalesced), so that the tool step
+  // and frame below read and write it at shared-memory latency
+  static_assert(sizeof(DevScene) % sizeof(double) == 0, "the scene record copies as doubles");
+  for (int i = threadIdx.x; i < (int)(sizeof(DevScene) / sizeof(double)); i += blockDim.x)
+    reinterpret_cast<double *>(&S.sc)[i] = reinterpret_cast<const double *>(&g)[i];
+  // this substep's per-brick wrench partials: 256 strides over the bricks, a
+  // fixed shuffle tree over each 32 of them, then the eight in order (the
+  // same sums for every node tile size, the CTA's thread count)
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int v = wid; v < 8; v += nw) {
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    if (g.has_blade)
+      for (int j = 32 * v + lane; j < g.n_brick; j += 256) {
+        const double *q = w.wpart + (size_t)(g.brick_begin + j) * 6;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) acc[k] += q[k];
+      }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      double y = acc[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) y += __shfl_down_sync(FULL, y, o);
+      if (lane == 0) S.part[k][v] = y;
+    }
+  }
+  __syncthreads();
+  if (wid == 0) {
+    if (lane < 6) {
+      double t = 0.0;
+      for (int i = 0; i < 8; ++i) t += S.part[lane][i];
+      S.W[lane] = t;
+    }
+    __syncwarp();
+    tool_step(w, S.sc, S.T, S.W, lane);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kToolWords; i += blockDim.x)
+    reinterpret_cast<int *>(w.scenes_next + sid)[kToolWord0 + i] = reinterpret_cast<const int *>(&S.sc)[kToolWord0 + i];
+}
+
+// take over the tool step that next_tool has left (one CTA; no other CTA of
+// the launch may read the record's tool block, step or frozen)
+__device__ __forceinline__ void commit_tool(const World &w, int sid) {
+  const bool frozen = w.scenes[sid].frozen != 0;
+  __syncthreads();
+  if (frozen) return;
+  for (int i = threadIdx.x; i < kToolWords; i += blockDim.x)
+    reinterpret_cast<int *>(w.scenes + sid)[kToolWord0 + i] =
+        reinterpret_cast<const int *>(w.scenes_next + sid)[kToolWord0 + i];
+}
+
 // --------------------------------------------------------------------------
-// k_musl_node: per slot, MUSL sums of the covering bricks, coupling, v*
+// k_musl_node: per slot, MUSL sums of the covering bricks, coupling, v*; its
+// first n_scenes CTAs take the scenes' tool steps
 // --------------------------------------------------------------------------
 __global__ void k_musl_node(World w, LaunchSet ls) {
   chain_wait();
-  __shared__ NodeS<3> N;
-  const int4 t = ls.ntiles[blockIdx.x];
+  __shared__ __align__(16) unsigned char raw[sizeof(NodeS<3>) > sizeof(ToolS) ? sizeof(NodeS<3>) : sizeof(ToolS)];
+  if ((int)blockIdx.x < ls.n_scenes) {
+    next_tool(w, ls.scene_ids[blockIdx.x], *reinterpret_cast<ToolS *>(raw));
+    return;
+  }
+  NodeS<3> &N = *reinterpret_cast<NodeS<3> *>(raw);
+  const int4 t = ls.ntiles[blockIdx.x - ls.n_scenes];
   const int i = threadIdx.x;
   const DevScene &sc = w.scenes[t.x];
   if (sc.frozen) return;
@@ -1311,15 +1573,6 @@ __device__ void world_inv_inertia(const DevScene &sc, double Iw[9]) {
   matmul_d(tmp, RT, Iw);
 }
 
-__device__ const DevSeg *seg_at(const DevScene &sc, long long step) {
-  long long acc = 0;
-  for (int i = 0; i < sc.nseg; ++i) {
-    acc += sc.seg[i].n_steps;
-    if (step < acc) return &sc.seg[i];
-  }
-  return nullptr;
-}
-
 // Sets up substep sc.step: prescribed twist, cut, D reset, blade frame.
 __device__ void prepare_substep(DevScene &sc) {
   if (!sc.has_blade) {
@@ -1426,235 +1679,6 @@ __global__ void k_get_wrenches(World w, const int *ids, int n, double *out) {
   for (int k = 0; k < 6; ++k) out[(size_t)idx * 6 + k] = sc.lastW[k];
 }
 
-// The tool step by one warp on the shared-memory copy of the scene record:
-// wrench history, interval-averaged rigid tool step, and the frame of the
-// next substep.  Float64 operations are slow here (about 2 lanes per clock
-// and SM), so each component of a vector or matrix is its own lane's, in the
-// expression of the one-thread code: a serial thread spent most of the
-// kernel's 16.5 us (a 16,000-particle scene) on some 400 of them; 9.2 us now.
-__device__ __forceinline__ double matmul_at(const double A[9], const double B[9], int k) {
-  const int i = k / 3, j = k % 3;
-  return A[3 * i] * B[j] + A[3 * i + 1] * B[3 + j] + A[3 * i + 2] * B[6 + j];
-}
-
-struct ToolTmp {
-  double Fa[3], Ta[3], th[3], A[9], Iw[9], K[9], K2[9], Rinc[9];
-};
-
-__device__ __forceinline__ void prepare_substep_warp(DevScene &sc, ToolTmp &T, int lane) {
-  if (!sc.has_blade) {
-    if (lane == 0) {
-      sc.cut = -1;
-      sc.reset_D = 0;
-    }
-    return;
-  }
-  const DevSeg *sg = seg_at(sc, sc.step);
-  const int cut = sg ? sg->cut_id : -1;
-  const bool dynamic = sc.mass > 0.0;
-  const int reset = (cut >= 0 && cut != sc.cur_cut) ? 1 : 0;
-  if (!dynamic && sg && lane < 3) {
-    sc.vB[lane] = sg->v[lane];
-    sc.wB[lane] = sg->w[lane];
-  }
-  if (lane == 0) {
-    sc.cut = cut;
-    sc.reset_D = reset;
-  }
-  // edge point and blade axes: lane 3 q + i holds component i of vector q
-  if (lane < 12) {
-    const int q = lane / 3, i = lane % 3;
-    const double *v = q == 0 ? sc.edgeT : q == 1 ? sc.nT : q == 2 ? sc.eT : sc.dT;
-    const double y = __dadd_rn(__dadd_rn(__dmul_rn(sc.R[3 * i], v[0]), __dmul_rn(sc.R[3 * i + 1], v[1])),
-                               __dmul_rn(sc.R[3 * i + 2], v[2]));
-    double *o = q == 0 ? sc.dxe : q == 1 ? sc.dn : q == 2 ? sc.de : sc.dd;
-    o[i] = q == 0 ? __dadd_rn(sc.xB[i], y) : y;
-  }
-  __syncwarp();
-  if (lane < 3) {
-    const int i = lane, j = (lane + 1) % 3, k = (lane + 2) % 3;
-    const double rj = __dsub_rn(sc.dxe[j], sc.xB[j]), rk = __dsub_rn(sc.dxe[k], sc.xB[k]);
-    const double wr = __dsub_rn(__dmul_rn(sc.wB[j], rk), __dmul_rn(sc.wB[k], rj));
-    sc.dve[i] = __dadd_rn(sc.vB[i], wr);
-  }
-  if (dynamic && lane < 9) T.A[lane] = matmul_at(sc.R, sc.Ib_inv, lane);
-  __syncwarp();
-  if (reset) {  // a new cut begins: keep its plane for the cut faces
-    if (lane < 3) sc.cutpl[cut][lane] = sc.dn[lane];
-    if (lane == 3) {
-      sc.cutpl[cut][3] = __dadd_rn(__dadd_rn(__dmul_rn(sc.dn[0], sc.dxe[0]), __dmul_rn(sc.dn[1], sc.dxe[1])),
-                                   __dmul_rn(sc.dn[2], sc.dxe[2]));
-      sc.cutpl_set |= 1u << cut;
-    }
-  }
-  if (lane < 3) {
-    const int i = lane;
-    sc.fxe[i] = (float)sc.dxe[i];
-    sc.fn[i] = (float)sc.dn[i];
-    sc.fe[i] = (float)sc.de[i];
-    sc.fd[i] = (float)sc.dd[i];
-    sc.fve[i] = (float)sc.dve[i];
-    sc.fc[i] = (float)(sc.dxe[i] - sc.half_height * sc.dd[i]);
-    sc.fxB[i] = (float)sc.xB[i];
-    sc.fvB[i] = (float)sc.vB[i];
-    sc.fwB[i] = (float)sc.wB[i];
-  }
-  if (lane == 3) {
-    sc.fhext[0] = (float)sc.half_thick;
-    sc.fhext[1] = (float)sc.half_len;
-    sc.fhext[2] = (float)sc.half_height;
-    sc.fL = (float)sc.L_d;
-    sc.fmu_s = (float)sc.mu_s;
-    sc.fmu_d = (float)sc.mu_d;
-    sc.finv_mass = dynamic ? (float)(1.0 / sc.mass) : 0.f;
-  }
-  if (lane < 9) {  // world inverse inertia R Ib^-1 R^T
-    const int i = lane / 3, j = lane % 3;
-    sc.fIinv[lane] =
-        dynamic ? (float)(T.A[3 * i] * sc.R[3 * j] + T.A[3 * i + 1] * sc.R[3 * j + 1] + T.A[3 * i + 2] * sc.R[3 * j + 2])
-                : 0.f;
-  }
-}
-
-__device__ __forceinline__ void tool_step(const World &w, DevScene &sc, ToolTmp &T, const double W[6], int lane) {
-  // labels committed by k_fupd this substep -> rebuild the slot table
-  if (lane == 0) {
-    sc.need_rebuild = sc.label_pending ? 1 : 0;
-    sc.label_pending = 0;
-  }
-  if (sc.has_blade) {
-    const long long st = sc.step;
-    if (st < sc.hist_cap && lane < 6) w.whist[(size_t)(sc.hist_begin + st) * 6 + lane] = W[lane];
-    const int cnt = sc.acc_cnt + 1;
-    if (lane < 3) {
-      sc.accF[lane] += W[lane];
-      sc.accT[lane] += W[3 + lane];
-    }
-    __syncwarp();
-    if (cnt >= sc.rigid_interval) {
-      const double H = sc.dt_d * cnt;
-      if (lane < 3) {
-        T.Fa[lane] = sc.accF[lane] / cnt;
-        T.Ta[lane] = sc.accT[lane] / cnt;
-      }
-      if (sc.mass > 0.0) {
-        const DevSeg *tg = seg_at(sc, st);
-        if (lane < 9) T.A[lane] = matmul_at(sc.R, sc.Ib_inv, lane);
-        __syncwarp();
-        if (lane < 9) {
-          const int i = lane / 3, j = lane % 3;
-          T.Iw[lane] = T.A[3 * i] * sc.R[3 * j] + T.A[3 * i + 1] * sc.R[3 * j + 1] + T.A[3 * i + 2] * sc.R[3 * j + 2];
-        }
-        __syncwarp();
-        if (lane < 3) {
-          const int k = lane;
-          const double dw = T.Iw[3 * k] * T.Ta[0] + T.Iw[3 * k + 1] * T.Ta[1] + T.Iw[3 * k + 2] * T.Ta[2];
-          const double vt = tg ? tg->v[k] : 0.0, wt = tg ? tg->w[k] : 0.0;
-          sc.vB[k] += H * (sc.kv * (vt - sc.vB[k]) + T.Fa[k] / sc.mass);
-          sc.wB[k] += H * (sc.kv * (wt - sc.wB[k]) + dw);
-        }
-      }
-      __syncwarp();
-      if (lane < 3) T.th[lane] = H * sc.wB[lane];
-      __syncwarp();
-      // rotation increment exp(th): I + sin a K + (1 - cos a) K^2
-      const double th0 = T.th[0], th1 = T.th[1], th2 = T.th[2];
-      const double a = sqrt(th0 * th0 + th1 * th1 + th2 * th2);
-      if (a > 0) {
-        const double k0 = th0 / a, k1 = th1 / a, k2 = th2 / a;
-        if (lane == 0) {
-          T.K[0] = T.K[4] = T.K[8] = 0;
-          T.K[1] = -k2;
-          T.K[2] = k1;
-          T.K[3] = k2;
-          T.K[5] = -k0;
-          T.K[6] = -k1;
-          T.K[7] = k0;
-        }
-        __syncwarp();
-        if (lane < 9) {
-          const double sa = sin(a), ca = 1.0 - cos(a);
-          double r = (lane % 4 == 0) ? 1.0 : 0.0;
-          r += sa * T.K[lane] + ca * matmul_at(T.K, T.K, lane);
-          T.Rinc[lane] = r;
-        }
-      } else if (lane < 9) {
-        T.Rinc[lane] = (lane % 4 == 0) ? 1.0 : 0.0;
-      }
-      __syncwarp();
-      const double Rn = lane < 9 ? matmul_at(T.Rinc, sc.R, lane) : 0.0;
-      __syncwarp();
-      if (lane < 9) sc.R[lane] = Rn;
-      if (lane < 3) {
-        sc.xB[lane] += H * sc.vB[lane];
-        sc.lastW[lane] = T.Fa[lane];
-        sc.lastW[3 + lane] = T.Ta[lane];
-        sc.accF[lane] = sc.accT[lane] = 0.0;
-      }
-    }
-    __syncwarp();
-    if (lane == 0) {
-      sc.acc_cnt = cnt >= sc.rigid_interval ? 0 : cnt;
-      if (sc.cut >= 0) sc.cur_cut = sc.cut;
-    }
-  }
-  if (lane == 0) {
-    sc.step++;
-    if (sc.stop_at >= 0 && sc.step >= sc.stop_at) sc.frozen = 1;
-  }
-  __syncwarp();
-  prepare_substep_warp(sc, T, lane);
-}
-
-__global__ void k_tool(World w, LaunchSet ls) {
-  chain_wait();
-  const int sid = ls.scene_ids[blockIdx.x];
-  DevScene &g = w.scenes[sid];
-  if (g.frozen) {  // a scene that has taken its substeps: nothing moves, nothing to rebuild
-    if (threadIdx.x == 0) g.need_rebuild = 0;
-    return;
-  }
-  // the scene record into shared memory (coalesced), so that the tool step
-  // and frame below read and write it at shared-memory latency
-  __shared__ DevScene sc;
-  __shared__ ToolTmp T;
-  __shared__ double part[6][8], W[6];
-  static_assert(sizeof(DevScene) % sizeof(double) == 0, "the scene record copies as doubles");
-  constexpr int kWords = (int)(sizeof(DevScene) / sizeof(double));
-  // this substep's per-brick wrench partials: threads stride the bricks, a
-  // fixed shuffle tree, then the warps in order
-  double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  if (g.has_blade)
-    for (int j = threadIdx.x; j < g.n_brick; j += blockDim.x) {
-      const double *q = w.wpart + (size_t)(g.brick_begin + j) * 6;
-#pragma unroll
-      for (int k = 0; k < 6; ++k) acc[k] += q[k];
-    }
-  for (int i = threadIdx.x; i < kWords; i += blockDim.x)
-    reinterpret_cast<double *>(&sc)[i] = reinterpret_cast<const double *>(&g)[i];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    double v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-    if (lane == 0) part[k][wid] = v;
-  }
-  __syncthreads();
-  if (wid == 0) {
-    if (lane < 6) {
-      double t = 0.0;
-      for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += part[lane][i];
-      W[lane] = t;
-    }
-    __syncwarp();
-    tool_step(w, sc, T, W, lane);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kWords; i += blockDim.x)
-    reinterpret_cast<double *>(&g)[i] = reinterpret_cast<const double *>(&sc)[i];
-}
-
 // --------------------------------------------------------------------------
 // logical-grid slot table (rebuilt after label changes)
 // --------------------------------------------------------------------------
@@ -1735,51 +1759,54 @@ __global__ void k_recount(World w, LaunchSet ls, int force) {
   chain_wait();
   const int4 t = ls.ntiles[blockIdx.x];
   DevScene &sc = w.scenes[t.x];
-  if (!force && !sc.need_rebuild) return;
+  if (!force && !sc.label_pending) return;
   const int lane = threadIdx.x & 31;
   const int warp = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = gridDim.y * (blockDim.x >> 5);
   for (int li = warp; li < t.z; li += nw)
     if (force || w.N.dirty[t.y + li]) recount_node<KR>(w, sc, t.y + li, lane);
 }
 
-// Slot counts of a node tile's nodes and their sum.  Nodes next to a newly
-// labelled particle (dirty) are recounted, a warp each (COUNTED: k_recount
-// has done so), the others keep their distinct codes from the last rebuild.
-template <int KR, bool COUNTED>
+// Slot counts of a node tile's nodes and their sum.
+__device__ __forceinline__ void count_tile(const World &w, const int4 &t, int *sm) {
+  const int i = threadIdx.x;
+  int cnt = 0;
+  if (i < t.z) {
+    cnt = w.N.ncodes[t.y + i];
+    w.N.slot_cnt[t.y + i] = (uint8_t)cnt;
+  }
+  int total;
+  block_excl_scan(cnt, sm, total);
+  if (i == 0) w.N.tile_sum[t.w] = total;
+}
+
+// The same with the nodes next to a newly labelled particle (dirty) recounted
+// first, a warp each; the others keep their distinct codes from the last
+// rebuild.
+template <int KR>
 __global__ void k_slot_count(World w, LaunchSet ls, int force) {
   chain_wait();
   const int4 t = ls.ntiles[blockIdx.x];
   DevScene &sc = w.scenes[t.x];
-  if (!force && !sc.need_rebuild) return;
+  if (!force && !sc.label_pending) return;
   __shared__ int sm[33];
+  __shared__ int dlist[512];   // node tile <= 512 nodes
+  __shared__ int ndirty;
   const int i = threadIdx.x;
-  const int node = t.y + i;
-  int cnt = 0;
-  if (!COUNTED) {
-    __shared__ int dlist[512];   // node tile <= 512 nodes
-    __shared__ int ndirty;
-    if (i == 0) ndirty = 0;
-    __syncthreads();
-    if (i < t.z && (force != 0 || w.N.dirty[node] != 0)) dlist[atomicAdd(&ndirty, 1)] = i;
-    __syncthreads();
-    const int lane = i & 31, wid = i >> 5, nw = blockDim.x >> 5;
-    for (int j = wid; j < ndirty; j += nw) recount_node<KR>(w, sc, t.y + dlist[j], lane);
-    __syncthreads();
-  }
-  if (i < t.z) {
-    cnt = w.N.ncodes[node];
-    w.N.slot_cnt[node] = (uint8_t)cnt;
-  }
-  int total;
-  block_excl_scan(cnt, sm, total);
-  if (threadIdx.x == 0) w.N.tile_sum[t.w] = total;
+  if (i == 0) ndirty = 0;
+  __syncthreads();
+  if (i < t.z && (force != 0 || w.N.dirty[t.y + i] != 0)) dlist[atomicAdd(&ndirty, 1)] = i;
+  __syncthreads();
+  const int lane = i & 31, wid = i >> 5, nw = blockDim.x >> 5;
+  for (int j = wid; j < ndirty; j += nw) recount_node<KR>(w, sc, t.y + dlist[j], lane);
+  __syncthreads();
+  count_tile(w, t, sm);
 }
 
 // per brick: slot count and first tile slot of each tile node, and the
 // tile's slot total (after the per-node counts are final)
-// (one warp per brick, BTILE_WARPS bricks per CTA: lane l takes the tile's
-// nodes 7l .. 7l + 6, an exclusive warp scan orders them)
-#define BTILE_WARPS 8
+// (one warp per brick: lane l takes the tile's nodes 7l .. 7l + 6, an
+// exclusive warp scan orders them)
+#define BTILE_WARPS 8  // bricks per CTA of k_brick_tiles
 
 // Distinct codes of a brick's particles and each particle's index in
 // the list (one warp; a lane keeps the codes of its particles lane + 32 j in
@@ -1826,14 +1853,11 @@ __device__ __forceinline__ int list_brick_codes(const World &w, DevScene &sc, co
 }
 
 template <int PPC>
-__global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, LaunchSet ls, int force) {
-  chain_wait();
-  const int lane = threadIdx.x & 31;
-  const int bi = blockIdx.x * BTILE_WARPS + (threadIdx.x >> 5);
+__device__ __forceinline__ void brick_tile_slots(const World &w, const LaunchSet &ls, int bi, int lane, int force) {
   if (bi >= ls.n_btiles) return;
   const int4 bt = ls.btiles[bi];
   DevScene &sc = w.scenes[bt.x];
-  if (!force && !sc.need_rebuild) return;
+  if (!force && !sc.label_pending) return;
   int ncode;
   if (force || w.B.bdirty[bt.y]) {
     ncode = list_brick_codes<PPC * BR3 / 32>(w, sc, bt, lane);
@@ -1853,7 +1877,7 @@ __global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, Launc
     if (t < TN) {
       const int nx = c0x + t % TE, ny = c0y + (t / TE) % TE, nz = c0z + t / (TE * TE);
       if (nx < sc.nn[0] && ny < sc.nn[1] && nz < sc.nn[2])
-        cnt[j] = w.N.slot_cnt[sc.node_begin + (nz * sc.nn[1] + ny) * sc.nn[0] + nx];
+        cnt[j] = w.N.ncodes[sc.node_begin + (nz * sc.nn[1] + ny) * sc.nn[0] + nx];
     }
     mine += cnt[j];
   }
@@ -1878,12 +1902,8 @@ __global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, Launc
   if (lane == 31) w.B.ptot[bt.y] = incl;
 }
 
-// per scene: slot offsets of the node tiles, and partial-sum ranges of the bricks
-__global__ void k_slot_scan(World w, LaunchSet ls, int force) {
-  chain_wait();
-  DevScene &sc = w.scenes[ls.scene_ids[blockIdx.x]];
-  if (!force && !sc.need_rebuild) return;
-  __shared__ int sm[33];
+// slot offsets of a scene's node tiles (one CTA): exclusive sums in place
+__device__ __forceinline__ void tile_offsets(const World &w, DevScene &sc, int *sm) {
   int carry = 0;
   for (int base = 0; base < sc.n_ntile; base += blockDim.x) {
     const int j = base + threadIdx.x;
@@ -1894,6 +1914,14 @@ __global__ void k_slot_scan(World w, LaunchSet ls, int force) {
     carry += total;
     __syncthreads();
   }
+  if (threadIdx.x == 0) {
+    sc.n_slots = carry;
+    if (carry > sc.slot_cap) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
+  }
+}
+
+// partial-sum ranges of a scene's bricks (one CTA)
+__device__ __forceinline__ void brick_ranges(const World &w, DevScene &sc, int *sm) {
   int pcarry = 0;
   bool pover = false;
   for (int base = 0; base < sc.n_brick; base += blockDim.x) {
@@ -1910,25 +1938,79 @@ __global__ void k_slot_scan(World w, LaunchSet ls, int force) {
     __syncthreads();
   }
   if (pover) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
-  if (threadIdx.x == 0) {
-    sc.n_slots = carry;
-    if (carry > sc.slot_cap) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
-  }
 }
 
+// Sums over a scene stand between the counts and the slots: a CTA per scene
+// takes them beside the work that does not wait for them, the tiles' in the
+// launch of the bricks' tiles, the bricks' in that of the slots.  (A launch of
+// its own for both was 3 us of a 16,000-particle scene, 8 of the 256-scene
+// batch and 10 of a 477,000-particle scene.)
+template <int PPC>
+__global__ void __launch_bounds__(32 * BTILE_WARPS) k_brick_tiles(World w, LaunchSet ls, int force) {
+  chain_wait();
+  if ((int)blockIdx.x < ls.n_scenes) {
+    __shared__ int sm[33];
+    DevScene &sc = w.scenes[ls.scene_ids[blockIdx.x]];
+    if (force || sc.label_pending) tile_offsets(w, sc, sm);
+    return;
+  }
+  brick_tile_slots<PPC>(w, ls, (blockIdx.x - ls.n_scenes) * BTILE_WARPS + (threadIdx.x >> 5), threadIdx.x & 31,
+                        force);
+}
+
+// After k_recount: the counts of the node tiles and, in further CTAs, the
+// tiles of the bricks, which wait for the nodes' codes alone.
+template <int PPC>
+__global__ void __launch_bounds__(512) k_count_tiles(World w, LaunchSet ls, int force) {
+  chain_wait();
+  if ((int)blockIdx.x < ls.n_ntiles) {
+    __shared__ int sm[33];
+    const int4 t = ls.ntiles[blockIdx.x];
+    if (force || w.scenes[t.x].label_pending) count_tile(w, t, sm);
+    return;
+  }
+  brick_tile_slots<PPC>(w, ls, (blockIdx.x - ls.n_ntiles) * (blockDim.x >> 5) + (threadIdx.x >> 5),
+                        threadIdx.x & 31, force);
+}
+
+// Slots of the nodes, and in the first n_scenes CTAs the bricks' partial-sum
+// ranges and the commit of the tool step (not when forced: no substep).
+// OFFSETS: tile_sum holds the tiles' slot offsets (tile_offsets), otherwise
+// their counts, which each CTA sums up to its own tile.
+template <bool OFFSETS>
 __global__ void k_slot_fill(World w, LaunchSet ls, int force) {
   chain_wait();
-  const int4 t = ls.ntiles[blockIdx.x];
-  DevScene &sc = w.scenes[t.x];
-  if (!force && !sc.need_rebuild) return;
   __shared__ int sm[33];
+  if ((int)blockIdx.x < ls.n_scenes) {
+    const int sid = ls.scene_ids[blockIdx.x];
+    DevScene &sc = w.scenes[sid];
+    if (force || sc.label_pending) brick_ranges(w, sc, sm);
+    if (!force) commit_tool(w, sid);
+    return;
+  }
+  const int4 t = ls.ntiles[blockIdx.x - ls.n_scenes];
+  DevScene &sc = w.scenes[t.x];
+  if (!force && !sc.label_pending) return;
   const int i = threadIdx.x;
   const int node = t.y + i;
   const int cnt = i < t.z ? (int)w.N.slot_cnt[node] : 0;
   int total;
   const int ex = block_excl_scan(cnt, sm, total);
+  int tile0;
+  if (OFFSETS) {
+    tile0 = w.N.tile_sum[t.w];
+  } else {
+    int before = 0;
+    for (int j = sc.ntile_begin + i; j < t.w; j += blockDim.x) before += w.N.tile_sum[j];
+    __syncthreads();
+    block_excl_scan(before, sm, tile0);
+    if (t.w == sc.ntile_begin + sc.n_ntile - 1 && i == 0) {
+      sc.n_slots = tile0 + total;
+      if (tile0 + total > sc.slot_cap) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
+    }
+  }
   if (i < t.z) {
-    int off = w.N.tile_sum[t.w] + ex;
+    int off = tile0 + ex;
     const bool fits = off + cnt <= sc.slot_cap;
     if (!fits) {
       w.N.slot_cnt[node] = 0;
@@ -2074,6 +2156,8 @@ cudaError_t bm_launch_prepare(const World &w, const LaunchSet &ls, cudaStream_t 
   return cudaGetLastError();
 }
 
+// k_tool and k_slot_scan have no launch (k_musl_node, k_brick_tiles and
+// k_slot_fill do their work) and so no time of their own
 const char *const bm_kernel_names[BM_NUM_KERNELS] = {
     "k_p2g_brick", "k_p2g_node", "k_g2p_musl", "k_musl_node", "k_fupd",
     "k_tool", "k_slot_count", "k_slot_scan", "k_slot_fill", "k_brick_tiles",
@@ -2092,35 +2176,34 @@ static inline void rec(cudaEvent_t *ev, int k, int after, cudaStream_t st) {
 // all recounted after a restore 24 -> 7 us; the 256-scene batch takes 47 us
 // in one launch.
 #define RECOUNT_CTAS (4 * 152)
-template <int KR>
-static void launch_count(const World &w, const LaunchSet &ls, cudaStream_t st, int force) {
+template <int PPC>
+static void launch_slots(const World &w, const LaunchSet &ls, cudaStream_t st, int force, cudaEvent_t *ev) {
+  rec(ev, 6, 0, st);
   if (ls.n_ntiles > RECOUNT_CTAS) {
-    chain_launch(k_slot_count<KR, false>, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
-    return;
+    chain_launch(k_slot_count<PPC>, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
+    rec(ev, 6, 1, st);
+    rec(ev, 9, 0, st);
+    const int tgrid = (ls.n_btiles + BTILE_WARPS - 1) / BTILE_WARPS;
+    chain_launch(k_brick_tiles<PPC>, dim3(ls.n_scenes + tgrid), 32 * BTILE_WARPS, 0, st, w, ls, force);
+    rec(ev, 9, 1, st);
+    rec(ev, 8, 0, st);
+    chain_launch(k_slot_fill<true>, dim3(ls.n_scenes + ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
+  } else {
+    const int parts = min(max(RECOUNT_CTAS / ls.n_ntiles, 1), 16), nw = ls.ntile_size / 32;
+    chain_launch(k_recount<PPC>, dim3((unsigned)ls.n_ntiles, (unsigned)parts), 256, 0, st, w, ls, force);
+    chain_launch(k_count_tiles<PPC>, dim3(ls.n_ntiles + (ls.n_btiles + nw - 1) / nw), ls.ntile_size, 0, st, w, ls,
+                 force);
+    rec(ev, 6, 1, st);
+    rec(ev, 8, 0, st);
+    chain_launch(k_slot_fill<false>, dim3(ls.n_scenes + ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
   }
-  const int parts = min(max(RECOUNT_CTAS / ls.n_ntiles, 1), 16);
-  chain_launch(k_recount<KR>, dim3((unsigned)ls.n_ntiles, (unsigned)parts), 256, 0, st, w, ls, force);
-  chain_launch(k_slot_count<KR, true>, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
+  rec(ev, 8, 1, st);
 }
-
 static cudaError_t launch_rebuild(const World &w, const LaunchSet &ls, cudaStream_t st, int force,
                                   cudaEvent_t *ev) {
   if (ls.n_ntiles == 0) return cudaSuccess;
-  rec(ev, 6, 0, st);
-  if (ls.ppc16) launch_count<16>(w, ls, st, force);
-  else launch_count<8>(w, ls, st, force);
-  rec(ev, 6, 1, st);
-  rec(ev, 9, 0, st);
-  const int tgrid = (ls.n_btiles + BTILE_WARPS - 1) / BTILE_WARPS;
-  if (ls.ppc16) chain_launch(k_brick_tiles<16>, dim3(tgrid), 32 * BTILE_WARPS, 0, st, w, ls, force);
-  else chain_launch(k_brick_tiles<8>, dim3(tgrid), 32 * BTILE_WARPS, 0, st, w, ls, force);
-  rec(ev, 9, 1, st);
-  rec(ev, 7, 0, st);
-  chain_launch(k_slot_scan, dim3(ls.n_scenes), 256, 0, st, w, ls, force);
-  rec(ev, 7, 1, st);
-  rec(ev, 8, 0, st);
-  chain_launch(k_slot_fill, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls, force);
-  rec(ev, 8, 1, st);
+  if (ls.ppc16) launch_slots<16>(w, ls, st, force, ev);
+  else launch_slots<8>(w, ls, st, force, ev);
   return cudaGetLastError();
 }
 
@@ -2250,7 +2333,7 @@ static void launch_bricks(const World &w, const LaunchSet &ls, cudaStream_t st, 
   }
   rec(ev, 2, 1, st);
   rec(ev, 3, 0, st);
-  chain_launch(k_musl_node, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls);
+  chain_launch(k_musl_node, dim3(ls.n_scenes + ls.n_ntiles), ls.ntile_size, 0, st, w, ls);
   rec(ev, 3, 1, st);
   rec(ev, 4, 0, st);
   if (ls.any_lattice) bm_launch_fupd_lat(w, ls, st);
@@ -2299,9 +2382,6 @@ cudaError_t bm_launch_substep_ev(const World &w, const LaunchSet &ls, cudaStream
   if (ls.n_btiles == 0) return cudaSuccess;
   if (ls.any_pair && w.H.n_buckets > 0) launch_pairs(w, ls, st, ev);
   launch_bricks(w, ls, st, ev);
-  rec(ev, 5, 0, st);
-  chain_launch(k_tool, dim3(ls.n_scenes), 256, 0, st, w, ls);
-  rec(ev, 5, 1, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_rebuild(w, ls, st, 0, ev);

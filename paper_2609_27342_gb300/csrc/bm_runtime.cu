@@ -274,6 +274,7 @@ void carve_pools(WorldH *W) {
   bp.binfo = W->get<int>(W->cap_brick);
   bp.bdirty = W->get<uint8_t>(W->cap_brick);
   W->w.scenes = W->get<DevScene>(W->cap_scenes);
+  W->w.scenes_next = W->get<DevScene>(W->cap_scenes);
   W->w.wpart = W->get<double>(W->cap_brick * 6);
   W->w.whist = W->get<double>(std::max<int64_t>(W->cap_hist, 1) * 6);
   W->d_btiles = W->get<int4>(W->cap_brick);
@@ -1066,7 +1067,6 @@ int bm_add_blade(bm_scene_t s, const bm_blade_desc *b, int *blade_id) {
   t.step = cur.step;
   t.err = cur.err;
   t.n_slots = cur.n_slots;
-  t.need_rebuild = cur.need_rebuild;
   t.stop_at = cur.stop_at;
   t.frozen = cur.frozen;
   CK(cudaMemcpy(W->w.scenes + s->slot, &t, sizeof t, cudaMemcpyHostToDevice));
@@ -1425,7 +1425,6 @@ int bm_checkpoint_restore(bm_scene_t s, const void *src, int src_on_device) {
   set_ranges(s, sv);
   sv.slot_cap = (int)s->slot_cap;
   sv.label_pending = 0;
-  sv.need_rebuild = 0;
   sv.lattice = s->lattice;     // decided by the scene's positions, not by the saved record
   sv.stop_at = s->stop_at;     // the stop substep is a control of the caller's, not state
   sv.frozen = (sv.stop_at >= 0 && sv.step >= sv.stop_at) ? 1 : 0;
