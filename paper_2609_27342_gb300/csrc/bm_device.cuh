@@ -475,6 +475,18 @@ __device__ __forceinline__ int block_excl_scan(int v, int *sm, int &total) {
 __device__ __forceinline__ int pic(int j, int c) { return j * BR3 + (c ^ ((j & 7) << 2)); }
 
 #define BT 192  // threads per brick CTA: 64 cells x 3 z-offsets
+// Sets of few bricks leave most of the chip idle and a brick's CTA is a chain
+// of latencies.  Their CTAs have several groups of threads (WIDE of BT in the
+// P2G and the general kernels): the particles take a third or less of the
+// rounds, and the scatter's sums go side by side, momentum and force as well
+// as the codes, each by one thread in the narrow form's order.  Substep of one
+// cut scene, us, narrow -> wide:
+//   lattice  80 bricks 77 -> 66, 210: 81 -> 74, 336: 86 -> 84, 432: 89 -> 96
+//   jittered 80 bricks 180 -> 115, 336: 197 -> 130, 630: 199 -> 179
+//   16/cell  80 bricks 176 -> 100, 336: 187 -> 127, 630: 216 -> 200
+#define WIDE 4
+#define WIDE_BRICKS_LAT (2 * 152)
+#define WIDE_BRICKS (4 * 152)
 
 __device__ __forceinline__ void node_coords(const DevScene &sc, int li, int &ix, int &iy, int &iz) {
   ix = li % sc.nn[0];
@@ -767,22 +779,33 @@ __device__ __forceinline__ void pre_particle(const DevScene &sc, const PPool &P,
   P.pend[p] = pend;
 }
 
+// Per-particle reaction wrenches of a brick (wrc[k][i], rows of `stride`, one
+// per particle) as the sums that BT threads striding over the particles would
+// hold; for CTAs of more threads.  Thread t < BT returns its sums in wr.
+__device__ __forceinline__ void stride_wrench(const float *wrc, int stride, int n, float wr[6]) {
+  for (int i = threadIdx.x; i < n && threadIdx.x < BT; i += BT)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) wr[k] += wrc[k * stride + i];
+}
+
 // Per-brick wrench partial of this substep: float32 sums inside the brick
 // (fixed shuffle tree, warps in order), one double per component; bricks
-// without tool contact write zeros.  All threads of the CTA (W warps) call it.
+// without tool contact write zeros.  All threads of the CTA call it; those of
+// its first W warps hold sums.
 template <int W>
 __device__ __forceinline__ void brick_wrench(const World &w, int brick, const float wr[6], bool anyc,
                                              float (*red)[W]) {
   const int tid = threadIdx.x;
   if (__syncthreads_or(anyc)) {
     const int lane = tid & 31, wid = tid >> 5;
+    if (wid < W)
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      float v = wr[k];
+      for (int k = 0; k < 6; ++k) {
+        float v = wr[k];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-      if (lane == 0) red[k][wid] = v;
-    }
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
+        if (lane == 0) red[k][wid] = v;
+      }
     __syncthreads();
     if (tid < 6) {
       double s = 0.0;

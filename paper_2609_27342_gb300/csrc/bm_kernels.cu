@@ -38,11 +38,16 @@ namespace {
 // k_p2g_brick: the brick's share of P2G (Eq. 2) into its node tile, per
 // logical grid, from the particles' A, J, v staged in shared memory.
 // --------------------------------------------------------------------------
-template <int PPC>
+// G groups of BT threads: G = 1, or an even number
+template <int PPC, int G>
 struct K2S {
+  static constexpr int NP = (G + 1) / 2;  // passes side by side, two groups each
   BrickTile T;
   float part[18][PPC * BR3];   // the brick's particles (fx, v, A, J), [particle-in-cell][cell]
-  float sz[7][3][TZ];          // one pass's (node, z-offset) sums
+  union {
+    float sz[NP][7][3][TZ];    // the passes' (node, z-offset) sums
+    float wrc[6][G > 1 ? PPC * BR3 : 1];  // before: each particle's reaction wrench (G > 1)
+  };
   unsigned long long cmask[BR3];  // several codes: which of the brick's codes each cell's particles carry
   float red[6][BT / 32];       // wrench partials of the warps
   int cs[BR3 + 1];
@@ -68,8 +73,8 @@ __device__ __forceinline__ void cell_codes(const uint8_t *pid, const int *cs, un
 // consecutive words: the fractional offset, v, and the P2G inputs A and J
 // that pre_particle computes from x, v, F, D, u_t and the codes.  The caller
 // provides the barrier that publishes it.
-template <int PPC, bool INELASTIC>
-__device__ void stage_particles(const World &w, const DevScene &sc, const int4 &bt, bool coded, K2S<PPC> &S,
+template <int PPC, int G, bool INELASTIC>
+__device__ void stage_particles(const World &w, const DevScene &sc, const int4 &bt, bool coded, K2S<PPC, G> &S,
                                 float wr[6], bool &clamped, bool &anyc) {
   const PPool &P = w.P;
   // each thread fetches its next particle's flag one iteration ahead, so the
@@ -85,7 +90,15 @@ __device__ void stage_particles(const World &w, const DevScene &sc, const int4 &
     const uint2 code = id < BM_BRICK_CODES ? S.T.bcode[id] : make_uint2(0u, 0u);
     const float f0 = P.fx[0][p], f1 = P.fx[1][p], f2 = P.fx[2][p];
     float A[9], J[3];
-    pre_particle<INELASTIC>(sc, P, p, tf, x, v, code.x, code.y, A, J, wr, clamped, anyc);
+    if (G == 1) {
+      pre_particle<INELASTIC>(sc, P, p, tf, x, v, code.x, code.y, A, J, wr, clamped, anyc);
+    } else {
+      float wp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      pre_particle<INELASTIC>(sc, P, p, tf, x, v, code.x, code.y, A, J, wp, clamped, anyc);
+      if (sc.has_blade)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) S.wrc[k][i] = wp[k];
+    }
     const int c = cell_of(S.cs, i);
     const int si = pic(i - S.cs[c], c);
     S.part[0][si] = f0;
@@ -103,29 +116,36 @@ __device__ void stage_particles(const World &w, const DevScene &sc, const int4 &
   }
 }
 
-template <int PPC, int MB, bool INELASTIC>
-__global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
+template <int PPC, int MB, bool INELASTIC, int G>
+__global__ void __launch_bounds__(BT * G, MB) k_p2g_brick(World w, LaunchSet ls) {
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
-  K2S<PPC> &S = *reinterpret_cast<K2S<PPC> *>(smraw);
+  K2S<PPC, G> &S = *reinterpret_cast<K2S<PPC, G> *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];  // scene, pool brick, first particle, count
   DevScene &scm = w.scenes[bt.x];
   const DevScene &sc = scm;
   if (sc.frozen || sc.lattice) return;
-  const int tid = threadIdx.x;
+  constexpr int NT = BT * G, NP = K2S<PPC, G>::NP;
+  const int tid = threadIdx.x, grp = tid / BT;
   const int lb = bt.y - sc.brick_begin;
   const BrickInfo B(w, bt, PPC * BR3);
   const bool several = B.nbc > 1;
   const int *csg = w.N.cell_start + sc.cell_begin + lb * BR3;
-  for (int i = tid; i <= BR3; i += BT) S.cs[i] = csg[i] - bt.z;
-  brick_tile(w, bt.y, B.nbc, S.T, BT);
+  for (int i = tid; i <= BR3; i += NT) S.cs[i] = csg[i] - bt.z;
+  brick_tile(w, bt.y, B.nbc, S.T, NT);
   __syncthreads();
   float wr[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   bool clamped = false, anyc = false;
-  stage_particles<PPC, INELASTIC>(w, sc, bt, several, S, wr, clamped, anyc);
+  stage_particles<PPC, G, INELASTIC>(w, sc, bt, several, S, wr, clamped, anyc);
   if (clamped) atomicOr(&scm.err, BM_ERRBIT_INVERTED);
-  if (!B.uniform) brick_slots<true>(w, S.T, B.nbc, B.pbase, BT);
-  if (sc.has_blade) brick_wrench(w, bt.y, wr, anyc, S.red);
+  if (!B.uniform) brick_slots<true>(w, S.T, B.nbc, B.pbase, NT);
+  if (sc.has_blade) {
+    if (G > 1) {
+      __syncthreads();
+      stride_wrench(S.wrc[0], PPC * BR3, bt.w, wr);
+    }
+    brick_wrench(w, bt.y, wr, anyc, S.red);
+  }
   __syncthreads();
   if (several) {
     cell_codes(S.pid, S.cs, S.cmask);
@@ -139,16 +159,19 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
   // layers, and each tile node adds its <= 3 layer sums and writes the slot
   // of the pass's code.  Every float sum has one owner: no atomics, and each
   // partial-sum entry is written exactly once.
-  const int c = tid % BR3, oz = tid / BR3;
+  const int c = tid % BR3, oz = tid % BT / BR3;
   const int cx = c & 3, cy = (c >> 2) & 3, cz = c >> 4;
   const int n_c = S.cs[c + 1] - S.cs[c];
   const unsigned long long codes = several ? S.cmask[c] : 0ull;
   const bool filt = (codes & (codes - 1)) != 0;  // the cell's particles carry several codes
-  for (int b = 0; b < B.npass; ++b) {
-    const bool has = n_c > 0 && (!several || ((codes >> b) & 1u));
+  for (int b0 = 0; b0 < B.npass; b0 += NP) {
+    // G > 1: an even group takes the momentum sums of its pass, the next the force sums
+    const int b = b0 + grp / 2;
+    const bool has = n_c > 0 && b < B.npass && (!several || ((codes >> b) & 1u));
+    float(*sz)[3][TZ] = S.sz[grp / 2];
     // two walks over the cell's particles, each reducing its own values, so
     // that fewer sums are live at once: (m N, m v N), then A grad N + N J
-    {
+    if (b < B.npass && (G == 1 || grp % 2 == 0)) {
       float a[3][3][4];
 #pragma unroll
       for (int i = 0; i < 3; ++i)
@@ -183,9 +206,9 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
         }
       }
       xy_reduce<4>(a, cx, cy);
-      stage_layer<4, TZ>(S.sz, a, cx, cy, cz, oz);
+      stage_layer<4, TZ>(sz, a, cx, cy, cz, oz);
     }
-    {
+    if (b < B.npass && (G == 1 || grp % 2 == 1)) {
       float a[3][3][3];
 #pragma unroll
       for (int i = 0; i < 3; ++i)
@@ -227,18 +250,20 @@ __global__ void __launch_bounds__(BT, MB) k_p2g_brick(World w, LaunchSet ls) {
         }
       }
       xy_reduce<3>(a, cx, cy);
-      stage_layer<3, TZ>(S.sz + 4, a, cx, cy, cz, oz);
+      stage_layer<3, TZ>(sz + 4, a, cx, cy, cz, oz);
     }
     __syncthreads();
-    for (int t = tid; t < TN; t += BT) {
-      const long long e = B.entry(w, S.T, b, t);
+    for (int t = tid; t < NP * TN; t += NT) {
+      const int q = NP == 1 ? 0 : t / TN, nd = t - q * TN;
+      if (b0 + q >= B.npass) break;
+      const long long e = B.entry(w, S.T, b0 + q, nd);
       if (e < 0) continue;
       float acc[7];
-      gather_z<7, TZ>(S.sz, t, acc);
+      gather_z<7, TZ>(S.sz[q], nd, acc);
       w.B.pm[e] = make_float4(acc[0], acc[1], acc[2], acc[3]);
       w.B.pd[e] = make_float4(acc[4], acc[5], acc[6], 0.f);
     }
-    if (b + 1 < B.npass) __syncthreads();  // the next pass overwrites the z stage
+    if (b0 + NP < B.npass) __syncthreads();  // the next pass overwrites the z stage
   }
 }
 
@@ -459,7 +484,7 @@ __device__ __forceinline__ int tile_slot(const World &w, const BrickTile &T, int
   return a == NOSLOT ? -1 : T.lo[t] + a;
 }
 
-template <int PPC>
+template <int PPC, int G>
 struct K4S {
   BrickTile T;
   union {
@@ -467,7 +492,7 @@ struct K4S {
       float4 tvo[TSCAP];      // v_old xyz, m of the tile slots (G2P)
       float4 tvn[TSCAP];      // v_new xyz
     };
-    float sz[3][3][TN];       // then: one MUSL pass's (node, z-offset) sums
+    float sz[G][3][3][TN];    // then: each group's MUSL pass's (node, z-offset) sums
   };
   float pf[3][PPC * BR3];
   float pv[3][PPC * BR3];
@@ -476,36 +501,37 @@ struct K4S {
   uint8_t pid[PPC * BR3];
 };
 
-template <int PPC, int MB>
-__global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
+template <int PPC, int MB, int G>
+__global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls) {
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
-  K4S<PPC> &S = *reinterpret_cast<K4S<PPC> *>(smraw);
+  K4S<PPC, G> &S = *reinterpret_cast<K4S<PPC, G> *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];
   DevScene &scm = w.scenes[bt.x];
   const DevScene &sc = scm;
   if (sc.frozen || sc.lattice) return;
   const PPool &P = w.P;
-  const int tid = threadIdx.x;
+  constexpr int NT = BT * G;
+  const int tid = threadIdx.x, grp = tid / BT;
   const int lb = bt.y - sc.brick_begin;
   const BrickInfo B(w, bt, PPC * BR3);
   const bool several = B.nbc > 1, single = B.single;
   const int total = w.B.ptot[bt.y];
   const bool in_smem = total <= TSCAP;  // otherwise G2P reads the pool slots directly
   const int *csg = w.N.cell_start + sc.cell_begin + lb * BR3;
-  for (int i = tid; i <= BR3; i += BT) S.cs[i] = csg[i] - bt.z;
-  brick_tile(w, bt.y, B.nbc, S.T, BT);
+  for (int i = tid; i <= BR3; i += NT) S.cs[i] = csg[i] - bt.z;
+  brick_tile(w, bt.y, B.nbc, S.T, NT);
   __syncthreads();
-  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, B.pbase, BT);
+  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, B.pbase, NT);
   if (single) {  // by node: a particle's node t holds its (only) logical grid
-    for (int t = tid; t < TN; t += BT) {
+    for (int t = tid; t < TN; t += NT) {
       const bool has = S.T.cnt[t] != 0;
       const int g = S.T.goff[t];
       S.tvo[t] = has ? w.S.vold[g] : make_float4(0.f, 0.f, 0.f, 0.f);
       S.tvn[t] = has ? w.S.vnew[g] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   } else if (in_smem) {
-    for (int t = tid; t < TN; t += BT) {
+    for (int t = tid; t < TN; t += NT) {
       const int n = S.T.cnt[t], lo = S.T.lo[t], g = S.T.goff[t];
       for (int a = 0; a < n; ++a) {
         S.tvo[lo + a] = w.S.vold[g + a];
@@ -517,7 +543,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
   // ---- phase 0: G2P ----
   const float beta = sc.beta, dt = sc.dt;
   bool bad = false;
-  for (int i = tid; i < bt.w; i += BT) {
+  for (int i = tid; i < bt.w; i += NT) {
     const int p = bt.z + i;
     const int c = cell_of(S.cs, i);
     const int lx = c & 3, ly = (c >> 2) & 3, lz = c >> 4;
@@ -616,7 +642,7 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
   if (bad) atomicOr(&scm.err, BM_ERRBIT_NONFINITE);
   // ---- phase 1: MUSL sums m v^{n+1} N, one pass per code of the brick,
   // reduced as in k_p2g_brick (xy_reduce, z stage, <= 3 layer sums per node) ----
-  const int c = tid % BR3, oz = tid / BR3;
+  const int c = tid % BR3, oz = tid % BT / BR3;
   const int cx = c & 3, cy = (c >> 2) & 3, cz = c >> 4;
   const int n_c = S.cs[c + 1] - S.cs[c];
   __syncthreads();  // G2P reads of the tile velocities are done: the z stage may reuse them
@@ -626,8 +652,9 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
   }
   const unsigned long long codes = several ? S.cmask[c] : 0ull;
   const bool filt = (codes & (codes - 1)) != 0;
-  for (int b = 0; b < B.npass; ++b) {
-    const bool has = n_c > 0 && (!several || ((codes >> b) & 1u));
+  for (int b0 = 0; b0 < B.npass; b0 += G) {
+    const int b = b0 + grp;
+    const bool has = n_c > 0 && b < B.npass && (!several || ((codes >> b) & 1u));
     float a[3][3][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -656,17 +683,21 @@ __global__ void __launch_bounds__(BT, MB) k_g2p_musl(World w, LaunchSet ls) {
         }
       }
     }
-    xy_reduce<3>(a, cx, cy);
-    stage_layer<3, TN>(S.sz, a, cx, cy, cz, oz);
+    if (b < B.npass) {
+      xy_reduce<3>(a, cx, cy);
+      stage_layer<3, TN>(S.sz[grp], a, cx, cy, cz, oz);
+    }
     __syncthreads();
-    for (int t = tid; t < TN; t += BT) {
-      const long long e = B.entry(w, S.T, b, t);
+    for (int t = tid; t < G * TN; t += NT) {
+      const int q = G == 1 ? 0 : t / TN, nd = t - q * TN;
+      if (b0 + q >= B.npass) break;
+      const long long e = B.entry(w, S.T, b0 + q, nd);
       if (e < 0) continue;
       float acc[3];
-      gather_z<3, TN>(S.sz, t, acc);
+      gather_z<3, TN>(S.sz[q], nd, acc);
       w.B.pm[e] = make_float4(acc[0], acc[1], acc[2], 0.f);
     }
-    if (b + 1 < B.npass) __syncthreads();  // the next pass overwrites the z stage
+    if (b0 + G < B.npass) __syncthreads();  // the next pass overwrites the z stage
   }
 }
 
@@ -886,12 +917,31 @@ __device__ __forceinline__ void next_tool(const World &w, int sid, ToolS &S) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int v = wid; v < 8; v += nw) {
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (g.has_blade)
-      for (int j = 32 * v + lane; j < g.n_brick; j += 256) {
-        const double *q = w.wpart + (size_t)(g.brick_begin + j) * 6;
+    if (g.has_blade) {
+      const double2 *q = reinterpret_cast<const double2 *>(w.wpart) + (size_t)g.brick_begin * 3;
+      const int nb = g.n_brick;
+      int j = 32 * v + lane;
+      for (; j + 256 < nb; j += 512) {  // two strides' loads in flight
+        double2 a[3], b[3];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) acc[k] += q[k];
+        for (int k = 0; k < 3; ++k) {
+          a[k] = q[(size_t)j * 3 + k];
+          b[k] = q[(size_t)(j + 256) * 3 + k];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          acc[2 * k] = acc[2 * k] + a[k].x + b[k].x;
+          acc[2 * k + 1] = acc[2 * k + 1] + a[k].y + b[k].y;
+        }
       }
+      if (j < nb)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const double2 a = q[(size_t)j * 3 + k];
+          acc[2 * k] += a.x;
+          acc[2 * k + 1] += a.y;
+        }
+    }
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
       double y = acc[k];
@@ -1002,8 +1052,8 @@ struct K1S {
   int any;
 };
 
-template <int MB, bool INELASTIC>
-__global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
+template <int MB, bool INELASTIC, int NG>
+__global__ void __launch_bounds__(BT * NG, MB) k_fupd(World w, LaunchSet ls) {
   chain_wait();
   __shared__ K1S S;
   const int4 bt = ls.btiles[blockIdx.x];
@@ -1011,6 +1061,7 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
   const DevScene &sc = scm;
   if (sc.frozen || sc.lattice) return;
   const PPool &P = w.P;
+  constexpr int NT = BT * NG;
   const int tid = threadIdx.x;
   const int lb = bt.y - sc.brick_begin;
   int c0x, c0y, c0z;
@@ -1019,14 +1070,14 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
   const BrickInfo B(w, bt, 0);
   const bool several = B.nbc > 1, single = B.single;
   const bool in_smem = w.B.ptot[bt.y] <= TSCAP;
-  brick_tile(w, bt.y, B.nbc, S.T, BT);
+  brick_tile(w, bt.y, B.nbc, S.T, NT);
   __syncthreads();
-  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, -1, BT);
+  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, -1, NT);
   if (single) {  // by node
-    for (int t = tid; t < TN; t += BT)
+    for (int t = tid; t < TN; t += NT)
       S.tvs[t] = S.T.cnt[t] ? w.S.vstar[S.T.goff[t]] : make_float4(0.f, 0.f, 0.f, 0.f);
   } else if (in_smem) {
-    for (int t = tid; t < TN; t += BT) {
+    for (int t = tid; t < TN; t += NT) {
       const int n = S.T.cnt[t], lo = S.T.lo[t], g = S.T.goff[t];
       for (int a = 0; a < n; ++a) S.tvs[lo + a] = w.S.vstar[g + a];
     }
@@ -1035,7 +1086,7 @@ __global__ void __launch_bounds__(BT, MB) k_fupd(World w, LaunchSet ls) {
   const float c = sc.dt * sc.inv_dx;
   const int cut = sc.cut;
   bool any = false;
-  for (int i = tid; i < bt.w; i += BT) {
+  for (int i = tid; i < bt.w; i += NT) {
     const int p = bt.z + i;
     int bx, by, bz;
     particle_base(P.base[p], bx, by, bz);
@@ -2245,9 +2296,17 @@ static cudaError_t brick_smem(K *kernel, int bytes) {
 
 template <int PPC, int C>
 static cudaError_t set_smem_attrs() {
-  cudaError_t e = brick_smem(k_p2g_brick<PPC, OccP2G<C, false>::v, false>, (int)sizeof(K2S<PPC>));
-  if (e == cudaSuccess) e = brick_smem(k_p2g_brick<PPC, OccP2G<C, true>::v, true>, (int)sizeof(K2S<PPC>));
-  if (e == cudaSuccess) e = brick_smem(k_g2p_musl<PPC, OccG2P<C>::v>, (int)sizeof(K4S<PPC>));
+  cudaError_t e = brick_smem(k_p2g_brick<PPC, OccP2G<C, false>::v, false, 1>, (int)sizeof(K2S<PPC, 1>));
+  if (e == cudaSuccess) e = brick_smem(k_p2g_brick<PPC, OccP2G<C, true>::v, true, 1>, (int)sizeof(K2S<PPC, 1>));
+  if (e == cudaSuccess) e = brick_smem(k_g2p_musl<PPC, OccG2P<C>::v, 1>, (int)sizeof(K4S<PPC, 1>));
+  return e;
+}
+
+template <int PPC>
+static cudaError_t set_wide_smem_attrs() {
+  cudaError_t e = brick_smem(k_p2g_brick<PPC, 1, false, WIDE>, (int)sizeof(K2S<PPC, WIDE>));
+  if (e == cudaSuccess) e = brick_smem(k_p2g_brick<PPC, 1, true, WIDE>, (int)sizeof(K2S<PPC, WIDE>));
+  if (e == cudaSuccess) e = brick_smem(k_g2p_musl<PPC, 1, WIDE>, (int)sizeof(K4S<PPC, WIDE>));
   return e;
 }
 
@@ -2264,35 +2323,47 @@ cudaError_t bm_kernels_init() {
   if (e == cudaSuccess) e = set_smem_attrs<16, 0>();
   if (e == cudaSuccess) e = set_smem_attrs<16, 1>();
   if (e == cudaSuccess) e = set_smem_attrs<16, 2>();
+  if (e == cudaSuccess) e = set_wide_smem_attrs<8>();
+  if (e == cudaSuccess) e = set_wide_smem_attrs<16>();
   if (e == cudaSuccess) e = bm_lattice_init();
   status = e;
   device = dev;
   return e;
 }
 
+template <int PPC, int MB, int G>
+static void launch_p2g(const World &w, const LaunchSet &ls, cudaStream_t st) {
+  chain_launch(k_p2g_brick<PPC, MB, false, G>, dim3(ls.n_btiles), BT * G, sizeof(K2S<PPC, G>), st, w, ls);
+}
+template <int PPC, int MB, int G>
+static void launch_p2g_inelastic(const World &w, const LaunchSet &ls, cudaStream_t st) {
+  chain_launch(k_p2g_brick<PPC, MB, true, G>, dim3(ls.n_btiles), BT * G, sizeof(K2S<PPC, G>), st, w, ls);
+}
+
 template <int PPC, int C>
 static void launch_p2g(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  if (ls.any_inelastic)
-    chain_launch(k_p2g_brick<PPC, OccP2G<C, true>::v, true>, dim3(ls.n_btiles), BT, sizeof(K2S<PPC>), st, w, ls);
-  else
-    chain_launch(k_p2g_brick<PPC, OccP2G<C, false>::v, false>, dim3(ls.n_btiles), BT, sizeof(K2S<PPC>), st, w, ls);
+  if (ls.any_inelastic) launch_p2g_inelastic<PPC, OccP2G<C, true>::v, 1>(w, ls, st);
+  else launch_p2g<PPC, OccP2G<C, false>::v, 1>(w, ls, st);
 }
 
-template <int PPC, int C>
+template <int PPC, int MB, int G>
 static void launch_g2p(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  chain_launch(k_g2p_musl<PPC, OccG2P<C>::v>, dim3(ls.n_btiles), BT, sizeof(K4S<PPC>), st, w, ls);
+  chain_launch(k_g2p_musl<PPC, MB, G>, dim3(ls.n_btiles), BT * G, sizeof(K4S<PPC, G>), st, w, ls);
 }
 
-template <int C>
+template <int MB, int G>
 static void launch_fupd(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  if (ls.any_inelastic) chain_launch(k_fupd<OccFupd<C>::v, true>, dim3(ls.n_btiles), BT, 0, st, w, ls);
-  else chain_launch(k_fupd<OccFupd<C>::v, false>, dim3(ls.n_btiles), BT, 0, st, w, ls);
+  if (ls.any_inelastic) chain_launch(k_fupd<MB, true, G>, dim3(ls.n_btiles), BT * G, 0, st, w, ls);
+  else chain_launch(k_fupd<MB, false, G>, dim3(ls.n_btiles), BT * G, 0, st, w, ls);
 }
 
 template <int PPC>
 static void launch_p2g_general(const World &w, const LaunchSet &ls, cudaStream_t st) {
   const int c = ls.variant % 3;
-  if (c == 0) launch_p2g<PPC, 0>(w, ls, st);
+  if (ls.n_btiles <= WIDE_BRICKS) {
+    if (ls.any_inelastic) launch_p2g_inelastic<PPC, 1, WIDE>(w, ls, st);
+    else launch_p2g<PPC, 1, WIDE>(w, ls, st);
+  } else if (c == 0) launch_p2g<PPC, 0>(w, ls, st);
   else if (c == 1) launch_p2g<PPC, 1>(w, ls, st);
   else launch_p2g<PPC, 2>(w, ls, st);
 }
@@ -2300,16 +2371,18 @@ static void launch_p2g_general(const World &w, const LaunchSet &ls, cudaStream_t
 template <int PPC>
 static void launch_g2p_general(const World &w, const LaunchSet &ls, cudaStream_t st) {
   const int c = (ls.variant / 3) % 3;
-  if (c == 0) launch_g2p<PPC, 0>(w, ls, st);
-  else if (c == 1) launch_g2p<PPC, 1>(w, ls, st);
-  else launch_g2p<PPC, 2>(w, ls, st);
+  if (ls.n_btiles <= WIDE_BRICKS) launch_g2p<PPC, 1, WIDE>(w, ls, st);
+  else if (c == 0) launch_g2p<PPC, OccG2P<0>::v, 1>(w, ls, st);
+  else if (c == 1) launch_g2p<PPC, OccG2P<1>::v, 1>(w, ls, st);
+  else launch_g2p<PPC, OccG2P<2>::v, 1>(w, ls, st);
 }
 
 static void launch_fupd_general(const World &w, const LaunchSet &ls, cudaStream_t st) {
   const int c = ls.variant / 9;
-  if (c == 0) launch_fupd<0>(w, ls, st);
-  else if (c == 1) launch_fupd<1>(w, ls, st);
-  else launch_fupd<2>(w, ls, st);
+  if (ls.n_btiles <= WIDE_BRICKS) launch_fupd<1, WIDE>(w, ls, st);
+  else if (c == 0) launch_fupd<OccFupd<0>::v, 1>(w, ls, st);
+  else if (c == 1) launch_fupd<OccFupd<1>::v, 1>(w, ls, st);
+  else launch_fupd<OccFupd<2>::v, 1>(w, ls, st);
 }
 
 // Each brick kernel in its lattice and its general form, as the set's scenes

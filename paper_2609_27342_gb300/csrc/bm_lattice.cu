@@ -149,9 +149,14 @@ constexpr int PT = BT;  // the wrench sums of a brick keep their threads
 
 // a particle's scatter inputs, four 16-byte chunks (XORed by bm_lat_xor):
 // A0 A3 A1 A4 | A2 A5 J0 J1 | A6 A7 A8 J2 | v0 v1 v2
+template <int G>
 struct P2GS {
+  static constexpr int NP = (G + 1) / 2;  // passes side by side, two groups of PT threads each
   float4 part[LP][4];
-  float sz[7][3][TZ];      // one pass's (node, z-offset) sums
+  union {
+    float sz[NP][7][3][TZ];  // the passes' (node, z-offset) sums
+    float wrc[6][G > 1 ? LP : 1];  // before: each particle's reaction wrench (G > 1)
+  };
   LatTile T;
   float red[6][PT / 32];
   __align__(8) uint8_t cid[LP];  // code index of each particle, 8 cell + number
@@ -162,9 +167,9 @@ struct P2GS {
 // are formed once for both x planes.
 struct CellOz {
   int c, cx, cy, cz, oz, p0;
-  __device__ __forceinline__ CellOz(int tid) {
-    c = tid % BR3;
-    oz = tid / BR3;
+  __device__ __forceinline__ CellOz(int t) {  // t < 3 BR3
+    c = t % BR3;
+    oz = t / BR3;
     cx = c & 3;
     cy = (c >> 2) & 3;
     cz = c >> 4;
@@ -175,7 +180,8 @@ struct CellOz {
   }
 };
 
-__device__ __forceinline__ void p2g_momentum(P2GS &S, const CellOz &q, unsigned m) {
+template <int G>
+__device__ __forceinline__ void p2g_momentum(const P2GS<G> &S, const CellOz &q, unsigned m, float (*sz)[3][TZ]) {
   f2 a[3][3][2];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -218,10 +224,11 @@ __device__ __forceinline__ void p2g_momentum(P2GS &S, const CellOz &q, unsigned 
       unpack2(a[i][j][1], s[i][j][2], s[i][j][3]);
     }
   xy_reduce<4>(s, q.cx, q.cy);
-  stage_layer<4, TZ>(S.sz, s, q.cx, q.cy, q.cz, q.oz);
+  stage_layer<4, TZ>(sz, s, q.cx, q.cy, q.cz, q.oz);
 }
 
-__device__ __forceinline__ void p2g_force(P2GS &S, const CellOz &q, unsigned m) {
+template <int G>
+__device__ __forceinline__ void p2g_force(const P2GS<G> &S, const CellOz &q, unsigned m, float (*sz)[3][TZ]) {
   f2 a[3][3];
   float a2[3][3];
 #pragma unroll
@@ -269,37 +276,46 @@ __device__ __forceinline__ void p2g_force(P2GS &S, const CellOz &q, unsigned m) 
       s[i][j][2] = a2[i][j];
     }
   xy_reduce<3>(s, q.cx, q.cy);
-  stage_layer<3, TZ>(S.sz + 4, s, q.cx, q.cy, q.cz, q.oz);
+  stage_layer<3, TZ>(sz + 4, s, q.cx, q.cy, q.cz, q.oz);
 }
 
-template <int MB, bool INELASTIC>
-__global__ void __launch_bounds__(PT, MB) k_p2g_lat(World w, LaunchSet ls) {
+template <int MB, bool INELASTIC, int G>
+__global__ void __launch_bounds__(PT * G, MB) k_p2g_lat(World w, LaunchSet ls) {
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
-  P2GS &S = *reinterpret_cast<P2GS *>(smraw);
+  P2GS<G> &S = *reinterpret_cast<P2GS<G> *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];  // scene, pool brick, first particle, count
   DevScene &scm = w.scenes[bt.x];
   const DevScene &sc = scm;
   if (sc.frozen || !sc.lattice) return;
   const PPool &P = w.P;
-  const int tid = threadIdx.x;
+  constexpr int NT = PT * G, NP = P2GS<G>::NP;
+  const int tid = threadIdx.x, grp = tid / PT;
   const BrickInfo B(w, bt, LP);
-  lat_tile(w, bt.y, B.nbc, S.T, PT);
+  lat_tile(w, bt.y, B.nbc, S.T, NT);
   if (B.mask && tid < LP / 4) reinterpret_cast<unsigned *>(S.cid)[tid] = 0xffffffffu;
   __syncthreads();
   float wr[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   bool clamped = false, anyc = false;
   uint8_t tf_next = tid < bt.w ? P.tflag[bt.z + tid] : 0;  // one iteration ahead, as in stage_particles
-  for (int i = tid; i < bt.w; i += PT) {
+  for (int i = tid; i < bt.w; i += NT) {
     const int p = bt.z + i;
     const uint8_t tf = tf_next;
-    if (i + PT < bt.w) tf_next = P.tflag[p + PT];
+    if (i + NT < bt.w) tf_next = P.tflag[p + NT];
     const float x[3] = {P.x[0][p], P.x[1][p], P.x[2][p]};
     const float v[3] = {P.v[0][p], P.v[1][p], P.v[2][p]};
     const int c = P.cid[p], q = P.lpos[p];
     const uint2 code = c < BM_BRICK_CODES ? S.T.bcode[c] : make_uint2(0u, 0u);
     float A[9], J[3];
-    pre_particle<INELASTIC>(sc, P, p, tf, x, v, code.x, code.y, A, J, wr, clamped, anyc);
+    if (G == 1) {
+      pre_particle<INELASTIC>(sc, P, p, tf, x, v, code.x, code.y, A, J, wr, clamped, anyc);
+    } else {
+      float wp[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      pre_particle<INELASTIC>(sc, P, p, tf, x, v, code.x, code.y, A, J, wp, clamped, anyc);
+      if (sc.has_blade)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) S.wrc[k][i] = wp[k];
+    }
     const int xo = bm_lat_xor(q);
     S.part[q][0 ^ xo] = make_float4(A[0], A[3], A[1], A[4]);
     S.part[q][1 ^ xo] = make_float4(A[2], A[5], J[0], J[1]);
@@ -308,24 +324,36 @@ __global__ void __launch_bounds__(PT, MB) k_p2g_lat(World w, LaunchSet ls) {
     if (B.mask) S.cid[place_cell8(q)] = (uint8_t)c;
   }
   if (clamped) atomicOr(&scm.err, BM_ERRBIT_INVERTED);
-  if (!B.uniform) brick_slots<true>(w, S.T, B.nbc, B.pbase, PT);
-  if (sc.has_blade) brick_wrench(w, bt.y, wr, anyc, S.red);
+  if (!B.uniform) brick_slots<true>(w, S.T, B.nbc, B.pbase, NT);
+  if (sc.has_blade) {
+    if (G > 1) {
+      __syncthreads();
+      stride_wrench(S.wrc[0], LP, bt.w, wr);
+    }
+    brick_wrench(w, bt.y, wr, anyc, S.red);
+  }
   __syncthreads();
-  const CellOz q(tid);
-  for (int b = 0; b < B.npass; ++b) {
-    const unsigned m = B.mask ? cell_mask(S.cid, q.c, b) : 0xffu;
-    p2g_momentum(S, q, m);
-    p2g_force(S, q, m);
+  const CellOz q(tid % PT);
+  for (int b0 = 0; b0 < B.npass; b0 += NP) {
+    // G > 1: an even group takes the momentum sums of its pass, the next the force sums
+    const int b = b0 + grp / 2;
+    if (b < B.npass) {
+      const unsigned m = B.mask ? cell_mask(S.cid, q.c, b) : 0xffu;
+      if (G == 1 || grp % 2 == 0) p2g_momentum(S, q, m, S.sz[grp / 2]);
+      if (G == 1 || grp % 2 == 1) p2g_force(S, q, m, S.sz[grp / 2]);
+    }
     __syncthreads();
-    for (int t = tid; t < TN; t += PT) {
-      const long long e = B.entry(w, S.T, b, t);
+    for (int t = tid; t < NP * TN; t += NT) {
+      const int k = NP == 1 ? 0 : t / TN, nd = t - k * TN;
+      if (b0 + k >= B.npass) break;
+      const long long e = B.entry(w, S.T, b0 + k, nd);
       if (e < 0) continue;
       float acc[7];
-      gather_z<7, TZ>(S.sz, t, acc);
+      gather_z<7, TZ>(S.sz[k], nd, acc);
       w.B.pm[e] = make_float4(acc[0], acc[1], acc[2], acc[3]);
       w.B.pd[e] = make_float4(acc[4], acc[5], acc[6], 0.f);
     }
-    if (b + 1 < B.npass) __syncthreads();
+    if (b0 + NP < B.npass) __syncthreads();
   }
 }
 
@@ -335,12 +363,13 @@ __global__ void __launch_bounds__(PT, MB) k_p2g_lat(World w, LaunchSet ls) {
 constexpr int GT = 256;  // a thread per (base cell, x plane, y plane): its two z planes
 constexpr int TVR = 52;  // floats of one x-row of 6 tile nodes: (v_old, v_new, 2 spare) each, padded
 
+template <int G>
 struct G2PS {
   float4 pv[LP];           // v^{n+1} at pv_place
   union {
     float tv[36 * TVR];    // v_old and v_new of the pass's code at the tile's nodes
     float sz[3][3][TZ];    // then: one MUSL pass's (node, z-offset) sums
-  };
+  } g[G];                  // of each group of GT threads
   LatTile T;
   uint16_t inv[LP];        // particle (index in the brick) at each place
   __align__(8) uint8_t cid[LP];
@@ -349,7 +378,8 @@ struct G2PS {
 // bank-spread index of a place in arrays of one 16-byte word per particle
 __device__ __forceinline__ int pv_place(int p) { return p ^ (((p >> 4) & 1) << 1) ^ (((p >> 3) & 1) << 2); }
 
-__device__ __forceinline__ void musl_cell(G2PS &S, const CellOz &q, unsigned m) {
+template <int G>
+__device__ __forceinline__ void musl_cell(const G2PS<G> &S, const CellOz &q, unsigned m, float (*sz)[3][TZ]) {
   f2 a[3][3];
   float a2[3][3];
 #pragma unroll
@@ -394,34 +424,35 @@ __device__ __forceinline__ void musl_cell(G2PS &S, const CellOz &q, unsigned m) 
       s[i][j][2] = a2[i][j];
     }
   xy_reduce<3>(s, q.cx, q.cy);
-  stage_layer<3, TZ>(S.sz, s, q.cx, q.cy, q.cz, q.oz);
+  stage_layer<3, TZ>(sz, s, q.cx, q.cy, q.cz, q.oz);
 }
 
-template <int MB>
-__global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
+template <int MB, int G>
+__global__ void __launch_bounds__(GT * G, MB) k_g2p_lat(World w, LaunchSet ls) {
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
-  G2PS &S = *reinterpret_cast<G2PS *>(smraw);
+  G2PS<G> &S = *reinterpret_cast<G2PS<G> *>(smraw);
   const int4 bt = ls.btiles[blockIdx.x];
   DevScene &scm = w.scenes[bt.x];
   const DevScene &sc = scm;
   if (sc.frozen || !sc.lattice) return;
   const PPool &P = w.P;
-  const int tid = threadIdx.x;
+  constexpr int NT = GT * G;
+  const int tid = threadIdx.x % GT, grp = threadIdx.x / GT;  // a pass is a group's
   const BrickInfo B(w, bt, LP);
   // the general kernel multiplies the weights of a tile beyond its slot
   // window in another order: (wx wy) wz, not wx (wy wz)
   const bool wide = w.B.ptot[bt.y] > TSCAP;
-  lat_tile(w, bt.y, B.nbc, S.T, GT);
-  if (bt.w < LP) reinterpret_cast<unsigned *>(S.inv)[tid] = 0xffffffffu;
-  if (B.mask && tid < LP / 4) reinterpret_cast<unsigned *>(S.cid)[tid] = 0xffffffffu;
+  lat_tile(w, bt.y, B.nbc, S.T, NT);
+  if (bt.w < LP && grp == 0) reinterpret_cast<unsigned *>(S.inv)[tid] = 0xffffffffu;
+  if (B.mask && (int)threadIdx.x < LP / 4) reinterpret_cast<unsigned *>(S.cid)[tid] = 0xffffffffu;
   __syncthreads();
-  for (int i = tid; i < bt.w; i += GT) {
+  for (int i = threadIdx.x; i < bt.w; i += NT) {
     const int q = P.lpos[bt.z + i];
     S.inv[q] = (uint16_t)i;
     if (B.mask) S.cid[place_cell8(q)] = P.cid[bt.z + i];
   }
-  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, B.pbase, GT);
+  if (!B.uniform) brick_slots<false>(w, S.T, B.nbc, B.pbase, NT);
   __syncthreads();
   const int cell = tid >> 2, jx = (tid >> 1) & 1, jy = tid & 1;
   const int cx = cell & 3, cy = (cell >> 2) & 3, cz = cell >> 4;
@@ -433,7 +464,7 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
     const int i = S.inv[pq[j]];
     pi[j] = bt.z + i;
     pc[j] = i == 0xffff ? -1 : B.nbc > 1 ? S.cid[cell * 8 + (jx * 2 + jy) * 2 + j] : 0;
-    if (pc[j] >= 0)
+    if (pc[j] >= 0 && pc[j] % G == grp)
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         v0[j][a] = P.v[a][pi[j]];
@@ -442,8 +473,10 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
   }
   const float beta = sc.beta, dt = sc.dt;
   bool bad = false;
-  for (int b = 0; b < B.npass; ++b) {
-    if (tid < TN) {
+  for (int b0 = 0; b0 < B.npass; b0 += G) {
+    const int b = b0 + grp;
+    float *tv = S.g[grp].tv;
+    if (tid < TN && b < B.npass) {
       const int sl = B.slot(w, S.T, b, tid);
       float4 vo = make_float4(0.f, 0.f, 0.f, 0.f), vn = vo;
       if (sl != NOSLOT) {
@@ -451,12 +484,12 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
         vo = w.S.vold[g];
         vn = w.S.vnew[g];
       }
-      float *o = S.tv + (tid / TE) * TVR + (tid % TE) * 8;
+      float *o = tv + (tid / TE) * TVR + (tid % TE) * 8;
       *reinterpret_cast<float4 *>(o) = make_float4(vo.x, vo.y, vo.z, vn.x);
       *reinterpret_cast<float2 *>(o + 4) = make_float2(vn.y, vn.z);
     }
     __syncthreads();
-    if (pc[0] == b || pc[1] == b) {
+    if (pc[0] == b || pc[1] == b) {  // (no particle has a code beyond the last)
       float wx[3], wy[3], wz[2][3];
       plane_w(S.T.wt[0][2 * cx + jx], wx);
       plane_w(S.T.wt[1][2 * cy + jy], wy);
@@ -467,7 +500,7 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
       for (int j = 0; j < 2; ++j)
 #pragma unroll
         for (int k = 0; k < 3; ++k) acc[j][k] = 0ull;
-      const float *r = S.tv + (cz * TE + cy) * TVR + cx * 8;
+      const float *r = tv + (cz * TE + cy) * TVR + cx * 8;
 #pragma unroll
       for (int oz = 0; oz < 3; ++oz)
 #pragma unroll
@@ -512,26 +545,27 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
         S.pv[pv_place(pq[j])] = make_float4(vv[0], vv[1], vv[2], 0.f);
       }
     }
-    if (b + 1 < B.npass) __syncthreads();
+    if (b0 + G < B.npass) __syncthreads();
   }
   if (bad) atomicOr(&scm.err, BM_ERRBIT_NONFINITE);
   __syncthreads();  // v^{n+1} is complete, and the z stage may take the tile's place
   // ---- MUSL: sums of v^{n+1} N, one pass per code ----
-  for (int b = 0; b < B.npass; ++b) {
-    if (tid < 3 * BR3) {
+  for (int b0 = 0; b0 < B.npass; b0 += G) {
+    const int b = b0 + grp;
+    if (tid < 3 * BR3 && b < B.npass) {
       const CellOz q(tid);
-      musl_cell(S, q, B.mask ? cell_mask(S.cid, q.c, b) : 0xffu);
+      musl_cell(S, q, B.mask ? cell_mask(S.cid, q.c, b) : 0xffu, S.g[grp].sz);
     }
     __syncthreads();
-    if (tid < TN) {
+    if (tid < TN && b < B.npass) {
       const long long e = B.entry(w, S.T, b, tid);
       if (e >= 0) {
         float acc[3];
-        gather_z<3, TZ>(S.sz, tid, acc);
+        gather_z<3, TZ>(S.g[grp].sz, tid, acc);
         w.B.pm[e] = make_float4(acc[0], acc[1], acc[2], 0.f);
       }
     }
-    if (b + 1 < B.npass) __syncthreads();
+    if (b0 + G < B.npass) __syncthreads();
   }
 }
 
@@ -539,7 +573,6 @@ __global__ void __launch_bounds__(GT, MB) k_g2p_lat(World w, LaunchSet ls) {
 // k_fupd_lat: F += dt sum v* (x) grad N, and the commit of the side labels
 // --------------------------------------------------------------------------
 constexpr int FT = 192;
-constexpr int NPT = (LP + FT - 1) / FT;  // particles per thread
 
 struct FupdS {
   float4 tile[TN];         // v* of the pass's code
@@ -549,8 +582,8 @@ struct FupdS {
   int any;
 };
 
-template <int MB, bool INELASTIC>
-__global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
+template <int MB, bool INELASTIC, int NG>
+__global__ void __launch_bounds__(FT * NG, MB) k_fupd_lat(World w, LaunchSet ls) {
   chain_wait();
   __shared__ FupdS S;
   const int4 bt = ls.btiles[blockIdx.x];
@@ -558,6 +591,7 @@ __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
   const DevScene &sc = scm;
   if (sc.frozen || !sc.lattice) return;
   const PPool &P = w.P;
+  constexpr int NT = FT * NG, NPT = (LP + NT - 1) / NT;  // particles per thread
   const int tid = threadIdx.x;
   const BrickInfo B(w, bt, LP);
   if (tid == 0) S.any = 0;
@@ -565,7 +599,7 @@ __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
   int pq[NPT], pc[NPT];
 #pragma unroll
   for (int j = 0; j < NPT; ++j) {
-    const int i = tid + j * FT, p = bt.z + i;
+    const int i = tid + j * NT, p = bt.z + i;
     pc[j] = -1;
     if (i < bt.w) {
       pq[j] = P.lpos[p];
@@ -574,20 +608,20 @@ __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
       for (int k = 0; k < 9; ++k) F[j][k] = P.F[k][p];
     }
   }
-  lat_tile(w, bt.y, B.nbc, S.T, FT);
+  lat_tile(w, bt.y, B.nbc, S.T, NT);
   __syncthreads();
   if (!B.uniform) {
-    brick_slots<false>(w, S.T, B.nbc, -1, FT);
+    brick_slots<false>(w, S.T, B.nbc, -1, NT);
     __syncthreads();
   }
   const float c = sc.dt * sc.inv_dx;
   for (int b = 0; b < B.nbc; ++b) {
-    for (int t = tid; t < TN; t += FT) {
+    for (int t = tid; t < TN; t += NT) {
       const int sl = B.slot(w, S.T, b, t);
       S.tile[t] = sl != NOSLOT ? w.S.vstar[S.T.goff[t] + sl] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    for (int e = tid; e < 288; e += FT) {
+    for (int e = tid; e < 288; e += NT) {
       const int row = e >> 3, x = e & 7;
       float wx[3], dx[3];
       plane_wd(S.T.wt[0][x], wx, dx);
@@ -605,7 +639,7 @@ __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
 #pragma unroll
     for (int j = 0; j < NPT; ++j) {
       if (pc[j] != b) continue;
-      const int p = bt.z + tid + j * FT;
+      const int p = bt.z + tid + j * NT;
       int x, y, z;
       place_xyz(pq[j], x, y, z);
       float wy[3], dy[3], wz[3], dz[3];
@@ -638,7 +672,7 @@ __global__ void __launch_bounds__(FT, MB) k_fupd_lat(World w, LaunchSet ls) {
   }
   const int cut = sc.cut;
   bool any = false;
-  for (int i = tid; i < bt.w && cut >= 0; i += FT) {
+  for (int i = tid; i < bt.w && cut >= 0; i += NT) {
     const int p = bt.z + i;
     const uint8_t pend = P.pend[p];
     if (pend) {
@@ -676,26 +710,46 @@ cudaError_t lat_smem(K *kernel, size_t bytes) {
 // (0.342 at 3, 0.349 at 5), F update 0.442 -> 0.200 (0.206 at 5, 0.193 at 7,
 // which costs a 477k-particle scene 2 us of 22).
 constexpr int OCC_P2G = 4, OCC_G2P = 4, OCC_FUPD = 6;
+// groups of threads of the forms for sets of few bricks (WIDE_BRICKS_LAT)
+constexpr int GWIDE = 2, FWIDE = 3;
 
 }  // namespace
 
 cudaError_t bm_lattice_init() {
-  cudaError_t e = lat_smem(k_p2g_lat<OCC_P2G, false>, sizeof(P2GS));
-  if (e == cudaSuccess) e = lat_smem(k_p2g_lat<OCC_P2G, true>, sizeof(P2GS));
-  if (e == cudaSuccess) e = lat_smem(k_g2p_lat<OCC_G2P>, sizeof(G2PS));
+  cudaError_t e = lat_smem(k_p2g_lat<OCC_P2G, false, 1>, sizeof(P2GS<1>));
+  if (e == cudaSuccess) e = lat_smem(k_p2g_lat<OCC_P2G, true, 1>, sizeof(P2GS<1>));
+  if (e == cudaSuccess) e = lat_smem(k_p2g_lat<1, false, WIDE>, sizeof(P2GS<WIDE>));
+  if (e == cudaSuccess) e = lat_smem(k_p2g_lat<1, true, WIDE>, sizeof(P2GS<WIDE>));
+  if (e == cudaSuccess) e = lat_smem(k_g2p_lat<OCC_G2P, 1>, sizeof(G2PS<1>));
+  if (e == cudaSuccess) e = lat_smem(k_g2p_lat<1, GWIDE>, sizeof(G2PS<GWIDE>));
   return e;
 }
 
+template <int MB, int G>
+static void p2g_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
+  if (ls.any_inelastic) chain_launch(k_p2g_lat<MB, true, G>, dim3(ls.n_btiles), PT * G, sizeof(P2GS<G>), st, w, ls);
+  else chain_launch(k_p2g_lat<MB, false, G>, dim3(ls.n_btiles), PT * G, sizeof(P2GS<G>), st, w, ls);
+}
+
 void bm_launch_p2g_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  if (ls.any_inelastic) chain_launch(k_p2g_lat<OCC_P2G, true>, dim3(ls.n_btiles), PT, sizeof(P2GS), st, w, ls);
-  else chain_launch(k_p2g_lat<OCC_P2G, false>, dim3(ls.n_btiles), PT, sizeof(P2GS), st, w, ls);
+  if (ls.n_btiles <= WIDE_BRICKS_LAT) p2g_lat<1, WIDE>(w, ls, st);
+  else p2g_lat<OCC_P2G, 1>(w, ls, st);
 }
 
 void bm_launch_g2p_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  chain_launch(k_g2p_lat<OCC_G2P>, dim3(ls.n_btiles), GT, sizeof(G2PS), st, w, ls);
+  if (ls.n_btiles <= WIDE_BRICKS_LAT)
+    chain_launch(k_g2p_lat<1, GWIDE>, dim3(ls.n_btiles), GT * GWIDE, sizeof(G2PS<GWIDE>), st, w, ls);
+  else
+    chain_launch(k_g2p_lat<OCC_G2P, 1>, dim3(ls.n_btiles), GT, sizeof(G2PS<1>), st, w, ls);
+}
+
+template <int MB, int G>
+static void fupd_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
+  if (ls.any_inelastic) chain_launch(k_fupd_lat<MB, true, G>, dim3(ls.n_btiles), FT * G, 0, st, w, ls);
+  else chain_launch(k_fupd_lat<MB, false, G>, dim3(ls.n_btiles), FT * G, 0, st, w, ls);
 }
 
 void bm_launch_fupd_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  if (ls.any_inelastic) chain_launch(k_fupd_lat<OCC_FUPD, true>, dim3(ls.n_btiles), FT, 0, st, w, ls);
-  else chain_launch(k_fupd_lat<OCC_FUPD, false>, dim3(ls.n_btiles), FT, 0, st, w, ls);
+  if (ls.n_btiles <= WIDE_BRICKS_LAT) fupd_lat<1, FWIDE>(w, ls, st);
+  else fupd_lat<OCC_FUPD, 1>(w, ls, st);
 }
