@@ -30,6 +30,7 @@
 
 #include "bm_device.cuh"
 #include "bm_internal.cuh"
+#include "bm_tool.cuh"
 
 
 namespace {
@@ -307,8 +308,7 @@ __device__ __forceinline__ void covering_entries(const World &w, const DevScene 
 // several (near a cut) are dealt out one to a thread, and the coupling reads
 // the node's other slots from shared memory: walked by a thread per node,
 // with its sums in local memory, they kept the whole warp waiting (k_p2g_node
-// 137 -> 86 us for the 256-scene batch mid-cut, 18.4 -> 10.4 us for a
-// 16,000-particle scene; k_musl_node 72 -> 66 and 12.4 -> 9.1 us).
+// 137 -> 86 us for the 256-scene batch mid-cut, k_musl_node 72 -> 66).
 // --------------------------------------------------------------------------
 #define NODE_WIN 512                    // slots held in shared memory at a time
 #define NODE_STEP (NODE_WIN - BM_MAXS)  // a window takes the nodes whose first slot lies in one step
@@ -350,17 +350,26 @@ __device__ __forceinline__ void couple_slot(const NodeS<NC> &N, int lo, int ns, 
   for (int c = 0; c < NC; ++c) out[c] = Sa[c] + acc[c] * iM;
 }
 
-// The slots of the tile's nodes with several, window by window: `sum(node,
-// a, pool slot, m, S)` takes a slot's sums, `finish(pool slot, m, S)` its
-// result after the coupling.  All threads of the CTA call it.
-template <int NC, class Sum, class Finish>
-__device__ __forceinline__ void coupled_slots(const World &w, NodeS<NC> &N, int node0, int cnt, Sum sum,
-                                              Finish finish) {
-  const int i = threadIdx.x;
+// A node tile: `single(node)` takes a node with one slot, by its own thread.
+// The slots of the nodes with several go window by window: `sum(node, a, pool
+// slot, m, S)` takes a slot's sums, `finish(pool slot, m, S)` its result after
+// the coupling.  All threads of the CTA call it; thread i < nt holds the slot
+// count of node i.  Each of `single` and `sum` is a chain of dependent loads;
+// a CTA with threads beyond nt (sets of few tiles) has these take the slots
+// while the first nt take the single nodes.
+template <int NC, class Single, class Sum, class Finish>
+__device__ __forceinline__ void tile_nodes(const World &w, NodeS<NC> &N, int node0, int nt, int cnt, Single single,
+                                           Sum sum, Finish finish) {
+  const int i = threadIdx.x, t0 = (int)blockDim.x > nt ? nt : 0;
+  if (t0 == 0 && cnt == 1) single(node0 + i);
+  if (!__syncthreads_or(cnt > 1)) {
+    if (t0 != 0 && cnt == 1) single(node0 + i);
+    return;
+  }
   const int mine = cnt > 1 ? cnt : 0;
   int total;
   const int first = block_excl_scan(mine, N.scan, total);
-  N.first[i] = first;
+  if (i < nt) N.first[i] = first;
   for (int w0 = 0; w0 < total; w0 += NODE_STEP) {
     for (int s = i; s < NODE_WIN; s += blockDim.x) N.owner[s] = 0xffff;
     __syncthreads();
@@ -368,17 +377,21 @@ __device__ __forceinline__ void coupled_slots(const World &w, NodeS<NC> &N, int 
       for (int a = 0; a < mine; ++a) N.owner[first - w0 + a] = (uint16_t)i;
     __syncthreads();
     const int ns = min(NODE_WIN, total - w0);
-    for (int s = i; s < ns; s += blockDim.x) {
-      const int o = N.owner[s];
-      if (o == 0xffff) continue;
-      const int a = s - (N.first[o] - w0);
-      const int slot = w.N.slot_off[node0 + o] + a;
-      N.code[s] = w.S.code[slot];
-      float m, S[NC];
-      sum(node0 + o, a, slot, m, S);
-      N.m[s] = m;
+    if (i < t0) {
+      if (w0 == 0 && cnt == 1) single(node0 + i);
+    } else {
+      for (int s = i - t0; s < ns; s += blockDim.x - t0) {
+        const int o = N.owner[s];
+        if (o == 0xffff) continue;
+        const int a = s - (N.first[o] - w0);
+        const int slot = w.N.slot_off[node0 + o] + a;
+        N.code[s] = w.S.code[slot];
+        float m, S[NC];
+        sum(node0 + o, a, slot, m, S);
+        N.m[s] = m;
 #pragma unroll
-      for (int c = 0; c < NC; ++c) N.S[s][c] = S[c];
+        for (int c = 0; c < NC; ++c) N.S[s][c] = S[c];
+      }
     }
     __syncthreads();
     for (int s = i; s < ns; s += blockDim.x) {
@@ -400,9 +413,8 @@ __global__ void k_p2g_node(World w, LaunchSet ls) {
   const int i = threadIdx.x;
   const DevScene &sc = w.scenes[t.x];
   if (sc.frozen) return;
-  const int node = t.y + i;
-  const int cnt = i < t.z ? w.N.slot_cnt[node] : 0;
-  if (cnt == 1) {
+  const int cnt = i < t.z ? w.N.slot_cnt[t.y + i] : 0;
+  auto single = [&](int node) {
     const int off = w.N.slot_off[node];
     int ix, iy, iz;
     node_coords(sc, node - sc.node_begin, ix, iy, iz);
@@ -429,10 +441,9 @@ __global__ void k_p2g_node(World w, LaunchSet ls) {
     }
     w.S.vold[off] = o;
     w.S.vnew[off] = nw;
-  }
-  if (!__syncthreads_or(cnt > 1)) return;
-  coupled_slots<6>(
-      w, N, t.y, cnt,
+  };
+  tile_nodes<6>(
+      w, N, t.y, ls.ntile_size, cnt, single,
       [&](int nd, int sl, int, float &m, float (&S)[6]) {
         int ix, iy, iz;
         node_coords(sc, nd - sc.node_begin, ix, iy, iz);
@@ -502,11 +513,16 @@ struct K4S {
 };
 
 template <int PPC, int MB, int G>
-__global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls) {
+__global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls, int tools) {
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   K4S<PPC, G> &S = *reinterpret_cast<K4S<PPC, G> *>(smraw);
-  const int4 bt = ls.btiles[blockIdx.x];
+  if (G > 1 && (int)blockIdx.x < tools) {
+    next_tool(w, ls.scene_ids[blockIdx.x], *reinterpret_cast<ToolS *>(smraw));
+    return;
+  }
+  static_assert(sizeof(ToolS) <= sizeof(K4S<PPC, G>), "the tool step fits");
+  const int4 bt = ls.btiles[blockIdx.x - tools];
   DevScene &scm = w.scenes[bt.x];
   const DevScene &sc = scm;
   if (sc.frozen || sc.lattice) return;
@@ -701,299 +717,23 @@ __global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls) 
   }
 }
 
-__device__ const DevSeg *seg_at(const DevScene &sc, long long step) {
-  long long acc = 0;
-  for (int i = 0; i < sc.nseg; ++i) {
-    acc += sc.seg[i].n_steps;
-    if (step < acc) return &sc.seg[i];
-  }
-  return nullptr;
-}
-
-// The tool step by one warp on the shared-memory copy of the scene record:
-// wrench history, interval-averaged rigid tool step, and the frame of the
-// next substep.  Float64 operations are slow here (about 2 lanes per clock
-// and SM), so each component of a vector or matrix is its own lane's, in the
-// expression of the one-thread code: a serial thread spent most of the
-// kernel's 16.5 us (a 16,000-particle scene) on some 400 of them; 9.2 us now.
-__device__ __forceinline__ double matmul_at(const double A[9], const double B[9], int k) {
-  const int i = k / 3, j = k % 3;
-  return A[3 * i] * B[j] + A[3 * i + 1] * B[3 + j] + A[3 * i + 2] * B[6 + j];
-}
-
-struct ToolTmp {
-  double Fa[3], Ta[3], th[3], A[9], Iw[9], K[9], K2[9], Rinc[9];
-};
-
-__device__ __forceinline__ void prepare_substep_warp(DevScene &sc, ToolTmp &T, int lane) {
-  if (!sc.has_blade) {
-    if (lane == 0) {
-      sc.cut = -1;
-      sc.reset_D = 0;
-    }
-    return;
-  }
-  const DevSeg *sg = seg_at(sc, sc.step);
-  const int cut = sg ? sg->cut_id : -1;
-  const bool dynamic = sc.mass > 0.0;
-  const int reset = (cut >= 0 && cut != sc.cur_cut) ? 1 : 0;
-  if (!dynamic && sg && lane < 3) {
-    sc.vB[lane] = sg->v[lane];
-    sc.wB[lane] = sg->w[lane];
-  }
-  if (lane == 0) {
-    sc.cut = cut;
-    sc.reset_D = reset;
-  }
-  // edge point and blade axes: lane 3 q + i holds component i of vector q
-  if (lane < 12) {
-    const int q = lane / 3, i = lane % 3;
-    const double *v = q == 0 ? sc.edgeT : q == 1 ? sc.nT : q == 2 ? sc.eT : sc.dT;
-    const double y = __dadd_rn(__dadd_rn(__dmul_rn(sc.R[3 * i], v[0]), __dmul_rn(sc.R[3 * i + 1], v[1])),
-                               __dmul_rn(sc.R[3 * i + 2], v[2]));
-    double *o = q == 0 ? sc.dxe : q == 1 ? sc.dn : q == 2 ? sc.de : sc.dd;
-    o[i] = q == 0 ? __dadd_rn(sc.xB[i], y) : y;
-  }
-  __syncwarp();
-  if (lane < 3) {
-    const int i = lane, j = (lane + 1) % 3, k = (lane + 2) % 3;
-    const double rj = __dsub_rn(sc.dxe[j], sc.xB[j]), rk = __dsub_rn(sc.dxe[k], sc.xB[k]);
-    const double wr = __dsub_rn(__dmul_rn(sc.wB[j], rk), __dmul_rn(sc.wB[k], rj));
-    sc.dve[i] = __dadd_rn(sc.vB[i], wr);
-  }
-  if (dynamic && lane < 9) T.A[lane] = matmul_at(sc.R, sc.Ib_inv, lane);
-  __syncwarp();
-  if (reset) {  // a new cut begins: keep its plane for the cut faces
-    if (lane < 3) sc.cutpl[cut][lane] = sc.dn[lane];
-    if (lane == 3) {
-      sc.cutpl[cut][3] = __dadd_rn(__dadd_rn(__dmul_rn(sc.dn[0], sc.dxe[0]), __dmul_rn(sc.dn[1], sc.dxe[1])),
-                                   __dmul_rn(sc.dn[2], sc.dxe[2]));
-      sc.cutpl_set |= 1u << cut;
-    }
-  }
-  if (lane < 3) {
-    const int i = lane;
-    sc.fxe[i] = (float)sc.dxe[i];
-    sc.fn[i] = (float)sc.dn[i];
-    sc.fe[i] = (float)sc.de[i];
-    sc.fd[i] = (float)sc.dd[i];
-    sc.fve[i] = (float)sc.dve[i];
-    sc.fc[i] = (float)(sc.dxe[i] - sc.half_height * sc.dd[i]);
-    sc.fxB[i] = (float)sc.xB[i];
-    sc.fvB[i] = (float)sc.vB[i];
-    sc.fwB[i] = (float)sc.wB[i];
-  }
-  if (lane == 3) {
-    sc.fhext[0] = (float)sc.half_thick;
-    sc.fhext[1] = (float)sc.half_len;
-    sc.fhext[2] = (float)sc.half_height;
-    sc.fL = (float)sc.L_d;
-    sc.fmu_s = (float)sc.mu_s;
-    sc.fmu_d = (float)sc.mu_d;
-    sc.finv_mass = dynamic ? (float)(1.0 / sc.mass) : 0.f;
-  }
-  if (lane < 9) {  // world inverse inertia R Ib^-1 R^T
-    const int i = lane / 3, j = lane % 3;
-    sc.fIinv[lane] =
-        dynamic ? (float)(T.A[3 * i] * sc.R[3 * j] + T.A[3 * i + 1] * sc.R[3 * j + 1] + T.A[3 * i + 2] * sc.R[3 * j + 2])
-                : 0.f;
-  }
-}
-
-__device__ __forceinline__ void tool_step(const World &w, DevScene &sc, ToolTmp &T, const double W[6], int lane) {
-  if (sc.has_blade) {
-    const long long st = sc.step;
-    if (st < sc.hist_cap && lane < 6) w.whist[(size_t)(sc.hist_begin + st) * 6 + lane] = W[lane];
-    const int cnt = sc.acc_cnt + 1;
-    if (lane < 3) {
-      sc.accF[lane] += W[lane];
-      sc.accT[lane] += W[3 + lane];
-    }
-    __syncwarp();
-    if (cnt >= sc.rigid_interval) {
-      const double H = sc.dt_d * cnt;
-      if (lane < 3) {
-        T.Fa[lane] = sc.accF[lane] / cnt;
-        T.Ta[lane] = sc.accT[lane] / cnt;
-      }
-      if (sc.mass > 0.0) {
-        const DevSeg *tg = seg_at(sc, st);
-        if (lane < 9) T.A[lane] = matmul_at(sc.R, sc.Ib_inv, lane);
-        __syncwarp();
-        if (lane < 9) {
-          const int i = lane / 3, j = lane % 3;
-          T.Iw[lane] = T.A[3 * i] * sc.R[3 * j] + T.A[3 * i + 1] * sc.R[3 * j + 1] + T.A[3 * i + 2] * sc.R[3 * j + 2];
-        }
-        __syncwarp();
-        if (lane < 3) {
-          const int k = lane;
-          const double dw = T.Iw[3 * k] * T.Ta[0] + T.Iw[3 * k + 1] * T.Ta[1] + T.Iw[3 * k + 2] * T.Ta[2];
-          const double vt = tg ? tg->v[k] : 0.0, wt = tg ? tg->w[k] : 0.0;
-          sc.vB[k] += H * (sc.kv * (vt - sc.vB[k]) + T.Fa[k] / sc.mass);
-          sc.wB[k] += H * (sc.kv * (wt - sc.wB[k]) + dw);
-        }
-      }
-      __syncwarp();
-      if (lane < 3) T.th[lane] = H * sc.wB[lane];
-      __syncwarp();
-      // rotation increment exp(th): I + sin a K + (1 - cos a) K^2
-      const double th0 = T.th[0], th1 = T.th[1], th2 = T.th[2];
-      const double a = sqrt(th0 * th0 + th1 * th1 + th2 * th2);
-      if (a > 0) {
-        const double k0 = th0 / a, k1 = th1 / a, k2 = th2 / a;
-        if (lane == 0) {
-          T.K[0] = T.K[4] = T.K[8] = 0;
-          T.K[1] = -k2;
-          T.K[2] = k1;
-          T.K[3] = k2;
-          T.K[5] = -k0;
-          T.K[6] = -k1;
-          T.K[7] = k0;
-        }
-        __syncwarp();
-        if (lane < 9) {
-          const double sa = sin(a), ca = 1.0 - cos(a);
-          double r = (lane % 4 == 0) ? 1.0 : 0.0;
-          r += sa * T.K[lane] + ca * matmul_at(T.K, T.K, lane);
-          T.Rinc[lane] = r;
-        }
-      } else if (lane < 9) {
-        T.Rinc[lane] = (lane % 4 == 0) ? 1.0 : 0.0;
-      }
-      __syncwarp();
-      const double Rn = lane < 9 ? matmul_at(T.Rinc, sc.R, lane) : 0.0;
-      __syncwarp();
-      if (lane < 9) sc.R[lane] = Rn;
-      if (lane < 3) {
-        sc.xB[lane] += H * sc.vB[lane];
-        sc.lastW[lane] = T.Fa[lane];
-        sc.lastW[3 + lane] = T.Ta[lane];
-        sc.accF[lane] = sc.accT[lane] = 0.0;
-      }
-    }
-    __syncwarp();
-    if (lane == 0) {
-      sc.acc_cnt = cnt >= sc.rigid_interval ? 0 : cnt;
-      if (sc.cut >= 0) sc.cur_cut = sc.cut;
-    }
-  }
-  if (lane == 0) {
-    sc.step++;
-    if (sc.stop_at >= 0 && sc.step >= sc.stop_at) sc.frozen = 1;
-  }
-  __syncwarp();
-  prepare_substep_warp(sc, T, lane);
-}
-
-// The tool step of a scene, as one CTA of k_musl_node: it needs the wrench
-// partials, which P2G has left, and nothing later in the substep; k_fupd still
-// reads this substep's frame, so the result goes to the scene's record in
-// scenes_next and commit_tool takes it over when the particles are done.  As a
-// kernel of its own after k_fupd it was 9.2 us of a 16,000-particle scene's 98 us
-// substep and 16 of the 256-scene batch's 1,460.
-struct ToolS {
-  DevScene sc;
-  ToolTmp T;
-  double part[6][8], W[6];
-};
-
-// the part of the record that the tool step writes, in words
-constexpr int kToolWord0 = (int)(offsetof(DevScene, xB) / sizeof(int));
-constexpr int kToolWords = (int)(offsetof(DevScene, err) / sizeof(int)) - kToolWord0;
-
-__device__ __forceinline__ void next_tool(const World &w, int sid, ToolS &S) {
-  DevScene &g = w.scenes[sid];
-  // the labels of the last substep are in the slot table; k_fupd sets this anew
-  if (threadIdx.x == 0) g.label_pending = 0;
-  if (g.frozen) return;  // a scene that has taken its substeps: nothing moves
-  // the scene record into shared memory (coalesced), so that the tool step
-  // and frame below read and write it at shared-memory latency
-  static_assert(sizeof(DevScene) % sizeof(double) == 0, "the scene record copies as doubles");
-  for (int i = threadIdx.x; i < (int)(sizeof(DevScene) / sizeof(double)); i += blockDim.x)
-    reinterpret_cast<double *>(&S.sc)[i] = reinterpret_cast<const double *>(&g)[i];
-  // this substep's per-brick wrench partials: 256 strides over the bricks, a
-  // fixed shuffle tree over each 32 of them, then the eight in order (the
-  // same sums for every node tile size, the CTA's thread count)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int v = wid; v < 8; v += nw) {
-    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (g.has_blade) {
-      const double2 *q = reinterpret_cast<const double2 *>(w.wpart) + (size_t)g.brick_begin * 3;
-      const int nb = g.n_brick;
-      int j = 32 * v + lane;
-      for (; j + 256 < nb; j += 512) {  // two strides' loads in flight
-        double2 a[3], b[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          a[k] = q[(size_t)j * 3 + k];
-          b[k] = q[(size_t)(j + 256) * 3 + k];
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          acc[2 * k] = acc[2 * k] + a[k].x + b[k].x;
-          acc[2 * k + 1] = acc[2 * k + 1] + a[k].y + b[k].y;
-        }
-      }
-      if (j < nb)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const double2 a = q[(size_t)j * 3 + k];
-          acc[2 * k] += a.x;
-          acc[2 * k + 1] += a.y;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      double y = acc[k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) y += __shfl_down_sync(FULL, y, o);
-      if (lane == 0) S.part[k][v] = y;
-    }
-  }
-  __syncthreads();
-  if (wid == 0) {
-    if (lane < 6) {
-      double t = 0.0;
-      for (int i = 0; i < 8; ++i) t += S.part[lane][i];
-      S.W[lane] = t;
-    }
-    __syncwarp();
-    tool_step(w, S.sc, S.T, S.W, lane);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kToolWords; i += blockDim.x)
-    reinterpret_cast<int *>(w.scenes_next + sid)[kToolWord0 + i] = reinterpret_cast<const int *>(&S.sc)[kToolWord0 + i];
-}
-
-// take over the tool step that next_tool has left (one CTA; no other CTA of
-// the launch may read the record's tool block, step or frozen)
-__device__ __forceinline__ void commit_tool(const World &w, int sid) {
-  const bool frozen = w.scenes[sid].frozen != 0;
-  __syncthreads();
-  if (frozen) return;
-  for (int i = threadIdx.x; i < kToolWords; i += blockDim.x)
-    reinterpret_cast<int *>(w.scenes + sid)[kToolWord0 + i] =
-        reinterpret_cast<const int *>(w.scenes_next + sid)[kToolWord0 + i];
-}
-
 // --------------------------------------------------------------------------
 // k_musl_node: per slot, MUSL sums of the covering bricks, coupling, v*; its
-// first n_scenes CTAs take the scenes' tool steps
+// first `tools` CTAs take the scenes' tool steps (none if G2P did)
 // --------------------------------------------------------------------------
-__global__ void k_musl_node(World w, LaunchSet ls) {
+__global__ void k_musl_node(World w, LaunchSet ls, int tools) {
   chain_wait();
   __shared__ __align__(16) unsigned char raw[sizeof(NodeS<3>) > sizeof(ToolS) ? sizeof(NodeS<3>) : sizeof(ToolS)];
-  if ((int)blockIdx.x < ls.n_scenes) {
+  if ((int)blockIdx.x < tools) {
     next_tool(w, ls.scene_ids[blockIdx.x], *reinterpret_cast<ToolS *>(raw));
     return;
   }
   NodeS<3> &N = *reinterpret_cast<NodeS<3> *>(raw);
-  const int4 t = ls.ntiles[blockIdx.x - ls.n_scenes];
+  const int4 t = ls.ntiles[blockIdx.x - tools];
   const int i = threadIdx.x;
   const DevScene &sc = w.scenes[t.x];
   if (sc.frozen) return;
-  const int node = t.y + i;
-  const int cnt = i < t.z ? w.N.slot_cnt[node] : 0;
+  const int cnt = i < t.z ? w.N.slot_cnt[t.y + i] : 0;
   auto sums = [&](int nd, int sl, float (&S)[3]) {
     int ix, iy, iz;
     node_coords(sc, nd - sc.node_begin, ix, iy, iz);
@@ -1011,7 +751,7 @@ __global__ void k_musl_node(World w, LaunchSet ls) {
       S[2] += a[k].z;
     }
   };
-  if (cnt == 1) {
+  auto single = [&](int node) {
     const int off = w.N.slot_off[node];
     float S[3];
     sums(node, 0, S);
@@ -1022,10 +762,9 @@ __global__ void k_musl_node(World w, LaunchSet ls) {
       vs = make_float4(S[0] * im, S[1] * im, S[2] * im, 0.f);
     }
     w.S.vstar[off] = vs;
-  }
-  if (!__syncthreads_or(cnt > 1)) return;
-  coupled_slots<3>(
-      w, N, t.y, cnt,
+  };
+  tile_nodes<3>(
+      w, N, t.y, ls.ntile_size, cnt, single,
       [&](int nd, int sl, int slot, float &m, float (&S)[3]) {
         sums(nd, sl, S);
         m = w.S.vold[slot].w;
@@ -2348,7 +2087,8 @@ static void launch_p2g(const World &w, const LaunchSet &ls, cudaStream_t st) {
 
 template <int PPC, int MB, int G>
 static void launch_g2p(const World &w, const LaunchSet &ls, cudaStream_t st) {
-  chain_launch(k_g2p_musl<PPC, MB, G>, dim3(ls.n_btiles), BT * G, sizeof(K4S<PPC, G>), st, w, ls);
+  const int tools = ls.any_lattice ? 0 : g2p_tools(ls);  // the lattice form's if both run
+  chain_launch(k_g2p_musl<PPC, MB, G>, dim3(tools + ls.n_btiles), BT * G, sizeof(K4S<PPC, G>), st, w, ls, tools);
 }
 
 template <int MB, int G>
@@ -2385,6 +2125,17 @@ static void launch_fupd_general(const World &w, const LaunchSet &ls, cudaStream_
   else launch_fupd<OccFupd<2>::v, 1>(w, ls, st);
 }
 
+// Threads of a node tile's CTA beyond its nodes, for sets of few tiles (sets of
+// many are bound by the loads themselves: 256-scene batch, 16,000 tiles,
+// 1,451 -> 1,592 us a substep).  k_p2g_node of a cut 16,000-particle scene 10.1 ->
+// 6.2 us, k_musl_node 8.8 -> 6.2; a 477,000-particle scene of some 500 tiles
+// 141 -> 139 us a substep.
+#define NODE_TEAM_TILES (4 * 152)
+#define NODE_TEAM 256
+static int node_threads(const LaunchSet &ls) {
+  return ls.ntile_size + (ls.n_ntiles <= NODE_TEAM_TILES ? NODE_TEAM : 0);
+}
+
 // Each brick kernel in its lattice and its general form, as the set's scenes
 // need (each form returns at once for the other's scenes).
 static void launch_bricks(const World &w, const LaunchSet &ls, cudaStream_t st, cudaEvent_t *ev) {
@@ -2396,7 +2147,7 @@ static void launch_bricks(const World &w, const LaunchSet &ls, cudaStream_t st, 
   }
   rec(ev, 0, 1, st);
   rec(ev, 1, 0, st);
-  chain_launch(k_p2g_node, dim3(ls.n_ntiles), ls.ntile_size, 0, st, w, ls);
+  chain_launch(k_p2g_node, dim3(ls.n_ntiles), node_threads(ls), 0, st, w, ls);
   rec(ev, 1, 1, st);
   rec(ev, 2, 0, st);
   if (ls.any_lattice) bm_launch_g2p_lat(w, ls, st);
@@ -2406,7 +2157,8 @@ static void launch_bricks(const World &w, const LaunchSet &ls, cudaStream_t st, 
   }
   rec(ev, 2, 1, st);
   rec(ev, 3, 0, st);
-  chain_launch(k_musl_node, dim3(ls.n_scenes + ls.n_ntiles), ls.ntile_size, 0, st, w, ls);
+  const int tools = g2p_tools(ls) ? 0 : ls.n_scenes;
+  chain_launch(k_musl_node, dim3(tools + ls.n_ntiles), node_threads(ls), 0, st, w, ls, tools);
   rec(ev, 3, 1, st);
   rec(ev, 4, 0, st);
   if (ls.any_lattice) bm_launch_fupd_lat(w, ls, st);

@@ -36,6 +36,7 @@
 // codes' particles are skipped.
 #include "bm_device.cuh"
 #include "bm_internal.cuh"
+#include "bm_tool.cuh"
 
 namespace {
 
@@ -428,11 +429,16 @@ __device__ __forceinline__ void musl_cell(const G2PS<G> &S, const CellOz &q, uns
 }
 
 template <int MB, int G>
-__global__ void __launch_bounds__(GT * G, MB) k_g2p_lat(World w, LaunchSet ls) {
+__global__ void __launch_bounds__(GT * G, MB) k_g2p_lat(World w, LaunchSet ls, int tools) {
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   G2PS<G> &S = *reinterpret_cast<G2PS<G> *>(smraw);
-  const int4 bt = ls.btiles[blockIdx.x];
+  if (G > 1 && (int)blockIdx.x < tools) {
+    next_tool(w, ls.scene_ids[blockIdx.x], *reinterpret_cast<ToolS *>(smraw));
+    return;
+  }
+  static_assert(sizeof(ToolS) <= sizeof(G2PS<G>), "the tool step fits");
+  const int4 bt = ls.btiles[blockIdx.x - tools];
   DevScene &scm = w.scenes[bt.x];
   const DevScene &sc = scm;
   if (sc.frozen || !sc.lattice) return;
@@ -737,10 +743,11 @@ void bm_launch_p2g_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
 }
 
 void bm_launch_g2p_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
+  const int tools = g2p_tools(ls);
   if (ls.n_btiles <= WIDE_BRICKS_LAT)
-    chain_launch(k_g2p_lat<1, GWIDE>, dim3(ls.n_btiles), GT * GWIDE, sizeof(G2PS<GWIDE>), st, w, ls);
+    chain_launch(k_g2p_lat<1, GWIDE>, dim3(tools + ls.n_btiles), GT * GWIDE, sizeof(G2PS<GWIDE>), st, w, ls, tools);
   else
-    chain_launch(k_g2p_lat<OCC_G2P, 1>, dim3(ls.n_btiles), GT, sizeof(G2PS<1>), st, w, ls);
+    chain_launch(k_g2p_lat<OCC_G2P, 1>, dim3(ls.n_btiles), GT, sizeof(G2PS<1>), st, w, ls, 0);
 }
 
 template <int MB, int G>

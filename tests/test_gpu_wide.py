@@ -2,8 +2,9 @@
 
 A scene stepped alone takes the forms with several groups of threads per
 brick; in a batch filled up with copies of a larger body it takes the
-one-group forms.  Every sum has the same terms in the same order in both, so
-the scene must come out with the same bits.
+one-group forms, and the tool step another kernel's CTAs.  Every sum has the
+same terms in the same order in both, so the scene must come out with the same
+bits.
 """
 import numpy as np
 import pytest
@@ -32,12 +33,13 @@ def _lattice(cells, k):
     return np.stack(np.meshgrid(*ax, indexing="ij"), -1).reshape(-1, 3)
 
 
-def _scene(X, blade, **kw):
+def _scene(X, blade, mass=0.0, **kw):
     size = X.max(0) - X.min(0) + DX
     # the edge stands in the top layer: contact, reaction and labels from the first substeps
     edge = (X[:, 0].mean() + 2e-4, X[:, 1].mean(), X[:, 2].max() - 0.2 * DX)
     b = bi.Blade(pose_x=tuple(float(t) for t in edge), half_length=float(size.max()),
-                 segments=[bi.Segment(40, v=(0.0, 0.0, -1.5), cut_id=0)]) if blade else None
+                 mass=mass, inertia=tuple(4e-5 * mass * np.diag((1.0, 2.0, 3.0)).ravel()), rigid_interval=2 if mass else 1,
+                 segments=[bi.Segment(40, v=(0.0, 0.0, -1.5), omega=(0.5, 2.0, -1.0), cut_id=0)]) if blade else None
     return bi.Scene(X=X, dx=DX, origin=(-DX / 2,) * 3, V0=DX ** 3 / 8, dt=1e-4, E=1e5, nu=0.3, blade=b, **kw)
 
 
@@ -48,6 +50,7 @@ def _scene(X, blade, **kw):
     ((9, 5, 6), (2, 2, 2), 0.1, 3, {}), ((4, 4, 4), (2, 2, 2), 0.1, 12, {}), ((7, 5, 3), (4, 2, 2), 0.0, 3, {}),
     ((7, 5, 3), (2, 2, 2), 0.1, 2, dict(yield_stress=2e3, viscosity=5.0)),
     ((9, 5, 6), (2, 2, 2), 0.0, 2, dict(yield_stress=2e3, viscosity=5.0)),
+    ((9, 5, 6), (2, 2, 2), 0.1, 2, dict(mass=0.05)),
 ])
 def test_few_and_many_bricks_agree_bitwise(pkg, cells, k, jitter, codes, kw):
     rng = np.random.default_rng(3)
@@ -80,14 +83,16 @@ def test_few_and_many_bricks_agree_bitwise(pkg, cells, k, jitter, codes, kw):
         else:
             assert pkg.footprint(sc)[2] <= 2 * 152
             s.step(8)
-        got.append((s.read(*FIELDS), s.tool_wrench() if codes < 12 else 0, s.info().error_bits, s.info().n_slots))
+        got.append((s.read(*FIELDS), s.tool_wrench() if codes < 12 else 0, s.info().error_bits, s.info().n_slots,
+                    s.tool_state() if codes < 12 else np.zeros(1)))
         s.close()
         if many:
             f.close()
             b.close()
     for name in FIELDS:
         assert np.array_equal(got[0][0][name], got[1][0][name]), name
-    assert np.array_equal(got[0][1], got[1][1]) and got[0][2:] == got[1][2:]
+    assert np.array_equal(got[0][1], got[1][1]) and got[0][2:4] == got[1][2:4]
+    assert np.array_equal(got[0][4], got[1][4])
     assert got[0][2] == 0
     if codes < 12 and n > 1:
         assert np.any(got[0][1] != 0)
