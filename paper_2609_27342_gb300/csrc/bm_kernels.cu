@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls, 
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   K4S<PPC, G> &S = *reinterpret_cast<K4S<PPC, G> *>(smraw);
-  if (G > 1 && (int)blockIdx.x < tools) {
+  if ((int)blockIdx.x < tools) {
     next_tool(w, ls.scene_ids[blockIdx.x], *reinterpret_cast<ToolS *>(smraw));
     return;
   }
@@ -1082,35 +1082,32 @@ __global__ void k_pair_sort(World w) {
   }
 }
 
-// Whether two particles' reference stencils overlap (base cells at most two
-// cells apart on every axis): such a pair interacts through the grid, and is
-// a contact pair only once a cut separates it (self-contact exclusion).
-__device__ __forceinline__ bool share_stencil(uint32_t bp, uint32_t bq) {
-  int px, py, pz, qx, qy, qz;
-  particle_base(bp, px, py, pz);
-  particle_base(bq, qx, qy, qz);
-  return abs(px - qx) <= 2 && abs(py - qy) <= 2 && abs(pz - qz) <= 2;
-}
-
-// Candidate lists of the particles in entries [c0, c1) of one bucket (at most
+// Candidate lists of the particles in entries [c0, c1) of the buckets (at most
 // 32, lane i holding entry c0 + i), by one warp.  The particles are taken in
 // groups of one cell (and scene); a group shares its 27 neighbour cells
 // (dz, dy, dx in -1..1, x fastest), whose bucket entries are laid end to end
-// and tested 64 at a time, two per lane, against each member in turn (read
-// from the warp's shared memory: five shuffles a member for every 32 entries
-// were a third of the kernel's instructions): an
+// and tested 64 at a time, two per lane, against each member in turn: an
 // entry counts when it belongs to the neighbour cell (its key; a bucket's
 // hash may be shared), is another particle and lies within r_l = 2 R_p +
 // skin.  A ballot gives each accepted entry its place, so every list is in
 // (cell, pool index) order, as a walk of the cells in order would give;
-// bit 31 of an entry marks a pair whose reference stencils overlap, and a
-// list of only such pairs is marked by NBR_SHARED in its count.
+// bit 31 of an entry marks a pair whose reference stencils overlap (base
+// cells at most two apart on every axis): such a pair interacts through the
+// grid, and is a contact pair only once a cut separates it (self-contact
+// exclusion).  A list of only such pairs is marked by NBR_SHARED in its count.
+// The kernel is bound by instructions (more warps per SM change nothing):
+// members are read from shared memory, the cell of an entry is the rank of
+// its start among the non-empty cells', and base cells are compared unpacked.
 #define NBR_SHARED 0x80
 #define LIST_WARPS 8
+#define LIST_UNIT 16  // entries per warp and round
+#define LIST_OCC 4
 
 struct ListMembers {
   float4 me[32];
-  uint32_t base[32];
+  int4 base[32];               // base cell + 2
+  int2 cell[27];               // of the non-empty neighbour cells: first entry and place in the row
+  unsigned long long key[27];
 };
 
 __device__ __forceinline__ void bucket_lists(const World &w, ListMembers &M, int c0, int c1, int lane) {
@@ -1118,10 +1115,11 @@ __device__ __forceinline__ void bucket_lists(const World &w, ListMembers &M, int
   const bool mine = lane < c1 - c0;
   const float4 me = mine ? P.hent[c0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
   const unsigned long long mkey = mine ? P.hentk[c0 + lane] : ~0ull;
+  int bx, by, bz;
+  particle_base(mine ? P.hbase[c0 + lane] : 0u, bx, by, bz);
   __syncwarp();
   M.me[lane] = me;
-  M.base[lane] = mine ? P.hbase[c0 + lane] : 0u;
-  __syncwarp();
+  M.base[lane] = make_int4(bx + 2, by + 2, bz + 2, 0);
   const int mscene = (int)(mkey >> 48);
   int mx = 0, my = 0, mz = 0;
   if (mine) {
@@ -1131,7 +1129,7 @@ __device__ __forceinline__ void bucket_lists(const World &w, ListMembers &M, int
     mz = (int)floorf(me.z * ih);
   }
   int cnt = 0;
-  bool apart = false;  // some pair of the lane's list shares no stencil
+  unsigned apart = 0;  // bit m: lane saw a pair of member m that shares no stencil
   unsigned todo = __ballot_sync(FULL, mine);
   while (todo) {
     const int lead = __ffs(todo) - 1;
@@ -1160,40 +1158,43 @@ __device__ __forceinline__ void bucket_lists(const World &w, ListMembers &M, int
     }
     const int T = __shfl_sync(FULL, incl, 31);
     const int excl = incl - sz;
+    const unsigned full = __ballot_sync(FULL, sz > 0);
+    if (sz > 0) {
+      const int r = __popc(full & ((1u << lane) - 1u));
+      M.cell[r] = make_int2(a0, excl);
+      M.key[r] = nk;
+    }
+    __syncwarp();
+    int before = -1;  // rank of the last cell that starts before the window
     for (int base = 0; base < T; base += 64) {
       float4 e[2];
-      uint32_t eb[2];
+      int ebx[2], eby[2], ebz[2];
       bool valid[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int j = base + 32 * h + lane;
-        // neighbour cell of candidate j: the last cell whose entries start at or before j
-        int L = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-          const int t = L + step;
-          const int ex = __shfl_sync(FULL, excl, t < 27 ? t : 26);
-          if (t < 27 && ex <= j) L = t;
-        }
-        const int aL = __shfl_sync(FULL, a0, L), exL = __shfl_sync(FULL, excl, L);
-        const unsigned long long kL = __shfl_sync(FULL, nk, L);
+        // the cell of candidate j is the last one that starts at or before j
+        const int w0 = base + 32 * h, j = w0 + lane;
+        const unsigned starts =
+            __reduce_or_sync(FULL, sz > 0 && excl >= w0 && excl < w0 + 32 ? 1u << (excl - w0) : 0u);
+        const int L = before + __popc(starts & (0xffffffffu >> (31 - lane)));
+        before += __popc(starts);
+        const int2 cl = M.cell[L];
         const bool inr = j < T;
-        const int k = aL + (j - exL);
+        const int k = cl.x + (j - cl.y);
         e[h] = inr ? P.hent[k] : make_float4(0.f, 0.f, 0.f, 0.f);
         const unsigned long long ek = inr ? P.hentk[k] : 0ull;
-        eb[h] = inr ? P.hbase[k] : 0u;
-        valid[h] = inr && ek == kL;
+        particle_base(inr ? P.hbase[k] : 0u, ebx[h], eby[h], ebz[h]);
+        valid[h] = inr && ek == M.key[L];
       }
       unsigned g = grp;
       while (g) {
         const int m = __ffs(g) - 1;
         g &= g - 1;
         const float4 mp = M.me[m];
-        const uint32_t bp = M.base[m];
+        const int4 bp = M.base[m];
         const int p = __float_as_int(mp.w);
-        int c = __shfl_sync(FULL, cnt, m);
-        const int c_in = c;
-        bool far = false;
+        const int c_in = __shfl_sync(FULL, cnt, m);
+        int c = c_in;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int q = __float_as_int(e[h].w);
@@ -1202,23 +1203,22 @@ __device__ __forceinline__ void bucket_lists(const World &w, ListMembers &M, int
           const unsigned am = __ballot_sync(FULL, acc);
           if (acc) {
             const int pos = c + __popc(am & ((1u << lane) - 1u));
-            const bool share = share_stencil(bp, eb[h]);
-            far |= !share;
+            const bool share = (unsigned)(bp.x - ebx[h]) <= 4u && (unsigned)(bp.y - eby[h]) <= 4u &&
+                               (unsigned)(bp.z - ebz[h]) <= 4u;
+            if (!share) apart |= 1u << m;
             if (pos < BM_NBR) P.nbr[(size_t)p * BM_NBR + pos] = share ? (int)((uint32_t)q | 0x80000000u) : q;
           }
           c += __popc(am);
         }
-        const bool any_far = __any_sync(FULL, far);
-        if (lane == m) {
-          cnt += c - c_in;
-          apart |= any_far;
-        }
+        if (lane == m) cnt = c;
       }
     }
+    __syncwarp();
   }
+  apart = __reduce_or_sync(FULL, apart);
   if (mine) {
     const int p = __float_as_int(me.w);
-    P.nbr_n[p] = (uint8_t)(min(cnt, BM_NBR) | (apart ? 0 : NBR_SHARED));
+    P.nbr_n[p] = (uint8_t)(min(cnt, BM_NBR) | ((apart >> lane) & 1u ? 0 : NBR_SHARED));
     P.xb[0][p] = me.x;
     P.xb[1][p] = me.y;
     P.xb[2][p] = me.z;
@@ -1227,27 +1227,17 @@ __device__ __forceinline__ void bucket_lists(const World &w, ListMembers &M, int
 }
 
 // candidate lists of every particle of the scenes that rebuild them: each
-// warp takes groups of 32 buckets (grid-stride) and builds the lists of the
-// particles of each non-empty one, 32 entries at a time.  The positions of
+// warp takes LIST_UNIT consecutive entries (grid-stride).  The positions of
 // the build are kept.
-__global__ void __launch_bounds__(32 * LIST_WARPS) k_pair_list(World w) {
+__global__ void __launch_bounds__(32 * LIST_WARPS, LIST_OCC) k_pair_list(World w) {
   chain_wait();
   if (!*w.H.build) return;
   __shared__ ListMembers members[LIST_WARPS];
-  const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-  const int nb = w.H.n_buckets;
-  for (int b0 = warp * 32; b0 < nb; b0 += nwarps * 32) {
-    const int b = b0 + lane;
-    const int e0 = b < nb ? w.H.bucket_start[b] : 0, e1 = b < nb ? w.H.bucket_start[b + 1] : 0;
-    unsigned todo = __ballot_sync(FULL, e1 > e0);
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int k0 = __shfl_sync(FULL, e0, src), k1 = __shfl_sync(FULL, e1, src);
-      for (int c = k0; c < k1; c += 32) bucket_lists(w, members[threadIdx.x >> 5], c, min(k1, c + 32), lane);
-    }
-  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int total = w.H.bucket_start[w.H.n_buckets];
+  const int step = gridDim.x * LIST_WARPS * LIST_UNIT;
+  for (int c = (blockIdx.x * LIST_WARPS + wid) * LIST_UNIT; c < total; c += step)
+    bucket_lists(w, members[wid], c, min(total, c + LIST_UNIT), lane);
 }
 
 // Pair impulses (Eq. 10-13), one thread per particle walking its list
@@ -1692,41 +1682,45 @@ __device__ __forceinline__ void brick_tile_slots(const World &w, const LaunchSet
   if (lane == 31) w.B.ptot[bt.y] = incl;
 }
 
+// Exclusive sums of v[0..n) by one CTA, each thread a run of consecutive
+// values, so that the CTA scans once however many there are: `out(j, sum
+// before j, v[j])`.  Returns the total.  (In steps of a value per thread, two
+// barriers each, a 477,000-particle scene's 1,000 bricks kept k_slot_fill at 12 us.)
+template <class Out>
+__device__ __forceinline__ int cta_offsets(const int *v, int n, int *sm, Out out) {
+  const int per = (n + blockDim.x - 1) / blockDim.x;
+  const int j0 = threadIdx.x * per, j1 = min(j0 + per, n);
+  int mine = 0;
+#pragma unroll 4
+  for (int j = j0; j < j1; ++j) mine += v[j];
+  int total;
+  int before = block_excl_scan(mine, sm, total);
+  for (int j = j0; j < j1; ++j) {
+    const int q = v[j];
+    out(j, before, q);
+    before += q;
+  }
+  return total;
+}
+
 // slot offsets of a scene's node tiles (one CTA): exclusive sums in place
 __device__ __forceinline__ void tile_offsets(const World &w, DevScene &sc, int *sm) {
-  int carry = 0;
-  for (int base = 0; base < sc.n_ntile; base += blockDim.x) {
-    const int j = base + threadIdx.x;
-    const int v = j < sc.n_ntile ? w.N.tile_sum[sc.ntile_begin + j] : 0;
-    int total;
-    const int ex = block_excl_scan(v, sm, total);
-    if (j < sc.n_ntile) w.N.tile_sum[sc.ntile_begin + j] = carry + ex;
-    carry += total;
-    __syncthreads();
-  }
+  int *ts = w.N.tile_sum + sc.ntile_begin;
+  const int total = cta_offsets(ts, sc.n_ntile, sm, [&](int j, int before, int) { ts[j] = before; });
   if (threadIdx.x == 0) {
-    sc.n_slots = carry;
-    if (carry > sc.slot_cap) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
+    sc.n_slots = total;
+    if (total > sc.slot_cap) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
   }
 }
 
 // partial-sum ranges of a scene's bricks (one CTA)
 __device__ __forceinline__ void brick_ranges(const World &w, DevScene &sc, int *sm) {
-  int pcarry = 0;
   bool pover = false;
-  for (int base = 0; base < sc.n_brick; base += blockDim.x) {
-    const int j = base + threadIdx.x;
-    const int v = j < sc.n_brick ? w.B.ptot[sc.brick_begin + j] : 0;
-    int total;
-    const int ex = block_excl_scan(v, sm, total);
-    if (j < sc.n_brick) {
-      const bool fits = pcarry + ex + v <= sc.ppool_cap;
-      w.B.poff[sc.brick_begin + j] = fits ? sc.ppool_begin + pcarry + ex : -1;
-      pover |= !fits;
-    }
-    pcarry += total;
-    __syncthreads();
-  }
+  cta_offsets(w.B.ptot + sc.brick_begin, sc.n_brick, sm, [&](int j, int before, int v) {
+    const bool fits = before + v <= sc.ppool_cap;
+    w.B.poff[sc.brick_begin + j] = fits ? sc.ppool_begin + before : -1;
+    pover |= !fits;
+  });
   if (pover) atomicOr(&sc.err, BM_ERRBIT_SLOT_OVERFLOW);
 }
 
@@ -2195,8 +2189,7 @@ static void launch_pairs(const World &w, const LaunchSet &ls, cudaStream_t st, c
   chain_launch(k_pair_sort, dim3((nb / 2 + 255) / 256), 256, 0, st, w);  // at least a thread per particle
   rec(ev, 16, 1, st);
   rec(ev, 18, 0, st);
-  const int lgrid = (nb / 32 + 7) / 8;  // 8 warps per CTA, a warp per 32 buckets, at most 8 CTAs per SM
-  chain_launch(k_pair_list, dim3(lgrid < 152 * 8 ? lgrid : 152 * 8), 32 * LIST_WARPS, 0, st, w);
+  chain_launch(k_pair_list, dim3(152 * LIST_OCC), 32 * LIST_WARPS, 0, st, w);
   rec(ev, 18, 1, st);
   rec(ev, 17, 0, st);
   chain_launch(k_pair, dim3(ls.n_btiles, 4), 128, 0, st, w, ls);

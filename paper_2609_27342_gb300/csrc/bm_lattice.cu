@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(GT * G, MB) k_g2p_lat(World w, LaunchSet ls, i
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   G2PS<G> &S = *reinterpret_cast<G2PS<G> *>(smraw);
-  if (G > 1 && (int)blockIdx.x < tools) {
+  if ((int)blockIdx.x < tools) {
     next_tool(w, ls.scene_ids[blockIdx.x], *reinterpret_cast<ToolS *>(smraw));
     return;
   }
@@ -747,7 +747,7 @@ void bm_launch_g2p_lat(const World &w, const LaunchSet &ls, cudaStream_t st) {
   if (ls.n_btiles <= WIDE_BRICKS_LAT)
     chain_launch(k_g2p_lat<1, GWIDE>, dim3(tools + ls.n_btiles), GT * GWIDE, sizeof(G2PS<GWIDE>), st, w, ls, tools);
   else
-    chain_launch(k_g2p_lat<OCC_G2P, 1>, dim3(ls.n_btiles), GT, sizeof(G2PS<1>), st, w, ls, 0);
+    chain_launch(k_g2p_lat<OCC_G2P, 1>, dim3(tools + ls.n_btiles), GT, sizeof(G2PS<1>), st, w, ls, tools);
 }
 
 template <int MB, int G>

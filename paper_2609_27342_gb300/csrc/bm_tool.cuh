@@ -288,6 +288,9 @@ __device__ __forceinline__ void commit_tool(const World &w, int sid) {
 }
 
 // Leading CTAs of G2P that take the scenes' tool steps; 0: k_musl_node does.
-inline int g2p_tools(const LaunchSet &ls) { return ls.n_btiles <= WIDE_BRICKS_LAT ? ls.n_scenes : 0; }
+#ifndef G2P_TOOLS
+#define G2P_TOOLS 152
+#endif
+inline int g2p_tools(const LaunchSet &ls) { return ls.n_scenes <= G2P_TOOLS ? ls.n_scenes : 0; }
 
 }  // namespace
