@@ -132,49 +132,72 @@ __device__ __forceinline__ void couple_T(int ns, const uint2 *codes, const float
     for (int c = 0; c < NC; ++c) S[b][c] = out[b][c];
 }
 
-// Walk the particles of code c in the stencil of scene-local node li with the
-// warp's lanes: for each of the 9 (y, z) rows of base cells the particles of
-// its three cells lie together in the pool (in two pieces where the row
-// crosses a brick), and consecutive lanes take consecutive particles, so the
-// reads of the NV values val[.][particle - p_begin] coalesce.  (A lane per
-// cell touched 27 sectors with every read, and the kernels were bound by
-// that.)  fn(values, N, grad N) for each.
-template <int NV, class Fn>
-__device__ __forceinline__ void walk_rows(const World &w, const DevScene &sc, int li, int lane, uint2 c,
-                                          float *const (&val)[NV], Fn fn) {
+// The 9 (y, z) rows of three base cells in a node's stencil: the particles of
+// a row lie together in the pool, in two pieces where it crosses a brick.
+struct Row {
+  int first;       // place of its first particle when the rows are laid end to end
+  int a0, na, b0;  // first piece: pool particle and count; second piece
+};
+
+// Fills rows[0..9) (and rows[9].first, the total) of scene-local node li by
+// one warp, a row per lane: walked one row after the other, the dependent
+// reads of the cell ranges were a third of the node kernels' time.
+__device__ __forceinline__ void node_rows(const World &w, const DevScene &sc, int li, int lane, Row *rows) {
   const int ix = li % sc.nn[0], iy = (li / sc.nn[0]) % sc.nn[1], iz = li / (sc.nn[0] * sc.nn[1]);
   const int *cs = w.N.cell_start + sc.cell_begin;
   const int x0 = max(ix - 2, 0), x1 = min(ix, sc.nb[0] - 1);
   const int xs = min(x0 | 3, x1);  // last cell of the first piece
-  const int pb = sc.p_begin;
-  for (int oz = 0; oz < 3; ++oz)
-    for (int oy = 0; oy < 3; ++oy) {
-      const int by = iy - oy, bz = iz - oz;
-      if (by < 0 || bz < 0 || by >= sc.nb[1] || bz >= sc.nb[2] || x0 > x1) continue;
-      const int a0 = cs[cell_at(sc, x0, by, bz)], a1 = cs[cell_at(sc, xs, by, bz) + 1];
-      int b0 = 0, b1 = 0;
-      if (xs < x1) {
-        b0 = cs[cell_at(sc, xs + 1, by, bz)];
-        b1 = cs[cell_at(sc, x1, by, bz) + 1];
-      }
-      const int na = a1 - a0, n = na + b1 - b0;
-      for (int i = lane; i < n; i += 32) {
-        const int p = i < na ? a0 + i : b0 + (i - na);
-        float v[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) v[k] = val[k][p - pb];
-        const float f0 = w.P.fx[0][p], f1 = w.P.fx[1][p], f2 = w.P.fx[2][p];
-        const int ox = ix - (int)(w.P.base[p] & 1023u);
-        if (w.P.s1[p] != c.x || w.P.s2[p] != c.y) continue;
-        float wx, wy, wz, dx, dy, dz;
-        wgt(ox, f0, wx, dx);
-        wgt(oy, f1, wy, dy);
-        wgt(oz, f2, wz, dz);
-        const float N = wx * wy * wz;
-        const float gN[3] = {dx * wy * wz * sc.inv_dx, wx * dy * wz * sc.inv_dx, wx * wy * dz * sc.inv_dx};
-        fn(v, N, gN);
-      }
+  int a0 = 0, na = 0, b0 = 0, n = 0;
+  const int by = iy - lane % 3, bz = iz - lane / 3;
+  if (lane < 9 && by >= 0 && bz >= 0 && by < sc.nb[1] && bz < sc.nb[2] && x0 <= x1) {
+    a0 = cs[cell_at(sc, x0, by, bz)];
+    na = cs[cell_at(sc, xs, by, bz) + 1] - a0;
+    n = na;
+    if (xs < x1) {
+      b0 = cs[cell_at(sc, xs + 1, by, bz)];
+      n += cs[cell_at(sc, x1, by, bz) + 1] - b0;
     }
+  }
+  int incl = n;
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane < 9) rows[lane] = Row{incl - n, a0, na, b0};
+  if (lane == 8) rows[9].first = incl;
+}
+
+// Walk the particles of code c in the stencil of scene-local node li with nt
+// threads (t of them this one), the rows laid end to end: consecutive threads
+// take consecutive particles, so the reads of the NV values
+// val[.][particle - p_begin] coalesce.  (A lane per cell touched 27 sectors
+// with every read.)  fn(values, N, grad N) for each.
+template <int NV, class Fn>
+__device__ __forceinline__ void walk_rows(const World &w, const DevScene &sc, int li, const Row *rows, int t, int nt,
+                                          uint2 c, float *const (&val)[NV], Fn fn) {
+  const int ix = li % sc.nn[0];
+  const int pb = sc.p_begin, total = rows[9].first;
+  int r = 0;
+  for (int j = t; j < total; j += nt) {
+    while (rows[r + 1].first <= j) ++r;
+    const Row q = rows[r];
+    const int i = j - q.first;
+    const int p = i < q.na ? q.a0 + i : q.b0 + (i - q.na);
+    float v[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = val[k][p - pb];
+    const float f0 = w.P.fx[0][p], f1 = w.P.fx[1][p], f2 = w.P.fx[2][p];
+    const int ox = ix - (int)(w.P.base[p] & 1023u);
+    if (w.P.s1[p] != c.x || w.P.s2[p] != c.y) continue;
+    float wx, wy, wz, dx, dy, dz;
+    wgt(ox, f0, wx, dx);
+    wgt(r % 3, f1, wy, dy);
+    wgt(r / 3, f2, wz, dz);
+    const float N = wx * wy * wz;
+    const float gN[3] = {dx * wy * wz * sc.inv_dx, wx * dy * wz * sc.inv_dx, wx * wy * dz * sc.inv_dx};
+    fn(v, N, gN);
+  }
 }
 
 // sum over the warp's lanes in a fixed butterfly order (every lane gets it)
@@ -184,29 +207,37 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// The per-node adjoint kernels run one warp per node: the lanes walk the
-// node's particles (walk_rows), their sums are combined by
-// warp_sum, one pass per logical grid of the node (codes fixed), and lane 0
-// applies the transposed coupling to the node's slot sums.
-constexpr int kAdjNodesPerBlock = kAdjBlock / 32;
+// The per-node adjoint kernels give a node kAdjTeam threads, which walk its
+// particles (walk_rows); their sums are combined by warp_sum and in warp
+// order, one pass per logical grid of the node (codes fixed), and one thread
+// applies the transposed coupling to the node's slot sums.  The kernels wait
+// on memory: with a warp per node, the rows one after the other, they took
+// 19.4 us each for the 32,000-particle calibration cuboid; 15.7 and 14.4 with
+// 64 threads, 16.0 and 14.6 with 128.
+constexpr int kAdjTeam = 64;
+constexpr int kAdjNodesPerBlock = kAdjBlock / kAdjTeam;
+constexpr int kAdjWarps = kAdjTeam / 32;  // per node
 
 // per node: slot masses, adjoint of v* from F' = F + dt sum v* (x) grad N,
 // then through v* = C p* / m
 __global__ void __launch_bounds__(kAdjBlock) k_adj_musl(World w, AdjWork aw) {
   chain_wait();
-  __shared__ float red[kAdjNodesPerBlock][BM_MAXS][4];
+  __shared__ float red[kAdjNodesPerBlock][kAdjWarps][BM_MAXS][4];
+  __shared__ Row rows[kAdjNodesPerBlock][10];
   const DevScene &sc = w.scenes[aw.slot];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int li = blockIdx.x * kAdjNodesPerBlock + wid;
-  if (li >= sc.n_node) return;
+  const int t = threadIdx.x % kAdjTeam, team = threadIdx.x / kAdjTeam;
+  const int lane = threadIdx.x & 31, wid = t >> 5;
+  const int li = blockIdx.x * kAdjNodesPerBlock + team;
   const int node = sc.node_begin + li;
-  const int off = w.N.slot_off[node], ns = w.N.slot_cnt[node];
-  if (ns == 0) return;
+  const int ns = li < sc.n_node ? w.N.slot_cnt[node] : 0;
+  const int off = ns > 0 ? w.N.slot_off[node] : 0;
+  if (ns > 0 && wid == 0) node_rows(w, sc, li, lane, rows[team]);
+  __syncthreads();
   const float dt = sc.dt, mp = sc.mp;
   for (int a = 0; a < ns; ++a) {
     const uint2 ca = w.S.code[off + a];
     float m = 0.f, S0 = 0.f, S1 = 0.f, S2 = 0.f;
-    walk_rows(w, sc, li, lane, ca, aw.Fb, [&](const float *F, float N, const float *gN) {
+    walk_rows(w, sc, li, rows[team], t, kAdjTeam, ca, aw.Fb, [&](const float *F, float N, const float *gN) {
       m += N * mp;
       S0 += dt * (F[0] * gN[0] + F[1] * gN[1] + F[2] * gN[2]);
       S1 += dt * (F[3] * gN[0] + F[4] * gN[1] + F[5] * gN[2]);
@@ -217,21 +248,27 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_musl(World w, AdjWork aw) {
     S1 = warp_sum(S1);
     S2 = warp_sum(S2);
     if (lane == 0) {
-      red[wid][a][0] = m;
-      red[wid][a][1] = S0;
-      red[wid][a][2] = S1;
-      red[wid][a][3] = S2;
+      red[team][wid][a][0] = m;
+      red[team][wid][a][1] = S0;
+      red[team][wid][a][2] = S1;
+      red[team][wid][a][3] = S2;
     }
   }
-  if (lane != 0) return;
+  __syncthreads();
+  if (t != 0) return;
   uint2 codes[BM_MAXS];
   float m[BM_MAXS], S[BM_MAXS][3];
   for (int a = 0; a < ns; ++a) {
     codes[a] = w.S.code[off + a];
-    m[a] = red[wid][a][0];
+    float q[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < kAdjWarps; ++k)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) q[r] += red[team][k][a][r];
+    m[a] = q[0];
     const float im = m[a] > 0.f ? 1.0f / m[a] : 0.f;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) S[a][r] = red[wid][a][1 + r] * im;
+    for (int r = 0; r < 3; ++r) S[a][r] = q[1 + r] * im;
   }
   couple_T<3>(ns, codes, m, S);
   const int rel = off - sc.slot_begin;
@@ -284,14 +321,17 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_v1(World w, AdjWork aw) {
 // N (p + dp)/m, then through Eq. 8 transposed
 __global__ void __launch_bounds__(kAdjBlock) k_adj_g2p(World w, AdjWork aw) {
   chain_wait();
-  __shared__ float red[kAdjNodesPerBlock][BM_MAXS][6];
+  __shared__ float red[kAdjNodesPerBlock][kAdjWarps][BM_MAXS][6];
+  __shared__ Row rows[kAdjNodesPerBlock][10];
   const DevScene &sc = w.scenes[aw.slot];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int li = blockIdx.x * kAdjNodesPerBlock + wid;
-  if (li >= sc.n_node) return;
+  const int t = threadIdx.x % kAdjTeam, team = threadIdx.x / kAdjTeam;
+  const int lane = threadIdx.x & 31, wid = t >> 5;
+  const int li = blockIdx.x * kAdjNodesPerBlock + team;
   const int node = sc.node_begin + li;
-  const int off = w.N.slot_off[node], ns = w.N.slot_cnt[node];
-  if (ns == 0) return;
+  const int ns = li < sc.n_node ? w.N.slot_cnt[node] : 0;
+  const int off = ns > 0 ? w.N.slot_off[node] : 0;
+  if (ns > 0 && wid == 0) node_rows(w, sc, li, lane, rows[team]);
+  __syncthreads();
   const int rel = off - sc.slot_begin;
   const float dt = sc.dt, beta = sc.beta;
   float *const val[6] = {aw.v1b[0], aw.v1b[1], aw.v1b[2], aw.xb[0], aw.xb[1], aw.xb[2]};
@@ -300,7 +340,7 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_g2p(World w, AdjWork aw) {
     const float ma = aw.sm[rel + a];
     float S[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (ma > 0.f)
-      walk_rows(w, sc, li, lane, ca, val, [&](const float *v, float N, const float *) {
+      walk_rows(w, sc, li, rows[team], t, kAdjTeam, ca, val, [&](const float *v, float N, const float *) {
         const float q = N / ma;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
@@ -311,18 +351,23 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_g2p(World w, AdjWork aw) {
       });
 #pragma unroll
     for (int r = 0; r < 6; ++r) {
-      const float t = warp_sum(S[r]);
-      if (lane == 0) red[wid][a][r] = t;
+      const float y = warp_sum(S[r]);
+      if (lane == 0) red[team][wid][a][r] = y;
     }
   }
-  if (lane != 0) return;
+  __syncthreads();
+  if (t != 0) return;
   uint2 codes[BM_MAXS];
   float m[BM_MAXS], S[BM_MAXS][6];
   for (int a = 0; a < ns; ++a) {
     codes[a] = w.S.code[off + a];
     m[a] = aw.sm[rel + a];
 #pragma unroll
-    for (int r = 0; r < 6; ++r) S[a][r] = red[wid][a][r];
+    for (int r = 0; r < 6; ++r) {
+      S[a][r] = 0.f;
+#pragma unroll
+      for (int k = 0; k < kAdjWarps; ++k) S[a][r] += red[team][k][a][r];
+    }
   }
   couple_T<6>(ns, codes, m, S);
   for (int a = 0; a < ns; ++a)
@@ -755,7 +800,7 @@ cudaError_t bm_launch_adjoint_substep(const World &w, const void *work, const do
   aw.fbar[1] = fbar[1];
   aw.fbar[2] = fbar[2];
   if (n_p == 0) return cudaSuccess;
-  // per-node kernels: a warp per node; per-particle kernels: a thread per particle
+  // per-node kernels: kAdjTeam threads per node; per-particle kernels: a thread per particle
   const int gn = (n_node + kAdjNodesPerBlock - 1) / kAdjNodesPerBlock, gp = (n_p + kAdjBlock - 1) / kAdjBlock;
   chain_launch(k_adj_musl, dim3((unsigned)gn), kAdjBlock, 0, st, w, aw);
   chain_launch(k_adj_v1, dim3((unsigned)gp), kAdjBlock, 0, st, w, aw);

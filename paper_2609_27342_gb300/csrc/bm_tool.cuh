@@ -198,10 +198,7 @@ __device__ __forceinline__ void tool_step(const World &w, DevScene &sc, ToolTmp 
 // reads this substep's frame, so the result goes to the scene's record in
 // scenes_next and commit_tool takes it over when the particles are done.  As a
 // kernel of its own after k_fupd it was 9.2 us of a 16,000-particle scene's 98 us
-// substep and 16 of the 256-scene batch's 1,460.  It takes about as long as
-// G2P in a small scene, whose k_musl_node is shorter (4 us without it), so the
-// wide forms of G2P run it; a large set's node tiles and bricks outlast it and
-// hold less of an SM in k_musl_node.
+// substep and 16 of the 256-scene batch's 1,460.
 struct ToolS {
   DevScene sc;
   ToolTmp T;
@@ -288,9 +285,11 @@ __device__ __forceinline__ void commit_tool(const World &w, int sid) {
 }
 
 // Leading CTAs of G2P that take the scenes' tool steps; 0: k_musl_node does.
-#ifndef G2P_TOOLS
-#define G2P_TOOLS 152
-#endif
+// A tool step takes about as long as G2P in a small scene and longer than its
+// k_musl_node (6 us); a 477,000-particle scene's k_musl_node is 18 us with it, 14
+// without.  For the 256-scene batch the two places measure the same (1,447 and
+// 1,449 us a substep), and there k_musl_node's CTAs hold less of an SM.
+constexpr int G2P_TOOLS = 152;
 inline int g2p_tools(const LaunchSet &ls) { return ls.n_scenes <= G2P_TOOLS ? ls.n_scenes : 0; }
 
 }  // namespace
