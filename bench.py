@@ -63,23 +63,22 @@ KERNEL_MODEL = {
     "k_musl_node": {"bytes": (0, 12, 86, 0), "flops": (0, 0, 20, 0)},
     "k_fupd": {"bytes": (97, 0, 54, 1080), "flops": (650, 0, 0, 0)},
 }
-# the substep's small kernels (bytes only): the tool step reads the bricks'
-# wrench partials (48 B per brick); the slot rebuild reads each node's dirty
+# the substep's small kernels (bytes only; the tool step and the sums over a
+# scene run as extra CTAs of these and of k_musl_node or k_g2p_musl, some 56 B
+# per brick): the slot rebuild reads each node's dirty
 # flag and code count and writes its slot count (3 B per node), writes each
 # brick's tile descriptors (4 B per tile node) and partial-sum range, and,
 # per node, the slot offset and the first-slot entries of the <= 8 covering
 # bricks (36 B) and each slot's code (8 B); the recount of the dirty nodes'
 # codes (the particles of 27 cells each) comes on top
 SMALL_KERNEL_BYTES = {
-    "k_tool": (0, 0, 0, 48),
     "k_slot_count": (0, 3, 0, 0),
     "k_brick_tiles": (0, 0, 0, 4 * 216 + 8),
-    "k_slot_scan": (0, 0, 0, 8),
     "k_slot_fill": (0, 37, 8, 0),
 }
 STEP_ALGORITHMIC_BYTES = 156  # per particle-substep: the state the method must move
 LATE_FIRST = 900              # first substep of the late timing window (of the 1,000-substep rollout)
-LAUNCHES_PER_SUBSTEP = 10     # kernels one batched substep launches (no pair contact)
+LAUNCHES_PER_SUBSTEP = 8      # kernels one batched substep launches (no pair contact)
 
 
 def log(*a):
@@ -157,8 +156,9 @@ def code_hash(text: str) -> str:
 
 
 def kernel_source_hash() -> str:
-    src = os.path.join(ROOT, "paper_2609_27342_gb300", "csrc", "bm_kernels.cu")
-    return code_hash(open(src).read())
+    csrc = os.path.join(ROOT, "paper_2609_27342_gb300", "csrc")
+    return code_hash("\n".join(open(os.path.join(csrc, f)).read() for f in
+                               ("bm_kernels.cu", "bm_lattice.cu", "bm_device.cuh", "bm_tool.cuh")))
 
 
 def ncu_traffic(kernel: str, units: dict):

@@ -12,8 +12,11 @@
 //                re-scatter
 //   k_musl_node  per node: MUSL sums, coupling, v*
 //   k_fupd       F update, commit of the new side labels
-//   k_tool       per scene: wrench, rigid tool step, next frame
-//   k_slot_*     compact logical-grid slots (Sec. III-G) after label changes
+//   k_recount, k_slot_*, k_brick_tiles, k_count_tiles
+//                compact logical-grid slots (Sec. III-G) after label changes
+// The tool step (bm_tool.cuh: wrench, rigid motion, next frame) runs as extra
+// CTAs of G2P or k_musl_node.  The brick kernels here take any scene;
+// bm_lattice.cu has their forms for lattice bodies.
 //   k_pair_*     material-material contact (Eq. 10-13): the rebuild test,
 //                spatial hash and candidate lists, and the pair impulses,
 //                ahead of P2G
