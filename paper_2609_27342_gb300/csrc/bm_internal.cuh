@@ -124,7 +124,7 @@ struct DevScene {
   double accF[3], accT[3];
   int acc_cnt, cur_cut;
   double lastW[6];
-  // frame of the current substep (written by the tool kernel / set-up)
+  // frame of the current substep (committed with the tool step / set-up)
   int cut, reset_D;
   double dxe[3], dn[3], de[3], dd[3], dve[3];
   float fxe[3], fn[3], fe[3], fd[3], fve[3], fc[3], fxB[3], fvB[3], fwB[3];

@@ -1,10 +1,9 @@
 """Brick kernels of sets of few bricks against those of larger sets, bit for bit.
 
 A scene stepped alone takes the forms with several groups of threads per
-brick; in a batch filled up with copies of a larger body it takes the
-one-group forms, and the tool step another kernel's CTAs.  Every sum has the
-same terms in the same order in both, so the scene must come out with the same
-bits.
+brick; in a batch filled up with a larger body it takes the one-group forms
+and the slot rebuild's other launches.  Every sum has the same terms in the
+same order in both, so the scene must come out with the same bits.
 """
 import numpy as np
 import pytest
@@ -65,7 +64,7 @@ def test_few_and_many_bricks_agree_bitwise(pkg, cells, k, jitter, codes, kw):
                  F=(np.eye(3).ravel() + 0.02 * rng.standard_normal((n, 9))).astype(np.float32),
                  mask1=np.where(code % 2 == 1, 1 << cut, 0).astype(np.uint32),
                  mask2=np.where((code % 2 == 0) & (code > 0), 1 << cut, 0).astype(np.uint32))
-    filler = _scene(_lattice((36, 36, 36), (1, 1, 1)), False)   # 729 bricks or more
+    filler = _scene(_lattice((42, 42, 42), (1, 1, 1)), False)   # over 1,000 bricks and 608 node tiles
     got = []
     for many in (False, True):
         s = pkg.Scene(sc)
@@ -75,7 +74,7 @@ def test_few_and_many_bricks_agree_bitwise(pkg, cells, k, jitter, codes, kw):
             fp = [pkg.footprint(q) for q in specs]
             b = pkg.Batch(max_particles=sum(q.n for q in specs), max_nodes=sum(f[1] for f in fp),
                           max_scenes=2, max_bricks=sum(f[2] for f in fp))
-            assert fp[1][2] > 4 * 152
+            assert fp[1][2] > 4 * 152 and fp[1][1] > 4 * 152 * 128
             f = pkg.Scene(filler)
             b.add(f)
             b.add(s)
