@@ -349,7 +349,12 @@ int rebuild_tiles(WorldH *W) {
   return BM_OK;
 }
 
-// brick tiles of one scene inside the world's list (scenes are listed in order)
+// The tile lists for a launch: a member that was destroyed has left them and
+// the members' places in them out of step.
+int current_tiles(WorldH *W) { return W->tiles_dirty ? rebuild_tiles(W) : BM_OK; }
+
+// brick tiles of one scene inside the world's list (scenes are listed in order;
+// the list must be current)
 int scene_btile_begin(const WorldH *W, const bm_scene_s *s) {
   int b = 0;
   for (const bm_scene_s *m : W->members) {
@@ -1106,10 +1111,8 @@ int bm_get_tool_state(bm_scene_t s, int blade_id, double pose[12], double twist[
 int bm_step(bm_scene_t s, int n_substeps) {
   if (!valid_scene(s) || n_substeps < 0) return fail(BM_E_INVALID, "bad scene or step count");
   WorldH *W = s->world;
-  if (W->tiles_dirty) {
-    int r = rebuild_tiles(W);
-    if (r) return r;
-  }
+  int tr = current_tiles(W);
+  if (tr) return tr;
   LaunchSet ls = scene_set(W, s);
   for (int k = 0; k < n_substeps; ++k) CK(bm_launch_substep(W->w, ls, W->st));
   return BM_OK;
@@ -1216,6 +1219,8 @@ int bm_write_state(bm_scene_t s, uint32_t field_mask, const void *const *src, in
                   cudaMemcpyHostToDevice));
   }
   if (masks) {
+    int tr = current_tiles(W);
+    if (tr) return tr;
     CK(bm_launch_rebuild(W->w, scene_set(W, s), W->st, 1));
     CK(cudaStreamSynchronize(W->st));
   }
@@ -1388,6 +1393,8 @@ int bm_checkpoint_restore(bm_scene_t s, const void *src, int src_on_device) {
   if (h.magic != kCkMagic || h.n != s->n || h.hist_cap != s->hist_cap || h.bytes != (int64_t)total ||
       h.pair != (s->desc.pair_contact ? 1 : 0))
     return fail(BM_E_INVALID, "checkpoint does not belong to this scene");
+  int tr = current_tiles(W);  // ahead of set_ranges below: the record's tile range is part of it
+  if (tr) return tr;
   const PPool &P = W->w.P;
   if ((int)secs.size() < kCopyMax && on_world_device(W, src)) {
     CopySet c{};
@@ -1808,10 +1815,8 @@ int bm_batch_step(bm_batch_t b, int n_substeps) {
   if (!b || n_substeps < 0) return fail(BM_E_INVALID, "bad batch or step count");
   WorldH *W = b->world;
   if (W->members.empty() || n_substeps == 0) return BM_OK;
-  if (W->tiles_dirty) {
-    int r = rebuild_tiles(W);
-    if (r) return r;
-  }
+  int tr = current_tiles(W);
+  if (tr) return tr;
   LaunchSet ls = world_set(W);
   auto graph_for = [&](int k, cudaGraphExec_t *out) -> int {
     auto it = W->graphs.find(k);
@@ -1857,10 +1862,8 @@ int bm_batch_profile(bm_batch_t b, int n_substeps, double *ms, int *launches, in
   if (!b || n_substeps <= 0 || !ms || cap < BM_NUM_KERNELS) return fail(BM_E_INVALID, "bad arguments");
   WorldH *W = b->world;
   if (W->members.empty()) return 0;
-  if (W->tiles_dirty) {
-    int r = rebuild_tiles(W);
-    if (r) return r;
-  }
+  int tr = current_tiles(W);
+  if (tr) return tr;
   LaunchSet ls = world_set(W);
   std::vector<cudaEvent_t> ev(2 * BM_NUM_KERNELS);
   for (auto &e : ev) CK(cudaEventCreate(&e));
@@ -1905,10 +1908,8 @@ int bm_batch_set_tool_states(bm_batch_t b, const double *states, int n, int on_d
   if (!b || !states) return fail(BM_E_INVALID, "bad batch or states");
   WorldH *W = b->world;
   if (n != (int)W->members.size()) return fail(BM_E_INVALID, "state count must equal the member count");
-  if (W->tiles_dirty) {
-    int r = rebuild_tiles(W);
-    if (r) return r;
-  }
+  int tr = current_tiles(W);
+  if (tr) return tr;
   const double *src = states;
   if (!on_device) {
     CK(cudaMemcpyAsync(W->d_stage, states, sizeof(double) * 18 * (size_t)n, cudaMemcpyHostToDevice, W->st));
@@ -1922,10 +1923,8 @@ int bm_batch_tool_wrenches(bm_batch_t b, double *out, int n, int on_device) {
   if (!b || !out) return fail(BM_E_INVALID, "bad batch or output");
   WorldH *W = b->world;
   if (n != (int)W->members.size()) return fail(BM_E_INVALID, "output count must equal the member count");
-  if (W->tiles_dirty) {
-    int r = rebuild_tiles(W);
-    if (r) return r;
-  }
+  int tr = current_tiles(W);
+  if (tr) return tr;
   double *dst = on_device ? out : W->d_stage;
   CK(bm_launch_get_wrenches(W->w, W->d_scene_ids, n, dst, W->st));
   if (!on_device) {
