@@ -1247,6 +1247,8 @@ struct CkSection {
   size_t bytes;
 };
 
+constexpr int kCkSectionsMax = 50;  // with pair contact and a wrench history
+
 std::vector<CkSection> ck_layout(const bm_scene_s *s, size_t *total) {
   const PPool &P = s->world->w.P;
   const int64_t n = s->n, pb = s->p_begin;
@@ -1298,7 +1300,7 @@ namespace {
 // 16,000-particle scene took 0.25 ms of host calls and copy start-up for
 // 3 MB.  A section is copied in 16-byte words where both sides are aligned
 // for it (a scene alone in its pools), else in 4-byte words or bytes.
-constexpr int kCopyMax = 64;     // sections per launch (45 with pair contact and a wrench history)
+constexpr int kCopyMax = 64;     // pieces per launch
 constexpr int kCopyBlock = 256;
 struct CopySet {
   char *dst[kCopyMax];
@@ -1356,7 +1358,7 @@ int bm_checkpoint_save(bm_scene_t s, void *dst, int dst_on_device) {
   CkHeader h{kCkMagic, s->n, s->p_begin, s->hist_cap, (int64_t)total, s->desc.pair_contact ? 1 : 0, 0};
   char *d = (char *)dst;
   CK(cudaMemcpyAsync(d, &h, sizeof h, cudaMemcpyDefault, W->st));
-  if ((int)secs.size() < kCopyMax && on_world_device(W, dst)) {
+  if (on_world_device(W, dst)) {
     CopySet c{};
     auto add = [&](void *to, const void *from, size_t bytes) {
       c.dst[c.n] = (char *)to;
@@ -1382,34 +1384,51 @@ int bm_checkpoint_restore(bm_scene_t s, const void *src, int src_on_device) {
   std::vector<CkSection> secs = ck_layout(s, &total);
   CK(cudaStreamSynchronize(W->st));
   const char *d = (const char *)src;
-  struct {
-    CkHeader h;
-    unsigned char gap[256 - sizeof(CkHeader)];
-    DevScene sv;
-  } rec;
-  static_assert(sizeof(CkHeader) < 256 && offsetof(decltype(rec), sv) == 256, "header and record are contiguous");
-  CK(cudaMemcpy(&rec, d, sizeof rec, cudaMemcpyDefault));
-  const CkHeader &h = rec.h;
+  // the header alone: only if it is this scene's does the buffer hold the rest
+  CkHeader h{};
+  CK(cudaMemcpy(&h, d, sizeof h, cudaMemcpyDefault));
   if (h.magic != kCkMagic || h.n != s->n || h.hist_cap != s->hist_cap || h.bytes != (int64_t)total ||
       h.pair != (s->desc.pair_contact ? 1 : 0))
     return fail(BM_E_INVALID, "checkpoint does not belong to this scene");
-  int tr = current_tiles(W);  // ahead of set_ranges below: the record's tile range is part of it
+  int tr = current_tiles(W);
   if (tr) return tr;
   const PPool &P = W->w.P;
-  if ((int)secs.size() < kCopyMax && on_world_device(W, src)) {
-    CopySet c{};
-    auto add = [&](void *to, const void *from, size_t bytes) {
-      c.dst[c.n] = (char *)to;
-      c.src[c.n] = (const char *)from;
-      c.bytes[c.n++] = (long long)bytes;
-    };
-    for (const CkSection &q : secs) add(q.pool, d + q.off, q.bytes);
-    add(P.pend + s->p_begin, nullptr, (size_t)s->n);
+  // The stop substep is a control of the caller's, not state: a scene restored
+  // ahead of it runs on.
+  int frozen = 0;
+  if (s->stop_at >= 0) {
+    long long step = 0;
+    CK(cudaMemcpy(&step, d + ck_align(sizeof h) + offsetof(DevScene, step), sizeof step, cudaMemcpyDefault));
+    frozen = step >= s->stop_at ? 1 : 0;
+  }
+  CopySet c{};
+  auto add = [&](void *to, const void *from, size_t bytes) {
+    c.dst[c.n] = (char *)to;
+    c.src[c.n] = (const char *)from;
+    c.bytes[c.n++] = (long long)bytes;
+  };
+  for (const CkSection &q : secs) add(q.pool, d + q.off, q.bytes);
+  add(P.pend + s->p_begin, nullptr, (size_t)s->n);
+  // The scene's record but for what belongs to its place and its particles'
+  // arrangement and not to its state: the ranges at the record's start, the
+  // stop substep with `frozen`, and `lattice` at its end.
+  char *rec = (char *)(W->w.scenes + s->slot);
+  auto add_record = [&](size_t from, size_t to) { add(rec + from, d + ck_align(sizeof h) + from, to - from); };
+  static_assert(offsetof(DevScene, nb) == 16 * sizeof(int), "the ranges of set_ranges and the scene's counts come first");
+  add_record(offsetof(DevScene, nb), offsetof(DevScene, stop_at));
+  add(rec + offsetof(DevScene, frozen), nullptr, sizeof(int));
+  add_record(offsetof(DevScene, err), offsetof(DevScene, label_pending));
+  add(rec + offsetof(DevScene, label_pending), nullptr, sizeof(int));
+  static_assert(kCkSectionsMax + 5 <= kCopyMax, "a restore is one launch");
+  if (on_world_device(W, src)) {
     CK(launch_copies(c, W->st));
   } else {
-    for (const CkSection &c : secs) CK(cudaMemcpyAsync(c.pool, d + c.off, c.bytes, cudaMemcpyDefault, W->st));
-    CK(cudaMemsetAsync(P.pend + s->p_begin, 0, s->n, W->st));
+    for (int i = 0; i < c.n; ++i)
+      CK(c.src[i] ? cudaMemcpyAsync(c.dst[i], c.src[i], c.bytes[i], cudaMemcpyDefault, W->st)
+                  : cudaMemsetAsync(c.dst[i], 0, c.bytes[i], W->st));
   }
+  if (frozen)
+    CK(cudaMemcpyAsync(rec + offsetof(DevScene, frozen), &frozen, sizeof frozen, cudaMemcpyHostToDevice, W->st));
   // pair-history partners and contact candidates are pool indices of the
   // world the save was made in
   if (s->desc.pair_contact && h.p_begin != s->p_begin) {
@@ -1428,14 +1447,6 @@ int bm_checkpoint_restore(bm_scene_t s, const void *src, int src_on_device) {
     for (auto &v : nb) v = rebase_candidate(v, (int)h.p_begin, (int)s->p_begin);
     CK(cudaMemcpy(np, nb.data(), sizeof(int) * nb.size(), cudaMemcpyHostToDevice));
   }
-  DevScene &sv = rec.sv;
-  set_ranges(s, sv);
-  sv.slot_cap = (int)s->slot_cap;
-  sv.label_pending = 0;
-  sv.lattice = s->lattice;     // decided by the scene's positions, not by the saved record
-  sv.stop_at = s->stop_at;     // the stop substep is a control of the caller's, not state
-  sv.frozen = (sv.stop_at >= 0 && sv.step >= sv.stop_at) ? 1 : 0;
-  CK(cudaMemcpyAsync(W->w.scenes + s->slot, &sv, sizeof sv, cudaMemcpyHostToDevice, W->st));
   CK(bm_launch_rebuild(W->w, scene_set(W, s), W->st, 1));
   CK(cudaStreamSynchronize(W->st));
   return BM_OK;
