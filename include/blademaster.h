@@ -422,7 +422,9 @@ int bm_surface_create(bm_scene_t s, const int lattice[3], bm_surface_t *out);
 /* Rebuild the topology from the scene's current side codes (rebuild != 0)
  * and re-embed every vertex in the current motion field; returns the vertex
  * and triangle counts.  Enqueued on the scene's stream; synchronises to
- * return the counts. */
+ * return the counts.  Without memory for the arrays it returns BM_E_OOM and the
+ * counts of what the surface still holds: the last update's, or none, and then
+ * the next call rebuilds whatever `rebuild` is. */
 int bm_surface_update(bm_surface_t f, int rebuild, int64_t *n_vertices, int64_t *n_triangles);
 /* Copy the last update's output: vertices [n_vertices][3] current
  * positions, reference [n_vertices][3] reference positions, triangles

@@ -1986,6 +1986,7 @@ struct bm_surface_s {
   void *pack = nullptr;                // in vbuf: records on their way to the host
   int64_t vcap = 0, tcap = 0;
   int64_t nv = 0, nt = 0;
+  bool built = false;                  // the arrays hold nv vertices and nt triangles
   void release_all(cudaStream_t st) {
     if (st) cudaStreamSynchronize(st);
     for (void *p : fixed) al.release(p);
@@ -2008,7 +2009,8 @@ T *surf_get(bm_surface_s *f, int64_t count) {
 
 // vertex arrays: ref[3], cur[3] floats, anchor int, masks 2 x uint32, cell
 // int, 3 words to pack records in for a host read (13 words per vertex), and
-// the cell ordinal (a byte)
+// the cell ordinal (a byte).  What a replaced array held is gone, whatever
+// comes of the update that replaced it.
 int surf_grow_vertices(bm_surface_s *f, int64_t nv) {
   if (nv <= f->vcap) return BM_OK;
   int64_t cap = std::max<int64_t>(nv + nv / 4, 1024);
@@ -2017,6 +2019,8 @@ int surf_grow_vertices(bm_surface_s *f, int64_t nv) {
   f->al.release(f->vbuf);
   f->vbuf = b;
   f->vcap = cap;
+  f->nv = f->nt = 0;
+  f->built = false;
   float *fb = (float *)b;
   for (int a = 0; a < 3; ++a) {
     f->sp.ref[a] = fb + (size_t)a * cap;
@@ -2039,6 +2043,8 @@ int surf_grow_tris(bm_surface_s *f, int64_t nt) {
   f->al.release(f->tbuf);
   f->tbuf = b;
   f->tcap = cap;
+  f->nv = f->nt = 0;
+  f->built = false;
   f->sp.tri = (int *)b;
   return BM_OK;
 }
@@ -2180,17 +2186,22 @@ int bm_surface_update(bm_surface_t f, int rebuild, int64_t *n_vertices, int64_t 
   sp.p_begin = (int)s->p_begin;  // the scene may have moved between worlds
   sp.slot = s->slot;
   cudaStream_t st = W->st;
-  if (rebuild || f->vbuf == nullptr) {
+  if (rebuild || !f->built) {
     CK(bm_launch_surface_count(W->w, sp, st));
     int tot[2] = {0, 0};  // vertices, triangles
     CK(cudaMemcpyAsync(tot, sp.totals, sizeof tot, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     int rc = surf_grow_vertices(f, tot[0]);
     if (!rc) rc = surf_grow_tris(f, tot[1]);
-    if (rc) return rc;
+    if (rc) {  // the counts are of what can still be read
+      if (n_vertices) *n_vertices = f->nv;
+      if (n_triangles) *n_triangles = f->nt;
+      return rc;
+    }
     CK(bm_launch_surface_write(W->w, sp, tot[0], (int)s->n_node, st));
     f->nv = tot[0];
     f->nt = tot[1];
+    f->built = true;
   }
   CK(bm_launch_surface_embed(W->w, sp, (int)f->nv, (int)s->n_node, st));
   CK(cudaStreamSynchronize(st));

@@ -35,8 +35,9 @@ class Surface:
         """Rebuild the topology from the current codes (``rebuild``) and
         re-embed the vertices in the current motion field."""
         nv, nt = C.c_int64(), C.c_int64()
-        A.check(self._L.bm_surface_update(self._h, int(bool(rebuild)), C.byref(nv), C.byref(nt)))
-        self.n_vertices, self.n_triangles = nv.value, nt.value
+        rc = self._L.bm_surface_update(self._h, int(bool(rebuild)), C.byref(nv), C.byref(nt))
+        self.n_vertices, self.n_triangles = nv.value, nt.value  # of what is left, where it failed
+        A.check(rc)
         return self.n_vertices, self.n_triangles
 
     def read(self) -> Dict[str, np.ndarray]:
