@@ -479,14 +479,11 @@ __device__ __forceinline__ int pic(int j, int c) { return j * BR3 + (c ^ ((j & 7
 // of latencies.  Their CTAs have several groups of threads (WIDE of BT in the
 // P2G and the general kernels): the particles take a third or less of the
 // rounds, and the scatter's sums go side by side, momentum and force as well
-// as the codes, each by one thread in the narrow form's order.  Substep of one
-// cut scene, us, narrow -> wide:
-//   lattice  80 bricks 77 -> 66, 210: 81 -> 74, 336: 86 -> 84, 432: 89 -> 96
-//   jittered 80 bricks 180 -> 115, 336: 197 -> 130, 630: 199 -> 179
-//   16/cell  80 bricks 176 -> 100, 336: 187 -> 127, 630: 216 -> 200
+// as the codes, each by one thread in the narrow form's order.
 #define WIDE 4
+// Lattice forms: substep of one cut scene, us, narrow -> wide: 80 bricks
+// 77 -> 66, 210: 81 -> 74, 336: 86 -> 84, 432: 89 -> 96.
 #define WIDE_BRICKS_LAT (2 * 152)
-#define WIDE_BRICKS (4 * 152)
 
 __device__ __forceinline__ void node_coords(const DevScene &sc, int li, int &ix, int &iy, int &iz) {
   ix = li % sc.nn[0];

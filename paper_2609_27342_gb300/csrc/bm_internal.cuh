@@ -240,7 +240,7 @@ struct LaunchSet {
   int any_pair;             // some scene has pair contact
   int any_inelastic;        // some scene has plasticity or viscosity
   int any_lattice, any_general;  // some scene takes the lattice kernels; some the general ones
-  int pair_n_particles;     // particles of pair-contact scenes (hash sizing)
+  int gen_bricks, gen_particles;  // of the scenes that take the general kernels
 };
 
 // surface reconstruction (bm_surface.cu, Sec. III-F) over a scene's sub-cell

@@ -2094,10 +2094,33 @@ static void launch_fupd(const World &w, const LaunchSet &ls, cudaStream_t st) {
   else chain_launch(k_fupd<MB, false, G>, dim3(ls.n_btiles), BT * G, 0, st, w, ls);
 }
 
+// Whether the general kernels take their wide form (WIDE).  One wide CTA fills
+// an SM, so its time is that of the waves of 152 bricks, some 20 us a substep
+// each, hardly depending on a brick's particles; the narrow form holds 600
+// bricks at once and takes a round for every 192 particles of a brick.  So a set
+// of sparse bricks goes over to the narrow form earlier.  Substep, us, narrow /
+// wide, bodies mid-cut of b bricks with p particles in a brick:
+//   p  33: b 125  61 /  53, 175  60 /  61, 245  62 /  69
+//   p 150: b 175  87 /  65, 245  86 /  75, 343  89 /  87, 392  92 /  93
+//   p 320: b 245  98 /  75, 343 102 /  88, 512 109 / 109, 648 112 / 127
+//   p 650: b 245 154 /  96, 392 165 / 124, 576 182 / 159, 729 203 / 194
+// and sets of one-brick scenes, every brick cut:
+//   p  64: b 100  73 /  71, 200  84 / 104, 600 122 / 201
+//   p 216: b 100  88 /  72, 200 107 / 114, 300 113 / 122
+//   p 512: b 200 122 / 115, 300 130 / 124, 400 147 / 164
+// The kernels' CTAs of the set's lattice bricks leave at once, but a wide one
+// holds the SM meanwhile: jittered scenes of 54 bricks beside lattice scenes, one
+// of 648 bricks 171 / 132, 3,456 410 / 394, 13,554 1,208 / 1,338, four of 1,080
+// 213 / 199, 3,456 411 / 414.
+static bool wide_general(const LaunchSet &ls) {
+  const int waves = 1 + ls.gen_particles / ls.gen_bricks / 128;
+  return ls.gen_bricks <= 152 * (waves < 4 ? waves : 4) && ls.n_btiles <= 8 * 152;
+}
+
 template <int PPC>
 static void launch_p2g_general(const World &w, const LaunchSet &ls, cudaStream_t st) {
   const int c = ls.variant % 3;
-  if (ls.n_btiles <= WIDE_BRICKS) {
+  if (wide_general(ls)) {
     if (ls.any_inelastic) launch_p2g_inelastic<PPC, 1, WIDE>(w, ls, st);
     else launch_p2g<PPC, 1, WIDE>(w, ls, st);
   } else if (c == 0) launch_p2g<PPC, 0>(w, ls, st);
@@ -2108,7 +2131,7 @@ static void launch_p2g_general(const World &w, const LaunchSet &ls, cudaStream_t
 template <int PPC>
 static void launch_g2p_general(const World &w, const LaunchSet &ls, cudaStream_t st) {
   const int c = (ls.variant / 3) % 3;
-  if (ls.n_btiles <= WIDE_BRICKS) launch_g2p<PPC, 1, WIDE>(w, ls, st);
+  if (wide_general(ls)) launch_g2p<PPC, 1, WIDE>(w, ls, st);
   else if (c == 0) launch_g2p<PPC, OccG2P<0>::v, 1>(w, ls, st);
   else if (c == 1) launch_g2p<PPC, OccG2P<1>::v, 1>(w, ls, st);
   else launch_g2p<PPC, OccG2P<2>::v, 1>(w, ls, st);
@@ -2116,7 +2139,7 @@ static void launch_g2p_general(const World &w, const LaunchSet &ls, cudaStream_t
 
 static void launch_fupd_general(const World &w, const LaunchSet &ls, cudaStream_t st) {
   const int c = ls.variant / 9;
-  if (ls.n_btiles <= WIDE_BRICKS) launch_fupd<1, WIDE>(w, ls, st);
+  if (wide_general(ls)) launch_fupd<1, WIDE>(w, ls, st);
   else if (c == 0) launch_fupd<OccFupd<0>::v, 1>(w, ls, st);
   else if (c == 1) launch_fupd<OccFupd<1>::v, 1>(w, ls, st);
   else launch_fupd<OccFupd<2>::v, 1>(w, ls, st);

@@ -423,6 +423,8 @@ LaunchSet scene_set(const WorldH *W, const bm_scene_s *s) {
   ls.any_inelastic = s->desc.yield_stress > 0 || s->desc.viscosity > 0;
   ls.any_lattice = s->lattice;
   ls.any_general = !s->lattice;
+  ls.gen_bricks = (int)s->n_brick;
+  ls.gen_particles = (int)s->n;
   return ls;
 }
 
@@ -442,6 +444,10 @@ LaunchSet world_set(const WorldH *W) {
     ls.ppc16 |= !s->lattice && s->ppc_max > 8;
     ls.any_lattice |= s->lattice;
     ls.any_general |= !s->lattice;
+    if (!s->lattice) {
+      ls.gen_bricks += (int)s->n_brick;
+      ls.gen_particles += (int)s->n;
+    }
   }
   return ls;
 }
