@@ -815,11 +815,21 @@ __device__ __forceinline__ void brick_wrench(const World &w, int brick, const fl
 }
 
 // --------------------------------------------------------------------------
-// One component of A grad N + N J = wx (A1 dyz + A2 wyd + J wyz) + dwx (A0 wyz)
-// in P2G, with the rounding of every operation spelled out, so that the
-// general and the lattice kernels agree bit for bit however the compiler
-// would contract the expression.
+// Terms of the transfer sums, with the rounding of every operation spelled
+// out: left to the compiler, a product and a sum are contracted in one
+// instantiation of a kernel (a launch bound, a particle count, general or
+// lattice) and not in another, and the forms of a kernel must agree bit for bit.
 // --------------------------------------------------------------------------
+// weight N = wx (wy wz) and a sum's next term
+__device__ __forceinline__ float weight(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_term(float sum, float N, float v) { return __fmaf_rn(N, v, sum); }
+// Eq. 17: v' = beta (v - v_old) + v_new, x' = x + dt v_new
+__device__ __forceinline__ float next_v(float beta, float v, float so, float sn) {
+  return __fmaf_rn(beta, __fsub_rn(v, so), sn);
+}
+__device__ __forceinline__ float next_x(float x, float dt, float sn) { return __fmaf_rn(dt, sn, x); }
+// One component of A grad N + N J = wx (A1 dyz + A2 wyd + J wyz) + dwx (A0 wyz)
+// in P2G
 __device__ __forceinline__ float force_u(float A1, float dyz, float A2, float wyd, float J, float wyz) {
   return __fmaf_rn(J, wyz, __fmaf_rn(A1, dyz, __fmul_rn(A2, wyd)));
 }

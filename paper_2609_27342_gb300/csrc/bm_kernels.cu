@@ -195,16 +195,16 @@ __global__ void __launch_bounds__(BT * G, MB) k_p2g_brick(World w, LaunchSet ls)
           const float v0 = S.part[3][si], v1 = S.part[4][si], v2 = S.part[5][si];
 #pragma unroll
           for (int oy = 0; oy < 3; ++oy) {
-            const float wyz = wy[oy] * wz;
-            const float M0 = v0 * wyz, M1 = v1 * wyz, M2 = v2 * wyz;
+            const float wyz = weight(wy[oy], wz);
+            const float M0 = weight(v0, wyz), M1 = weight(v1, wyz), M2 = weight(v2, wyz);
 #pragma unroll
             for (int ox = 0; ox < 3; ++ox) {
               float *q = a[oy][ox];
               const float wxx = wx[ox];
-              q[0] += wxx * wyz;
-              q[1] += wxx * M0;
-              q[2] += wxx * M1;
-              q[3] += wxx * M2;
+              q[0] = add_term(q[0], wxx, wyz);
+              q[1] = add_term(q[1], wxx, M0);
+              q[2] = add_term(q[2], wxx, M1);
+              q[3] = add_term(q[3], wxx, M2);
             }
           }
         }
@@ -582,18 +582,18 @@ __global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls, 
       for (int oz = 0; oz < 3; ++oz)
 #pragma unroll
         for (int oy = 0; oy < 3; ++oy) {
-          const float wyz = wy[oy] * wz[oz];
+          const float wyz = weight(wy[oy], wz[oz]);
 #pragma unroll
           for (int ox = 0; ox < 3; ++ox) {
             const int t = t0 + (oz * TE + oy) * TE + ox;
             const float4 vo = S.tvo[t], vn = S.tvn[t];
-            const float N = wx[ox] * wyz;
-            sn[0] += N * vn.x;
-            sn[1] += N * vn.y;
-            sn[2] += N * vn.z;
-            so[0] += N * vo.x;
-            so[1] += N * vo.y;
-            so[2] += N * vo.z;
+            const float N = weight(wx[ox], wyz);
+            sn[0] = add_term(sn[0], N, vn.x);
+            sn[1] = add_term(sn[1], N, vn.y);
+            sn[2] = add_term(sn[2], N, vn.z);
+            so[0] = add_term(so[0], N, vo.x);
+            so[1] = add_term(so[1], N, vo.y);
+            so[2] = add_term(so[2], N, vo.z);
           }
         }
     } else if (in_smem) {
@@ -604,19 +604,19 @@ __global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls, 
       for (int oz = 0; oz < 3; ++oz)
 #pragma unroll
         for (int oy = 0; oy < 3; ++oy) {
-          const float wyz = wy[oy] * wz[oz];
+          const float wyz = weight(wy[oy], wz[oz]);
 #pragma unroll
           for (int ox = 0; ox < 3; ++ox) {
             const int s = tile_slot(w, S.T, B.nbc, t0 + (oz * TE + oy) * TE + ox, id);
             const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
             const float4 vo = s >= 0 ? S.tvo[s] : zero, vn = s >= 0 ? S.tvn[s] : zero;
-            const float N = vo.w > 0.f ? wx[ox] * wyz : 0.f;
-            sn[0] += N * vn.x;
-            sn[1] += N * vn.y;
-            sn[2] += N * vn.z;
-            so[0] += N * vo.x;
-            so[1] += N * vo.y;
-            so[2] += N * vo.z;
+            const float N = vo.w > 0.f ? weight(wx[ox], wyz) : 0.f;
+            sn[0] = add_term(sn[0], N, vn.x);
+            sn[1] = add_term(sn[1], N, vn.y);
+            sn[2] = add_term(sn[2], N, vn.z);
+            so[0] = add_term(so[0], N, vo.x);
+            so[1] = add_term(so[1], N, vo.y);
+            so[2] = add_term(so[2], N, vo.z);
           }
         }
     } else
@@ -636,18 +636,18 @@ __global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls, 
             vn = w.S.vnew[g];
           }
           if (!(vo.w > 0.f)) continue;
-          const float N = wx[ox] * wy[oy] * wz[oz];
-          sn[0] += N * vn.x;
-          sn[1] += N * vn.y;
-          sn[2] += N * vn.z;
-          so[0] += N * vo.x;
-          so[1] += N * vo.y;
-          so[2] += N * vo.z;
+          const float N = weight(weight(wx[ox], wy[oy]), wz[oz]);
+          sn[0] = add_term(sn[0], N, vn.x);
+          sn[1] = add_term(sn[1], N, vn.y);
+          sn[2] = add_term(sn[2], N, vn.z);
+          so[0] = add_term(so[0], N, vo.x);
+          so[1] = add_term(so[1], N, vo.y);
+          so[2] = add_term(so[2], N, vo.z);
         }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const float vv = beta * (P.v[a][p] - so[a]) + sn[a];
-      const float xx = P.x[a][p] + dt * sn[a];
+      const float vv = next_v(beta, P.v[a][p], so[a], sn[a]);
+      const float xx = next_x(P.x[a][p], dt, sn[a]);
       P.v[a][p] = vv;
       P.x[a][p] = xx;
       S.pv[a][si] = vv;
@@ -691,13 +691,13 @@ __global__ void __launch_bounds__(BT * G, MB) k_g2p_musl(World w, LaunchSet ls, 
         const float v0 = S.pv[0][si], v1 = S.pv[1][si], v2 = S.pv[2][si];
 #pragma unroll
         for (int oy = 0; oy < 3; ++oy) {
-          const float wyz = wy[oy] * wz;
+          const float wyz = weight(wy[oy], wz);
 #pragma unroll
           for (int ox = 0; ox < 3; ++ox) {
-            const float N = wx[ox] * wyz;
-            a[oy][ox][0] += N * v0;
-            a[oy][ox][1] += N * v1;
-            a[oy][ox][2] += N * v2;
+            const float N = weight(wx[ox], wyz);
+            a[oy][ox][0] = add_term(a[oy][ox][0], N, v0);
+            a[oy][ox][1] = add_term(a[oy][ox][1], N, v1);
+            a[oy][ox][2] = add_term(a[oy][ox][2], N, v2);
           }
         }
       }

@@ -542,8 +542,8 @@ __global__ void __launch_bounds__(GT * G, MB) k_g2p_lat(World w, LaunchSet ls, i
         unpack2(acc[j][2], sn[1], sn[2]);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          vv[a] = beta * (v0[j][a] - so[a]) + sn[a];
-          const float xx = x0[j][a] + dt * sn[a];
+          vv[a] = next_v(beta, v0[j][a], so[a], sn[a]);
+          const float xx = next_x(x0[j][a], dt, sn[a]);
           P.v[a][pi[j]] = vv[a];
           P.x[a][pi[j]] = xx;
           bad |= !isfinite(vv[a]) || !isfinite(xx);

@@ -2,7 +2,8 @@
 
 Sparse sets: many one-brick scenes of few particles take the one-group forms at
 a brick count where fuller ones take several groups; each scene must come out
-as on its own, where it takes several.
+as on its own, where it takes several.  Occupancy variants: a set with a larger
+body runs the one-group forms at the variant's resident CTAs.
 """
 import numpy as np
 import pytest
@@ -69,4 +70,47 @@ def test_sparse_set_equals_the_scenes_alone_bitwise(pkg):
         s.close()
     for s in ss:
         s.close()
+    b.close()
+
+
+# 12 codes: more than the slot tables hold, and tiles beyond the slot window
+@pytest.mark.parametrize("cells,per_axis,codes,kw", [
+    ((9, 5, 6), (2, 2, 2), 1, {}), ((7, 5, 3), (4, 2, 2), 1, dict(jitter=0.0)),
+    ((9, 5, 6), (2, 2, 2), 1, dict(yield_stress=2e3, viscosity=5.0)),
+    ((7, 5, 3), (4, 2, 2), 1, dict(yield_stress=2e3, viscosity=5.0)),
+    ((4, 4, 4), (2, 2, 2), 12, dict(blade=False)), ((4, 4, 4), (4, 2, 2), 12, dict(blade=False)),
+])
+def test_occupancy_variants_agree_bitwise(pkg, cells, per_axis, codes, kw):
+    sc = _scene(cells, per_axis, **kw)
+    filler = _scene((42, 42, 42), (1, 1, 1), blade=False)
+    b, n, bricks = _batch(pkg, [sc, filler])
+    assert bricks > 4 * 152
+    s, f = pkg.Scene.in_batch(b, sc), pkg.Scene.in_batch(b, filler)
+    q = np.floor(sc.X / DX).astype(int)
+    code = (q[:, 0] % 4 + 4 * (q[:, 1] % 3)) * (codes > 1)    # columns of cells; 0: none, odd / even: side 1 / 2 of a cut
+    bit = 1 << (1 + (code + 1) // 2)
+    s.write(mask1=np.where(code % 2 == 1, bit, 0).astype(np.uint32),
+            mask2=np.where((code % 2 == 0) & (code > 0), bit, 0).astype(np.uint32), **_state(s.n, 3))
+    cut = f.spec.X[:, 0] < f.spec.X[:, 0].mean()     # several codes in some of its bricks
+    f.write(mask1=np.where(cut, 2, 0).astype(np.uint32), mask2=np.where(cut, 0, 2).astype(np.uint32), **_state(f.n, 4))
+    ck = s.checkpoint(), f.checkpoint()
+    want = None
+    # default, one other choice of each kernel, and the two others of all three
+    for variant in (0, 1, 2, 3, 6, 9, 18, 13, 26):
+        s.restore(ck[0])
+        f.restore(ck[1])
+        b.set_tiles(4, 128, variant)
+        b.step(8)
+        got = [g.read(*FIELDS) for g in (s, f)] + [s.tool_wrench() if codes == 1 else 0,
+                                                   s.info().error_bits, f.info().error_bits]
+        assert got[3] == 0 and got[4] == 0
+        if want is None:
+            want = got
+            assert codes > 1 or (np.any(want[2] != 0) and np.any(want[0]["mask1"] | want[0]["mask2"]))
+        for i in (0, 1):
+            for k in FIELDS:
+                assert np.array_equal(got[i][k], want[i][k]), (variant, i, k)
+        assert np.array_equal(got[2], want[2]), variant
+    s.close()
+    f.close()
     b.close()
