@@ -1385,14 +1385,20 @@ cudaError_t launch_copies(const CopySet &c, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// whether p is memory of the world's device, to which a kernel may copy
-bool on_world_device(const WorldH *W, const void *p) {
-  cudaPointerAttributes at{};
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+// Whether [p, p + bytes) is memory of the world's device, by both of its ends,
+// so that a kernel may copy it; other buffers are left to cudaMemcpy, which
+// also refuses what it cannot copy.
+bool on_world_device(const WorldH *W, const void *p, size_t bytes) {
+  const char *ends[2] = {(const char *)p, (const char *)p + (bytes ? bytes - 1 : 0)};
+  for (const char *q : ends) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, q) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != W->device) return false;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == W->device;
+  return true;
 }
 }  // namespace
 }
@@ -1406,7 +1412,7 @@ int bm_checkpoint_save(bm_scene_t s, void *dst, int dst_on_device) {
   CkHeader h{kCkMagic, s->n, s->p_begin, s->hist_cap, (int64_t)total, s->desc.pair_contact ? 1 : 0, 0};
   char *d = (char *)dst;
   CK(cudaMemcpyAsync(d, &h, sizeof h, cudaMemcpyDefault, W->st));
-  if (on_world_device(W, dst)) {
+  if (on_world_device(W, dst, total)) {
     CopySet c{};
     auto add = [&](void *to, const void *from, size_t bytes) {
       c.dst[c.n] = (char *)to;
@@ -1468,7 +1474,7 @@ int bm_checkpoint_restore(bm_scene_t s, const void *src, int src_on_device) {
   add_record(offsetof(DevScene, err), offsetof(DevScene, label_pending));
   add(rec + offsetof(DevScene, label_pending), nullptr, sizeof(int));
   static_assert(kCkSectionsMax + 5 <= kCopyMax, "a restore is one launch");
-  if (on_world_device(W, src)) {
+  if (on_world_device(W, src, total)) {
     CK(launch_copies(c, W->st));
   } else {
     for (int i = 0; i < c.n; ++i)
@@ -2265,11 +2271,13 @@ int bm_surface_read(bm_surface_t f, float *vertices, float *reference, int32_t *
   const size_t nv = (size_t)f->nv, nt = (size_t)f->nt;
   const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   // struct-of-arrays on the device, [n][3] / [n][2] at the ABI: packed by a
-  // kernel, for the host by way of the vertex arrays' spare words (a copy of
-  // 4-byte rows per column took 16 us each)
+  // kernel, straight into device memory, otherwise by way of the vertex arrays'
+  // spare words (a copy of 4-byte rows per column took 16 us each)
   auto records = [&](void *dst, const void *const *cols, int nc) -> cudaError_t {
-    cudaError_t e = bm_launch_surface_pack(cols, nc, (int)nv, dst_on_device ? dst : f->pack, st);
-    if (e == cudaSuccess && !dst_on_device) e = cudaMemcpyAsync(dst, f->pack, sizeof(uint32_t) * nc * nv, kind, st);
+    const size_t bytes = sizeof(uint32_t) * nc * nv;
+    const bool direct = dst_on_device && on_world_device(f->scene->world, dst, bytes);
+    cudaError_t e = bm_launch_surface_pack(cols, nc, (int)nv, direct ? dst : f->pack, st);
+    if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(dst, f->pack, bytes, kind, st);
     return e;
   };
   if (nv && vertices) {

@@ -89,3 +89,61 @@ def test_restore_keeps_place_and_stop_substep(pkg, device):
     s.close()
     other.close()
     b.close()
+
+
+@pytest.mark.parametrize("where", ["device", "device+4", "device+1", "pinned", "managed"])
+def test_any_buffer_holds_a_checkpoint(pkg, where):
+    """Device memory in one launch, by 16-byte words, 4-byte words or bytes as
+    its alignment allows; other memory section by section."""
+    import torch
+    from paper_2609_27342_gb300 import _abi as A
+    sc = bi.single_cut_cuboid(size=(0.04, 0.02, 0.02), edge_z0=0.0201, speed=1.0, n_down=100)
+    s = pkg.Scene(sc)
+    s.step(20)
+    n = s.checkpoint_size()
+    keep = None
+    if where == "managed":
+        rt = C.CDLL("libcudart.so.13")
+        p = C.c_void_p()
+        assert rt.cudaMallocManaged(C.byref(p), C.c_size_t(n), C.c_uint(1)) == 0
+        ptr, on_device = p.value, 1
+    else:
+        off = int(where.partition("+")[2] or 0)
+        keep = torch.empty(n + 256, dtype=torch.uint8, device="cpu", pin_memory=True) if where == "pinned" else \
+            torch.empty(n + 256, dtype=torch.uint8, device="cuda")
+        keep.fill_(0x5a)
+        torch.cuda.synchronize()
+        ptr, on_device = keep.data_ptr() + off, int(keep.is_cuda)
+    L = A.load()
+    A.check(L.bm_checkpoint_save(s.handle, C.c_void_p(ptr), on_device))
+    if keep is not None:    # nothing is written outside the checkpoint
+        assert bool((keep[:off] == 0x5a).all()) and bool((keep[off + n:] == 0x5a).all())
+    s.step(6)
+    want = s.read("x", "v", "F", "D", "ut", "mask1", "mask2")
+    tool = s.tool_state()
+    s.step(3)
+    A.check(L.bm_checkpoint_restore(s.handle, C.c_void_p(ptr), on_device))
+    s.step(6)
+    for k, v in s.read(*want).items():
+        assert np.array_equal(v, want[k]), k
+    assert np.array_equal(s.tool_state(), tool)
+    s.close()
+    if where == "managed":
+        assert rt.cudaFree(p) == 0
+
+
+def test_surface_read_into_device_memory(pkg):
+    import torch
+    from paper_2609_27342_gb300.surface import Surface
+    s = pkg.Scene(bi.Scene(X=bi.lattice_cuboid((0.03, 0.02, 0.02), 5e-3), dx=5e-3))
+    f = Surface(s)
+    nv, nt = f.update()
+    want = f.read()
+    v = torch.zeros(nv + 1, 3, device="cuda")
+    t = torch.zeros(nt, 3, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    f.read_into(v[1:], t)
+    assert np.array_equal(v[1:].cpu().numpy(), want["vertices"]) and bool((v[0] == 0).all())
+    assert np.array_equal(t.cpu().numpy(), want["triangles"])
+    f.close()
+    s.close()
