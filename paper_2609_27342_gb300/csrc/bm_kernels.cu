@@ -1334,31 +1334,124 @@ __global__ void k_pair(World w, LaunchSet ls) {
 }
 
 // --------------------------------------------------------------------------
-// frames outside a substep, a warp per scene: of the scenes as they are, and
-// after a tool state was set
+// tool: rigid interval, frame of the next substep (float64, one thread)
 // --------------------------------------------------------------------------
-#define FRAME_WARPS 4
-__global__ void __launch_bounds__(32 * FRAME_WARPS) k_prepare(World w, LaunchSet ls) {
+__device__ void matvec_rn(const double M[9], const double x[3], double y[3]) {
+  for (int i = 0; i < 3; ++i)
+    y[i] = __dadd_rn(__dadd_rn(__dmul_rn(M[3 * i], x[0]), __dmul_rn(M[3 * i + 1], x[1])),
+                     __dmul_rn(M[3 * i + 2], x[2]));
+}
+
+__device__ void matmul_d(const double A[9], const double B[9], double C[9]) {
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j)
+      C[3 * i + j] = A[3 * i] * B[j] + A[3 * i + 1] * B[3 + j] + A[3 * i + 2] * B[6 + j];
+}
+
+__device__ void world_inv_inertia(const DevScene &sc, double Iw[9]) {
+  double RT[9], tmp[9];
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) RT[3 * i + j] = sc.R[3 * j + i];
+  matmul_d(sc.R, sc.Ib_inv, tmp);
+  matmul_d(tmp, RT, Iw);
+}
+
+// Sets up substep sc.step: prescribed twist, cut, D reset, blade frame.
+__device__ void prepare_substep(DevScene &sc) {
+  if (!sc.has_blade) {
+    sc.cut = -1;
+    sc.reset_D = 0;
+    return;
+  }
+  const DevSeg *sg = seg_at(sc, sc.step);
+  const int cut = sg ? sg->cut_id : -1;
+  const bool dynamic = sc.mass > 0.0;
+  if (!dynamic && sg)
+    for (int i = 0; i < 3; ++i) {
+      sc.vB[i] = sg->v[i];
+      sc.wB[i] = sg->w[i];
+    }
+  sc.cut = cut;
+  sc.reset_D = (cut >= 0 && cut != sc.cur_cut) ? 1 : 0;
+  double t[3];
+  matvec_rn(sc.R, sc.edgeT, t);
+  for (int i = 0; i < 3; ++i) sc.dxe[i] = __dadd_rn(sc.xB[i], t[i]);
+  matvec_rn(sc.R, sc.nT, sc.dn);
+  matvec_rn(sc.R, sc.eT, sc.de);
+  matvec_rn(sc.R, sc.dT, sc.dd);
+  double r[3] = {__dsub_rn(sc.dxe[0], sc.xB[0]), __dsub_rn(sc.dxe[1], sc.xB[1]),
+                 __dsub_rn(sc.dxe[2], sc.xB[2])};
+  double wr[3] = {__dsub_rn(__dmul_rn(sc.wB[1], r[2]), __dmul_rn(sc.wB[2], r[1])),
+                  __dsub_rn(__dmul_rn(sc.wB[2], r[0]), __dmul_rn(sc.wB[0], r[2])),
+                  __dsub_rn(__dmul_rn(sc.wB[0], r[1]), __dmul_rn(sc.wB[1], r[0]))};
+  for (int i = 0; i < 3; ++i) sc.dve[i] = __dadd_rn(sc.vB[i], wr[i]);
+  if (sc.reset_D) {  // a new cut begins: keep its plane for the cut faces
+    for (int i = 0; i < 3; ++i) sc.cutpl[cut][i] = sc.dn[i];
+    sc.cutpl[cut][3] = __dadd_rn(__dadd_rn(__dmul_rn(sc.dn[0], sc.dxe[0]), __dmul_rn(sc.dn[1], sc.dxe[1])),
+                                 __dmul_rn(sc.dn[2], sc.dxe[2]));
+    sc.cutpl_set |= 1u << cut;
+  }
+  for (int i = 0; i < 3; ++i) {
+    sc.fxe[i] = (float)sc.dxe[i];
+    sc.fn[i] = (float)sc.dn[i];
+    sc.fe[i] = (float)sc.de[i];
+    sc.fd[i] = (float)sc.dd[i];
+    sc.fve[i] = (float)sc.dve[i];
+    sc.fc[i] = (float)(sc.dxe[i] - sc.half_height * sc.dd[i]);
+    sc.fxB[i] = (float)sc.xB[i];
+    sc.fvB[i] = (float)sc.vB[i];
+    sc.fwB[i] = (float)sc.wB[i];
+  }
+  sc.fhext[0] = (float)sc.half_thick;
+  sc.fhext[1] = (float)sc.half_len;
+  sc.fhext[2] = (float)sc.half_height;
+  sc.fL = (float)sc.L_d;
+  sc.fmu_s = (float)sc.mu_s;
+  sc.fmu_d = (float)sc.mu_d;
+  if (dynamic) {
+    double Iw[9];
+    world_inv_inertia(sc, Iw);
+    for (int k = 0; k < 9; ++k) sc.fIinv[k] = (float)Iw[k];
+    sc.finv_mass = (float)(1.0 / sc.mass);
+  } else {
+    for (int k = 0; k < 9; ++k) sc.fIinv[k] = 0.f;
+    sc.finv_mass = 0.f;
+  }
+}
+
+__device__ void rot_exp(const double th[3], double Rm[9]) {
+  double a = sqrt(th[0] * th[0] + th[1] * th[1] + th[2] * th[2]);
+  for (int k = 0; k < 9; ++k) Rm[k] = (k % 4 == 0) ? 1.0 : 0.0;
+  if (!(a > 0)) return;
+  double k0 = th[0] / a, k1 = th[1] / a, k2 = th[2] / a;
+  double K[9] = {0, -k2, k1, k2, 0, -k0, -k1, k0, 0};
+  double K2[9];
+  matmul_d(K, K, K2);
+  double sa = sin(a), ca = 1.0 - cos(a);
+  for (int k = 0; k < 9; ++k) Rm[k] += sa * K[k] + ca * K2[k];
+}
+
+__global__ void k_prepare(World w, LaunchSet ls) {
   chain_wait();
-  __shared__ ToolTmp T[FRAME_WARPS];
-  const int wid = threadIdx.x >> 5, idx = blockIdx.x * FRAME_WARPS + wid;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= ls.n_scenes) return;
-  prepare_substep_warp(w.scenes[ls.scene_ids[idx]], T[wid], threadIdx.x & 31);
+  prepare_substep(w.scenes[ls.scene_ids[idx]]);
 }
 
 // tool states {x_B, R, v_B, omega_B} of several scenes, then their frames
-__global__ void __launch_bounds__(32 * FRAME_WARPS) k_set_tools(World w, const int *ids, int n, const double *states) {
+__global__ void k_set_tools(World w, const int *ids, int n, const double *states) {
   chain_wait();
-  __shared__ ToolTmp T[FRAME_WARPS];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, idx = blockIdx.x * FRAME_WARPS + wid;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n) return;
   DevScene &sc = w.scenes[ids[idx]];
-  if (lane < 18) {
-    double *to = lane < 3 ? sc.xB + lane : lane < 12 ? sc.R + (lane - 3) : lane < 15 ? sc.vB + (lane - 12) : sc.wB + (lane - 15);
-    *to = states[(size_t)idx * 18 + lane];
+  const double *q = states + (size_t)idx * 18;
+  for (int k = 0; k < 3; ++k) sc.xB[k] = q[k];
+  for (int k = 0; k < 9; ++k) sc.R[k] = q[3 + k];
+  for (int k = 0; k < 3; ++k) {
+    sc.vB[k] = q[12 + k];
+    sc.wB[k] = q[15 + k];
   }
-  __syncwarp();
-  prepare_substep_warp(sc, T[wid], lane);
+  prepare_substep(sc);
 }
 
 __global__ void k_get_wrenches(World w, const int *ids, int n, double *out) {
@@ -1846,7 +1939,7 @@ __global__ void k_code(World w, int p_begin, int n, int64_t *out) {
 // ----------------------------------------------------------------------------
 cudaError_t bm_launch_prepare(const World &w, const LaunchSet &ls, cudaStream_t st) {
   if (ls.n_scenes == 0) return cudaSuccess;
-  chain_launch(k_prepare, dim3((unsigned)((ls.n_scenes + FRAME_WARPS - 1) / FRAME_WARPS)), 32 * FRAME_WARPS, 0, st, w, ls);
+  chain_launch(k_prepare, dim3((unsigned)((ls.n_scenes + 63) / 64)), 64, 0, st, w, ls);
   return cudaGetLastError();
 }
 
@@ -2166,8 +2259,7 @@ cudaError_t bm_launch_read(const World &w, int scene_slot, int p_begin, int n, u
 cudaError_t bm_launch_set_tools(const World &w, const int *scene_ids, int n, const double *states,
                                 cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  chain_launch(k_set_tools, dim3((unsigned)((n + FRAME_WARPS - 1) / FRAME_WARPS)), 32 * FRAME_WARPS, 0, st, w, scene_ids, n,
-               states);
+  chain_launch(k_set_tools, dim3((unsigned)((n + 63) / 64)), 64, 0, st, w, scene_ids, n, states);
   return cudaGetLastError();
 }
 
