@@ -16,8 +16,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libblademaster.so")
 SOURCES = ["bm_kernels.cu", "bm_lattice.cu", "bm_runtime.cu", "bm_adjoint.cu", "bm_surface.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler",
-         "-ffp-contract=off", "-diag-suppress", "177"]
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off"]
 
 
 def nvcc() -> str:

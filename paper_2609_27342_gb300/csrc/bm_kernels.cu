@@ -1334,7 +1334,11 @@ __global__ void k_pair(World w, LaunchSet ls) {
 }
 
 // --------------------------------------------------------------------------
-// tool: rigid interval, frame of the next substep (float64, one thread)
+// frames outside a substep (float64, a thread per scene): of the scenes as
+// they are, and after a tool state was set.  prepare_substep_warp (bm_tool.cuh)
+// in the same operations, so that setting a tool to the state it is in changes
+// no bit; with the warp form here too, k_musl_node, which carries the tool step,
+// is compiled to a slower kernel (14.5 -> 16.2 us for a 477,000-particle scene).
 // --------------------------------------------------------------------------
 __device__ void matvec_rn(const double M[9], const double x[3], double y[3]) {
   for (int i = 0; i < 3; ++i)
@@ -1417,18 +1421,6 @@ __device__ void prepare_substep(DevScene &sc) {
     for (int k = 0; k < 9; ++k) sc.fIinv[k] = 0.f;
     sc.finv_mass = 0.f;
   }
-}
-
-__device__ void rot_exp(const double th[3], double Rm[9]) {
-  double a = sqrt(th[0] * th[0] + th[1] * th[1] + th[2] * th[2]);
-  for (int k = 0; k < 9; ++k) Rm[k] = (k % 4 == 0) ? 1.0 : 0.0;
-  if (!(a > 0)) return;
-  double k0 = th[0] / a, k1 = th[1] / a, k2 = th[2] / a;
-  double K[9] = {0, -k2, k1, k2, 0, -k0, -k1, k0, 0};
-  double K2[9];
-  matmul_d(K, K, K2);
-  double sa = sin(a), ca = 1.0 - cos(a);
-  for (int k = 0; k < 9; ++k) Rm[k] += sa * K[k] + ca * K2[k];
 }
 
 __global__ void k_prepare(World w, LaunchSet ls) {

@@ -30,9 +30,11 @@ __device__ __forceinline__ double matmul_at(const double A[9], const double B[9]
 }
 
 struct ToolTmp {
-  double Fa[3], Ta[3], th[3], A[9], Iw[9], K[9], K2[9], Rinc[9];
+  double Fa[3], Ta[3], th[3], A[9], Iw[9], K[9], Rinc[9];
 };
 
+// Frame of substep sc.step, by one warp: prescribed twist, cut, D reset, blade axes
+// (prepare_substep in bm_kernels.cu restates it).
 __device__ __forceinline__ void prepare_substep_warp(DevScene &sc, ToolTmp &T, int lane) {
   if (!sc.has_blade) {
     if (lane == 0) {
