@@ -2101,12 +2101,14 @@ static void launch_fupd(const World &w, const LaunchSet &ls, cudaStream_t st) {
 //   p 216: b 100  88 /  72, 200 107 / 114, 300 113 / 122
 //   p 512: b 200 122 / 115, 300 130 / 124, 400 147 / 164
 // The kernels' CTAs of the set's lattice bricks leave at once, but a wide one
-// holds the SM meanwhile: jittered scenes of 54 bricks beside lattice scenes, one
-// of 648 bricks 171 / 132, 3,456 410 / 394, 13,554 1,208 / 1,338, four of 1,080
-// 213 / 199, 3,456 411 / 414.
+// holds the SM meanwhile, so beyond 608 bricks in all two waves are the limit
+// and beyond 1,216 none: b jittered bricks of 16,000-particle scenes among n,
+// narrow / wide: b 54 n 648 171 / 132, n 3,456 410 / 394, n 13,554 1,208 / 1,338;
+// b 216 n 1,080 213 / 199, n 3,456 411 / 414; b 432 n 864 204 / 213.
 static bool wide_general(const LaunchSet &ls) {
+  const int most = ls.n_btiles <= 4 * 152 ? 4 : ls.n_btiles <= 8 * 152 ? 2 : 0;
   const int waves = 1 + ls.gen_particles / ls.gen_bricks / 128;
-  return ls.gen_bricks <= 152 * (waves < 4 ? waves : 4) && ls.n_btiles <= 8 * 152;
+  return ls.gen_bricks <= 152 * (waves < most ? waves : most);
 }
 
 template <int PPC>
