@@ -324,7 +324,8 @@ void carve_pools(WorldH *W) {
   W->d_scene_ids = W->get<int>(W->cap_scenes);
   W->d_slot_ids = W->get<int>(W->cap_scenes);
   W->d_stage = W->get<double>((int64_t)W->cap_scenes * 18);
-  W->io_bytes = std::min<size_t>(sizeof(float) * 9 * (size_t)P, kStageBytes);
+  // the longest field: F, with pair contact the history's displacements
+  W->io_bytes = std::min<size_t>(sizeof(float) * (W->pair ? 3 * BM_HIST : 9) * (size_t)P, kStageBytes);
   W->io = W->get<char>((int64_t)W->io_bytes);
 }
 

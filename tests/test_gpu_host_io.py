@@ -29,9 +29,9 @@ def _scene(cells, **kw):
 
 
 # one cell; F at the 4 MiB staging buffer's end and beyond it (36 B a particle);
-# the pair history, longer than the buffer of a small scene
+# the pair history (192 B a particle) within it and beyond
 @pytest.mark.parametrize("cells,kw", [((1, 1, 1), {}), ((48, 16, 18), {}), ((48, 16, 19), {}), ((48, 16, 20), {}),
-                                      ((4, 4, 4), dict(pair_contact=True))])
+                                      ((4, 4, 4), dict(pair_contact=True)), ((14, 14, 16), dict(pair_contact=True))])
 def test_host_and_device_io_agree(pkg, cells, kw):
     import torch
     sc = _scene(cells, **kw)
