@@ -46,23 +46,32 @@ SMS = 152
 FP32_LANES = 128
 FALLBACK_HBM_GBS = 6800.0
 
-# Per-kernel compulsory traffic (bytes) and FP32 work (flop, FMA = 2) per
-# particle, per node, per occupied slot and per 4x4x4-cell brick: the reads
-# and writes of each kernel's own inputs and outputs, with brick-tile
-# partials counted at 3.375 tiles per slot (6^3 tile nodes per 4^3 cells).
+# Per-kernel compulsory traffic (bytes) and FP32 work (flop: add, multiply,
+# divide, root, log 1, FMA 2; comparisons 0) per particle, per node, per
+# occupied slot and per 4x4x4-cell brick: the reads and writes of each kernel's
+# own inputs and outputs, with brick-tile partials counted at 3.375 tiles per
+# slot (6^3 tile nodes per 4^3 cells).  The batch's bodies are lattices: the
+# brick kernels' rows are those of their lattice forms (k_p2g_lat, k_g2p_lat,
+# k_fupd_lat), which read a particle's place (2 B) and the brick's 24 plane
+# offsets instead of the particle's offset and masks and form no weights.
 KERNEL_MODEL = {
     # contact, labels and stress are computed in the P2G brick kernel's
-    # staging phase: it reads x, v, F, masks, the fractional offset and the
-    # D/u_t flag (81 B) and writes the pending label; D and u_t (16 B) are
-    # read only for flagged particles and written only where they change, so
-    # they are not counted (the cell of a particle comes from the brick's
-    # cell ranges, not from memory)
-    "k_p2g_brick": {"bytes": (82, 0, 108, 2000), "flops": (1470, 0, 0, 0)},
+    # staging phase: it reads x, v, F, the place, the code index and the D/u_t
+    # flag (64 B) and writes the pending label; D and u_t (16 B) are read only
+    # for flagged particles and written only where they change, so they are
+    # not counted.  Flop: momentum sums 252, force sums 513, stress 92, reach
+    # of the blade, floor, gravity and label band 87; per brick the reduction
+    # of 7 values (18 adds by 192 threads) and the tile sums
+    "k_p2g_brick": {"bytes": (65, 0, 108, 1900), "flops": (944, 0, 0, 27200)},
     "k_p2g_node": {"bytes": (0, 12, 140, 0), "flops": (0, 0, 40, 0)},
-    "k_g2p_musl": {"bytes": (68, 0, 162, 1080), "flops": (570, 0, 0, 0)},
+    # place, x, v in; x, v out.  Flop: gather 360, update 15, MUSL sums 198
+    "k_g2p_musl": {"bytes": (50, 0, 162, 1860), "flops": (573, 0, 0, 11700)},
     "k_musl_node": {"bytes": (0, 12, 86, 0), "flops": (0, 0, 20, 0)},
-    "k_fupd": {"bytes": (97, 0, 54, 1080), "flops": (650, 0, 0, 0)},
+    # place, pending label, F in; F out.  Per brick the sums along x of 36 node
+    # rows and 8 planes
+    "k_fupd": {"bytes": (75, 0, 54, 1860), "flops": (207, 0, 0, 10400)},
 }
+LATTICE_FORM = {"k_p2g_brick": "k_p2g_lat", "k_g2p_musl": "k_g2p_lat", "k_fupd": "k_fupd_lat"}
 # the substep's small kernels (bytes only; the tool step and the sums over a
 # scene run as extra CTAs of these and of k_musl_node or k_g2p_musl, some 56 B
 # per brick): the slot rebuild reads each node's dirty
@@ -289,7 +298,7 @@ def run_native(args):
         from paper_2609_27342_gb300.autotune import autotune
         probe = [pkg.Scene(s, stream=stream) for s in scenes]
         tb = make_batch(probe)
-        tuned = autotune(tb, stream)
+        tuned = autotune(tb, stream, occ_choices=(0,))  # the lattice kernels have one occupancy each
         tb.close()
         for o in probe:
             o.close()
@@ -355,7 +364,7 @@ def run_native(args):
     roof["alu_peak_measured_tflops"] = round(fma.value, 2)
     roof["alu_frac_of_measured"] = round(tfs / fma.value, 4) if fma.value > 0 else None
     traffic = ncu_traffic(dom, units)
-    roof.update({"kernel": dom, "traffic": traffic, "algorithmic_bytes": alg_bytes,
+    roof.update({"kernel": LATTICE_FORM.get(dom, dom), "traffic": traffic, "algorithmic_bytes": alg_bytes,
                  "algorithmic_flops": alg_flops, "avg_launch_ms": round(ktimes[dom], 4),
                  "hbm_frac": round(hbm_frac, 4), "alu_frac": round(alu_frac, 4),
                  "kernel_ms": {k: round(v, 4) for k, v in ktimes.items()}})

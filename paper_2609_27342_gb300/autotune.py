@@ -2,15 +2,19 @@
 
 The batched substep has launch parameters that do not change its results
 (every sum is taken in a fixed order, and the kernel variants share their
-arithmetic): the occupancy of each brick kernel (resident CTAs per SM of the
-per-brick P2G, G2P+MUSL and F-update kernels, i.e. registers per thread
+arithmetic): the occupancy of each general brick kernel (resident CTAs per SM
+of the per-brick P2G, G2P+MUSL and F-update kernels, i.e. registers per thread
 against latency hiding; one of three choices each, encoded in the brick
 variant as p2g + 3 g2p + 9 fupd), the node tile (threads per CTA of the
 per-node kernels) and the number of substeps captured in one CUDA graph.  The
 tuner times candidate shapes on the batch itself with CUDA events on the
 batch's stream and keeps the fastest: one brick kernel's occupancy at a time
 (the kernels run one after the other, so their choices are independent),
-then the node tile, then the graph chunk.
+then the node tile, then the graph chunk.  The lattice forms of the brick
+kernels and the forms for sets of few bricks have one occupancy each: in a
+batch that runs only these, the occupancy probes time equal kernels (pass
+``occ_choices=(0,)`` to leave them out), and the margin keeps the default
+unless their noise exceeds it.
 
 Every probe advances the simulation: tuning is a warm-up of the batch, not a
 side computation.
@@ -78,8 +82,9 @@ def autotune(batch, stream, key: Optional[tuple] = None, substeps: int = 16, rou
     ``baseline`` shape (graph chunk, node tile, variant) and ranked by its
     time relative to their mean; a candidate replaces the shape it would
     change only when it is faster by more than ``margin`` (see ``pick``).
-    ``stream`` is the torch stream the batch launches on.  With ``key`` the result is cached for this process and a
-    later call with the same key only applies it."""
+    ``stream`` is the torch stream the batch launches on.  With ``key`` the
+    result is cached for this process and a later call with the same key only
+    applies it."""
     if key is not None and key in _cache:
         b = _cache[key]["best"]
         batch.set_tiles(b["graph_chunk"], b["node_tile"], b["brick_variant"])

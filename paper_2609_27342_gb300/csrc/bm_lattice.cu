@@ -20,7 +20,7 @@
 //   * the F update forms the sums along x once per (node row, x plane) and
 //     not once per particle.
 // The kernels are bound by instructions and shared-memory reads, not by DRAM
-// (about 70 B per particle each).  Two other forms were measured and left:
+// (78, 47 and 57 B per particle).  Two other forms were measured and left:
 // one axis at a time for the whole brick (7 multiply-adds per particle and
 // value; P2G 0.39 ms) rounds differently, and an x-row of cells per thread
 // (no shuffles, but 9 reads per particle; P2G 0.97 ms) is slower.
